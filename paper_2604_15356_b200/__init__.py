@@ -34,7 +34,7 @@ def sources():
 def build(force=False, verbose=False):
     """Compile libplc.so for sm_100a with nvcc (in-tree)."""
     srcs = sources()
-    deps = srcs + [os.path.join(_CSRC, "plc_common.cuh"), os.path.join(_INC, "plc.h")]
+    deps = srcs + [os.path.join(_CSRC, h) for h in ("plc_common.cuh", "plc_coder.cuh")] + [os.path.join(_INC, "plc.h")]
     if not force and os.path.exists(_SO) and all(os.path.getmtime(_SO) >= os.path.getmtime(d) for d in deps):
         return _SO
     cmd = ["nvcc", "-t", "0", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -1,12 +1,43 @@
 // C ABI of libplc (see include/plc.h): argument checks, context scratch, kernel launches.
 #include <atomic>
+#include <cstring>
 #include <new>
 #include <vector>
 
-#include "plc_common.cuh"
+#include "plc_coder.cuh"
 #include <cmath>
 
 namespace plc {
+bool build_coder_tables(CoderTables* t) {
+    memset(t, 0, sizeof(*t));
+    for (int id = 0; id < kNumTables; ++id) {
+        uint32_t f[kNumSym], c[kNumSym + 1] = {0};
+        build_freqs(id + kQMin, f);
+        for (int i = 0; i < kNumSym; ++i) {
+            const int hi = (i & 1) ? (i + 1) / 2 : -(i / 2);
+            EncEntry& e = t->enc.enc[id][i == kEsc ? kEsc : hi + kHiMax];
+            e.rcp = f[i] == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / f[i]);
+            e.fc = f[i] | (c[i] << 16);
+            t->dec.fc[id][i] = e.fc;
+            c[i + 1] = c[i] + f[i];
+        }
+        t->dec.fc[id][kNumSym] = c[kNumSym] << 16;
+        uint8_t* first = t->dec.first[id];
+        memset(first, 0xff, sizeof(t->dec.first[id]));
+        int z = 0;
+        for (uint32_t slot = 0; slot < kProbM; ++slot) {               // r = 2^15 - slot falls: an interval's first slot comes first
+            while (c[z + 1] <= slot) ++z;
+            const uint32_t r = kProbM - slot;
+            int e = 0;
+            while ((r >> e) > 1) ++e;
+            const int at = e * 16 + (int)(((r << 4) >> e) - 16);
+            if (first[at] == 0xff) first[at] = (uint8_t)z;
+            if (z > first[at] + 1) return false;
+        }
+    }
+    return true;
+}
+
 static std::atomic<unsigned long long> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
 }  // namespace plc
@@ -31,6 +62,7 @@ struct plc_ctx {
     cudaEvent_t side_ev[2];         // fork / join of the side stream
     unsigned int* side_ticket;      // work counter of the side stream's launches
     Counters* counters;
+    CoderTables* tables;            // the coder's frequency tables
     uint8_t* dense_scratch;         // dense variant: P, Tb, n2b, mu, s1; linear variant: P, Ebar, s1, A_layer, mu
     size_t dense_bytes;
     const __half* lin_E;            // linear variant (Sec. 7.1): caller's E [V][dm], A [L][2H*d][dm], c [L][2H*d]
@@ -68,6 +100,13 @@ cudaEvent_t* prof_pair(plc_ctx* c, int which) {
 }  // namespace
 
 namespace {
+
+// The coder's tables, built once per process.
+const CoderTables* host_tables() {
+    static CoderTables t;
+    static const bool ok = build_coder_tables(&t);
+    return ok ? &t : nullptr;
+}
 
 plc_status status_code(unsigned int w) {
     if (w & kStTimeout) return PLC_E_CUDA;
@@ -140,6 +179,7 @@ CodecArgs base_args(const plc_ctx* c) {
     a.sh.zero_q = c->cfg.zero_rate_D > 0.0f
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
+    a.tables = c->tables;
     a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs;
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
@@ -239,7 +279,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
     c->staging_words_per_warp = 4ull * cfg->chunk_pos * cfg->head_dim + 64;
     const int warps = codec_grid_warps(0);
     bool ok = (!T_dev || cudaMalloc(&c->rownorm2, sizeof(float) * (size_t)rows) == cudaSuccess) &&
-              cudaMalloc(&c->staging, sizeof(uint16_t) * c->staging_words_per_warp * warps) == cudaSuccess &&
+              cudaMalloc(&c->staging, sizeof(uint16_t) * c->staging_words_per_warp * warps + 16) == cudaSuccess &&
               cudaMalloc(&c->ticket, sizeof(unsigned int) * kTicketWords) == cudaSuccess &&
               cudaMalloc(&c->status, sizeof(unsigned int)) == cudaSuccess &&
               cudaMallocHost(&c->status_host, sizeof(unsigned int)) == cudaSuccess &&
@@ -248,7 +288,10 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
               cudaEventCreateWithFlags(&c->side_ev[0], cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&c->side_ev[1], cudaEventDisableTiming) == cudaSuccess &&
               cudaMalloc(&c->side_ticket, sizeof(unsigned int)) == cudaSuccess &&
-              cudaMalloc(&c->counters, sizeof(Counters)) == cudaSuccess;
+              cudaMalloc(&c->counters, sizeof(Counters)) == cudaSuccess &&
+              cudaMalloc(&c->tables, sizeof(CoderTables)) == cudaSuccess;
+    const CoderTables* tables = host_tables();
+    if (ok) ok = tables && cudaMemcpy(c->tables, tables, sizeof(CoderTables), cudaMemcpyHostToDevice) == cudaSuccess;
     if (ok) ok = cudaMemset(c->status, 0, sizeof(unsigned int)) == cudaSuccess &&
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
     if (ok && T_dev) ok = launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, 0) == cudaSuccess &&
@@ -282,7 +325,7 @@ plc_status plc_destroy(plc_ctx* c) {
     if (c->poll_stream) cudaStreamDestroy(c->poll_stream);
     if (c->side_stream) cudaStreamDestroy(c->side_stream);
     for (int i = 0; i < 2; ++i) if (c->side_ev[i]) cudaEventDestroy(c->side_ev[i]);
-    cudaFree(c->side_ticket);
+    cudaFree(c->side_ticket); cudaFree(c->tables);
     delete c;
     return PLC_OK;
 }

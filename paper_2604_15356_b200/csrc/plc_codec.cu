@@ -15,7 +15,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "plc_common.cuh"
+#include "plc_coder.cuh"
 
 namespace plc {
 namespace {
@@ -40,42 +40,6 @@ struct Geo {
     static constexpr int G = D / 32;       // components a lane owns
     static constexpr int ROWS = 32 / R;    // rows fetched by one warp-wide load
 };
-
-// Encoder tables are indexed by hi + 31 (hi in [-31, 31]; entry 63 = escape): the symbol's place in
-// the alphabet (0, +1, -1, +2, ...) only matters for the cumulative counts, which are kept.
-struct EncTables { EncEntry enc[kNumTables][kNumSym]; };
-// Decoder tables: cum[] for the search, fc[] = f | (c << 16) for the state update.
-struct DecTables { uint16_t cum[kNumTables][kNumSym + 2]; uint32_t fc[kNumTables][kNumSym]; };
-
-__device__ inline void build_enc_tables(EncTables* t) {
-    for (int id = threadIdx.x; id < kNumTables; id += blockDim.x) {
-        uint32_t f[kNumSym];
-        build_freqs(id + kQMin, f);
-        uint32_t c = 0;
-        for (int i = 0; i < kNumSym; ++i) {
-            uint32_t fi = f[i];
-            const int hi = (i & 1) ? (i + 1) / 2 : -(i / 2);            // alphabet order 0, +1, -1, +2, ...
-            const int at = i == kEsc ? kEsc : hi + kHiMax;
-            t->enc[id][at].rcp = fi == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / fi);
-            t->enc[id][at].fc = fi | (c << 16);
-            c += fi;
-        }
-    }
-}
-__device__ inline void build_dec_tables(DecTables* t) {
-    for (int id = threadIdx.x; id < kNumTables; id += blockDim.x) {
-        uint32_t f[kNumSym];
-        build_freqs(id + kQMin, f);
-        uint32_t c = 0;
-        for (int i = 0; i < kNumSym; ++i) {
-            t->cum[id][i] = (uint16_t)c;
-            t->fc[id][i] = f[i] | (c << 16);
-            c += f[i];
-        }
-        t->cum[id][kNumSym] = (uint16_t)c;
-        t->cum[id][kNumSym + 1] = 0xffff;
-    }
-}
 
 // component owned by (lane, g): 8 (lane mod R) + G (lane div R) + g
 template <int D>
@@ -207,149 +171,6 @@ __device__ __forceinline__ void pairs_ready() {
 
 __device__ __forceinline__ int scale_class(float sigma2, float floor2, float inv_delta2) {
     return class_from_v((sigma2 + floor2) * inv_delta2);
-}
-
-// Per-lane constants of the coder steps.
-struct LaneCode {
-    uint32_t lt;         // lanes below this one
-    int sh;              // 16 * (lane & 1): which half of a bit-plane word lanes 0 / 1 store
-    int hs;              // lane >> 4: which half of a bit-plane word this lane's bit sits in
-    uint32_t bit;        // 1 << (lane & 15): this lane's bit in that half
-    int lane;
-};
-__device__ __forceinline__ LaneCode lane_code(int lane) {
-    LaneCode lc;
-    lc.lt = lanemask_lt(); lc.sh = 16 * (lane & 1); lc.hs = lane >> 4; lc.bit = 1u << (lane & 15); lc.lane = lane;
-    return lc;
-}
-
-// One encoder step for the warp: every lane codes `sym` with S raw bit planes (S is the same in
-// all lanes).  Words are written back to front at stage[wp-1], stage[wp-2], ...; returns the new
-// wp.  In decoder order a step is: 2S plane words, the refill words of the lanes that renormalise
-// (lanes ascending), the raw high parts of escaped lanes (lanes ascending, low half first).
-template <int SC>
-__device__ __forceinline__ int encode_step(int sym, int s_dyn, const EncEntry* tbl, uint32_t& x, uint16_t* __restrict__ stage,
-                                           int wp, const LaneCode& lc, unsigned& n_escapes) {
-    const int S = SC >= 0 ? SC : s_dyn;                            // SC < 0: plane count known at run time only
-    const int S2 = 2 * S;
-    const int u = sym + (S ? (1 << (S - 1)) : 0);                  // |sym| <= 2^30, S <= 15: no overflow
-    const int hi = u >> S;                                         // bits below S of u are the raw part
-    const uint32_t at = (uint32_t)(hi + kHiMax);
-    const bool esc = at > 2u * kHiMax;                             // |hi| > 31
-    const EncEntry e = tbl[min(at, (uint32_t)kEsc)];
-    const uint32_t f = e.fc & 0xffffu;
-    const bool emit = x >= (f << 17);
-    const uint32_t emask = __ballot_sync(kFull, emit);
-    int base = wp - S2 - __popc(emask);
-    if (__any_sync(kFull, esc)) {                  // rare: raw 32-bit hi of the escaped lanes
-        const uint32_t xmask = __ballot_sync(kFull, esc);
-        const int n_esc = __popc(xmask);
-        base -= 2 * n_esc;
-        if (esc) {
-            const int at = base + S2 + __popc(emask) + 2 * __popc(xmask & lc.lt);
-            stage[at] = (uint16_t)((uint32_t)hi & 0xffffu);
-            stage[at + 1] = (uint16_t)((uint32_t)hi >> 16);
-        }
-        n_escapes += n_esc;
-    }
-    uint16_t* out = stage + base;
-    if (emit) out[S2 + __popc(emask & lc.lt)] = (uint16_t)(x & 0xffffu);
-    const uint32_t xe = emit ? x >> 16 : x;
-    uint32_t q = __umulhi(xe, e.rcp);
-    uint32_t r = xe - q * f;
-    if (r >= f) { ++q; r -= f; }
-    x = (q << kProbBits) + r + (e.fc >> 16);
-    if (S > 0) {
-        uint16_t* mine = out + lc.lane;            // lanes 0 and 1 store the two halves of every plane
-#pragma unroll
-        for (int b = 0; b < S; ++b) {
-            const uint32_t plane = __ballot_sync(kFull, (u >> b) & 1);
-            if (lc.lane < 2) mine[2 * b] = (uint16_t)(plane >> lc.sh);
-        }
-    }
-    return base;
-}
-
-// All G components of one position, last component first, dispatched on the number of planes.
-template <int G>
-__device__ __forceinline__ int encode_position(const int (&sym)[G], int s, bool mixed, const EncEntry* tbl, uint32_t& x,
-                                               uint16_t* __restrict__ stage, int wp, const LaneCode& lc, unsigned& n_escapes) {
-#define PLC_ENC_CASE(S_, LABEL)                                                                            \
-    LABEL:                                                                                                 \
-        _Pragma("unroll") for (int g = G - 1; g >= 0; --g)                                                 \
-            wp = encode_step<S_>(sym[g], s, tbl, x, stage, wp, lc, n_escapes);                             \
-        break;
-    // The plane counts that occur in practice get code of their own.  With a per-position step
-    // (`mixed`) neighbouring positions differ in plane count, and jumping between a dozen
-    // specialised bodies costs more in instruction fetch than they save: those take the loop.
-    switch (mixed ? -1 : s) {
-        PLC_ENC_CASE(0, case 0) PLC_ENC_CASE(1, case 1) PLC_ENC_CASE(2, case 2) PLC_ENC_CASE(3, case 3)
-        PLC_ENC_CASE(4, case 4) PLC_ENC_CASE(5, case 5) PLC_ENC_CASE(6, case 6) PLC_ENC_CASE(7, case 7)
-        PLC_ENC_CASE(-1, default)
-    }
-#undef PLC_ENC_CASE
-    return wp;
-}
-
-// One decoder step for the warp; words[-1 .. nwords) are readable (words[-1] is the last half of
-// the chunk's state block).  A read past the end is redirected to the chunk's last word; rp still
-// advances, so the caller's final check rp == nwords reports it.
-template <int SC>
-__device__ __forceinline__ int decode_step(int s_dyn, const uint16_t* cum, const uint32_t* fcs, uint32_t& x,
-                                           const uint16_t* __restrict__ words, int& rp, int last, const LaneCode& lc) {
-    const int S = SC >= 0 ? SC : s_dyn;
-    uint32_t lo = 0;
-    if (S > 0) {
-        const int S2 = 2 * S;
-        uint32_t v = 0;
-        if (lc.lane < S2) v = __ldg(words + min(rp + lc.lane, last));
-#pragma unroll
-        for (int b = 0; b < S; ++b) {
-            const uint32_t hw = __shfl_sync(kFull, v, 2 * b + lc.hs);
-            if (hw & lc.bit) lo |= 1u << b;
-        }
-        rp += S2;
-    }
-    const uint32_t slot = x & (kProbM - 1u);
-    const uint16_t* cp = cum;
-#pragma unroll
-    for (int step = 32; step > 0; step >>= 1)
-        if (cp[step] <= slot) cp += step;
-    const int zz = (int)(cp - cum);
-    const uint32_t fc = fcs[zz];
-    x = (fc & 0xffffu) * (x >> kProbBits) + slot - (fc >> 16);
-    const bool need = x < kRansL;
-    const uint32_t nmask = __ballot_sync(kFull, need);
-    if (need) x = (x << 16) | __ldg(words + min(rp + __popc(nmask & lc.lt), last));
-    rp += __popc(nmask);
-    const int t = (zz + 1) >> 1;
-    int hi = (zz & 1) ? t : -t;
-    if (__any_sync(kFull, zz == kEsc)) {
-        const bool esc = zz == kEsc;
-        const uint32_t xmask = __ballot_sync(kFull, esc);
-        if (esc) {
-            const int at = rp + 2 * __popc(xmask & lc.lt);
-            hi = (int)((uint32_t)__ldg(words + min(at, last)) | ((uint32_t)__ldg(words + min(at + 1, last)) << 16));
-        }
-        rp += 2 * __popc(xmask);
-    }
-    return S ? (int)(((uint32_t)hi << S) + lo - (1u << (S - 1))) : hi;
-}
-
-template <int G>
-__device__ __forceinline__ void decode_position(int (&sym)[G], int s, bool mixed, const uint16_t* cum, const uint32_t* fcs, uint32_t& x,
-                                                const uint16_t* __restrict__ words, int& rp, int last, const LaneCode& lc) {
-#define PLC_DEC_CASE(S_, LABEL)                                                                            \
-    LABEL:                                                                                                 \
-        _Pragma("unroll") for (int g = 0; g < G; ++g)                                                      \
-            sym[g] = decode_step<S_>(s, cum, fcs, x, words, rp, last, lc);                                 \
-        break;
-    switch (mixed ? -1 : s) {
-        PLC_DEC_CASE(0, case 0) PLC_DEC_CASE(1, case 1) PLC_DEC_CASE(2, case 2) PLC_DEC_CASE(3, case 3)
-        PLC_DEC_CASE(4, case 4) PLC_DEC_CASE(5, case 5) PLC_DEC_CASE(6, case 6) PLC_DEC_CASE(7, case 7)
-        PLC_DEC_CASE(-1, default)
-    }
-#undef PLC_DEC_CASE
 }
 
 // Lane 0's value for the whole warp, through a warp reduction: the result is provably the same in
@@ -501,6 +322,25 @@ __device__ __forceinline__ long long kv_elem(const KvView& v, int t, int H, int 
     return layer * v.sl + kv * v.skv + s * v.ss + head * v.sh + (long long)pos * v.sp;
 }
 
+// Copies n 16-bit words to a 16-byte aligned destination from a 2-byte aligned source, 16 bytes a lane
+// and step (`lane` of `lanes` threads; two-byte copies cost the tail of a chunk as much as a quarter of
+// its coding).  The source is read in aligned 32-bit words, up to two bytes before and behind the
+// range: the staging areas have that room.
+__device__ __forceinline__ void copy_words(uint8_t* dst, const uint16_t* src, int n, int lane, int lanes) {
+    const uint32_t* s4 = reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(src) & ~(uintptr_t)3);
+    const uint32_t sh = (reinterpret_cast<uintptr_t>(src) & 2) ? 16u : 0u;
+    const int n16 = n >> 3;                                   // whole 16-byte pieces
+#pragma unroll 2
+    for (int i = lane; i < n16; i += lanes) {
+        uint32_t w[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) w[j] = __ldcg(s4 + 4 * i + j);
+        reinterpret_cast<uint4*>(dst)[i] = make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                                                      __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+    }
+    for (int i = 8 * n16 + lane; i < n; i += lanes) reinterpret_cast<uint16_t*>(dst)[i] = __ldcg(src + i);
+}
+
 // Finishes an encoded chunk: reserves its place, writes states and words, index and counters.
 __device__ __forceinline__ void commit_chunk(const CodecArgs& a, long long slot, uint32_t x, const uint16_t* stage,
                                              int wp, int cap_words, int lane, int P, unsigned n_escapes, int n_skipped = 0) {
@@ -528,8 +368,7 @@ __device__ __forceinline__ void commit_chunk(const CodecArgs& a, long long slot,
     if (!fits || !aligned) return;
     uint8_t* dst = a.st.payload + off;
     reinterpret_cast<uint32_t*>(dst)[lane] = x;
-    uint16_t* dw = reinterpret_cast<uint16_t*>(dst + 128);
-    for (int i = lane; i < n_words; i += 32) dw[i] = __ldcg(stage + wp + i);
+    copy_words(dst + 128, stage + wp, n_words, lane, 32);
 }
 
 // Quantiser decision in binary32: sym = rint((kv - mu) * fl(1/delta)), clamped to +-2^30.
@@ -577,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const Co
     constexpr bool FROM_OPEN = SRC == kSrcOpen;
     constexpr bool DENSE = SRC == kSrcDense;
     __shared__ EncTables tb;
-    build_enc_tables(&tb);
+    load_tables(&tb, &a.tables->enc);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -702,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const Co
                     ideal += (float)(kProbBits + s) - log2f((float)f) + (at > 2u * kHiMax ? 32.f : 0.f);
                 }
             }
-            wp = encode_position<G>(sym, s, FLEX && a.step_exp != nullptr, tb.enc[qp - kQMin], x, stage, wp, lc, n_escapes);
+            wp = encode_position<G>(sym, s, tb.enc[qp - kQMin], x, stage, wp, lc, n_escapes);
         }
         if (FLEX && a.dbg.ideal) {
             ideal = warp_sum(ideal);
@@ -717,7 +556,7 @@ template <int D, bool DENSE, bool ZR, bool FLEX>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     __shared__ DecTables tb;
-    build_dec_tables(&tb);
+    load_tables(&tb, &a.tables->dec);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -747,6 +586,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const Co
         const uint16_t* words = reinterpret_cast<const uint16_t*>(src + 128);
         const int nwords = (int)((nbytes - 128u) >> 1);
         const int last = nwords - 1;                 // -1 for a chunk of states only: words[-1] is inside the chunk
+        auto read_word = [&](int i) { return (uint32_t)__ldg(words + min(i, last)); };   // past the end: the last word
         int rp = 0;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D + 8 * (lane % Geo<D>::R));
         const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
@@ -797,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const Co
             } else {
                 int s, qp;
                 class_params(q, s, qp);
-                decode_position<G>(sym, s, FLEX && a.step_exp != nullptr, tb.cum[qp - kQMin], tb.fc[qp - kQMin], x, words, rp, last, lc);
+                decode_position<G>(sym, s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, read_word, rp, lc);
 #pragma unroll
                 for (int g = 0; g < G; ++g) out[g] = __fmaf_rn((float)sym[g], delta_p, mu[g]);
             }

@@ -35,12 +35,6 @@ struct EncEntry {
     uint32_t rcp, fc;
 };
 
-// Per-class tables as they sit in shared memory.
-struct __align__(16) Tables {
-    EncEntry enc[kNumTables][kNumSym];      // 20 KB
-    uint16_t cum[kNumTables][kNumSym + 2];  // c[0..64], padded: 5280 B
-};
-
 // Two 32-bit constants per table id: theta = round(2^32 exp(-sqrt2/s')), rho = round(2^32
 // exp(-sqrt2/(2 s'))), s' = 2^(qp/8).  Literal so that encoder and decoder builds agree bit for bit.
 __host__ __device__ inline void table_constants(int qp, uint32_t& theta, uint32_t& rho) {
@@ -124,23 +118,6 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Fills the shared-memory tables; call with all threads of the block, then __syncthreads().
-__device__ inline void build_tables_smem(Tables* t) {
-    for (int id = threadIdx.x; id < kNumTables; id += blockDim.x) {
-        uint32_t f[kNumSym];
-        build_freqs(id + kQMin, f);
-        uint32_t c = 0;
-        for (int i = 0; i < kNumSym; ++i) {
-            uint32_t fi = f[i];
-            t->enc[id][i].rcp = fi == 1 ? 0xffffffffu : (uint32_t)((1ull << 32) / fi);
-            t->enc[id][i].fc = fi | (c << 16);
-            t->cum[id][i] = (uint16_t)c;
-            c += fi;
-        }
-        t->cum[id][kNumSym] = (uint16_t)c;       // 2^15 wraps to 0x8000: fits uint16
-        t->cum[id][kNumSym + 1] = 0xffff;
-    }
-}
 #endif
 
 // Host-side launch counter shared by all translation units.
@@ -197,8 +174,11 @@ struct DebugDev {
     int ideal;             // non-zero: add every coded component's model code length to Counters::ideal_bits
 };
 
+struct CoderTables;                                // plc_coder.cuh
+
 struct CodecArgs {
     CodecShape sh;
+    const CoderTables* tables;                     // frequency tables of the coder
     const __half* T; const float* rownorm2;        // [tables][V][d], [tables][V]
     const int2* pairs;                             // [S*n][Kp]
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
