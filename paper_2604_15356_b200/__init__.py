@@ -12,7 +12,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 _SO = os.path.join(_HERE, "libplc.so")
-_SOURCES = ["plc_api.cu", "plc_topk.cu", "plc_prefix.cu", "plc_codec.cu", "plc_dense.cu", "plc_static.cu", "plc_trie.cu"]
+_SOURCES = ["plc_api.cu", "plc_topk.cu", "plc_prefix.cu", "plc_codec.cu", "plc_coop.cu", "plc_dense.cu", "plc_static.cu", "plc_trie.cu"]
 
 OK, E_INVALID, E_SHAPE, E_ALIGN, E_CAPACITY, E_CORRUPT, E_STATE, E_CUDA = range(8)
 PRED_TOPK, PRED_DENSE, PRED_LINEAR = 0, 1, 2
@@ -34,7 +34,7 @@ def sources():
 def build(force=False, verbose=False):
     """Compile libplc.so for sm_100a with nvcc (in-tree)."""
     srcs = sources()
-    deps = srcs + [os.path.join(_CSRC, h) for h in ("plc_common.cuh", "plc_coder.cuh")] + [os.path.join(_INC, "plc.h")]
+    deps = srcs + [os.path.join(_CSRC, h) for h in ("plc_common.cuh", "plc_coder.cuh", "plc_codec.cuh")] + [os.path.join(_INC, "plc.h")]
     if not force and os.path.exists(_SO) and all(os.path.getmtime(_SO) >= os.path.getmtime(d) for d in deps):
         return _SO
     cmd = ["nvcc", "-t", "0", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -401,7 +401,7 @@ static plc_status run_dense(plc_ctx* c, CodecArgs a, const void* logits_dev, boo
         cudaEvent_t* pg = prof_pair(c, 2);
         if (dense_layer(c->T + l * layer_elems, sh, c->dense_scratch, off, c->status, st, pg ? pg[0] : nullptr,
                         pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
-        a.dense_layer = l;
+        a.dense_t0 = l * sh.tables; a.dense_nt = sh.tables;
         a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[4]) + (size_t)l * sh.tables;
         cudaEvent_t* pk = prof_pair(c, encode ? 0 : 1);
         if (pk) cudaEventRecord(pk[0], st);
@@ -425,7 +425,7 @@ static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bo
         cudaEvent_t* pg = prof_pair(c, 2);
         if (linear_layer(c->lin_A + (size_t)l * sh.ncols * sh.dm, sh, c->dense_scratch, off, c->status, st,
                          pg ? pg[0] : nullptr, pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
-        a.dense_layer = l;
+        a.dense_t0 = l * sh.tables; a.dense_nt = sh.tables;
         a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[3]) + (size_t)l * sh.tables;
         a.mu_bias = c->lin_c + (size_t)l * sh.ncols;
         cudaEvent_t* pk = prof_pair(c, encode ? 0 : 1);

@@ -14,6 +14,8 @@
 //     that holds the smallest symbol of that interval, and no interval of any of the 40 tables holds
 //     more than one symbol boundary (checked on the host for every slot when the tables are built).
 #pragma once
+#include <type_traits>
+
 #include "plc_common.cuh"
 
 namespace plc {
@@ -91,24 +93,90 @@ __device__ __forceinline__ uint32_t push_state(uint32_t x, bool emit, EncEntry e
     return r >= f ? y + mf : y;
 }
 
+// The planes of a position travel in groups of GP steps whose planes fit one transpose (GP * S <= 32);
+// plane_group<G>(S) is that GP, kPlaneWords<G> the most groups a position has (S <= 15).
+template <int G>
+constexpr int kPlaneWords = G <= 2 ? 1 : G / 2;
+template <int G, class F>
+__device__ __forceinline__ void by_plane_group(int S, F&& f) {             // calls f(integral_constant<GP>)
+    if (G <= 2 || G * S <= 32) f(std::integral_constant<int, G>{});
+    else if (G == 4 || G * S <= 64) f(std::integral_constant<int, (G >= 2 ? G / 2 : 1)>{});
+    else f(std::integral_constant<int, (G >= 4 ? G / 4 : 1)>{});
+}
+
+// What a position's symbols put into the stream, before the state is known: table entries and, per
+// group, lane j's plane.
+template <int G>
+struct Prepared {
+    EncEntry e[G];
+    uint32_t plane[kPlaneWords<G>];
+};
+template <int G>
+__device__ __forceinline__ void prepare_position(const int (&u)[G], const uint32_t (&at)[G], int S, const EncEntry* tbl, const LaneCode& lc,
+                                                 Prepared<G>& pr) {
+#pragma unroll
+    for (int g = 0; g < G; ++g) pr.e[g] = tbl[at[g]];
+#pragma unroll
+    for (int i = 0; i < kPlaneWords<G>; ++i) pr.plane[i] = 0;
+    if (S > 0) {
+        const uint32_t mask = (1u << S) - 1u;
+        by_plane_group<G>(S, [&](auto gp) {
+            constexpr int GP = decltype(gp)::value;
+#pragma unroll
+            for (int i = 0; i < G / GP; ++i) {
+                uint32_t packed = 0;
+#pragma unroll
+                for (int k = 0; k < GP; ++k) packed |= ((uint32_t)u[i * GP + k] & mask) << (k * S);
+                pr.plane[i] = transpose32(packed, lc);
+            }
+        });
+    }
+}
+
+// Splits symbols (S planes a component) into u = sym + 2^(S-1) and table places; true if none escapes.
+template <int G>
+__device__ __forceinline__ bool split_symbols(const int (&sym)[G], int S, int (&u)[G], uint32_t (&at)[G]) {
+    const int half = (1 << S) >> 1;                        // |sym| <= 2^30, S <= 15: no overflow
+    uint32_t worst = 0;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        u[g] = sym[g] + half;
+        at[g] = (uint32_t)((u[g] >> S) + kHiMax);
+        worst = max(worst, at[g]);
+    }
+    return !__any_sync(kFull, worst > 2u * kHiMax);
+}
+
 // Words of the stream are written back to front: stage[wp - 1], stage[wp - 2], ...  In decoder order a
 // step is: 2S plane words, the refill words of the lanes that renormalise (lanes ascending), the raw
-// high parts of escaped lanes (lanes ascending, low half first).
-template <int GP>
-__device__ __forceinline__ void put_planes(const uint32_t* lo, const int* base, int S, uint16_t* __restrict__ stage, const LaneCode& lc) {
-    uint32_t packed = 0;
+// high parts of escaped lanes (lanes ascending, low half first).  Last component first; returns the
+// new wp.
+template <int G>
+__device__ __forceinline__ int push_position(const Prepared<G>& pr, int S, uint32_t& x, uint16_t* __restrict__ stage, int wp, const LaneCode& lc) {
+    int base[G];
 #pragma unroll
-    for (int i = 0; i < GP; ++i) packed |= lo[i] << (i * S);
-    const uint32_t plane = transpose32(packed, lc);
-    // lane j = i * S + b: plane b of step i, at halfword base[i] + 2 b = (base[i] - 2 i S) + 2 j
-    int off[GP];
-#pragma unroll
-    for (int i = 0; i < GP; ++i) off[i] = base[i] - 2 * i * S;
-    if (lc.lane < GP * S) {
-        uint16_t* p = stage + (of_my_step<GP>(off, lc.lane, S) + 2 * lc.lane);
-        p[0] = (uint16_t)plane;
-        p[1] = (uint16_t)(plane >> 16);
+    for (int g = G - 1; g >= 0; --g) {
+        const bool emit = x >= (pr.e[g].fc << 17);         // f << 17: the count above f is shifted out
+        const uint32_t emask = __ballot_sync(kFull, emit);
+        wp -= __popc(emask);
+        if (emit) stage[wp + __popc(emask & lc.lt)] = (uint16_t)x;
+        x = push_state(x, emit, pr.e[g]);
+        wp -= 2 * S;
+        base[g] = wp - 2 * S * g;                          // lane j = g S + b of a group: halfword base + 2 j
     }
+    if (S > 0)
+        by_plane_group<G>(S, [&](auto gp) {
+            constexpr int GP = decltype(gp)::value;
+#pragma unroll
+            for (int i = 0; i < G / GP; ++i) {
+                if (lc.lane < GP * S) {
+                    uint16_t* p = stage + (of_my_step<GP>(base + i * GP, lc.lane, S) + 2 * (i * GP * S + lc.lane));
+                    p[0] = (uint16_t)pr.plane[i];
+                    p[1] = (uint16_t)(pr.plane[i] >> 16);
+                }
+            }
+        });
+    return wp;
 }
 
 // Positions with an escaped component, one step at a time.
@@ -145,54 +213,16 @@ __device__ __forceinline__ int encode_position_escapes(const int (&u)[G], int S,
     return wp;
 }
 
-// All G components of one position, last component first; S bit planes a component (the same in all
-// lanes).  Returns the new wp.
+// All G components of one position; S bit planes a component (the same in all lanes).
 template <int G>
 __device__ __forceinline__ int encode_position(const int (&sym)[G], int S, const EncEntry* tbl, uint32_t& x,
                                                uint16_t* __restrict__ stage, int wp, const LaneCode& lc, unsigned& n_escapes) {
-    const int half = (1 << S) >> 1;                        // |sym| <= 2^30, S <= 15: no overflow
     int u[G];
-    uint32_t at[G], worst = 0;
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        u[g] = sym[g] + half;
-        at[g] = (uint32_t)((u[g] >> S) + kHiMax);
-        worst = max(worst, at[g]);
-    }
-    if (__any_sync(kFull, worst > 2u * kHiMax)) return encode_position_escapes<G>(u, S, tbl, x, stage, wp, lc.lane, n_escapes);
-    EncEntry e[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) e[g] = tbl[at[g]];
-    int base[G];
-#pragma unroll
-    for (int g = G - 1; g >= 0; --g) {
-        const bool emit = x >= (e[g].fc << 17);            // f << 17: the count above f is shifted out
-        const uint32_t emask = __ballot_sync(kFull, emit);
-        wp -= __popc(emask);
-        if (emit) stage[wp + __popc(emask & lc.lt)] = (uint16_t)x;
-        x = push_state(x, emit, e[g]);
-        wp -= 2 * S;
-        base[g] = wp;
-    }
-    if (S > 0) {
-        const uint32_t mask = (1u << S) - 1u;
-        uint32_t lo[G];
-#pragma unroll
-        for (int g = 0; g < G; ++g) lo[g] = (uint32_t)u[g] & mask;
-        if (G * S <= 32) put_planes<G>(lo, base, S, stage, lc);
-        else if (G * S <= 64) {
-            if constexpr (G >= 2) {
-#pragma unroll
-                for (int g = 0; g < G; g += G / 2) put_planes<G / 2>(lo + g, base + g, S, stage, lc);
-            }
-        } else {
-            if constexpr (G >= 4) {
-#pragma unroll
-                for (int g = 0; g < G; g += G / 4) put_planes<G / 4>(lo + g, base + g, S, stage, lc);
-            }
-        }
-    }
-    return wp;
+    uint32_t at[G];
+    if (!split_symbols<G>(sym, S, u, at)) return encode_position_escapes<G>(u, S, tbl, x, stage, wp, lc.lane, n_escapes);
+    Prepared<G> pr;
+    prepare_position<G>(u, at, S, tbl, lc, pr);
+    return push_position<G>(pr, S, x, stage, wp, lc);
 }
 
 // Symbol of a slot: its fc entry and its place in the alphabet.
@@ -208,19 +238,6 @@ __device__ __forceinline__ uint32_t find_symbol(uint32_t x, const uint8_t* first
 __device__ __forceinline__ int hi_of(int zz) {                            // 0, +1, -1, +2, ...
     const int t = (zz + 1) >> 1;
     return (zz & 1) ? t : -t;
-}
-
-template <int GP, class Words>
-__device__ __forceinline__ uint32_t get_planes(const int* base, int S, const Words& words, const LaneCode& lc) {
-    int off[GP];
-#pragma unroll
-    for (int i = 0; i < GP; ++i) off[i] = base[i] - 2 * i * S;
-    uint32_t plane = 0;
-    if (lc.lane < GP * S) {
-        const int p = of_my_step<GP>(off, lc.lane, S) + 2 * lc.lane;
-        plane = words(p) | (words(p + 1) << 16);
-    }
-    return transpose32(plane, lc);
 }
 
 // Positions with an escaped component, one step at a time.
@@ -258,14 +275,15 @@ __device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, co
     }
 }
 
-// All G components of one position.  words(i) reads 16-bit word i of the chunk (any i: the reader keeps
-// the access in bounds; rp advances regardless, so the caller's final check of rp reports a short chunk).
+// The serial part of decoding a position: advances x and rp, gives every step's place in the word
+// stream and high part; false if a component escaped (x and rp are then as before the call).
+// words(i) reads 16-bit word i of the chunk (any i: the reader keeps the access in bounds; rp advances
+// regardless, so the caller's final check of rp reports a short chunk).
 template <int G, class Words>
-__device__ __forceinline__ void decode_position(int (&sym)[G], int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x,
-                                                const Words& words, int& rp, const LaneCode& lc) {
+__device__ __forceinline__ bool pull_position(int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x, const Words& words, int& rp,
+                                              const LaneCode& lc, int (&base)[G], int (&hi)[G]) {
     const uint32_t x0 = x;
     const int rp0 = rp;
-    int base[G], hi[G];
     bool esc = false;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -281,41 +299,46 @@ __device__ __forceinline__ void decode_position(int (&sym)[G], int S, const uint
         esc = esc || zz == kEsc;
         hi[g] = hi_of(zz);
     }
-    if (__any_sync(kFull, esc)) {                          // the words after the first escape were read wrongly: start over
-        x = x0; rp = rp0;
-        decode_position_escapes<G, Words>(sym, S, first, fcs, x, words, rp, lc.lane);
-        return;
-    }
+    if (!__any_sync(kFull, esc)) return true;
+    x = x0; rp = rp0;                                      // the words after the first escape were read wrongly
+    return false;
+}
+
+// The rest: a position's planes from the word stream, and its symbols.
+template <int G, class Words>
+__device__ __forceinline__ void join_position(const int (&base)[G], const int (&hi)[G], int S, const Words& words, const LaneCode& lc, int (&sym)[G]) {
     if (S == 0) {
 #pragma unroll
         for (int g = 0; g < G; ++g) sym[g] = hi[g];
         return;
     }
     const uint32_t mask = (1u << S) - 1u, half = (1u << S) >> 1;
-    auto join = [&](int g, uint32_t lo) { sym[g] = (int)(((uint32_t)hi[g] << S) + (lo & mask) - half); };
-    if (G * S <= 32) {
-        const uint32_t v = get_planes<G>(base, S, words, lc);
+    by_plane_group<G>(S, [&](auto gp) {
+        constexpr int GP = decltype(gp)::value;
 #pragma unroll
-        for (int g = 0; g < G; ++g) join(g, v >> (g * S));
-    } else if (G * S <= 64) {
-        if constexpr (G >= 2) {
+        for (int i = 0; i < G / GP; ++i) {
+            int off[GP];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t v = get_planes<G / 2>(base + h * (G / 2), S, words, lc);
-#pragma unroll
-                for (int g = 0; g < G / 2; ++g) join(h * (G / 2) + g, v >> (g * S));
+            for (int k = 0; k < GP; ++k) off[k] = base[i * GP + k] - 2 * k * S;
+            uint32_t plane = 0;
+            if (lc.lane < GP * S) {
+                const int p = of_my_step<GP>(off, lc.lane, S) + 2 * lc.lane;
+                plane = words(p) | (words(p + 1) << 16);
             }
-        }
-    } else {
-        if constexpr (G >= 4) {
+            const uint32_t v = transpose32(plane, lc);
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                const uint32_t v = get_planes<G / 4>(base + h * (G / 4), S, words, lc);
-#pragma unroll
-                for (int g = 0; g < G / 4; ++g) join(h * (G / 4) + g, v >> (g * S));
-            }
+            for (int k = 0; k < GP; ++k) sym[i * GP + k] = (int)(((uint32_t)hi[i * GP + k] << S) + ((v >> (k * S)) & mask) - half);
         }
-    }
+    });
+}
+
+// All G components of one position.
+template <int G, class Words>
+__device__ __forceinline__ void decode_position(int (&sym)[G], int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x,
+                                                const Words& words, int& rp, const LaneCode& lc) {
+    int base[G], hi[G];
+    if (pull_position<G>(S, first, fcs, x, words, rp, lc, base, hi)) join_position<G>(base, hi, S, words, lc, sym);
+    else decode_position_escapes<G>(sym, S, first, fcs, x, words, rp, lc.lane);
 }
 
 #endif  // __CUDACC__

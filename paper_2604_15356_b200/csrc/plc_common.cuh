@@ -189,9 +189,9 @@ struct CodecArgs {
     unsigned int* ticket;                          // kTicketWords work counters (zeroed by the launcher)
     int sched_nq, sched_g;                         // gather kernels: work queues, SMs that share one (set by the launcher)
     unsigned int* status; Counters* counters;
-    // dense variant: prediction read from buffers; one launch covers the 2*H tables of dense_layer
-    const float* mu_dense; const float* s1_dense; long long mu_ld, s1_ld; int dense_layer;
-    const __half* mu_bias;                         // optional [2*H][d] f16 added to mu (linear predictor's c), or null
+    // dense variant: prediction read from buffers; one launch covers tables [dense_t0, dense_t0 + dense_nt)
+    const float* mu_dense; const float* s1_dense; long long mu_ld, s1_ld; int dense_t0, dense_nt;
+    const __half* mu_bias;                         // optional [dense_nt][d] f16 added to mu (linear predictor's c), or null
     // append path: symbols come from / go to the open chunk
     int32_t* open_sym; int32_t* open_q; int open_slot; int open_count; int chunk_index;
     unsigned open_first, open_items;               // seal launch: the (table, session) items [open_first, open_first + open_items)
@@ -246,6 +246,7 @@ cudaError_t dense_layer(const __half* T_layer, const DenseShape& sh, uint8_t* sc
 cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, cudaStream_t st);
 cudaError_t launch_encode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_decode(const CodecArgs& a, cudaStream_t st);
+cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st);   // a block per chunk; queues set, tickets zeroed
 cudaError_t launch_append_quantise(const CodecArgs& a, cudaStream_t st);   // predict + quantise into the open chunk
 cudaError_t launch_append_seal(const CodecArgs& a, cudaStream_t st);       // code the open chunk
 

@@ -1,0 +1,439 @@
+// Predict / quantise / rANS with a whole block per (stream, chunk), for calls with few chunks.
+//
+// The kernels of plc_codec.cu give every chunk to one warp, which predicts a position and codes it
+// before it turns to the next: right while there are enough chunks to fill the GPU, but a call with
+// fewer chunks than resident warps then runs at the latency of one warp's chain (row gathers, the KV
+// load, the coder), about 1.8 us a position however little work there is.  Only the coder is serial
+// in a chunk, and of the coder only the state and the word cursor; the rest is independent from
+// position to position.  Here warp 0 of a block carries the chunk's state and the other warps do
+// everything else, one position each and batch, two batches deep in shared memory with one barrier a
+// batch: encoding, they predict, quantise, look the table entries up and transpose the bit planes, so
+// that the coder's chain per step is one state update; decoding, they predict (the coder needs the
+// class) and, a batch later, fetch the planes whose places the coder has found and write the vectors.
+// The decoder's words come through a ring in shared memory filled by asynchronous copies, so no
+// refill waits for global memory.
+#include <algorithm>
+
+#include "plc_codec.cuh"
+
+namespace plc {
+namespace {
+
+constexpr int kCoopMaxWarps = 16;
+constexpr int kRingBytes = 8192, kRingBlock = 512;       // word ring of a decoding coder; bytes one warp-wide copy brings
+constexpr int kSkipped = -1000000;                       // class mark of a zero-rate position
+
+struct SlotMeta { int q, e, escaped, pad; };             // class (or kSkipped), step exponent, whether a component escapes
+
+// The words of a chunk, read through the ring.  `ready` bytes have landed, `fetched` are on their way.
+struct RingWords {
+    const uint16_t* ring;
+    __device__ __forceinline__ uint32_t operator()(int i) const { return ring[i & (kRingBytes / 2 - 1)]; }
+};
+__device__ __forceinline__ void ring_fetch(uint16_t* ring, const uint8_t* src, int total, int rp, int& fetched, int lane) {
+    while (fetched < total && fetched + kRingBlock <= 2 * rp + kRingBytes) {
+        const int at = fetched + 16 * lane;
+        if (at < total) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(ring) + (at & (kRingBytes - 1)));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src + at), "r"(min(16, total - at)) : "memory");
+        }
+        fetched += kRingBlock;
+    }
+}
+
+// A position's slot, 16 (or 8) bytes a lane at a time.  Encoding: the table entries and planes of a
+// Prepared position (u itself where a component escapes); decoding: the steps' high parts (the symbols
+// themselves where one escapes) and, behind them, the steps' places in the word stream.
+template <int G>
+constexpr int kEncSlotWords = 32 * (2 * G + kPlaneWords<G>);
+template <int G>
+constexpr int kDecSlotWords = 32 * G + 8;
+template <int G>
+__device__ __forceinline__ void slot_put_ints(int* slot, int lane, const int (&v)[G]) {
+    if constexpr (G >= 4) {
+#pragma unroll
+        for (int i = 0; i < G / 4; ++i) reinterpret_cast<int4*>(slot)[i * 32 + lane] = make_int4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < G; ++i) slot[i * 32 + lane] = v[i];
+    }
+}
+template <int G>
+__device__ __forceinline__ void slot_get_ints(const int* slot, int lane, int (&v)[G]) {
+    if constexpr (G >= 4) {
+#pragma unroll
+        for (int i = 0; i < G / 4; ++i) {
+            const int4 w = reinterpret_cast<const int4*>(slot)[i * 32 + lane];
+            v[4 * i] = w.x; v[4 * i + 1] = w.y; v[4 * i + 2] = w.z; v[4 * i + 3] = w.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < G; ++i) v[i] = slot[i * 32 + lane];
+    }
+}
+template <int G>
+__device__ __forceinline__ void slot_put(int* slot, int lane, const Prepared<G>& pr) {
+    if constexpr (G >= 2) {
+#pragma unroll
+        for (int i = 0; i < G / 2; ++i)
+            reinterpret_cast<uint4*>(slot)[i * 32 + lane] = make_uint4(pr.e[2 * i].rcp, pr.e[2 * i].fc, pr.e[2 * i + 1].rcp, pr.e[2 * i + 1].fc);
+    } else {
+        reinterpret_cast<uint2*>(slot)[lane] = make_uint2(pr.e[0].rcp, pr.e[0].fc);
+    }
+#pragma unroll
+    for (int i = 0; i < kPlaneWords<G>; ++i) slot[64 * G + i * 32 + lane] = (int)pr.plane[i];
+}
+template <int G>
+__device__ __forceinline__ void slot_get(const int* slot, int lane, Prepared<G>& pr) {
+    if constexpr (G >= 2) {
+#pragma unroll
+        for (int i = 0; i < G / 2; ++i) {
+            const uint4 w = reinterpret_cast<const uint4*>(slot)[i * 32 + lane];
+            pr.e[2 * i] = EncEntry{w.x, w.y}; pr.e[2 * i + 1] = EncEntry{w.z, w.w};
+        }
+    } else {
+        const uint2 w = reinterpret_cast<const uint2*>(slot)[lane];
+        pr.e[0] = EncEntry{w.x, w.y};
+    }
+#pragma unroll
+    for (int i = 0; i < kPlaneWords<G>; ++i) pr.plane[i] = (uint32_t)slot[64 * G + i * 32 + lane];
+}
+
+size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
+    const int NP = warps - 1, G = d / 32, planes = G <= 2 ? 1 : G / 2;
+    const int slot = enc ? 32 * (2 * G + planes) : 32 * G + 8;
+    return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : kRingBytes);
+}
+
+// All warps of the block meet here; the two roles reach it from different places in the code.
+__device__ __forceinline__ void block_barrier() { asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)blockDim.x) : "memory"); }
+
+// The block's current chunk.
+struct CoopItem {
+    Item it;
+    long long row0, kv0;                 // first row of the positions; element of the chunk's first vector
+    unsigned long long off;              // decoding: the chunk's bytes
+    unsigned nbytes;
+    int go;                              // 0: nothing to do for this chunk, -1: no chunks left
+};
+struct CoopShared {
+    CoopItem item;
+    SlotMeta meta[2][kCoopMaxWarps];
+    uint8_t* dst;                        // encoding: where the finished chunk's words go (null: nowhere)
+    int wp;
+};
+
+// Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a batch; the inputs
+// of the next are fetched while it works on one.
+template <int D, bool DENSE, bool ENC, class Tab>
+__device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
+                                             const LaneCode& lc) {
+    constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
+    const int lane = lc.lane;
+    const int P = sh.item.it.P, Kp = DENSE ? 0 : a.sh.Kp, n_batches = (P + NP - 1) / NP, c0 = first_comp<D>(lane);
+    const int t = sh.item.it.t, t0 = DENSE ? a.dense_t0 : 0;
+    const int first = ENC ? P - 1 : 0, dir = ENC ? -1 : 1;
+    const long long row0 = sh.item.row0;
+    const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+    const float* n2 = a.rownorm2 + (size_t)t * a.sh.V;
+    const bool zr = a.sh.zero_q != kZeroOff;
+    int buf = 0;
+    float m_next[G] = {}, s1_next = 0.f, ideal = 0.f;
+    uint32_t kv_next[(G + 1) / 2] = {};
+    // decoding: the position predicted a batch ago, whose vector is written when the coder has passed it
+    float mu_old[G] = {};
+    SlotMeta old{kSkipped, 0, 0, 0};
+    auto fetch = [&](int k, int into) {
+        const int p = first + dir * k;
+        if (DENSE) dense_fetch<D>(a, row0 + p, t - t0, c0, m_next, s1_next);
+        else prefetch_pairs(sp0 + into * Kp, a.pairs + (row0 + p) * Kp, Kp, lane);
+        if (ENC) load_half_raw<G>(reinterpret_cast<const __half*>(a.kv.base) + sh.item.kv0 + c0 + p * a.kv.sp, kv_next);
+    };
+    auto finish = [&](int b) {                                                 // decoding: position of batch b
+        const int p = b * NP + w;
+        if (b < 0 || p >= P) return;
+        int sym[G];
+        float out[G];
+        if (old.q == kSkipped) {                                               // zero-rate position: KV' = KV^
+#pragma unroll
+            for (int g = 0; g < G; ++g) { sym[g] = 0; out[g] = mu_old[g]; }
+        } else {
+            const int* slot = slots + ((b & 1) * NP + w) * SW;
+            int hi[G];
+            slot_get_ints<G>(slot, lane, hi);
+            if (sh.meta[b & 1][w].escaped) {
+#pragma unroll
+                for (int g = 0; g < G; ++g) sym[g] = hi[g];
+            } else {
+                int base[G], s, qp;
+#pragma unroll
+                for (int g = 0; g < G; ++g) base[g] = slot[32 * G + g];
+                class_params(old.q, s, qp);
+                const uint16_t* words = reinterpret_cast<const uint16_t*>(a.st.payload + sh.item.off + 128);
+                const int last = (int)((sh.item.nbytes - 128u) >> 1) - 1;      // past the end: the last word
+                join_position<G>(base, hi, s, [&](int i) { return (uint32_t)__ldg(words + min(i, last)); }, lc, sym);
+            }
+            const float delta = a.step_exp ? ldexpf(a.sh.delta, old.e) : a.sh.delta;
+#pragma unroll
+            for (int g = 0; g < G; ++g) out[g] = __fmaf_rn((float)sym[g], delta, mu_old[g]);
+        }
+        store_vec<G>(a.kv.base, sh.item.kv0 + c0 + p * a.kv.sp, out, a.sh.out_dtype);
+        if (a.dbg.sym) {
+            const long long o = (row0 + p) * (2 * a.sh.L * a.sh.H) + t;
+#pragma unroll
+            for (int g = 0; g < G; ++g) a.dbg.sym[o * D + c0 + g] = sym[g];
+        }
+    };
+    if (w < P) fetch(w, 0);
+    for (int b = 0; b < n_batches; ++b) {
+        const int k = b * NP + w, p = first + dir * k;
+        float mu[G] = {};
+        SlotMeta sm{kSkipped, 0, 0, 0};
+        if (k < P) {
+            float sigma2;
+            uint32_t kv_raw[(G + 1) / 2];
+#pragma unroll
+            for (int i = 0; i < (G + 1) / 2; ++i) kv_raw[i] = kv_next[i];
+            if (DENSE) {
+                float m_cur[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) m_cur[g] = m_next[g];
+                const float s1_cur = s1_next;
+                if (k + NP < P) fetch(k + NP, 0);
+                dense_finish<D>(a, t - t0, c0, 1.0f / D, m_cur, s1_cur, mu, sigma2);
+            } else {
+                const int2* sp = sp0 + buf * Kp;
+                if (k + NP < P) { fetch(k + NP, buf ^ 1); pairs_ready<1>(); }
+                else pairs_ready<0>();
+                buf ^= 1;
+                predict<D>(col, n2, sp, Kp, lane, 1.0f / D, mu, sigma2);
+            }
+            float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
+            int zero_q = a.sh.zero_q;
+            if (a.step_exp) {                                                  // adaptive step delta * 2^e
+                sm.e = __ldg(a.step_exp + row0 + p);
+                inv_delta = ldexpf(inv_delta, -sm.e);
+                inv_delta2 = ldexpf(inv_delta2, -2 * sm.e);
+                if (zr) zero_q -= 8 * sm.e;
+            }
+            const int q = __reduce_max_sync(kFull, scale_class(sigma2, a.sh.sigma_floor * a.sh.sigma_floor, inv_delta2));   // same in all lanes
+            const bool skip = zr && q <= zero_q;
+            sm.q = skip ? kSkipped : q;
+            if constexpr (ENC) {
+                float kvv[G];
+                half_raw_to_float<G>(kv_raw, kvv);
+                int sym[G], u[G], s, qp;
+                uint32_t at[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) sym[g] = quantise(kvv[g], mu[g], inv_delta);
+                class_params(q, s, qp);
+                int* slot = slots + ((b & 1) * NP + w) * SW;
+                if (split_symbols<G>(sym, s, u, at)) {
+                    Prepared<G> pr;
+                    prepare_position<G>(u, at, s, tb.enc[qp - kQMin], lc, pr);
+                    slot_put<G>(slot, lane, pr);
+                } else {
+                    sm.escaped = 1;
+                    slot_put_ints<G>(slot, lane, u);
+                }
+                if (a.dbg.sym) {
+                    const long long o = (row0 + p) * (2 * a.sh.L * a.sh.H) + t;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) a.dbg.sym[o * D + c0 + g] = skip ? 0 : sym[g];
+                }
+                if (a.dbg.ideal && !skip) {              // log2(2^15 / f) + s raw bits (+ 32 per escape)
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const uint32_t f = tb.enc[qp - kQMin][min(at[g], (uint32_t)kEsc)].fc & 0xffffu;
+                        ideal += (float)(kProbBits + s) - log2f((float)f) + (at[g] > 2u * kHiMax ? 32.f : 0.f);
+                    }
+                }
+            }
+            if (a.dbg.q || a.dbg.mu) {
+                const long long o = (row0 + p) * (2 * a.sh.L * a.sh.H) + t;
+                if (a.dbg.q && lane == 0) a.dbg.q[o] = q;
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    if (a.dbg.mu) a.dbg.mu[o * D + c0 + g] = mu[g];
+            }
+            if (lane == 0) sh.meta[b & 1][w] = sm;
+            __syncwarp();                                                      // readers of the pair slot are done
+        }
+        block_barrier();
+        if constexpr (!ENC) {
+            finish(b - 1);
+#pragma unroll
+            for (int g = 0; g < G; ++g) mu_old[g] = mu[g];
+            old = sm;
+        }
+    }
+    block_barrier();
+    if constexpr (!ENC) finish(n_batches - 1);
+    if (ENC && a.dbg.ideal) {
+        ideal = warp_sum(ideal);
+        if (lane == 0) atomicAdd(&a.counters->ideal_bits, (double)ideal);
+    }
+}
+
+// Coder of the block's chunk, one batch behind the predictions.
+template <int D, bool ENC, class Tab>
+__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const LaneCode& lc) {
+    constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
+    const int lane = lc.lane;
+    const int P = sh.item.it.P, n_batches = (P + NP - 1) / NP;
+    uint32_t x = kRansL;
+    if constexpr (ENC) {
+        uint16_t* stage = a.staging + (long long)blockIdx.x * a.staging_words_per_warp;
+        const int cap_words = (int)a.staging_words_per_warp;
+        int wp = cap_words, n_skipped = 0;
+        unsigned n_escapes = 0;
+        for (int b = 0; b < n_batches; ++b) {
+            block_barrier();                                                   // batch b is there
+            const int cnt = min(NP, P - b * NP);
+            const int* slot = slots + (b & 1) * NP * SW;
+            Prepared<G> next;
+            slot_get<G>(slot, lane, next);
+            SlotMeta sm = sh.meta[b & 1][0];
+            for (int j = 0; j < cnt; ++j, slot += SW) {
+                const Prepared<G> pr = next;
+                const SlotMeta m = sm;
+                if (j + 1 < cnt) { slot_get<G>(slot + SW, lane, next); sm = sh.meta[b & 1][j + 1]; }
+                if (m.q == kSkipped) { ++n_skipped; continue; }
+                int s, qp;
+                class_params(m.q, s, qp);
+                if (!m.escaped) {
+                    wp = push_position<G>(pr, s, x, stage, wp, lc);
+                } else {
+                    int u[G];
+                    slot_get_ints<G>(slot, lane, u);
+                    wp = encode_position_escapes<G>(u, s, tb.enc[qp - kQMin], x, stage, wp, lane, n_escapes);
+                }
+            }
+        }
+        block_barrier();
+        uint8_t* dst = reserve_chunk(a, sh.item.it.slot, x, cap_words - wp, lane, P, n_escapes, n_skipped);
+        if (lane == 0) { sh.dst = dst; sh.wp = wp; }
+    } else {
+        const uint8_t* src = a.st.payload + sh.item.off;
+        x = reinterpret_cast<const uint32_t*>(src)[lane];
+        bool bad = x < kRansL;
+        src += 128;
+        const int nwords = (int)((sh.item.nbytes - 128u) >> 1);
+        int rp = 0, fetched = 0, ready = 0;
+        ring_fetch(ring, src, 2 * nwords, 0, fetched, lane);
+        const RingWords words{ring};
+        for (int b = 0; b < n_batches; ++b) {
+            block_barrier();                                                   // the classes of batch b are there
+            const int cnt = min(NP, P - b * NP);
+            int* slot = slots + (b & 1) * NP * SW;
+            int q = sh.meta[b & 1][0].q;
+            for (int j = 0; j < cnt; ++j, slot += SW) {
+                const int qj = q;
+                if (j + 1 < cnt) q = sh.meta[b & 1][j + 1].q;
+                if (qj == kSkipped) continue;
+                // a position takes at most G * (2 * 15 + 32 + 64) words
+                if (min(2 * rp + 252 * G, 2 * nwords) > ready) {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncwarp();
+                    ready = fetched;
+                }
+                int s, qp, base[G], hi[G];
+                class_params(qj, s, qp);
+                if (pull_position<G>(s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, words, rp, lc, base, hi)) {
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+                        if (lane == g) slot[32 * G + g] = base[g];
+                } else {
+                    decode_position_escapes<G>(hi, s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, words, rp, lane);
+                    if (lane == 0) sh.meta[b & 1][j].escaped = 1;
+                }
+                slot_put_ints<G>(slot, lane, hi);
+                __syncwarp();                                                  // readers of the ring are done
+                ring_fetch(ring, src, 2 * nwords, rp, fetched, lane);
+            }
+        }
+        block_barrier();
+        bad = bad || x != kRansL || rp != nwords;
+        if (__any_sync(kFull, bad) && lane == 0) atomicOr(a.status, kStCorrupt);
+        asm volatile("cp.async.wait_all;" ::: "memory");                       // of a damaged chunk: nothing may land later
+    }
+}
+
+// 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
+template <int D, bool DENSE, bool ENC>
+__global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
+    using Tab = std::conditional_t<ENC, EncTables, DecTables>;
+    __shared__ Tab tb;
+    __shared__ CoopShared sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NP = (blockDim.x >> 5) - 1;   // NP predicting warps
+    const int Kp = DENSE ? 0 : a.sh.Kp;
+    int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
+    uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
+    const LaneCode lc = lane_code(lane);
+    load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->dec));
+    const int Wl = DENSE ? a.dense_nt : 2 * a.sh.L * a.sh.H;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks, total = (unsigned)Wl * per_table;
+    QueueCursor qc = DENSE ? QueueCursor{0, 0} : queue_of_this_sm(a);
+
+    for (;;) {
+        if (warp == 0) {
+            const unsigned item = DENSE ? next_ticket(a.ticket, lane) : next_queued(a, qc, per_table, Wl, lane);
+            if (lane == 0) {
+                CoopItem ci{};
+                ci.go = -1;
+                if (item < total) {
+                    ci.it = bulk_item(a, item, DENSE ? a.dense_t0 : 0);
+                    ci.go = ci.it.P > 0;
+                    ci.row0 = (long long)ci.it.s * a.n + ci.it.p0;
+                    ci.kv0 = kv_elem(a.kv, ci.it.t, a.sh.H, ci.it.s, ci.it.p0);
+                    if (ENC && !ci.go) { a.st.chunk_offset[ci.it.slot] = 0; a.st.chunk_bytes[ci.it.slot] = 0; }
+                    if (!ENC && ci.go) {
+                        ci.off = a.st.chunk_offset[ci.it.slot];
+                        ci.nbytes = a.st.chunk_bytes[ci.it.slot];
+                        if (ci.nbytes < 128u || (ci.nbytes & 1u) || (ci.off & 15ull) || ci.off + ci.nbytes > a.st.capacity) {
+                            atomicOr(a.status, kStCorrupt);
+                            ci.go = 0;
+                        }
+                    }
+                }
+                sh.item = ci;
+            }
+        }
+        __syncthreads();
+        const int go = sh.item.go;
+        if (go < 0) break;
+        if (go > 0) {
+            if (warp == 0) coop_code<D, ENC>(a, sh, tb, slots, ring, NP, lc);
+            else coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
+        }
+        __syncthreads();                                                       // the chunk is coded; its item has been read
+        if (ENC && go > 0 && sh.dst)
+            copy_words(sh.dst, a.staging + (long long)blockIdx.x * a.staging_words_per_warp + sh.wp,
+                       (int)a.staging_words_per_warp - sh.wp, threadIdx.x, blockDim.x);
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
+    return dispatch_d(a.sh.d, [&](auto D) {
+        constexpr int d = decltype(D)::value;
+        const bool dense = a.mu_dense != nullptr;
+        auto kern = dense ? (encode ? coop_kernel<d, true, true> : coop_kernel<d, true, false>)
+                          : (encode ? coop_kernel<d, false, true> : coop_kernel<d, false, false>);
+        const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
+        int warps = items <= 2ll * sm_count() ? kCoopMaxWarps : kCoopMaxWarps / 2;
+        if (coop_smem(warps, a.sh.Kp, d, dense, encode) > 96 * 1024) warps = kCoopMaxWarps / 2;
+        const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int occ = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem) != cudaSuccess || occ < 1) occ = 1;
+        const long long blocks = std::min<long long>(items, (long long)sm_count() * occ);
+        kern<<<(unsigned)blocks, warps * 32, smem, st>>>(a);
+        count_launch();
+        return cudaGetLastError();
+    });
+}
+
+}  // namespace plc
