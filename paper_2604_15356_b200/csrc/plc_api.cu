@@ -1,4 +1,5 @@
 // C ABI of libplc (see include/plc.h): argument checks, context scratch, kernel launches.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 #include <new>
@@ -548,14 +549,19 @@ static plc_status rotq_impl(plc_ctx* c, const plc_kv_view* kv, int elem_bytes, c
     const unsigned long long W = 2ull * c->cfg.n_layers * c->cfg.n_kv_heads;
     if (4ull * rotq_words(c, p->bits) * W * (unsigned long long)S * (unsigned long long)n > capacity) return PLC_E_CAPACITY;
     if (S == 0 || n == 0) return PLC_OK;
-    const int mc = (n + c->cfg.chunk_pos - 1) / c->cfg.chunk_pos;
+    // Records have fixed places, so the positions a warp walks in one go are only a matter of scheduling:
+    // four goes a resident warp (a go pays for its ticket and a cold start, about a position's worth),
+    // from 8 positions up to the chunk length.
+    const long long per_go = (long long)W * S * n / (4ll * codec_grid_warps(0));
+    const int cp = (int)std::min<long long>(std::max<long long>(per_go, 8), std::max(c->cfg.chunk_pos, 8));
+    const int mc = (n + cp - 1) / cp;
     if ((long long)W * S * mc >= (1ll << 32)) return PLC_E_SHAPE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     rc = run_topk_for(c, logits_dev, S, n, pb, pe, st);
     if (rc) return rc;
     CodecArgs a = base_args(c);
     a.kv = to_dev(kv); a.S = S; a.n = n; a.pos_begin = pb; a.pos_end = pe; a.pairs = c->pairs;
-    a.st.max_chunks = mc;
+    a.st.max_chunks = mc; a.sh.chunk_pos = cp;
     RotqArgs r{};
     r.bits = p->bits; r.rec_words = rotq_words(c, p->bits);
     for (int i = 0; i < 8; ++i) r.sign_bits[i] = p->sign_bits[i];
