@@ -285,7 +285,7 @@ def run_codec(args, torch, plc, workloads, dev, name, over, steps, warmup, dist=
     barrier()
     t_start = torch.cuda.Event(enable_timing=True); t_end = torch.cuda.Event(enable_timing=True)
     t_start.record()
-    gemm_k = []
+    gemm_k = None
     for i in range(steps):
         st.total_bytes.zero_()
         ev[3 * i].record()
@@ -299,7 +299,7 @@ def run_codec(args, torch, plc, workloads, dev, name, over, steps, warmup, dist=
     ek, n_ek = ctx.kernel_ms(0)
     dk, n_dk = ctx.kernel_ms(1)
     if dense or linear:
-        gemm_k.append(ctx.kernel_ms(2)[0])
+        gemm_k = ctx.kernel_ms(2)
     launches = plc.launch_count() - launches0
     clocks = sampler.stop()
     total_ms = t_start.elapsed_time(t_end)
@@ -335,18 +335,19 @@ def run_codec(args, torch, plc, workloads, dev, name, over, steps, warmup, dist=
     if roofline["traffic"] is not None:
         roofline["traffic_note"] = NCU_TRAFFIC_NOTE
     if dense or linear:
-        gm = statistics.mean(gemm_k)
+        gm, n_gemm = gemm_k
+        per_launch = 2.0 * L * steps / n_gemm                          # layers one contraction covers (small batches: several)
         tpeak, tkind = tensor_peak()
         if dense:      # 2 * rows * V * (2H*d) flop per layer and direction
-            flop = 2.0 * S * n * V * (2 * H * d)
+            flop = 2.0 * S * n * V * (2 * H * d) * per_launch
         else:          # per layer: rows x (2H*d) x d_model
-            flop = 2.0 * S * n * d_model * (2 * H * d)
+            flop = 2.0 * S * n * d_model * (2 * H * d) * per_launch
         roofline = {"kernel": "dense_gemm_kernel", "bound": "tensor", "achieved": flop / (gm / 1e3) / 1e12, "peak": tpeak,
                     "unit": "TFLOP/s", "frac": flop / (gm / 1e3) / 1e12 / tpeak, "traffic": None, "peak_kind": tkind,
-                    "ms_per_launch": gm, "flop_per_launch": flop, "launches_per_step": 2 * L,
-                    "coder_kernels_ms_last_layer": {"encode": ek_last, "decode": dk_last}}
+                    "ms_per_launch": gm, "flop_per_launch": flop, "launches_per_step": n_gemm // steps,
+                    "coder_kernels_ms_per_launch": {"encode": ek_last, "decode": dk_last}}
         if linear:
-            roofline["flop_per_step_all_contractions"] = 2 * (L * flop + 2.0 * S * n * V * d_model +
+            roofline["flop_per_step_all_contractions"] = 2 * (L * flop / per_launch + 2.0 * S * n * V * d_model +
                                                               2.0 * S * n * V * 256 * ((W + 255) // 256))
     e2e = None
     if want_e2e and not linear:

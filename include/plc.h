@@ -145,7 +145,9 @@ typedef struct plc_ctx plc_ctx;
 
 /* Creates a context for one parameter set and one candidate table.
  * T_dev: [L][2][H][V][d] f16, the stand-in for F_M(t_<i, t) of Def. 5 (one d-vector per layer, K/V,
- * head and candidate token); 16-byte aligned; must outlive the context (it is not copied).
+ * head and candidate token); 16-byte aligned; must outlive the context (it is not copied;
+ * PLC_PRED_DENSE contexts keep its bf16 transpose while that takes at most a quarter of the memory
+ * free at creation, and form a layer's at a time per call otherwise).
  * Synchronises the device once (it pre-computes the squared norm of every row of T).
  * Errors: PLC_E_INVALID / PLC_E_SHAPE / PLC_E_ALIGN on bad arguments, PLC_E_CUDA. */
 plc_status plc_create(plc_ctx** out, const plc_config* cfg, const void* T_dev);
@@ -154,8 +156,9 @@ plc_status plc_create(plc_ctx** out, const plc_config* cfg, const void* T_dev);
  * embedding, so that the expectation over the next token moves inside it):
  *     KV^ = c + A * Ebar,   Ebar = sum_v P(v) E(v)   over the whole vocabulary,
  *     sigma_mix^2 = sum_v P(v) ||c + A E(v)||^2 / d - ||KV^||^2 / d          (Thm. 2 with F := c + A E).
- * E_dev [V][d_model], A_dev [L][2][H][d][d_model], c_dev [L][2][H][d], all f16, 16-byte aligned, not
- * copied (they must outlive the context).  d_model: a multiple of 64, at most 16384.
+ * E_dev [V][d_model], A_dev [L][2][H][d][d_model], c_dev [L][2][H][d], all f16, 16-byte aligned; they
+ * must outlive the context (which keeps a bf16 copy of A while that takes at most a quarter of the
+ * memory free at creation, and converts a layer at a time per call otherwise).  d_model: a multiple of 64, at most 16384.
  * Arithmetic: P, E, A and Ebar are rounded to bfloat16 and contracted on the tensor cores with
  * binary32 accumulation; c is added in binary32. */
 typedef struct {
@@ -355,8 +358,9 @@ plc_status plc_table_constants(int32_t qp, uint32_t* theta, uint32_t* rho);
 plc_status plc_build_table(int32_t qp, uint32_t* f, uint32_t* c);
 /* With profiling on, plc_encode / plc_decode record CUDA events on the caller's stream directly
  * around their fused predict+code kernel (the top-K kernel that precedes it is outside);
- * plc_last_kernel_ms waits for the most recent such launch (which = 0 encode, 1 decode, 2 the dense
- * variant's tensor-core contraction of the last layer) and returns its duration.  PLC_E_STATE if
+ * plc_last_kernel_ms waits for the most recent such launch (which = 0 encode, 1 decode, 2 the dense and
+ * linear variants' tensor-core contraction of the last group of layers; small calls form all layers
+ * in one) and returns its duration.  PLC_E_STATE if
  * no such launch was recorded. */
 plc_status plc_set_profiling(plc_ctx* ctx, int32_t on);
 /* Work-queue layout the most recent top-K plc_encode / plc_decode of this context used: *n_queues

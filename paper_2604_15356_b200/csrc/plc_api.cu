@@ -70,9 +70,10 @@ struct plc_ctx {
     const __half* lin_A;
     const __half* lin_c;
     int lin_dm;
-    uint8_t* lin_model;             // linear: E transposed (bf16) and the candidate-norm table of every (layer, table);
-                                    // dense: the candidate-norm table alone
-    size_t lin_off[2];
+    uint8_t* model;                 // linear: E transposed, the candidate-norm table of every (layer, table), A (all bf16);
+                                    // dense: the candidate-norm table and T transposed (bf16)
+    size_t model_off[3];
+    bool resident;                  // the model holds A / the transposed T of every layer (otherwise converted a layer at a time per call)
     int last_nq, last_g;            // work-queue layout of the most recent top-K encode / decode launch
     int profiling;                  // record events around the codec kernels
     // Event pairs (start, stop) of the profiled launches since the last reset, per kind: 0 encode
@@ -191,31 +192,30 @@ DenseShape dense_shape(const plc_ctx* c, long long rows) {
     DenseShape sh;
     sh.rows = rows; sh.V = c->cfg.vocab; sh.d = c->cfg.head_dim; sh.tables = 2 * c->cfg.n_kv_heads;
     sh.ldv = (sh.V + 63) / 64 * 64;
-    sh.ncols = sh.tables * sh.d; sh.ncols_pad = (sh.ncols + 255) / 256 * 256;
-    sh.nt_all = c->cfg.n_layers * sh.tables; sh.nt_all_pad = (sh.nt_all + 255) / 256 * 256;
+    sh.ncols = sh.tables * sh.d; sh.nt_all = c->cfg.n_layers * sh.tables;
+    sh.resident = c->resident;
+    sh.group = sh.resident ? layers_per_group(c->cfg.n_layers, rows, sh.ncols) : 1;
     return sh;
 }
 
-LinearShape linear_shape(const plc_config& cfg, int dm, long long rows) {
+LinearShape linear_shape(const plc_ctx* c, long long rows) {
     LinearShape sh;
-    sh.rows = rows; sh.V = cfg.vocab; sh.d = cfg.head_dim; sh.dm = dm; sh.tables = 2 * cfg.n_kv_heads; sh.L = cfg.n_layers;
+    sh.rows = rows; sh.V = c->cfg.vocab; sh.d = c->cfg.head_dim; sh.dm = c->lin_dm; sh.tables = 2 * c->cfg.n_kv_heads; sh.L = c->cfg.n_layers;
     sh.ldv = (sh.V + 63) / 64 * 64;
-    sh.ncols = sh.tables * sh.d; sh.ncols_pad = (sh.ncols + 255) / 256 * 256;
-    sh.nt_all = sh.L * sh.tables; sh.nt_all_pad = (sh.nt_all + 255) / 256 * 256;
+    sh.ncols = sh.tables * sh.d; sh.nt_all = sh.L * sh.tables;
+    sh.resident = c->resident;
+    sh.group = sh.resident ? layers_per_group(sh.L, rows, sh.ncols) : 1;
     return sh;
+}
+
+// Whether a context keeps a second, bf16 copy of its model's weights: only while that leaves the caller
+// three quarters of the memory that is free when it is created.
+bool keep_weights(size_t bytes) {
+    size_t free_b = 0, total_b = 0;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4;
 }
 
 plc_status ensure_scratch(plc_ctx* c, size_t need) {
-    if (need <= c->dense_bytes) return PLC_OK;
-    if (c->dense_scratch) cudaFree(c->dense_scratch);
-    c->dense_scratch = nullptr; c->dense_bytes = 0;
-    if (cudaMalloc(&c->dense_scratch, need) != cudaSuccess) return PLC_E_CUDA;
-    c->dense_bytes = need;
-    return PLC_OK;
-}
-
-plc_status ensure_dense(plc_ctx* c, const DenseShape& sh, size_t* off) {
-    const size_t need = dense_scratch_bytes(sh, off);
     if (need <= c->dense_bytes) return PLC_OK;
     if (c->dense_scratch) cudaFree(c->dense_scratch);
     c->dense_scratch = nullptr; c->dense_bytes = 0;
@@ -297,19 +297,20 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
     if (ok && T_dev) ok = launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, 0) == cudaSuccess &&
                           cudaDeviceSynchronize() == cudaSuccess;
-    if (ok && T_dev && cfg->variant == PLC_PRED_DENSE) {     // candidate norms of every layer, once
+    if (ok && T_dev && cfg->variant == PLC_PRED_DENSE) {     // operands of every layer, once
+        c->resident = keep_weights((size_t)rows * cfg->head_dim * 2);
         const DenseShape sh = dense_shape(c, 0);
-        ok = (long long)cfg->n_layers * 2 * cfg->n_kv_heads <= 65536 &&
-             cudaMalloc(&c->lin_model, dense_model_bytes(sh)) == cudaSuccess &&
-             dense_prepare(c->T, cfg->n_layers, sh, c->lin_model, 0) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+        ok = sh.nt_all <= 65536 && cudaMalloc(&c->model, dense_model_bytes(sh, c->model_off)) == cudaSuccess &&
+             dense_prepare(c->T, sh, c->model, c->model_off, 0) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     }
     if (ok && lin) {
         c->lin_E = static_cast<const __half*>(lin->E_dev); c->lin_A = static_cast<const __half*>(lin->A_dev);
         c->lin_c = static_cast<const __half*>(lin->c_dev); c->lin_dm = lin->d_model;
-        const LinearShape sh = linear_shape(*cfg, lin->d_model, 0);
-        const size_t bytes = linear_model_bytes(sh, c->lin_off);
-        ok = cudaMalloc(&c->lin_model, bytes) == cudaSuccess &&
-             linear_prepare(c->lin_E, c->lin_A, c->lin_c, sh, c->lin_model, c->lin_off, c->status, 0) == cudaSuccess;
+        c->resident = keep_weights((size_t)cfg->n_layers * 2 * cfg->n_kv_heads * cfg->head_dim * lin->d_model * 2);
+        const LinearShape sh = linear_shape(c, 0);
+        const size_t bytes = linear_model_bytes(sh, c->model_off);
+        ok = cudaMalloc(&c->model, bytes) == cudaSuccess &&
+             linear_prepare(c->lin_E, c->lin_A, c->lin_c, sh, c->model, c->model_off, c->status, 0) == cudaSuccess;
     }
     if (!ok) { plc_destroy(c); return PLC_E_CUDA; }
     *out = c;
@@ -319,7 +320,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
 plc_status plc_destroy(plc_ctx* c) {
     if (!c) return PLC_E_INVALID;
     cudaFree(c->rownorm2); cudaFree(c->pairs); cudaFree(c->cand); cudaFree(c->step_exp); cudaFree(c->staging);
-    cudaFree(c->ticket); cudaFree(c->status); cudaFree(c->counters); cudaFree(c->dense_scratch); cudaFree(c->lin_model);
+    cudaFree(c->ticket); cudaFree(c->status); cudaFree(c->counters); cudaFree(c->dense_scratch); cudaFree(c->model);
     for (int k = 0; k < 3; ++k)
         for (cudaEvent_t e : c->prof_ev[k]) cudaEventDestroy(e);
     if (c->status_host) cudaFreeHost(c->status_host);
@@ -386,24 +387,23 @@ static plc_status run_topk_for(plc_ctx* c, const void* logits_dev, int S, int n,
     return launch_topk(a, st) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
 }
 
-// Dense variant: softmax once, then per layer the bf16 contraction and the coding of its 2H tables.
+// Dense variant: softmax once, then per group of layers the bf16 contraction and the coding of its tables.
 static plc_status run_dense(plc_ctx* c, CodecArgs a, const void* logits_dev, bool encode, cudaStream_t st) {
     const DenseShape sh = dense_shape(c, (long long)a.S * a.n);
-    if (sh.tables > 256) return PLC_E_SHAPE;              // one norm column per table, at most 256 per launch
-    size_t off[5];
-    plc_status rc = ensure_dense(c, sh, off);
+    if (sh.tables > 256) return PLC_E_SHAPE;              // one norm column per table, at most 256 per layer
+    size_t off[4];
+    plc_status rc = ensure_scratch(c, dense_scratch_bytes(sh, off));
     if (rc) return rc;
-    if (dense_begin(static_cast<const __half*>(logits_dev), sh, c->lin_model, c->dense_scratch, off, c->status, st) != cudaSuccess)
-        return PLC_E_CUDA;
-    a.mu_dense = reinterpret_cast<const float*>(c->dense_scratch + off[3]);
-    a.mu_ld = sh.ncols; a.s1_ld = sh.nt_all;
-    const size_t layer_elems = (size_t)sh.tables * sh.V * sh.d;
-    for (int l = 0; l < c->cfg.n_layers; ++l) {
+    if (dense_softmax(static_cast<const __half*>(logits_dev), sh, c->dense_scratch, off, st) != cudaSuccess) return PLC_E_CUDA;
+    a.mu_dense = reinterpret_cast<const float*>(c->dense_scratch + off[2]);
+    a.mu_ld = (long long)sh.group * sh.ncols; a.s1_ld = sh.nt_all;
+    for (int l = 0; l < c->cfg.n_layers; l += sh.group) {
+        const int nl = std::min(sh.group, c->cfg.n_layers - l);
         cudaEvent_t* pg = prof_pair(c, 2);
-        if (dense_layer(c->T + l * layer_elems, sh, c->dense_scratch, off, c->status, st, pg ? pg[0] : nullptr,
-                        pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
-        a.dense_t0 = l * sh.tables; a.dense_nt = sh.tables;
-        a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[4]) + (size_t)l * sh.tables;
+        if (dense_layers(c->T, l, nl, sh, c->model, c->model_off, c->dense_scratch, off, c->status, st, pg ? pg[0] : nullptr,
+                         pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
+        a.dense_t0 = l * sh.tables; a.dense_nt = nl * sh.tables;
+        a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[3]) + (size_t)l * sh.tables;
         cudaEvent_t* pk = prof_pair(c, encode ? 0 : 1);
         if (pk) cudaEventRecord(pk[0], st);
         if ((encode ? launch_encode(a, st) : launch_decode(a, st)) != cudaSuccess) return PLC_E_CUDA;
@@ -412,22 +412,23 @@ static plc_status run_dense(plc_ctx* c, CodecArgs a, const void* logits_dev, boo
     return PLC_OK;
 }
 
-// Linear-embedding variant (Sec. 7.1): Ebar and the variance term once, then per layer mu = Ebar A^T and the coding.
+// Linear-embedding variant (Sec. 7.1): Ebar and the variance term once, then per group of layers mu = Ebar A^T and the coding.
 static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bool encode, cudaStream_t st) {
-    const LinearShape sh = linear_shape(c->cfg, c->lin_dm, (long long)a.S * a.n);
-    size_t off[6];
+    const LinearShape sh = linear_shape(c, (long long)a.S * a.n);
+    size_t off[5];
     plc_status rc = ensure_scratch(c, linear_scratch_bytes(sh, off));
     if (rc) return rc;
-    if (linear_begin(static_cast<const __half*>(logits_dev), sh, c->lin_model, c->lin_off, c->dense_scratch, off, c->status, st) !=
+    if (linear_begin(static_cast<const __half*>(logits_dev), sh, c->model, c->model_off, c->dense_scratch, off, c->status, st) !=
         cudaSuccess) return PLC_E_CUDA;
-    a.mu_dense = reinterpret_cast<const float*>(c->dense_scratch + off[5]);
-    a.mu_ld = sh.ncols; a.s1_ld = sh.nt_all;
-    for (int l = 0; l < c->cfg.n_layers; ++l) {
+    a.mu_dense = reinterpret_cast<const float*>(c->dense_scratch + off[4]);
+    a.mu_ld = (long long)sh.group * sh.ncols; a.s1_ld = sh.nt_all;
+    for (int l = 0; l < c->cfg.n_layers; l += sh.group) {
+        const int nl = std::min(sh.group, c->cfg.n_layers - l);
         cudaEvent_t* pg = prof_pair(c, 2);
-        if (linear_layer(c->lin_A + (size_t)l * sh.ncols * sh.dm, sh, c->dense_scratch, off, c->status, st,
-                         pg ? pg[0] : nullptr, pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
-        a.dense_t0 = l * sh.tables; a.dense_nt = sh.tables;
-        a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[3]) + (size_t)l * sh.tables;
+        if (linear_layers(c->lin_A, l, nl, sh, c->model, c->model_off, c->dense_scratch, off, c->status, st,
+                          pg ? pg[0] : nullptr, pg ? pg[1] : nullptr) != cudaSuccess) return PLC_E_CUDA;
+        a.dense_t0 = l * sh.tables; a.dense_nt = nl * sh.tables;
+        a.s1_dense = reinterpret_cast<const float*>(c->dense_scratch + off[2]) + (size_t)l * sh.tables;
         a.mu_bias = c->lin_c + (size_t)l * sh.ncols;
         cudaEvent_t* pk = prof_pair(c, encode ? 0 : 1);
         if (pk) cudaEventRecord(pk[0], st);

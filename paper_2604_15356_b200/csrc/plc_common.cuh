@@ -211,38 +211,41 @@ struct RotqArgs {
 cudaError_t launch_rotq(const CodecArgs& a, const RotqArgs& r, bool encode, cudaStream_t st);
 constexpr int kTicketWords = 1024;               // one counter per work queue (at most one queue per SM)
 
-// Dense (full-vocabulary) prediction, one layer at a time.
+// Dense (full-vocabulary) prediction, a group of layers at a time.
 struct DenseShape {
     long long rows;        // S * n positions
     int V, d, tables;      // tables = 2 * H of one layer
-    int ldv;               // V rounded up to 64 (row pitch of P and Tb, in elements)
-    int ncols, ncols_pad;  // tables * d, rounded up to 256
-    int nt_all, nt_all_pad;   // L * tables (one variance column per layer and table), rounded up to 256
+    int ldv;               // V rounded up to 64 (row pitch of P, Tb and Nb, in elements)
+    int ncols;             // tables * d
+    int nt_all;            // L * tables (one variance column per layer and table)
+    int group;             // layers per contraction
+    bool resident;         // the context keeps the transposed bf16 table of every layer
 };
-size_t dense_scratch_bytes(const DenseShape& sh, size_t* off /*[5]: P, Tb, -, mu, s1*/);
-size_t dense_model_bytes(const DenseShape& sh);
-cudaError_t dense_prepare(const __half* T, int L, const DenseShape& sh, uint8_t* model, cudaStream_t st);
-cudaError_t dense_begin(const __half* logits, const DenseShape& sh, const uint8_t* model, uint8_t* scratch, const size_t* off,
-                        unsigned int* status, cudaStream_t st);
+int layers_per_group(int L, long long rows, int ncols);
+size_t dense_scratch_bytes(const DenseShape& sh, size_t* off /*[4]: P, Tb, mu, s1*/);
+size_t dense_model_bytes(const DenseShape& sh, size_t* off /*[2]: Nb_all, Tb_all*/);
+cudaError_t dense_prepare(const __half* T, const DenseShape& sh, uint8_t* model, const size_t* moff, cudaStream_t st);
 cudaError_t dense_softmax(const __half* logits, const DenseShape& sh, uint8_t* scratch, const size_t* off, cudaStream_t st);
+cudaError_t dense_layers(const __half* T, int l0, int nl, const DenseShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
+                         const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);   // events bracket the contraction
 // Linear-embedding predictor (Sec. 7.1).
 struct LinearShape {
     long long rows;
     int V, d, dm, tables, L;   // tables = 2*H per layer, dm = d_model (multiple of 64)
     int ldv;                   // V rounded up to 64
-    int ncols, ncols_pad;      // tables*d, rounded up to 256
-    int nt_all, nt_all_pad;    // L*tables, rounded up to 256
+    int ncols;                 // tables*d
+    int nt_all;                // L*tables
+    int group;                 // layers per contraction
+    bool resident;             // the context keeps A as bf16
 };
-size_t linear_model_bytes(const LinearShape& sh, size_t* off /*[2]*/);
-size_t linear_scratch_bytes(const LinearShape& sh, size_t* off /*[6]*/);
+size_t linear_model_bytes(const LinearShape& sh, size_t* off /*[3]*/);
+size_t linear_scratch_bytes(const LinearShape& sh, size_t* off /*[5]*/);
 cudaError_t linear_prepare(const __half* E, const __half* A, const __half* c, const LinearShape& sh, uint8_t* model,
                            const size_t* moff, unsigned int* status, cudaStream_t st);
 cudaError_t linear_begin(const __half* logits, const LinearShape& sh, const uint8_t* model, const size_t* moff,
                          uint8_t* scratch, const size_t* off, unsigned int* status, cudaStream_t st);
-cudaError_t linear_layer(const __half* A_layer, const LinearShape& sh, uint8_t* scratch, const size_t* off,
-                         unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
-cudaError_t dense_layer(const __half* T_layer, const DenseShape& sh, uint8_t* scratch, const size_t* off,
-                        unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);   // events bracket the contraction
+cudaError_t linear_layers(const __half* A, int l0, int nl, const LinearShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
+                          const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
 cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, cudaStream_t st);
 cudaError_t launch_encode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_decode(const CodecArgs& a, cudaStream_t st);

@@ -13,6 +13,7 @@
 // The decoder's words come through a ring in shared memory filled by asynchronous copies, so no
 // refill waits for global memory.
 #include <algorithm>
+#include <cstdlib>
 
 #include "plc_codec.cuh"
 
@@ -423,6 +424,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
                           : (encode ? coop_kernel<d, false, true> : coop_kernel<d, false, false>);
         const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
         int warps = items <= 2ll * sm_count() ? kCoopMaxWarps : kCoopMaxWarps / 2;
+        { static const char* e = getenv(dense ? "PLC_NWD" : "PLC_NW"); if (e) warps = atoi(e); }
         if (coop_smem(warps, a.sh.Kp, d, dense, encode) > 96 * 1024) warps = kCoopMaxWarps / 2;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

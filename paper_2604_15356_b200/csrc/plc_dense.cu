@@ -1,17 +1,20 @@
 // Full-vocabulary prediction (Def. 5 of the paper: KV^ = sum over the whole vocabulary of
 // P(t | t_<i) F(t_<i, t)) as a dense bf16 contraction on the 5th-generation tensor cores:
 //   MU[rows x (2H*d)] = P[rows x V] * Tb[(2H*d) x V]^T     per layer, fp32 accumulation in TMEM.
-// P = bf16(softmax(logits)); Tb = bf16(T) of the layer, transposed so that both operands are
-// K-major (V contiguous).  One CTA computes a 128 x 256 tile: a TMA producer thread fills a
-// 4-stage shared-memory ring (128B-swizzled boxes of 64 K-elements), one thread issues
-// tcgen05.mma (128x256x16) into 256 TMEM columns and releases ring slots with tcgen05.commit,
-// four warps read the accumulators back with tcgen05.ld and store the tile.  Single-CTA launch:
-// every TMA load lands in this CTA's own shared memory and the tensor maps cover this GPU's memory
-// only.  Every mbarrier wait is bounded; a wait that runs out sets an error bit and a CTA-wide
-// `failed` word: the producer stops and waits (bounded) for the copies it has in flight, the
-// epilogue stores nothing, and the CTA frees its TMEM and returns.
-// The variance term s1[row][table] = sum_v P[row][v] * bf16(||Tb_v||^2 / d) is a second launch of
-// the same kernel with a narrow N tile (one column per table).
+// P = bf16(softmax(logits)); Tb = bf16(T), transposed so that both operands are K-major (V contiguous).
+// One persistent CTA per SM walks 128 x 256 output tiles: a TMA producer thread fills a 4-stage
+// shared-memory ring (128B-swizzled boxes of 64 K-elements) across tile boundaries, one thread issues
+// tcgen05.mma (128 x N x 16, N <= 256) into one of two 256-column TMEM accumulators and releases ring
+// slots with tcgen05.commit, four warps read the other accumulator back with tcgen05.ld and store the
+// tile under the next tile's contraction.  Every output element is summed over K in one accumulator
+// in K order, whatever the number of rows or columns of the call: a row's prediction does not depend
+// on what else is in the batch (an encoder and a decoder may be called on different batches).
+// Single-CTA loads: every TMA load lands in this CTA's own shared memory and the tensor maps cover this
+// GPU's memory only.  Every mbarrier wait is bounded; a wait that runs out sets an error bit and a
+// CTA-wide `failed` word: all roles leave their loops, the producer waits (bounded) for the copies it
+// has in flight, nothing more is stored, and the CTA frees its TMEM and returns.
+// The variance terms s1[row][table] = sum_v P[row][v] * bf16(||Tb_v||^2 / d) are further columns of
+// the same contraction.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -82,32 +85,59 @@ __host__ __device__ constexpr uint32_t make_idesc(int bn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
 }
 
+// One range of output columns: column c is B row row0 + c of its map, stored as binary32 (out) or
+// bfloat16 (out16) with row pitch ldo.
+struct GemmSeg {
+    float* out;
+    __nv_bfloat16* out16;
+    long long ldo;
+    int ncols, row0, tiles;
+};
+struct GemmArgs {
+    GemmSeg seg[2];
+    int rows, num_kb, tiles_m, tiles_n;
+    unsigned int* status;
+};
+// Tiles are walked in groups of kTileGroup column tiles (row block next, column tile fastest): the CTAs
+// resident together then cover about 18 row blocks by 8 column tiles, the split of 148 tiles that
+// fetches least of both operands (each block of A once per group, each slab of B once per wave).
+constexpr int kTileGroup = 8;
+struct Tile { int m, seg, c0, n; };                        // row block, segment, first column, columns rounded up to 16
+__device__ __forceinline__ Tile tile_of(const GemmArgs& g, int id) {
+    const int per_group = g.tiles_m * kTileGroup, gi = id / per_group, r = id - gi * per_group;
+    const int wide = min(kTileGroup, g.tiles_n - gi * kTileGroup);
+    Tile t;
+    t.m = r / wide;
+    int nt = gi * kTileGroup + r % wide;
+    t.seg = nt >= g.seg[0].tiles;
+    if (t.seg) nt -= g.seg[0].tiles;
+    t.c0 = nt * kBN;
+    t.n = min(kBN, (g.seg[t.seg].ncols - t.c0 + 15) & ~15);
+    return t;
+}
+
 __global__ void __launch_bounds__(kGemmThreads, 1)
-dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                  float* __restrict__ out, long long ldo, int rows, int ncols, int num_kb, int bn, unsigned int* status) {
+dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b0,
+                  const __grid_constant__ CUtensorMap map_b1, const __grid_constant__ GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)kStages * kStageBytes);   // full[4], empty[4], tmem_full
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)kStages * kStageBytes);   // full[4], empty[4], tfull[2], tempty[2], drain
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
     volatile uint32_t* failed = tmem_slot + 1;        // set by any role whose wait ran out
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // Column tile fastest in launch order: the CTAs resident together then share their row blocks of A
-    // (each block of A is fetched from HBM once and found in L2 by the other column tiles), and B, the
-    // smaller operand, is what gets re-read from L2.
-    const int ntn = (int)gridDim.y;
-    const int lin = blockIdx.y * gridDim.x + blockIdx.x;
-    const int m0 = (lin / ntn) * kBM, n0 = (lin % ntn) * bn;
-    const uint32_t stage_tx = (uint32_t)(kABytes + bn * kBK * 2), idesc = make_idesc(bn);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages), tfull = smem_u32(bars + 2 * kStages);
+    const int total = g.tiles_m * g.tiles_n;
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages), tfull0 = smem_u32(bars + 2 * kStages),
+                   tempty0 = smem_u32(bars + 2 * kStages + 2), drain = smem_u32(bars + 2 * kStages + 4);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-        mbar_init(tfull, 1);
+        for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 4); }
+        mbar_init(drain, 1);
         *failed = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(256u) : "memory");
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2u * kBN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -119,53 +149,70 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
         // TMA producer
         int issued = 0;
         bool ok = true;
-        for (int kb = 0; kb < num_kb && ok; ++kb) {
-            const int s = kb % kStages;
-            const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
-            ok = !*failed && mbar_wait(empty0 + 8 * s, ph ^ 1u, status);
-            if (!ok) break;
-            mbar_expect_tx(full0 + 8 * s, stage_tx);
-            const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes);
-            tma_load_2d(sa, &map_a, kb * kBK, m0, full0 + 8 * s);
-            tma_load_2d(sa + kABytes, &map_b, kb * kBK, n0, full0 + 8 * s);
-            ++issued;
+        for (int id = blockIdx.x; id < total && ok; id += gridDim.x) {
+            const Tile t = tile_of(g, id);
+            const CUtensorMap* mb = t.seg ? &map_b1 : &map_b0;
+            const int brow = g.seg[t.seg].row0 + t.c0;
+            for (int kb = 0; kb < g.num_kb; ++kb) {
+                const int s = issued % kStages;
+                const uint32_t ph = (uint32_t)(issued / kStages) & 1u;
+                ok = !*failed && mbar_wait(empty0 + 8 * s, ph ^ 1u, g.status);
+                if (!ok) break;
+                mbar_expect_tx(full0 + 8 * s, kStageBytes);
+                const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes);
+                tma_load_2d(sa, &map_a, kb * kBK, t.m * kBM, full0 + 8 * s);
+                tma_load_2d(sa + kABytes, mb, kb * kBK, brow, full0 + 8 * s);
+                ++issued;
+            }
         }
-        if (!ok) {
-            // drain: the copies already issued still land in this CTA's shared memory
-            *failed = 1u;
-            for (int kb = issued > kStages ? issued - kStages : 0; kb < issued; ++kb)
-                mbar_wait(full0 + 8 * (kb % kStages), (uint32_t)(kb / kStages) & 1u, status);
-        }
+        if (!ok) *failed = 1u;
+        // the copies still in flight (none after a complete run: the last tile has consumed them) land before the CTA ends
+        if (!ok)
+            for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i)
+                mbar_wait(full0 + 8 * (i % kStages), (uint32_t)(i / kStages) & 1u, g.status);
     } else if (warp == 1 && lane == 0) {
         // MMA issuer
+        int used = 0, turn = 0;
         bool ok = true;
-        for (int kb = 0; kb < num_kb && ok; ++kb) {
-            const int s = kb % kStages;
-            const uint32_t ph = (uint32_t)(kb / kStages) & 1u;
-            ok = mbar_wait(full0 + 8 * s, ph, status);
-            if (!ok) { *failed = 1u; __threadfence_block(); break; }
+        for (int id = blockIdx.x; id < total && ok; id += gridDim.x, ++turn) {
+            const Tile t = tile_of(g, id);
+            const uint32_t idesc = make_idesc(t.n), acc = (uint32_t)turn & 1u, tmem_d = tmem_base + acc * kBN;
+            ok = !*failed && mbar_wait(tempty0 + 8 * acc, ((uint32_t)(turn >> 1) & 1u) ^ 1u, g.status);   // the epilogue has read it
+            if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes);
-            const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kABytes);
+            for (int kb = 0; kb < g.num_kb; ++kb, ++used) {
+                const int s = used % kStages;
+                ok = mbar_wait(full0 + 8 * s, (uint32_t)(used / kStages) & 1u, g.status);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t sa = smem_u32(smem + (size_t)s * kStageBytes);
+                const uint64_t da = smem_desc_sw128(sa), db = smem_desc_sw128(sa + kABytes);
 #pragma unroll
-            for (int k = 0; k < kBK / kUmmaK; ++k)
-                umma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, (kb | k) ? 1u : 0u);
-            umma_commit(empty0 + 8 * s);              // frees the ring slot when these MMAs have read it
+                for (int k = 0; k < kBK / kUmmaK; ++k)
+                    umma_bf16(tmem_d, da + 2 * k, db + 2 * k, idesc, (kb | k) ? 1u : 0u);
+                umma_commit(empty0 + 8 * s);          // frees the ring slot when these MMAs have read it
+            }
+            if (ok) umma_commit(tfull0 + 8 * acc);
         }
-        umma_commit(tfull);                           // arrives when the MMAs issued so far are done (all of them, or none pending)
+        if (!ok) *failed = 1u;
+        umma_commit(drain);                           // nothing issued is running when the TMEM is freed
+        mbar_wait(drain, 0, g.status);
     } else if (warp >= 2) {
         // epilogue: warp w reads TMEM lanes 32*(w%4) ... +31
-        bool ok = mbar_wait(tfull, 0, status);
-        if (!ok) *failed = 1u;
-        ok = ok && !*failed;                          // partial accumulators are never stored
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int q = warp & 3;
-        const int row = m0 + q * 32 + lane;
-        const bool vec_ok = ((ldo | ncols) & 3) == 0;
-        if (ok) {
-            for (int c = 0; c * 32 < bn; ++c) {
+        int turn = 0;
+        for (int id = blockIdx.x; id < total; id += gridDim.x, ++turn) {
+            const Tile t = tile_of(g, id);
+            const uint32_t acc = (uint32_t)turn & 1u;
+            const bool ok = !*failed && mbar_wait(tfull0 + 8 * acc, (uint32_t)(turn >> 1) & 1u, g.status);
+            if (!__all_sync(kFull, ok)) { *failed = 1u; break; }              // partial accumulators are never stored
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const GemmSeg& sg = g.seg[t.seg];
+            const int row = t.m * kBM + q * 32 + lane;
+            const bool vec_ok = ((sg.ldo | sg.ncols) & (sg.out16 ? 7 : 3)) == 0;
+            for (int c = 0; c * 32 < t.n; ++c) {
                 uint32_t r[32];
-                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32);
+                const uint32_t taddr = tmem_base + acc * kBN + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 32);
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                     "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -176,29 +223,50 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
                       "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                     : "r"(taddr) : "memory");
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const int col = n0 + c * 32;
-                if (row < rows && col < ncols) {
-                    float* dr = out + (long long)row * ldo + col;
+                const int col = t.c0 + c * 32, left = sg.ncols - col;
+                if (row >= g.rows) continue;
+                if (sg.out16) {
+                    __nv_bfloat16* dr = sg.out16 + (long long)row * sg.ldo + col;
+                    if (vec_ok) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (8 * j < left) {
+                                __nv_bfloat162 o[4];
+#pragma unroll
+                                for (int i = 0; i < 4; ++i)
+                                    o[i] = __floats2bfloat162_rn(__uint_as_float(r[8 * j + 2 * i]), __uint_as_float(r[8 * j + 2 * i + 1]));
+                                reinterpret_cast<uint4*>(dr)[j] = *reinterpret_cast<const uint4*>(o);
+                            }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j)
+                            if (j < left) dr[j] = __float2bfloat16_rn(__uint_as_float(r[j]));
+                    }
+                } else {
+                    float* dr = sg.out + (long long)row * sg.ldo + col;
                     if (vec_ok) {
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            if (col + 4 * j < ncols)
+                            if (4 * j < left)
                                 reinterpret_cast<float4*>(dr)[j] = make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
                                                                                 __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
                     } else {
 #pragma unroll
                         for (int j = 0; j < 32; ++j)
-                            if (col + j < ncols) dr[j] = __uint_as_float(r[j]);
+                            if (j < left) dr[j] = __uint_as_float(r[j]);
                     }
                 }
             }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tempty0 + 8 * acc) : "memory");
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 1) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2u * kBN) : "memory");
     }
 }
 
@@ -353,17 +421,34 @@ bool make_map(CUtensorMap* map, void* base, uint64_t inner, uint64_t outer, uint
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// out[rows x ncols] (fp32, pitch ldo) = A[rows x K] * B[nrows_b x K]^T, both bf16 with row pitch ldk (a
-// multiple of 64; K = ldk, zero padded); nrows_b is a multiple of the N tile bn.
-cudaError_t launch_gemm(const __nv_bfloat16* A, long long rows, const __nv_bfloat16* B, int nrows_b, int ldk, int bn,
-                        float* out, long long ldo, int ncols, unsigned int* status, cudaStream_t st) {
-    CUtensorMap ma, mb;
+// A column range of a contraction's result: ncols rows of B (bf16, row pitch as A's) from row0 on, and
+// where their columns go.
+struct GemmOut {
+    const __nv_bfloat16* B;
+    int nrows_b, row0, ncols;
+    float* out;
+    __nv_bfloat16* out16;
+    long long ldo;
+};
+// out[rows x ncols] = A[rows x K] * B[.. x K]^T for one or two column ranges, A and B bf16 with row pitch
+// ldk (a multiple of 64; K = ldk, zero padded).
+cudaError_t launch_gemm(const __nv_bfloat16* A, long long rows, int ldk, const GemmOut* o, int n_out, unsigned int* status, cudaStream_t st) {
+    CUtensorMap ma, mb[2];
     if (!make_map(&ma, const_cast<__nv_bfloat16*>(A), (uint64_t)ldk, (uint64_t)rows, (uint64_t)ldk, kBM)) return cudaErrorUnknown;
-    if (!make_map(&mb, const_cast<__nv_bfloat16*>(B), (uint64_t)ldk, (uint64_t)nrows_b, (uint64_t)ldk, (uint32_t)bn)) return cudaErrorUnknown;
+    GemmArgs g{};
+    for (int i = 0; i < n_out; ++i) {
+        if (!make_map(&mb[i], const_cast<__nv_bfloat16*>(o[i].B), (uint64_t)ldk, (uint64_t)o[i].nrows_b, (uint64_t)ldk, kBN)) return cudaErrorUnknown;
+        g.seg[i] = GemmSeg{o[i].out, o[i].out16, o[i].ldo, o[i].ncols, o[i].row0, (o[i].ncols + kBN - 1) / kBN};
+    }
+    if (n_out < 2) mb[1] = mb[0];
+    g.rows = (int)rows; g.num_kb = ldk / kBK; g.status = status;
+    g.tiles_m = (int)((rows + kBM - 1) / kBM); g.tiles_n = g.seg[0].tiles + g.seg[1].tiles;
     cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
     if (e != cudaSuccess) return e;
-    dim3 g((unsigned)((rows + kBM - 1) / kBM), (unsigned)(nrows_b / bn));
-    dense_gemm_kernel<<<g, kGemmThreads, kGemmSmem, st>>>(ma, mb, out, ldo, (int)rows, ncols, ldk / kBK, bn, status);
+    const long long tiles = (long long)g.tiles_m * g.tiles_n;
+    if (tiles >= (1ll << 31)) return cudaErrorInvalidValue;
+    const int sms = dense_sm_count();
+    dense_gemm_kernel<<<(unsigned)(tiles < sms ? tiles : sms), kGemmThreads, kGemmSmem, st>>>(ma, mb[0], mb[1], g);
     count_launch();
     return cudaGetLastError();
 }
@@ -376,10 +461,6 @@ __global__ void __launch_bounds__(256) cvt_f16_bf16_kernel(const __half* __restr
         const long long r = i / ld; const int c = (int)(i % ld);
         dst[i] = __float2bfloat16_rn(c < cols ? __half2float(src[r * cols + c]) : 0.f);
     }
-}
-__global__ void __launch_bounds__(256) cvt_f32_bf16_kernel(const float* __restrict__ src, long long n, __nv_bfloat16* __restrict__ dst) {
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
-        dst[i] = __float2bfloat16_rn(src[i]);
 }
 // Nb[t][v] = bf16(sum_j (tlin[v][t*d + j] + c[t][j])^2 / d): one warp per (v, t).
 __global__ void __launch_bounds__(256) tlin_norm_kernel(const float* __restrict__ tlin, long long ld_t, const __half* __restrict__ c,
@@ -400,40 +481,58 @@ __global__ void __launch_bounds__(256) tlin_norm_kernel(const float* __restrict_
 
 }  // namespace
 
-size_t dense_scratch_bytes(const DenseShape& sh, size_t* off /*[5]*/) {
-    auto up = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
+namespace {
+size_t up1k(size_t x) { return (x + 1023) & ~(size_t)1023; }
+
+cudaError_t transpose_tables(const __half* T, int tables, const DenseShape& sh, __nv_bfloat16* Tb, cudaStream_t st) {
+    for (int t0 = 0; t0 < tables; t0 += 32768) {                       // the grid's z extent is limited
+        const int nt = tables - t0 < 32768 ? tables - t0 : 32768;
+        transpose_bf16_kernel<<<dim3((sh.ldv + 31) / 32, sh.d / 32, nt), 256, 0, st>>>(T + (size_t)t0 * sh.V * sh.d, nt, sh.V, sh.d, sh.ldv,
+                                                                                      Tb + (size_t)t0 * sh.d * sh.ldv);
+        count_launch();
+    }
+    return cudaGetLastError();
+}
+}  // namespace
+
+// Layers whose predictions one contraction forms (and one coder launch then reads): as many as keep mu
+// within 1 GB.  Small calls take all layers at once: a layer of theirs fills neither the SMs nor the
+// coder (2048 positions x 8 layers, linear variant: 128 chunks a layer on 148 SMs).
+int layers_per_group(int L, long long rows, int ncols) {
+    const long long per_layer = rows * ncols * 4;
+    const long long n = per_layer > 0 ? (1ll << 30) / per_layer : L;
+    return (int)(n < 1 ? 1 : n > L ? L : n);
+}
+
+size_t dense_scratch_bytes(const DenseShape& sh, size_t* off /*[4]*/) {
     size_t o = 0;
-    off[0] = o; o += up((size_t)sh.rows * sh.ldv * 2);                 // P
-    off[1] = o; o += up((size_t)sh.ncols_pad * sh.ldv * 2);            // Tb
-    off[2] = o;                                                        // (unused)
-    off[3] = o; o += up((size_t)sh.rows * sh.ncols * 4);               // mu
-    off[4] = o; o += up((size_t)sh.rows * sh.nt_all * 4);              // s1 of every (layer, table)
+    off[0] = o; o += up1k((size_t)sh.rows * sh.ldv * 2);                          // P
+    off[1] = o; o += sh.resident ? 0 : up1k((size_t)sh.ncols * sh.ldv * 2);       // Tb of one layer
+    off[2] = o; o += up1k((size_t)sh.rows * sh.ncols * sh.group * 4);             // mu of a group of layers
+    off[3] = o; o += up1k((size_t)sh.rows * sh.nt_all * 4);                       // s1 of every (layer, table)
     return o;
 }
 
-size_t dense_model_bytes(const DenseShape& sh) { return (size_t)sh.nt_all_pad * sh.ldv * 2; }
-
-// Creation: Nb_all[l * tables + t][v] = bf16(sum_j bf16(T[l][t][v][j])^2 / d) for every layer; rows beyond
-// L * tables and columns beyond V are zero.
-cudaError_t dense_prepare(const __half* T, int L, const DenseShape& sh, uint8_t* model, cudaStream_t st) {
-    __nv_bfloat16* Nb = reinterpret_cast<__nv_bfloat16*>(model);
-    cudaError_t e = cudaMemsetAsync(Nb, 0, dense_model_bytes(sh), st);
-    if (e != cudaSuccess) return e;
-    const long long nrows = (long long)L * sh.tables * sh.V;
-    rownorm_bf16_kernel<<<blocks_for(nrows * 32), 256, 0, st>>>(T, nrows, sh.V, sh.d, sh.ldv, Nb);
-    count_launch();
-    return cudaGetLastError();
+size_t dense_model_bytes(const DenseShape& sh, size_t* off /*[2]: Nb_all, Tb_all*/) {
+    size_t o = 0;
+    off[0] = o; o += up1k((size_t)sh.nt_all * sh.ldv * 2);
+    off[1] = o; o += sh.resident ? up1k((size_t)sh.nt_all * sh.d * sh.ldv * 2) : 0;
+    return o;
 }
 
-// Per call: P = bf16(softmax(logits)) and the variance term of every layer in one contraction,
-// s1[row][l * tables + t] = sum_v P[row][v] Nb_all[l * tables + t][v].
-cudaError_t dense_begin(const __half* logits, const DenseShape& sh, const uint8_t* model, uint8_t* scratch, const size_t* off,
-                        unsigned int* status, cudaStream_t st) {
-    cudaError_t e = dense_softmax(logits, sh, scratch, off, st);
+// Creation: Nb_all[l * tables + t][v] = bf16(sum_j bf16(T[l][t][v][j])^2 / d) for every layer (columns beyond V
+// are zero) and, where the context keeps it, the transposed bf16 table of every layer.
+cudaError_t dense_prepare(const __half* T, const DenseShape& sh, uint8_t* model, const size_t* moff, cudaStream_t st) {
+    __nv_bfloat16* Nb = reinterpret_cast<__nv_bfloat16*>(model + moff[0]);
+    cudaError_t e = cudaMemsetAsync(Nb, 0, (size_t)sh.nt_all * sh.ldv * 2, st);
     if (e != cudaSuccess) return e;
-    return launch_gemm(reinterpret_cast<const __nv_bfloat16*>(scratch + off[0]), sh.rows,
-                       reinterpret_cast<const __nv_bfloat16*>(model), sh.nt_all_pad, sh.ldv, 256,
-                       reinterpret_cast<float*>(scratch + off[4]), sh.nt_all, sh.nt_all, status, st);
+    const long long nrows = (long long)sh.nt_all * sh.V;
+    rownorm_bf16_kernel<<<blocks_for(nrows * 32), 256, 0, st>>>(T, nrows, sh.V, sh.d, sh.ldv, Nb);
+    count_launch();
+    e = cudaGetLastError();
+    if (e == cudaSuccess && sh.resident)
+        e = transpose_tables(T, sh.nt_all, sh, reinterpret_cast<__nv_bfloat16*>(model + moff[1]), st);
+    return e;
 }
 
 cudaError_t dense_softmax(const __half* logits, const DenseShape& sh, uint8_t* scratch, const size_t* off, cudaStream_t st) {
@@ -448,58 +547,55 @@ cudaError_t dense_softmax(const __half* logits, const DenseShape& sh, uint8_t* s
     return cudaGetLastError();
 }
 
-// Prediction of one layer: fills mu [rows][ncols] in the scratch (the variance term of every layer was
-// formed by dense_begin).
-cudaError_t dense_layer(const __half* T_layer, const DenseShape& sh, uint8_t* scratch, const size_t* off,
-                        unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
-    __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(scratch + off[0]);
-    __nv_bfloat16* Tb = reinterpret_cast<__nv_bfloat16*>(scratch + off[1]);
-    float* mu = reinterpret_cast<float*>(scratch + off[3]);
-    cudaError_t e;
-    if (sh.ncols_pad > sh.ncols) {       // rows of Tb beyond the real columns must read as zero
-        e = cudaMemsetAsync(Tb + (size_t)sh.ncols * sh.ldv, 0, (size_t)(sh.ncols_pad - sh.ncols) * sh.ldv * 2, st);
+// Predictions of layers [l0, l0 + nl): mu [rows][sh.group * ncols] in the scratch; the first group (l0 = 0)
+// also forms the variance terms of every layer, s1[row][l * tables + t] = sum_v P[row][v] Nb_all[l * tables + t][v].
+cudaError_t dense_layers(const __half* T, int l0, int nl, const DenseShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
+                         const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
+    const __nv_bfloat16* P = reinterpret_cast<const __nv_bfloat16*>(scratch + off[0]);
+    GemmOut o[2] = {};
+    if (sh.resident) {
+        o[0] = GemmOut{reinterpret_cast<const __nv_bfloat16*>(model + moff[1]), sh.nt_all * sh.d, l0 * sh.ncols, nl * sh.ncols, nullptr, nullptr, 0};
+    } else {
+        __nv_bfloat16* Tb = reinterpret_cast<__nv_bfloat16*>(scratch + off[1]);
+        const cudaError_t e = transpose_tables(T + (size_t)l0 * sh.tables * sh.V * sh.d, sh.tables, sh, Tb, st);
         if (e != cudaSuccess) return e;
+        o[0] = GemmOut{Tb, sh.ncols, 0, sh.ncols, nullptr, nullptr, 0};
     }
-    dim3 tg((sh.ldv + 31) / 32, sh.d / 32, sh.tables);
-    transpose_bf16_kernel<<<tg, 256, 0, st>>>(T_layer, sh.tables, sh.V, sh.d, sh.ldv, Tb);
-    count_launch();
+    o[0].out = reinterpret_cast<float*>(scratch + off[2]); o[0].ldo = (long long)sh.group * sh.ncols;
+    o[1] = GemmOut{reinterpret_cast<const __nv_bfloat16*>(model + moff[0]), sh.nt_all, 0, sh.nt_all,
+                   reinterpret_cast<float*>(scratch + off[3]), nullptr, sh.nt_all};
     if (ev0) cudaEventRecord(ev0, st);
-    e = launch_gemm(P, sh.rows, Tb, sh.ncols_pad, sh.ldv, kBN, mu, (long long)sh.ncols, sh.ncols, status, st);
+    const cudaError_t e = launch_gemm(P, sh.rows, sh.ldv, o, l0 == 0 ? 2 : 1, status, st);
     if (ev1) cudaEventRecord(ev1, st);
     return e;
 }
 
 // ---------------------------------------------------------------------------------------------
 // Linear-embedding predictor (Sec. 7.1): KV^ ~ c + A Ebar, Ebar = sum_v p_v E(v).  Two chained
-// contractions on the same tensor-core kernel: Ebar = P * E (once per call, shared by all layers),
-// then per layer mu = Ebar * A_layer^T (K = d_model); the variance term of all layers is one more
-// contraction of P with the table of candidate norms ||c + A E(v)||^2 / d built at creation.
+// contractions on the same tensor-core kernel: Ebar = P * E (once per call, shared by all layers; the
+// variance terms of all layers, P times the table of candidate norms ||c + A E(v)||^2 / d built at
+// creation, are further columns of it), then mu = Ebar * A^T for a group of layers (K = d_model).
 
-size_t linear_model_bytes(const LinearShape& sh, size_t* off /*[2]: Ebt, NbAll*/) {
-    auto up = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
+size_t linear_model_bytes(const LinearShape& sh, size_t* off /*[3]: Ebt, NbAll, Ab_all*/) {
     size_t o = 0;
-    off[0] = o; o += up((size_t)sh.dm * sh.ldv * 2);
-    off[1] = o; o += up((size_t)sh.nt_all_pad * sh.ldv * 2);
+    off[0] = o; o += up1k((size_t)sh.dm * sh.ldv * 2);
+    off[1] = o; o += up1k((size_t)sh.nt_all * sh.ldv * 2);
+    off[2] = o; o += sh.resident ? up1k((size_t)sh.L * sh.ncols * sh.dm * 2) : 0;
     return o;
 }
 
-size_t linear_scratch_bytes(const LinearShape& sh, size_t* off /*[6]: P, Ef, Eb16, s1, Ab, mu*/) {
-    auto up = [](size_t x) { return (x + 1023) & ~(size_t)1023; };
+size_t linear_scratch_bytes(const LinearShape& sh, size_t* off /*[5]: P, Eb16, s1, Ab, mu*/) {
     size_t o = 0;
-    off[0] = o; o += up((size_t)sh.rows * sh.ldv * 2);
-    off[1] = o; o += up((size_t)sh.rows * sh.dm * 4);
-    off[2] = o; o += up((size_t)sh.rows * sh.dm * 2);
-    off[3] = o; o += up((size_t)sh.rows * sh.nt_all * 4);
-    off[4] = o; o += up((size_t)sh.ncols_pad * sh.dm * 2);
-    off[5] = o; o += up((size_t)sh.rows * sh.ncols * 4);
+    off[0] = o; o += up1k((size_t)sh.rows * sh.ldv * 2);
+    off[1] = o; o += up1k((size_t)sh.rows * sh.dm * 2);
+    off[2] = o; o += up1k((size_t)sh.rows * sh.nt_all * 4);
+    off[3] = o; o += sh.resident ? 0 : up1k((size_t)sh.ncols * sh.dm * 2);
+    off[4] = o; o += up1k((size_t)sh.rows * sh.ncols * sh.group * 4);
     return o;
 }
 
-static int tile_for(int n) { return n % 256 == 0 ? 256 : (n % 128 == 0 ? 128 : 64); }
-
-
-// Creation: E transposed to bf16 and the norm table of every (layer, table).  Allocates (and
-// frees) its temporaries; synchronises the stream.
+// Creation: E transposed to bf16, A as bf16 where the context keeps it, and the norm table of every
+// (layer, table).  Allocates (and frees) its temporaries; synchronises the stream.
 cudaError_t linear_prepare(const __half* E, const __half* A, const __half* c, const LinearShape& sh, uint8_t* model,
                            const size_t* moff, unsigned int* status, cudaStream_t st) {
     __nv_bfloat16* Ebt = reinterpret_cast<__nv_bfloat16*>(model + moff[0]);
@@ -507,10 +603,9 @@ cudaError_t linear_prepare(const __half* E, const __half* A, const __half* c, co
     __nv_bfloat16 *Eb = nullptr, *Ab = nullptr;
     float* tlin = nullptr;
     cudaError_t e = cudaMalloc(&Eb, (size_t)sh.V * sh.dm * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&Ab, (size_t)sh.ncols_pad * sh.dm * 2);
+    if (e == cudaSuccess && !sh.resident) e = cudaMalloc(&Ab, (size_t)sh.ncols * sh.dm * 2);
     if (e == cudaSuccess) e = cudaMalloc(&tlin, (size_t)sh.V * sh.ncols * 4);
-    if (e == cudaSuccess) e = cudaMemsetAsync(NbAll, 0, (size_t)sh.nt_all_pad * sh.ldv * 2, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(Ab, 0, (size_t)sh.ncols_pad * sh.dm * 2, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(NbAll, 0, (size_t)sh.nt_all * sh.ldv * 2, st);
     if (e == cudaSuccess) {
         dim3 tg((sh.ldv + 31) / 32, sh.dm / 32, 1);
         transpose_bf16_kernel<<<tg, 256, 0, st>>>(E, 1, sh.V, sh.dm, sh.ldv, Ebt);
@@ -518,8 +613,10 @@ cudaError_t linear_prepare(const __half* E, const __half* A, const __half* c, co
         count_launch(2);
         for (int l = 0; l < sh.L && e == cudaSuccess; ++l) {
             const __half* Al = A + (size_t)l * sh.ncols * sh.dm;
-            cvt_f16_bf16_kernel<<<blocks_for((long long)sh.ncols * sh.dm), 256, 0, st>>>(Al, sh.ncols, sh.dm, sh.dm, Ab);
-            e = launch_gemm(Eb, sh.V, Ab, sh.ncols_pad, sh.dm, 256, tlin, sh.ncols, sh.ncols, status, st);
+            __nv_bfloat16* Abl = sh.resident ? reinterpret_cast<__nv_bfloat16*>(model + moff[2]) + (size_t)l * sh.ncols * sh.dm : Ab;
+            cvt_f16_bf16_kernel<<<blocks_for((long long)sh.ncols * sh.dm), 256, 0, st>>>(Al, sh.ncols, sh.dm, sh.dm, Abl);
+            const GemmOut o{Abl, sh.ncols, 0, sh.ncols, tlin, nullptr, sh.ncols};
+            e = launch_gemm(Eb, sh.V, sh.dm, &o, 1, status, st);
             if (e != cudaSuccess) break;
             const long long pairs = (long long)sh.V * sh.tables;
             tlin_norm_kernel<<<blocks_for(pairs * 32), 256, 0, st>>>(
@@ -539,31 +636,27 @@ cudaError_t linear_begin(const __half* logits, const LinearShape& sh, const uint
     DenseShape ds{}; ds.rows = sh.rows; ds.V = sh.V; ds.ldv = sh.ldv;
     cudaError_t e = dense_softmax(logits, ds, scratch, off, st);
     if (e != cudaSuccess) return e;
-    const __nv_bfloat16* P = reinterpret_cast<const __nv_bfloat16*>(scratch + off[0]);
-    float* Ef = reinterpret_cast<float*>(scratch + off[1]);
-    __nv_bfloat16* Eb16 = reinterpret_cast<__nv_bfloat16*>(scratch + off[2]);
-    float* s1 = reinterpret_cast<float*>(scratch + off[3]);
-    e = launch_gemm(P, sh.rows, reinterpret_cast<const __nv_bfloat16*>(model + moff[0]), sh.dm, sh.ldv, tile_for(sh.dm),
-                    Ef, sh.dm, sh.dm, status, st);
-    if (e != cudaSuccess) return e;
-    cvt_f32_bf16_kernel<<<blocks_for(sh.rows * sh.dm), 256, 0, st>>>(Ef, sh.rows * sh.dm, Eb16);
-    count_launch();
-    return launch_gemm(P, sh.rows, reinterpret_cast<const __nv_bfloat16*>(model + moff[1]), sh.nt_all_pad, sh.ldv, 256,
-                       s1, sh.nt_all, sh.nt_all, status, st);
+    const GemmOut o[2] = {
+        {reinterpret_cast<const __nv_bfloat16*>(model + moff[0]), sh.dm, 0, sh.dm, nullptr, reinterpret_cast<__nv_bfloat16*>(scratch + off[1]), sh.dm},
+        {reinterpret_cast<const __nv_bfloat16*>(model + moff[1]), sh.nt_all, 0, sh.nt_all, reinterpret_cast<float*>(scratch + off[2]), nullptr, sh.nt_all}};
+    return launch_gemm(reinterpret_cast<const __nv_bfloat16*>(scratch + off[0]), sh.rows, sh.ldv, o, 2, status, st);
 }
 
-// Per layer: mu [rows][2H*d] = Ebar * A_layer^T (the bias c is added where mu is read).
-cudaError_t linear_layer(const __half* A_layer, const LinearShape& sh, uint8_t* scratch, const size_t* off,
-                         unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
-    __nv_bfloat16* Ab = reinterpret_cast<__nv_bfloat16*>(scratch + off[4]);
-    cudaError_t e = cudaSuccess;
-    if (sh.ncols_pad > sh.ncols) e = cudaMemsetAsync(Ab + (size_t)sh.ncols * sh.dm, 0, (size_t)(sh.ncols_pad - sh.ncols) * sh.dm * 2, st);
-    if (e != cudaSuccess) return e;
-    cvt_f16_bf16_kernel<<<blocks_for((long long)sh.ncols * sh.dm), 256, 0, st>>>(A_layer, sh.ncols, sh.dm, sh.dm, Ab);
-    count_launch();
+// Layers [l0, l0 + nl): mu [rows][sh.group * ncols] = Ebar * A^T (the bias c is added where mu is read).
+cudaError_t linear_layers(const __half* A, int l0, int nl, const LinearShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
+                          const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1) {
+    GemmOut o{};
+    if (sh.resident) {
+        o = GemmOut{reinterpret_cast<const __nv_bfloat16*>(model + moff[2]), sh.L * sh.ncols, l0 * sh.ncols, nl * sh.ncols, nullptr, nullptr, 0};
+    } else {
+        __nv_bfloat16* Ab = reinterpret_cast<__nv_bfloat16*>(scratch + off[3]);
+        cvt_f16_bf16_kernel<<<blocks_for((long long)sh.ncols * sh.dm), 256, 0, st>>>(A + (size_t)l0 * sh.ncols * sh.dm, sh.ncols, sh.dm, sh.dm, Ab);
+        count_launch();
+        o = GemmOut{Ab, sh.ncols, 0, sh.ncols, nullptr, nullptr, 0};
+    }
+    o.out = reinterpret_cast<float*>(scratch + off[4]); o.ldo = (long long)sh.group * sh.ncols;
     if (ev0) cudaEventRecord(ev0, st);
-    e = launch_gemm(reinterpret_cast<const __nv_bfloat16*>(scratch + off[2]), sh.rows, Ab, sh.ncols_pad, sh.dm, 256,
-                    reinterpret_cast<float*>(scratch + off[5]), sh.ncols, sh.ncols, status, st);
+    const cudaError_t e = launch_gemm(reinterpret_cast<const __nv_bfloat16*>(scratch + off[1]), sh.rows, sh.dm, &o, 1, status, st);
     if (ev1) cudaEventRecord(ev1, st);
     return e;
 }
