@@ -35,6 +35,16 @@ bool build_coder_tables(CoderTables* t) {
             if (first[at] == 0xff) first[at] = (uint8_t)z;
             if (z > first[at] + 1) return false;
         }
+        if (id < kWideFrom) {
+            memcpy(t->wide.first[id], first, sizeof(t->wide.first[id]));
+            memcpy(t->wide.fc[id], t->dec.fc[id], sizeof(t->wide.fc[id]));
+        } else {
+            for (int at = 0; at < 256; ++at) {
+                if (first[at] == 0xff) continue;
+                const int z0 = first[at];
+                t->wide.wide[id - kWideFrom][at] = make_uint2(f[z0] | (c[z0] << 16), (z0 + 1 < kNumSym ? f[z0 + 1] : 0u) | ((uint32_t)z0 << 16));
+            }
+        }
     }
     return true;
 }

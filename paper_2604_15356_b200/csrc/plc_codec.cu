@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const Co
             } else {
                 int s, qp;
                 class_params(q, s, qp);
-                decode_position<G>(sym, s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, read_word, rp, lc);
+                decode_position<G>(sym, s, Lookup{tb.first[qp - kQMin], tb.fc[qp - kQMin]}, x, read_word, rp, lc);
 #pragma unroll
                 for (int g = 0; g < G; ++g) out[g] = __fmaf_rn((float)sym[g], delta_p, mu[g]);
             }

@@ -13,6 +13,10 @@
 //     r = 2^15 - slot as a binary32 number, its exponent and top four mantissa bits index a byte table
 //     that holds the smallest symbol of that interval, and no interval of any of the 40 tables holds
 //     more than one symbol boundary (checked on the host for every slot when the tables are built).
+//     The eight tables that positions with bit planes use also exist in a wide form with everything an
+//     interval needs in one 8-byte entry (kernels with one coder a block have room for it).
+// Cycles of one warp alone, four steps with four planes each: encoding 618 before the state's chain was
+// taken out of the words' places, decoding 1080 before the wide form and the refill window.
 #pragma once
 #include <type_traits>
 
@@ -28,8 +32,13 @@ struct EncTables { EncEntry enc[kNumTables][kNumSym]; };
 constexpr int kFcStride = kNumSym + 4;
 struct DecTables { uint8_t first[kNumTables][256]; uint32_t fc[kNumTables][kFcStride]; };
 static_assert(sizeof(EncTables) % 16 == 0 && sizeof(DecTables) % 16 == 0, "tables are copied in 16-byte pieces");
-// Both, as a context keeps them in device memory.
-struct CoderTables { EncTables enc; DecTables dec; };
+// Decoder tables with the wide form (f0 | c0 << 16, f1 | z0 << 16: an interval's first symbol z0 and the
+// next) for table ids 8 .. 15, the ids of classes with bit planes; the others as above.
+constexpr int kWideFrom = 8 - kQMin;
+struct WideDecTables { uint8_t first[kWideFrom][256]; uint32_t fc[kWideFrom][kFcStride]; uint2 wide[kNumTables - kWideFrom][256]; };
+static_assert(sizeof(WideDecTables) % 16 == 0, "tables are copied in 16-byte pieces");
+// All of them, as a context keeps them in device memory.
+struct CoderTables { EncTables enc; DecTables dec; WideDecTables wide; };
 bool build_coder_tables(CoderTables* t);             // host; false if an interval held two boundaries
 
 #ifdef __CUDACC__
@@ -153,14 +162,21 @@ __device__ __forceinline__ bool split_symbols(const int (&sym)[G], int S, int (&
 // new wp.
 template <int G>
 __device__ __forceinline__ int push_position(const Prepared<G>& pr, int S, uint32_t& x, uint16_t* __restrict__ stage, int wp, const LaneCode& lc) {
+    // the state's chain first, the words' places (votes and counts) after it, so that no step waits for them
+    uint32_t low[G], emask[G];
+    bool emit[G];
+#pragma unroll
+    for (int g = G - 1; g >= 0; --g) {
+        emit[g] = x >= (pr.e[g].fc << 17);                 // f << 17: the count above f is shifted out
+        emask[g] = __ballot_sync(kFull, emit[g]);
+        low[g] = x;
+        x = push_state(x, emit[g], pr.e[g]);
+    }
     int base[G];
 #pragma unroll
     for (int g = G - 1; g >= 0; --g) {
-        const bool emit = x >= (pr.e[g].fc << 17);         // f << 17: the count above f is shifted out
-        const uint32_t emask = __ballot_sync(kFull, emit);
-        wp -= __popc(emask);
-        if (emit) stage[wp + __popc(emask & lc.lt)] = (uint16_t)x;
-        x = push_state(x, emit, pr.e[g]);
+        wp -= __popc(emask[g]);
+        if (emit[g]) stage[wp + __popc(emask[g] & lc.lt)] = (uint16_t)low[g];
         wp -= 2 * S;
         base[g] = wp - 2 * S * g;                          // lane j = g S + b of a group: halfword base + 2 j
     }
@@ -225,25 +241,45 @@ __device__ __forceinline__ int encode_position(const int (&sym)[G], int S, const
     return push_position<G>(pr, S, x, stage, wp, lc);
 }
 
-// Symbol of a slot: its fc entry and its place in the alphabet.
-__device__ __forceinline__ uint32_t find_symbol(uint32_t x, const uint8_t* first, const uint32_t* fcs, int& zz) {
-    const uint32_t slot = x & (kProbM - 1u);
-    const float r = 8421376.0f - __uint_as_float(0x4b000000u | slot);      // 2^23 + 2^15 - (2^23 + slot), exact
-    const int z = first[(__float_as_uint(r) >> 19) - 127u * 16u];
-    const uint32_t a = fcs[z], b = fcs[z + 1];
-    const bool next = slot >= (b >> 16);
-    zz = next ? z + 1 : z;
-    return next ? b : a;
+// One decoder step before its refill: the symbol (place in the alphabet) of state x and the next state.
+// r = 2^15 - slot as a float: 2^23 + 2^15 - (2^23 + slot), exact; its bits from the fourth mantissa bit up
+// number the intervals.
+__device__ __forceinline__ int interval_of(uint32_t slot) {
+    const float r = 8421376.0f - __uint_as_float(0x4b000000u | slot);
+    return (int)(__float_as_uint(r) >> 19) - 127 * 16;
 }
+struct Lookup {                                            // any table: two dependent look-ups
+    const uint8_t* first;
+    const uint32_t* fc;
+    __device__ __forceinline__ uint32_t operator()(uint32_t x, int& zz) const {
+        const uint32_t slot = x & (kProbM - 1u);
+        const int z = first[interval_of(slot)];
+        const uint32_t a = fc[z], b = fc[z + 1];
+        const bool next = slot >= (b >> 16);
+        zz = next ? z + 1 : z;
+        const uint32_t e = next ? b : a;
+        return (e & 0xffffu) * (x >> kProbBits) + slot - (e >> 16);
+    }
+};
+struct WideLookup {                                        // tables kept in wide form: one
+    const uint2* t;
+    __device__ __forceinline__ uint32_t operator()(uint32_t x, int& zz) const {
+        const uint32_t slot = x & (kProbM - 1u);
+        const uint2 w = t[interval_of(slot)];
+        const uint32_t f0 = w.x & 0xffffu, d = slot - (w.x >> 16), top = x >> kProbBits;
+        const bool next = d >= f0;
+        zz = (int)(w.y >> 16) + next;
+        return next ? (w.y & 0xffffu) * top + (d - f0) : f0 * top + d;
+    }
+};
 __device__ __forceinline__ int hi_of(int zz) {                            // 0, +1, -1, +2, ...
     const int t = (zz + 1) >> 1;
     return (zz & 1) ? t : -t;
 }
 
 // Positions with an escaped component, one step at a time.
-template <int G, class Words>
-__device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x,
-                                                        const Words& words, int& rp, int lane) {
+template <int G, class Find, class Words>
+__device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, const Find& find, uint32_t& x, const Words& words, int& rp, int lane) {
     const uint32_t lt = lanemask_lt();
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
@@ -255,8 +291,7 @@ __device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, co
         }
         rp += 2 * S;
         int zz;
-        const uint32_t fc = find_symbol(x, first, fcs, zz);
-        x = (fc & 0xffffu) * (x >> kProbBits) + (x & (kProbM - 1u)) - (fc >> 16);
+        x = find(x, zz);
         const bool need = x < kRansL;
         const uint32_t nmask = __ballot_sync(kFull, need);
         if (need) x = (x << 16) | words(rp + __popc(nmask & lt));
@@ -279,9 +314,9 @@ __device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, co
 // stream and high part; false if a component escaped (x and rp are then as before the call).
 // words(i) reads 16-bit word i of the chunk (any i: the reader keeps the access in bounds; rp advances
 // regardless, so the caller's final check of rp reports a short chunk).
-template <int G, class Words>
-__device__ __forceinline__ bool pull_position(int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x, const Words& words, int& rp,
-                                              const LaneCode& lc, int (&base)[G], int (&hi)[G]) {
+template <int G, class Find, class Words>
+__device__ __forceinline__ bool pull_position(int S, const Find& find, uint32_t& x, const Words& words, int& rp, const LaneCode& lc,
+                                              int (&base)[G], int (&hi)[G]) {
     const uint32_t x0 = x;
     const int rp0 = rp;
     bool esc = false;
@@ -289,12 +324,13 @@ __device__ __forceinline__ bool pull_position(int S, const uint8_t* first, const
     for (int g = 0; g < G; ++g) {
         base[g] = rp;
         rp += 2 * S;
+        const uint32_t window = words(rp + lc.lane);       // the step's refill words, fetched beside the look-up
         int zz;
-        const uint32_t fc = find_symbol(x, first, fcs, zz);
-        x = (fc & 0xffffu) * (x >> kProbBits) + (x & (kProbM - 1u)) - (fc >> 16);
+        x = find(x, zz);
         const bool need = x < kRansL;
         const uint32_t nmask = __ballot_sync(kFull, need);
-        if (need) x = (x << 16) | words(rp + __popc(nmask & lc.lt));
+        const uint32_t word = __shfl_sync(kFull, window, __popc(nmask & lc.lt));
+        x = need ? (x << 16) | word : x;
         rp += __popc(nmask);
         esc = esc || zz == kEsc;
         hi[g] = hi_of(zz);
@@ -333,12 +369,12 @@ __device__ __forceinline__ void join_position(const int (&base)[G], const int (&
 }
 
 // All G components of one position.
-template <int G, class Words>
-__device__ __forceinline__ void decode_position(int (&sym)[G], int S, const uint8_t* first, const uint32_t* fcs, uint32_t& x,
-                                                const Words& words, int& rp, const LaneCode& lc) {
+template <int G, class Find, class Words>
+__device__ __forceinline__ void decode_position(int (&sym)[G], int S, const Find& find, uint32_t& x, const Words& words, int& rp,
+                                                const LaneCode& lc) {
     int base[G], hi[G];
-    if (pull_position<G>(S, first, fcs, x, words, rp, lc, base, hi)) join_position<G>(base, hi, S, words, lc, sym);
-    else decode_position_escapes<G>(sym, S, first, fcs, x, words, rp, lc.lane);
+    if (pull_position<G>(S, find, x, words, rp, lc, base, hi)) join_position<G>(base, hi, S, words, lc, sym);
+    else decode_position_escapes<G>(sym, S, find, x, words, rp, lc.lane);
 }
 
 #endif  // __CUDACC__

@@ -21,21 +21,25 @@ namespace plc {
 namespace {
 
 constexpr int kCoopMaxWarps = 16;
-constexpr int kRingBytes = 8192, kRingBlock = 512;       // word ring of a decoding coder; bytes one warp-wide copy brings
+constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
+// Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; about four such are held.
+__host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 8192 : 4096; }
 constexpr int kSkipped = -1000000;                       // class mark of a zero-rate position
 
 struct SlotMeta { int q, e, escaped, pad; };             // class (or kSkipped), step exponent, whether a component escapes
 
 // The words of a chunk, read through the ring.  `ready` bytes have landed, `fetched` are on their way.
+template <int G>
 struct RingWords {
     const uint16_t* ring;
-    __device__ __forceinline__ uint32_t operator()(int i) const { return ring[i & (kRingBytes / 2 - 1)]; }
+    __device__ __forceinline__ uint32_t operator()(int i) const { return ring[i & (ring_bytes(G) / 2 - 1)]; }
 };
+template <int G>
 __device__ __forceinline__ void ring_fetch(uint16_t* ring, const uint8_t* src, int total, int rp, int& fetched, int lane) {
-    while (fetched < total && fetched + kRingBlock <= 2 * rp + kRingBytes) {
+    while (fetched < total && fetched + kRingBlock <= 2 * rp + ring_bytes(G)) {
         const int at = fetched + 16 * lane;
         if (at < total) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(ring) + (at & (kRingBytes - 1)));
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(ring) + (at & (ring_bytes(G) - 1)));
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src + at), "r"(min(16, total - at)) : "memory");
         }
         fetched += kRingBlock;
@@ -103,7 +107,7 @@ __device__ __forceinline__ void slot_get(const int* slot, int lane, Prepared<G>&
 size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
     const int NP = warps - 1, G = d / 32, planes = G <= 2 ? 1 : G / 2;
     const int slot = enc ? 32 * (2 * G + planes) : 32 * G + 8;
-    return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : kRingBytes);
+    return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G));
 }
 
 // All warps of the block meet here; the two roles reach it from different places in the code.
@@ -321,8 +325,8 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         src += 128;
         const int nwords = (int)((sh.item.nbytes - 128u) >> 1);
         int rp = 0, fetched = 0, ready = 0;
-        ring_fetch(ring, src, 2 * nwords, 0, fetched, lane);
-        const RingWords words{ring};
+        ring_fetch<G>(ring, src, 2 * nwords, 0, fetched, lane);
+        const RingWords<G> words{ring};
         for (int b = 0; b < n_batches; ++b) {
             block_barrier();                                                   // the classes of batch b are there
             const int cnt = min(NP, P - b * NP);
@@ -332,25 +336,29 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                 const int qj = q;
                 if (j + 1 < cnt) q = sh.meta[b & 1][j + 1].q;
                 if (qj == kSkipped) continue;
-                // a position takes at most G * (2 * 15 + 32 + 64) words
-                if (min(2 * rp + 252 * G, 2 * nwords) > ready) {
+                // a position's words, and the last refill window
+                if (min(2 * rp + 252 * G + 64, 2 * nwords) > ready) {
                     asm volatile("cp.async.wait_all;" ::: "memory");
                     __syncwarp();
                     ready = fetched;
                 }
                 int s, qp, base[G], hi[G];
                 class_params(qj, s, qp);
-                if (pull_position<G>(s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, words, rp, lc, base, hi)) {
+                auto step = [&](const auto& find) {
+                    if (pull_position<G>(s, find, x, words, rp, lc, base, hi)) {
 #pragma unroll
-                    for (int g = 0; g < G; ++g)
-                        if (lane == g) slot[32 * G + g] = base[g];
-                } else {
-                    decode_position_escapes<G>(hi, s, tb.first[qp - kQMin], tb.fc[qp - kQMin], x, words, rp, lane);
-                    if (lane == 0) sh.meta[b & 1][j].escaped = 1;
-                }
+                        for (int g = 0; g < G; ++g)
+                            if (lane == g) slot[32 * G + g] = base[g];
+                    } else {
+                        decode_position_escapes<G>(hi, s, find, x, words, rp, lane);
+                        if (lane == 0) sh.meta[b & 1][j].escaped = 1;
+                    }
+                };
+                if (qp - kQMin >= kWideFrom) step(WideLookup{tb.wide[qp - kQMin - kWideFrom]});
+                else step(Lookup{tb.first[qp - kQMin], tb.fc[qp - kQMin]});
                 slot_put_ints<G>(slot, lane, hi);
                 __syncwarp();                                                  // readers of the ring are done
-                ring_fetch(ring, src, 2 * nwords, rp, fetched, lane);
+                ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
             }
         }
         block_barrier();
@@ -363,7 +371,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
 template <int D, bool DENSE, bool ENC>
 __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
-    using Tab = std::conditional_t<ENC, EncTables, DecTables>;
+    using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
     __shared__ CoopShared sh;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NP = (blockDim.x >> 5) - 1;   // NP predicting warps
@@ -371,7 +379,7 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
     int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
     const LaneCode lc = lane_code(lane);
-    load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->dec));
+    load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->wide));
     const int Wl = DENSE ? a.dense_nt : 2 * a.sh.L * a.sh.H;
     const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks, total = (unsigned)Wl * per_table;
     QueueCursor qc = DENSE ? QueueCursor{0, 0} : queue_of_this_sm(a);
