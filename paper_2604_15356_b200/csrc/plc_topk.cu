@@ -1,23 +1,12 @@
-// Top-K softmax over per-position next-token logits (one thread block per row, rows strided over
-// the grid).  Selection is exact (logit descending, index ascending, -0 = +0).
+// Top-K softmax over per-position next-token logits.  Selection is exact (logit descending, index
+// ascending, -0 = +0).
 //
-// Fast path (K <= 16 per warp of the block: K <= 128 with 256 threads): pass 0 reads the row from HBM and keeps one
-// maximum per thread; the ceil(K / warps)-th largest thread maximum of every warp, minimised over the
-// warps, is a value with at least K row elements at or above it, i.e. a lower bound of the K-th
-// largest logit that needs no histogram.  Pass 1 (served by L2) sums exp(l - l_max) over the row
-// and notes the groups of 8 logits that hold an element at or above that bound; after the pass the
-// noted groups are taken apart, one per thread, into a candidate list (typically 1.2-2 K entries).
-// A list of at most 256 goes to global memory and a second kernel (one warp per row, bitonic sort in
-// registers) orders it and writes the K selected, their weights and Z_k; without the scratch for
-// that, or for longer lists, the block ranks by counting (long lists: sorted) itself.  Rows whose
-// candidates overflow the list (large tie groups, adversarial layouts) and larger K take the radix-select path:
-// a 4096-bin histogram of the order-preserving 16-bit key finds the bin that holds the K-th largest,
-// a 16-way refinement finds the key itself, and equal keys are taken in index order.
+// K <= 128, and calls that ask for no selected set (only lse / log2 P): topk_stream_kernel, which reads
+// a row once, any alignment (see there).  K > 128: topk_softmax_kernel, one block a row: a 4096-bin
+// histogram of the order-preserving 16-bit key finds the bin that holds the K-th largest, a 16-way
+// refinement finds the key itself, and equal keys are taken in index order.
 // Reductions use warp shuffles in a fixed order, so results are bit-reproducible from run to run.
-// Rows that fit a 64 KB shared-memory buffer (and rows of any length when no selection is asked for)
-// first go through topk_staged_kernel further down, which does the same row work on a copy of the
-// row in shared memory; this kernel then takes only what that one marks as left over.
-#include <type_traits>
+#include <algorithm>
 
 #include "plc_common.cuh"
 
@@ -26,7 +15,6 @@ namespace {
 
 constexpr int kBins = 4096;
 constexpr int kCandCap = 1024;
-constexpr int kHdrRedo = -2;                        // header mark: the row is left to the general kernel
 
 __device__ __forceinline__ uint32_t key_of(uint32_t u) {
     u &= 0xffffu;
@@ -43,7 +31,7 @@ constexpr uint32_t kKeyNegInf = 0x03ffu;            // key_of(0xfc00)
 
 template <int THREADS>
 struct __align__(16) Smem {
-    uint32_t hist[kBins];                           // fast path: candidate list (keys, then indices)
+    uint32_t hist[kBins];
     uint32_t sub[16];
     uint32_t sel_key[kCandCap];
     int32_t sel_idx[kCandCap];
@@ -51,12 +39,10 @@ struct __align__(16) Smem {
     int32_t cand_idx[kCandCap];
     float ek[kCandCap];
     uint32_t red_k[THREADS / 32];
-    uint32_t red_t[THREADS / 32];
     float red_s[THREADS / 32];
     int scan[THREADS / 32];
-    int nsel, ncand, bstar, count_above, cstar, thr, need, neq, running, nlist, nhit;
-    float row_max, row_sum, sum_k;
-    uint32_t theta;
+    int nsel, ncand, bstar, count_above, cstar, thr, need, neq, running;
+    float sum_k;
 };
 
 // Exclusive scan of one int per thread over the block (thread order); total to all threads.
@@ -274,25 +260,23 @@ __device__ void select_by_histogram(Smem<THREADS>& sm, const __half* row, int V,
     __syncthreads();
 }
 
-// Candidate list of the fast path: one order word per candidate, larger = earlier in (key
-// descending, index ascending); 32-bit words while indices fit 16 bits, 64-bit words otherwise.
-__device__ __forceinline__ void list_put(uint32_t* list, bool narrow, int slot, uint32_t key, int idx) {
-    if (narrow) list[slot] = (key << 16) | (0xffffu - (uint32_t)idx);
-    else reinterpret_cast<unsigned long long*>(list)[slot] = ((unsigned long long)key << 32) | (0xffffffffu - (uint32_t)idx);
+// Entry k of a row's pairs: candidate and weight.
+__device__ __forceinline__ void put_pair(const TopkArgs& a, long long rowi, int k, int idx, float w) {
+    a.pairs[rowi * a.Kp + k] = make_int2(idx, __float_as_int(w));
 }
-// Appends those of the two logits in `w` (indices i, i + 1) that reach the bound th2 (the bound in
-// both halves).  A warp gets here whenever any of its 256 logits of the moment qualifies, with one
-// or two lanes active, so the test is a packed compare and the key is formed for the hits only.
-__device__ __forceinline__ void collect2(uint32_t w, uint32_t th2, int i, bool narrow, int* nlist, uint32_t* list) {
-    const uint32_t ge = __hge2_mask(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&th2));
-    if (ge == 0) return;
-    if (ge & 0xffffu) {
-        const int slot = atomicAdd(nlist, 1);
-        if (slot < kCandCap) list_put(list, narrow, slot, key_of(w & 0xffffu), i);
-    }
-    if (ge >> 16) {
-        const int slot = atomicAdd(nlist, 1);
-        if (slot < kCandCap) list_put(list, narrow, slot, key_of(w >> 16), i + 1);
+
+// log2 P of the row's token and, for the adaptive step (Def. 7), b = max(1, floor(b0 h / hbar)) capped at
+// b0 + extra, decided in binary32.
+__device__ __forceinline__ void put_surprisal(const TopkArgs& a, long long rowi, const __half* row, float lse) {
+    const int tk = a.tokens[rowi];
+    const float v = (tk >= 0 && tk < a.V) ? (__half2float(row[tk]) - lse) * 1.44269504088896341f : __int_as_float(0x7fc00000);
+    if (a.logp2) a.logp2[rowi] = v;
+    if (a.step_exp || a.bits_out) {
+        const float r = __fmul_rn((float)a.b0, __fdiv_rn(-v, a.hbar));
+        int b = (r >= 1.0f) ? (int)floorf(r) : 1;
+        b = min(b, a.b0 + a.extra);
+        if (a.step_exp) a.step_exp[rowi] = a.b0 - b;
+        if (a.bits_out) a.bits_out[rowi] = b;
     }
 }
 
@@ -303,288 +287,297 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int V = a.V, K = a.K;
     const int ntiles = (V + THREADS * 8 - 1) / (THREADS * 8);
-    const int per_warp = (K + NW - 1) / NW;
-    // A warp can offer at most 32 thread maxima, and the bound is only tight while it asks for the
-    // upper half of them: beyond 16 per warp the candidates overflow the list on ordinary rows.
-    // Calls that want no selected set (only lse / log2 P of the tokens / step exponents) skip the selection.
-    const bool select = a.pairs || a.idx || a.w || a.zk;
-    const bool fast = select && per_warp <= 16 && K <= kCandCap;
-    // The candidate list of the fast path lives in the histogram's memory, which is idle there.
-    const bool narrow = V <= 65536;
-    uint32_t* list32 = sm.hist;
-    unsigned long long* list64 = reinterpret_cast<unsigned long long*>(sm.hist);
-
-    if (a.redo_only && *a.redo == 0) return;                             // nothing was left over
     for (long long rowi = blockIdx.x; rowi < a.N; rowi += gridDim.x) {
         if (a.pos_begin || a.pos_end) {
             int s = (int)(rowi / a.n_per_session), i = (int)(rowi % a.n_per_session);
             int b = a.pos_begin ? a.pos_begin[s] : 0, e = a.pos_end ? a.pos_end[s] : a.n_per_session;
             if (i < b || i >= e) continue;
         }
-        if (a.redo_only && __float_as_int(a.cand_hdr[rowi].z) != kHdrRedo) continue;
         const __half* row = a.logits + rowi * (long long)V;
-        if (tid == 0) { sm.nlist = 0; sm.nhit = 0; }
-
-        // Pass 0 (HBM): one maximum per thread.
+        // Pass 0 (HBM): the maximum.
         uint32_t tkey = 0;
-        if (VEC) {
-            uint32_t m2 = 0xfc00fc00u;                                   // (-inf, -inf)
-#pragma unroll 4
-            for (int t = 0; t < ntiles; ++t) {
-                const int i0 = t * (THREADS * 8) + tid * 8;
-                if (i0 < V) {
-                    const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
-                    m2 = hmax2_bits(m2, hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w)));
-                }
-            }
-            tkey = max(key_of(m2 & 0xffffu), key_of(m2 >> 16));
-            if (tid * 8 >= V) tkey = 0;                                   // this thread owns nothing
-        } else {
-            for (int t = 0; t < ntiles; ++t)
-                for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { tkey = max(tkey, key_of(bits)); });
-        }
-        // per warp: the largest and the per_warp-th largest thread maximum
-        const uint32_t wmax = __reduce_max_sync(kFull, tkey);
-        uint32_t wth = 0;
-        if (fast) {
-            uint32_t v = tkey;
-            for (int r = 0; r < per_warp; ++r) {
-                wth = __reduce_max_sync(kFull, v);
-                const uint32_t eq = __ballot_sync(kFull, v == wth);
-                if (lane == __ffs(eq) - 1) v = 0;
-            }
-        }
-        if (lane == 0) { sm.red_k[wid] = wmax; sm.red_t[wid] = wth; }
+        for (int t = 0; t < ntiles; ++t)
+            for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { tkey = max(tkey, key_of(bits)); });
+        tkey = __reduce_max_sync(kFull, tkey);
+        if (lane == 0) sm.red_k[wid] = tkey;
         __syncthreads();
-        uint32_t km = sm.red_k[0], theta = sm.red_t[0];
+        uint32_t km = sm.red_k[0];
 #pragma unroll
-        for (int w = 1; w < NW; ++w) { km = max(km, sm.red_k[w]); theta = min(theta, sm.red_t[w]); }
-        theta = max(theta, kKeyNegInf);
+        for (int w = 1; w < NW; ++w) km = max(km, sm.red_k[w]);
         const float lmax = val_of_key(km);
-
-        // Pass 1 (L2): sum of exp(l - l_max) over the row (fast exponential: its relative error of
-        // about 2e-6 at the arguments that matter is inside the tolerance of lse and Z_k) and, on
-        // the fast path, the elements at or above the bound.
+        // Pass 1 (L2): sum of exp(l - l_max).
         const float nb = -lmax * 1.44269504088896341f;
         float s = 0.f;
-        if (VEC) {
-            const uint32_t tb = bits_of_key(theta);
-            const uint32_t th2 = tb | (tb << 16);
-#pragma unroll 2
-            for (int t = 0; t < ntiles; ++t) {
-                const int i0 = t * (THREADS * 8) + tid * 8;
-                if (i0 < V) {
-                    const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
-                    const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
-                    const uint32_t top = hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w));
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&wds[j]));
-                        s += exp_rel(f.x, nb);
-                        s += exp_rel(f.y, nb);
-                    }
-                    // A group of 8 with a logit at or above the bound is only noted here (few lanes get
-                    // here, so anything longer would run once per group with the rest of the warp idle);
-                    // the noted groups are taken apart after the pass, one per thread.
-                    if (fast && !__hblt2(*reinterpret_cast<const __half2*>(&top), *reinterpret_cast<const __half2*>(&th2))) {
-                        const int slot = atomicAdd(&sm.nhit, 1);
-                        if (slot < kCandCap) sm.sel_idx[slot] = i0;          // sel_idx is idle on this path
-                    }
-                }
-            }
-        } else {
-            for (int t = 0; t < ntiles; ++t)
-                for_tile<VEC, THREADS>(row, V, t, [&](int i, uint32_t bits) {
-                    s += exp_rel(__half2float(__ushort_as_half((unsigned short)bits)), nb);
-                    const uint32_t key = key_of(bits);
-                    if (fast && key >= theta) {
-                        const int slot = atomicAdd(&sm.nlist, 1);
-                        if (slot < kCandCap) list_put(sm.hist, narrow, slot, key, i);
-                    }
-                });
-        }
+        for (int t = 0; t < ntiles; ++t)
+            for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { s += exp_rel(__half2float(__ushort_as_half((unsigned short)bits)), nb); });
         s = warp_sum(s);
         if (lane == 0) sm.red_s[wid] = s;
         __syncthreads();
         float sum_all = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) sum_all += sm.red_s[w];
-        if (VEC && fast) {
-            const int nhit = sm.nhit;
-            if (nhit > kCandCap) {
-                if (tid == 0) sm.nlist = kCandCap + 1;                    // too many: the radix select takes the row
-            } else {
-                const uint32_t tb = bits_of_key(theta);
-                const uint32_t th2 = tb | (tb << 16);
-                for (int t = tid; t < nhit; t += THREADS) {
-                    const int i0 = sm.sel_idx[t];
-                    const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
-                    const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) collect2(wds[j], th2, i0 + 2 * j, narrow, &sm.nlist, sm.hist);
-                }
-            }
-            __syncthreads();
+        select_by_histogram<VEC, THREADS>(sm, row, V, K, ntiles);
+        for (int k = tid; k < K; k += THREADS) sm.ek[k] = expf(val_of_key(sm.cand_key[k]) - lmax);
+        __syncthreads();
+        if (wid == 0) {
+            float p = 0.f;
+            for (int k = lane; k < K; k += 32) p += sm.ek[k];
+            p = warp_sum(p);
+            if (lane == 0) sm.sum_k = p;
         }
-        const int nlist = sm.nlist;
-        // Two-kernel selection: a list that one warp can sort goes to global memory as it is and
-        // topk_rank_kernel finishes the row (order, weights, Z_k); everything else stays here.
-        const bool handed = fast && a.cand && K <= 128 && nlist >= K && nlist <= kTopkListCap;
-        if (a.cand_hdr && tid == 0)
-            a.cand_hdr[rowi] = make_float4(lmax, sum_all, __int_as_float(handed ? nlist : -1), 0.f);
-        if (handed) {
-            if (narrow) {
-                uint32_t* dst = static_cast<uint32_t*>(a.cand) + rowi * kTopkListCap;
-                for (int c = tid; c < nlist; c += THREADS) dst[c] = list32[c];
-            } else {
-                unsigned long long* dst = static_cast<unsigned long long*>(a.cand) + rowi * kTopkListCap;
-                for (int c = tid; c < nlist; c += THREADS) dst[c] = list64[c];
-            }
-        } else if (fast && nlist >= K && nlist <= kCandCap) {
-            // Order the candidates (at least K of them); the first K are the result.  Short lists are
-            // ranked by counting (n^2 / THREADS compares per thread, no barriers), long ones sorted.
-            constexpr int kRankMax = 192;
-            if (nlist > kRankMax) {
-                int n_pad = 256;
-                while (n_pad < nlist) n_pad <<= 1;
-                if (narrow) {
-                    for (int c = nlist + tid; c < n_pad; c += THREADS) list32[c] = 0;    // pad: orders after everything
-                    __syncthreads();
-                    bitonic_desc<THREADS>(list32, n_pad);
-                    for (int k = tid; k < K; k += THREADS) {
-                        const uint32_t v = list32[k];
-                        sm.cand_key[k] = v >> 16; sm.cand_idx[k] = (int)(0xffffu - (v & 0xffffu));
-                    }
-                } else {
-                    for (int c = nlist + tid; c < n_pad; c += THREADS) list64[c] = 0;
-                    __syncthreads();
-                    bitonic_desc<THREADS>(list64, n_pad);
-                    for (int k = tid; k < K; k += THREADS) {
-                        const unsigned long long v = list64[k];
-                        sm.cand_key[k] = (uint32_t)(v >> 32); sm.cand_idx[k] = (int)(0xffffffffu - (uint32_t)v);
-                    }
-                }
-            } else if (narrow) {
-                const int n4 = (nlist + 3) & ~3;
-                for (int c = nlist + tid; c < n4; c += THREADS) list32[c] = 0;           // pad: orders after everything
-                __syncthreads();
-                for (int c = tid; c < nlist; c += THREADS) {
-                    const uint32_t mine = list32[c];
-                    int rank = 0;
-                    for (int j = 0; j < n4; j += 4) {
-                        const uint4 o = *reinterpret_cast<const uint4*>(list32 + j);
-                        rank += (o.x > mine) + (o.y > mine) + (o.z > mine) + (o.w > mine);
-                    }
-                    if (rank < K) { sm.cand_key[rank] = mine >> 16; sm.cand_idx[rank] = (int)(0xffffu - (mine & 0xffffu)); }
-                }
-            } else {
-                for (int c = tid; c < nlist; c += THREADS) {
-                    const unsigned long long mine = list64[c];
-                    int rank = 0;
-                    for (int j = 0; j < nlist; ++j) rank += list64[j] > mine;
-                    if (rank < K) { sm.cand_key[rank] = (uint32_t)(mine >> 32); sm.cand_idx[rank] = (int)(0xffffffffu - (uint32_t)mine); }
-                }
-            }
-            __syncthreads();
-        } else if (select) {
-            __syncthreads();
-            select_by_histogram<VEC, THREADS>(sm, row, V, K, ntiles);
+        __syncthreads();
+        const float sum_k = sm.sum_k;
+        for (int k = tid; k < K; k += THREADS) {
+            float w = sm.ek[k] / sum_k;
+            int idx = sm.cand_idx[k];
+            if (a.pairs) put_pair(a, rowi, k, idx, w);
+            if (a.idx) a.idx[rowi * K + k] = idx;
+            if (a.w) a.w[rowi * K + k] = w;
         }
-
-        float sum_k = 0.f;
-        if (select && !handed) {
-            for (int k = tid; k < K; k += THREADS) sm.ek[k] = expf(val_of_key(sm.cand_key[k]) - lmax);
-            __syncthreads();
-            if (wid == 0) {
-                float p = 0.f;
-                for (int k = lane; k < K; k += 32) p += sm.ek[k];
-                p = warp_sum(p);
-                if (lane == 0) sm.sum_k = p;
-            }
-            __syncthreads();
-            sum_k = sm.sum_k;
-            for (int k = tid; k < K; k += THREADS) {
-                float w = sm.ek[k] / sum_k;
-                int idx = sm.cand_idx[k];
-                if (a.pairs) a.pairs[rowi * a.Kp + k] = make_int2(idx, __float_as_int(w));
-                if (a.idx) a.idx[rowi * K + k] = idx;
-                if (a.w) a.w[rowi * K + k] = w;
-            }
-            if (a.pairs)
-                for (int k = K + tid; k < a.Kp; k += THREADS) a.pairs[rowi * a.Kp + k] = make_int2(sm.cand_idx[0], 0);
-        }
+        if (a.pairs)
+            for (int k = K + tid; k < a.Kp; k += THREADS) put_pair(a, rowi, k, sm.cand_idx[0], 0.f);
         if (tid == 0) {
             float lse = lmax + logf(sum_all);
             if (a.lse) a.lse[rowi] = lse;
-            if (a.zk && !handed) a.zk[rowi] = sum_k / sum_all;
-            if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) {
-                const int tk = a.tokens[rowi];
-                const float v = (tk >= 0 && tk < V) ? (__half2float(row[tk]) - lse) * 1.44269504088896341f : __int_as_float(0x7fc00000);
-                if (a.logp2) a.logp2[rowi] = v;
-                if (a.step_exp || a.bits_out) {
-                    // Def. 7: b = max(1, floor(b0 h / hbar)), capped at b0 + extra; decided in binary32
-                    const float r = __fmul_rn((float)a.b0, __fdiv_rn(-v, a.hbar));
-                    int b = (r >= 1.0f) ? (int)floorf(r) : 1;
-                    b = min(b, a.b0 + a.extra);
-                    if (a.step_exp) a.step_exp[rowi] = a.b0 - b;
-                    if (a.bits_out) a.bits_out[rowi] = b;
-                }
-            }
+            if (a.zk) a.zk[rowi] = sum_k / sum_all;
+            if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) put_surprisal(a, rowi, row, lse);
         }
         __syncthreads();
     }
 }
 
-// ---- rows that fit in shared memory -------------------------------------------------------------
-// The same row work as the fast path above, but the row is brought into shared memory ONCE by a
-// bulk asynchronous copy (one instruction of one thread, completion on an mbarrier) and both passes
-// and the taking apart of the noted groups read it there: the second pass costs no L2 round trips,
-// no registers hold loads in flight, and the copy of a block's next row runs under the tail of the
-// current one.  Three blocks per SM keep about 190 KB of copies or rows per SM in flight.  Rows
-// whose candidates do not fit the hand-over (ties, more than 256 at or above the bound) are marked
-// for the general kernel.  A call that wants no selection (lse / log2 P only) may have rows longer
-// than the buffer: they pass through it in chunks, one HBM read and no L2 pass at all.  Every wait
-// on the barrier is bounded.
-constexpr int kStageBytes = 64 * 1024;             // largest row buffer: V <= 32768 binary16 logits
-// A row longer than the buffer is staged in equal chunks (a multiple of 8 logits each); only calls
-// without a selection take such rows here: maximum and sum are carried from chunk to chunk.
-__host__ __device__ constexpr int stage_chunks(int V) { return (V * 2 + kStageBytes - 1) / kStageBytes; }
-__host__ __device__ constexpr int stage_chunk_elems(int V) {
-    return stage_chunks(V) <= 1 ? V : (((V + stage_chunks(V) - 1) / stage_chunks(V) + 7) & ~7);
-}
-__host__ __device__ constexpr int stage_buf_bytes(int V) { return (stage_chunk_elems(V) * 2 + 127) & ~127; }
-#ifndef PLC_STAGE_THREADS
-#define PLC_STAGE_THREADS 256
-#endif
-constexpr int kStageThreads = PLC_STAGE_THREADS;
-constexpr uint32_t kStageSpin = 1u << 24;
+// ---- rows streamed once, a warp (or a few warps) a row --------------------------------------------
+// The row is read from HBM once, straight into registers, by one warp when there are rows enough to
+// fill the GPU, by up to 32 warps (4 blocks of a cluster) otherwise; the warps of a row meet only at its
+// end, so nothing idles at barriers while others stream.  Per 8 logits and lane: one 16-byte load, a
+// packed maximum and the sum of exp relative to a running reference.  For the selection a lane only
+// leaves the maximum of every group of logits that it reads (a group: 8 logits, or 32 and a multiple
+// of it in long rows; at most 64 a lane) in shared memory.  At the row's end the K-th largest of those
+// maxima is the bound: at least K logits reach it, exactly K groups (and ties) hold such logits, and
+// only those groups, 2 to 10 % of the row, are read again.  The logits at or above the bound, a few
+// more than K, are ordered by counting.  A row with more than kListCap of them (ties) is selected by
+// counting passes over the row (slow_select).
+// Noting every group that reached a running bound instead, with votes or in columns, took 12000 to
+// 13000 instructions for a row of 32000 logits, twice what the sum takes; this takes about 3000.
+constexpr int kSlots = 64;                          // group maxima of a row, per lane
+constexpr int kCodes = 256;                         // groups that are read again
+constexpr int kListCap = 256;                       // logits at or above the bound
+constexpr int kFinal = 128;                         // K <= kFinal here
+constexpr int kBatch = 4;                           // 16-byte loads a lane has in flight per batch (two batches at a time)
+constexpr int kStreamWarps = 8;                     // most warps of a block
+constexpr int kMaxCluster = 4;
 
-struct __align__(16) StageSm {
-    unsigned long long bar;
-    uint32_t list[kCandCap];
-    int32_t hit[kCandCap];
-    uint32_t red_k[kStageThreads / 32];
-    uint32_t red_t[kStageThreads / 32];
-    float red_s[kStageThreads / 32];
-    int nlist, nhit;
+__device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
+    uint4 r;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ __half2 as_half2(uint32_t w) { return *reinterpret_cast<const __half2*>(&w); }
+__device__ __forceinline__ uint32_t top2_of(const uint4& r) { return hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w)); }
+__device__ __forceinline__ uint4 all4(uint32_t w) { return make_uint4(w, w, w, w); }
+constexpr uint32_t kNegInf2 = 0xfc00fc00u, kNoValue2 = 0xffffffffu;         // NaN: reaches no bound, loses every maximum
+__device__ __forceinline__ uint32_t top_key(uint32_t top2) { return max(key_of(top2 & 0xffffu), key_of(top2 >> 16)); }
+__device__ __forceinline__ uint32_t half_at(const uint4& r, int j) {       // j is a compile-time constant after unrolling
+    const uint32_t w = j < 2 ? r.x : j < 4 ? r.y : j < 6 ? r.z : r.w;
+    return (j & 1) ? w >> 16 : w & 0xffffu;
+}
+// Packed pairs of binary32 (sm_100 f32x2 instructions).
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long both(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1,%2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void parts(unsigned long long v, float& lo, float& hi) { asm("mov.b64 {%0,%1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+
+// Order words: larger = earlier in (key descending, index ascending); 32 bits while indices fit 16.
+template <class W>
+__device__ __forceinline__ W order_word(uint32_t key, int idx) {
+    if constexpr (sizeof(W) == 4) return (key << 16) | (0xffffu - (uint32_t)idx);
+    else return ((W)key << 32) | (0xffffffffu - (uint32_t)idx);
+}
+template <class W>
+__device__ __forceinline__ uint32_t key_of_word(W w) { return (uint32_t)(w >> (sizeof(W) * 4)); }
+template <class W>
+__device__ __forceinline__ int idx_of_word(W w) {
+    if constexpr (sizeof(W) == 4) return (int)(0xffffu - (w & 0xffffu));
+    else return (int)(0xffffffffu - (uint32_t)w);
+}
+
+// First place of this lane among the warp's `mine` items; total to all lanes.
+__device__ __forceinline__ int warp_excl_scan(int mine, int lane, int& total) {
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += t;
+    }
+    total = __shfl_sync(kFull, inc, 31);
+    return inc - mine;
+}
+
+// A row as head logits up to the first 16-byte boundary, nv whole 16-byte groups, and a tail.
+struct RowView {
+    const __half* row;
+    const uint4* body;
+    int V, head, nv;
+};
+__device__ __forceinline__ RowView row_view(const __half* row, int V) {
+    RowView r;
+    r.row = row; r.V = V;
+    r.head = min((int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(row) & 15u)) & 15u) >> 1, V);
+    r.nv = (V - r.head) >> 3;
+    r.body = reinterpret_cast<const uint4*>(row + r.head);
+    return r;
+}
+// The ends of the row as groups -1 (lane 0: the head) and nv (lane 1: the tail) of 8, kNoValue where the
+// row is not.
+__device__ __forceinline__ uint4 row_ends(const RowView& r, int lane) {
+    uint32_t w[4] = {kNoValue2, kNoValue2, kNoValue2, kNoValue2};
+    if (lane < 2) {
+        const int tail0 = r.head + 8 * r.nv, i0 = lane == 0 ? r.head - 8 : tail0;
+        const int b = lane == 0 ? 0 : tail0, e = lane == 0 ? r.head : r.V;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int i = i0 + j;
+            if (i >= b && i < e) {
+                const uint32_t h = (uint32_t)__half_as_ushort(r.row[i]);
+                w[j / 2] = (j & 1) ? (w[j / 2] & 0xffffu) | (h << 16) : (w[j / 2] & 0xffff0000u) | h;
+            }
+        }
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Exact selection by one warp reading the row from memory: bisection of the K-th largest key between `lo`
+// (at least K logits reach it) and the maximum by counting passes, then the K elements, equal keys in
+// index order, into the list (packed).  For rows whose ties overflow the lists.
+template <class W>
+__device__ __noinline__ void slow_select(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, int lane) {
+    const RowView r = row_view(row, V);
+    const uint32_t lt = lanemask_lt();
+    const uint4 ends = row_ends(r, lane);
+    auto key_at = [&](const uint4& q, int j) { const uint32_t h = half_at(q, j); return h == 0xffffu ? 0u : key_of(h); };   // 0: no value
+    auto count = [&](uint32_t t) {
+        int c = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) c += key_at(ends, j) >= t;
+#pragma unroll 2
+        for (int v = lane; v < r.nv; v += 32) {
+            const uint4 q = r.body[v];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) c += key_at(q, j) >= t;
+        }
+        return (int)__reduce_add_sync(kFull, c);
+    };
+    uint32_t hi = kmax + 1;                                              // nothing reaches it
+#pragma unroll 1
+    for (bool first = true; hi - lo > 1; first = false) {
+        const uint32_t mid = first ? lo + 1 : lo + ((hi - lo) >> 1);     // most often the bound itself is the key
+        if (count(mid) >= K) lo = mid; else hi = mid;
+    }
+    int need = K - count(lo + 1), n = 0;
+    const int last = (r.nv + 31) >> 5;
+#pragma unroll 1
+    for (int s = -1; s <= last; ++s) {                                   // head, body, tail: index order over the lanes
+        const int v = s < 0 ? -1 : s < last ? s * 32 + lane : r.nv;
+        const bool body = s >= 0 && s < last;
+        const bool have = body ? v < r.nv : lane == (s < 0 ? 0 : 1);
+        const uint4 q = !have ? all4(kNoValue2) : body ? r.body[v] : ends;
+        int eq = 0, all;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) eq += key_at(q, j) == lo;
+        int before = warp_excl_scan(eq, lane, all);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t key = key_at(q, j);
+            const bool ok = key > lo || (key == lo && before < need);
+            before += key == lo;
+            const uint32_t m = __ballot_sync(kFull, ok);
+            if (ok) list[n + __popc(m & lt)] = order_word<W>(key, r.head + 8 * v + j);
+            n += __popc(m);
+        }
+        need = max(0, need - all);
+    }
+    __syncwarp();
+}
+
+// Orders a list of n words into `sorted`: a word's place is the number of larger ones, which the team's
+// lanes count together, 16 bytes of the list at a time.
+template <class W, class Sync>
+__device__ __forceinline__ void order_list(W* list, int n, W* sorted, int tid, int threads, Sync&& sync) {
+    constexpr int PER = 16 / sizeof(W);
+    const int pad = (n + PER - 1) & ~(PER - 1);
+    if (n + tid < pad) list[n + tid] = 0;                                 // larger than nothing
+    sync();
+#pragma unroll 1
+    for (int i = tid; i < n; i += 3 * threads) {                          // three words a pass: lists are a few words longer than K
+        const int i2 = i + threads, i3 = i + 2 * threads;
+        const W w1 = list[i], w2 = i2 < n ? list[i2] : (W)0, w3 = i3 < n ? list[i3] : (W)0;
+        int rank1 = 0, rank2 = 0, rank3 = 0;
+        auto count = [&](W o) { rank1 += o > w1; rank2 += o > w2; rank3 += o > w3; };
+#pragma unroll 2
+        for (int j = 0; j < pad; j += PER) {
+            const uint4 o = *reinterpret_cast<const uint4*>(list + j);
+            if constexpr (sizeof(W) == 4) { count(o.x); count(o.y); count(o.z); count(o.w); }
+            else { count((W)o.y << 32 | o.x); count((W)o.w << 32 | o.z); }
+        }
+        sorted[rank1] = w1;
+        if (i2 < n) sorted[rank2] = w2;
+        if (i3 < n) sorted[rank3] = w3;
+    }
+    sync();
+}
+// Writes the row's K selected from the ordered list (one warp).
+template <class W>
+__device__ __forceinline__ void emit_selected(const TopkArgs& a, long long rowi, const W* sorted, float lmax, float sum_all, int lane) {
+    constexpr int R = kFinal / 32;
+    const int K = a.K;
+    W v[R];
+    float ek[R], p = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        v[r] = r * 32 + lane < K ? sorted[r * 32 + lane] : (W)0;
+        ek[r] = r * 32 + lane < K ? expf(val_of_key(key_of_word<W>(v[r])) - lmax) : 0.f;
+        if (r * 32 + lane < K) p += ek[r];
+    }
+    const float sum_k = warp_sum(p);
+    const int idx0 = __shfl_sync(kFull, idx_of_word<W>(v[0]), 0);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int k = r * 32 + lane;
+        if (k < K) {
+            const float w = ek[r] / sum_k;
+            const int idx = idx_of_word<W>(v[r]);
+            if (a.pairs) put_pair(a, rowi, k, idx, w);
+            if (a.idx) a.idx[rowi * K + k] = idx;
+            if (a.w) a.w[rowi * K + k] = w;
+        }
+    }
+    if (a.pairs)
+        for (int k = K + lane; k < a.Kp; k += 32) put_pair(a, rowi, k, idx0, 0.f);
+    if (a.zk && lane == 0) a.zk[rowi] = sum_k / sum_all;
+}
+
+constexpr int kCntCodes = 17, kCntList = 18;        // places of the running totals behind the bound's 17 counters
+struct StreamShared {                               // of the warps that share a row (the first block's copy counts)
+    float ref[kStreamWarps * kMaxCluster], sum[kStreamWarps * kMaxCluster];
+    uint32_t key[kStreamWarps * kMaxCluster];
+    int cnt[19];                                    // of the end of the row, which the first block's warps share: see kCntCodes
 };
 
-__device__ __forceinline__ bool stage_wait(uint32_t bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kStageSpin; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-// The row after `rowi` (stride: the grid) that lies inside its session's position range, or N.
-__device__ __forceinline__ long long stage_next_row(const TopkArgs& a, long long rowi) {
-    for (; rowi < a.N; rowi += gridDim.x) {
+// The row after `rowi` (stride: the rows in work at a time) inside its session's position range, or N.
+__device__ __forceinline__ long long next_row(const TopkArgs& a, long long rowi, long long stride) {
+    for (; rowi < a.N; rowi += stride) {
         if (!(a.pos_begin || a.pos_end)) return rowi;
         const int s = (int)(rowi / a.n_per_session), i = (int)(rowi % a.n_per_session);
         const int b = a.pos_begin ? a.pos_begin[s] : 0, e = a.pos_end ? a.pos_end[s] : a.n_per_session;
@@ -593,311 +586,345 @@ __device__ __forceinline__ long long stage_next_row(const TopkArgs& a, long long
     return a.N;
 }
 
-__global__ void __launch_bounds__(kStageThreads) topk_staged_kernel(TopkArgs a) {
-    constexpr int THREADS = kStageThreads, NW = THREADS / 32;
-    extern __shared__ __align__(128) unsigned char stage_raw[];
-    const __half* buf = reinterpret_cast<const __half*>(stage_raw);
-    StageSm& sm = *reinterpret_cast<StageSm*>(stage_raw + stage_buf_bytes(a.V));
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int Vrow = a.V, K = a.K;
-    const int nchunks = stage_chunks(Vrow), ce = stage_chunk_elems(Vrow);
-    const int per_warp = (K + NW - 1) / NW;
-    const bool select = a.pairs || a.idx || a.w || a.zk;            // the launcher sends only one-chunk rows of the fast path here with a selection
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&sm.bar);
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage_raw);
+// Shared memory of a row: group maxima (binary16, two slots a word), groups to read again, the list.
+template <class W>
+constexpr size_t stream_smem_per_row() { return 32 * kSlots * 2 + kCodes * 2 + kListCap * sizeof(W); }
 
-    auto fetch = [&](long long rowi, int c) {                        // one thread: the whole chunk in one copy
-        const uint32_t bytes = (uint32_t)min(ce, Vrow - c * ce) * 2u;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the buffer's last readers used ordinary loads
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(dst), "l"(a.logits + rowi * (long long)Vrow + (long long)c * ce), "r"(bytes), "r"(bar) : "memory");
-    };
+__device__ __forceinline__ uint32_t cluster_blocks() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Generic address of the cluster's first block's copy of a shared-memory object.
+template <class T>
+__device__ __forceinline__ T* at_first_block(T* p) {
+    T* r;
+    asm("mapa.u64 %0, %1, %2;" : "=l"(r) : "l"(p), "r"(0u));
+    return r;
+}
 
-    long long rowi = stage_next_row(a, blockIdx.x);
-    int c = 0;
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(1u) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (tid == 0 && rowi < a.N) fetch(rowi, 0);
-    uint32_t parity = 0;
-    float run_max = 0.f, run_sum = 0.f;                              // over the chunks of the row so far
-    while (rowi < a.N) {
-        int next_c = c + 1;
-        long long next = rowi;
-        if (next_c == nchunks) { next_c = 0; next = stage_next_row(a, rowi + gridDim.x); }
-        const int V = min(ce, Vrow - c * ce);                        // logits in the buffer
-        const int ntiles = (V + THREADS * 8 - 1) / (THREADS * 8);
-        if (tid == 0) { sm.nlist = 0; sm.nhit = 0; }
-        bool ok = stage_wait(bar, parity);
-        if (!ok) ok = stage_wait(bar, parity);                        // a copy in flight is waited for once more before giving up
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0 && a.status) atomicOr(a.status, kStTimeout);
-            return;
-        }
-        parity ^= 1u;
-
-        // Pass 0: one maximum per thread.
-        uint32_t m2 = 0xfc00fc00u;                                   // (-inf, -inf)
-#pragma unroll 4
-        for (int t = 0; t < ntiles; ++t) {
-            const int i0 = t * (THREADS * 8) + tid * 8;
-            if (i0 < V) {
-                const uint4 r = *reinterpret_cast<const uint4*>(buf + i0);
-                m2 = hmax2_bits(m2, hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w)));
-            }
-        }
-        uint32_t tkey = max(key_of(m2 & 0xffffu), key_of(m2 >> 16));
-        if (tid * 8 >= V) tkey = 0;                                   // this thread owns nothing
-        const uint32_t wmax = __reduce_max_sync(kFull, tkey);
-        uint32_t wth = 0;
-        if (select) {
-            uint32_t v = tkey;
-            for (int r = 0; r < per_warp; ++r) {
-                wth = __reduce_max_sync(kFull, v);
-                const uint32_t eq = __ballot_sync(kFull, v == wth);
-                if (lane == __ffs(eq) - 1) v = 0;
-            }
-        }
-        if (lane == 0) { sm.red_k[wid] = wmax; sm.red_t[wid] = wth; }
-        __syncthreads();
-        uint32_t km = sm.red_k[0], theta = sm.red_t[0];
-#pragma unroll
-        for (int w = 1; w < NW; ++w) { km = max(km, sm.red_k[w]); theta = min(theta, sm.red_t[w]); }
-        theta = max(theta, kKeyNegInf);
-        const float lmax = val_of_key(km);
-
-        // Pass 1: sum of exp(l - l_max); groups of 8 with an element at or above the bound are noted.
-        const float nb = -lmax * 1.44269504088896341f;
-        const uint32_t tb = bits_of_key(theta);
-        const uint32_t th2 = tb | (tb << 16);
-        float s = 0.f;
-#pragma unroll 2
-        for (int t = 0; t < ntiles; ++t) {
-            const int i0 = t * (THREADS * 8) + tid * 8;
-            if (i0 < V) {
-                const uint4 r = *reinterpret_cast<const uint4*>(buf + i0);
-                const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
-                const uint32_t top = hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w));
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&wds[j]));
-                    s += exp_rel(f.x, nb);
-                    s += exp_rel(f.y, nb);
-                }
-                if (select && !__hblt2(*reinterpret_cast<const __half2*>(&top), *reinterpret_cast<const __half2*>(&th2))) {
-                    const int slot = atomicAdd(&sm.nhit, 1);
-                    if (slot < kCandCap) sm.hit[slot] = i0;
-                }
-            }
-        }
-        s = warp_sum(s);
-        if (lane == 0) sm.red_s[wid] = s;
-        __syncthreads();
-        float sum_all = 0.f;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) sum_all += sm.red_s[w];
-        int nlist = 0;
-        if (select) {
-            const int nhit = sm.nhit;
-            if (nhit <= kCandCap) {
-                for (int t = tid; t < nhit; t += THREADS) {
-                    const int i0 = sm.hit[t];
-                    const uint4 r = *reinterpret_cast<const uint4*>(buf + i0);
-                    const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) collect2(wds[j], th2, i0 + 2 * j, true, &sm.nlist, sm.list);
-                }
-            }
+// SHARE: the warps of a cluster of blocks (of a block, if it is alone) share a row; otherwise every warp
+// has a row of its own.
+template <bool SELECT, bool SHARE, class W>
+__global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const TopkArgs a) {
+    extern __shared__ __align__(16) unsigned char stream_raw[];
+    __shared__ StreamShared local_sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int blocks = SHARE ? (int)cluster_blocks() : 1;
+    const int NW = SHARE ? nwarps * blocks : 1, wrow = SHARE ? (int)cluster_rank() * nwarps + warp : 0;   // warps of the row, this one's number
+    StreamShared& sh = *(SHARE && blocks > 1 ? at_first_block(&local_sh) : &local_sh);
+    auto meet = [&]() {
+        if (blocks > 1) {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        } else {
             __syncthreads();
-            nlist = nhit <= kCandCap ? sm.nlist : kCandCap + 1;
         }
-        // the buffer is free: the next copy runs under the rest of this row
-        if (tid == 0 && next < a.N) fetch(next, next_c);
+    };
+    unsigned char* raw = stream_raw + (SHARE ? 0 : (size_t)warp * stream_smem_per_row<W>());
+    uint32_t* slots = reinterpret_cast<uint32_t*>(raw);                                  // [kSlots / 2][32]
+    uint16_t* codes = reinterpret_cast<uint16_t*>(slots + 16 * kSlots);
+    W* list = reinterpret_cast<W*>(codes + kCodes);
+    uint16_t* my_slots = reinterpret_cast<uint16_t*>(SHARE && blocks > 1 ? at_first_block(slots) : slots);
+    if (SHARE && blocks > 1) meet();                                                      // all blocks of the cluster have started
+    const int K = a.K;
+    const long long group = SHARE ? blockIdx.x / blocks : (long long)blockIdx.x * nwarps + warp;
+    const long long stride = SHARE ? gridDim.x / blocks : (long long)gridDim.x * nwarps;
 
-        // maximum and sum over the chunks so far (the same values in every thread)
-        float lmax_row = lmax, sum_row = sum_all;
-        if (c > 0) {
-            lmax_row = fmaxf(run_max, lmax);
-            sum_row = (run_max > -INFINITY ? run_sum * expf(run_max - lmax_row) : 0.f) +
-                      (lmax > -INFINITY ? sum_all * expf(lmax - lmax_row) : 0.f);
-        }
-        run_max = lmax_row; run_sum = sum_row;
-
-        if (next_c == 0) {                                               // last chunk: the row is complete
-            const bool handed = select && nlist >= K && nlist <= kTopkListCap;
-            if (select) {
-                if (tid == 0) {
-                    a.cand_hdr[rowi] = make_float4(lmax_row, sum_row, __int_as_float(handed ? nlist : kHdrRedo), 0.f);
-                    if (!handed) atomicAdd(a.redo, 1u);
-                }
-                if (handed) {
-                    uint32_t* out = static_cast<uint32_t*>(a.cand) + rowi * kTopkListCap;
-                    for (int i = tid; i < nlist; i += THREADS) out[i] = sm.list[i];
-                }
+    for (long long rowi = next_row(a, group, stride); rowi < a.N; rowi = next_row(a, rowi + stride, stride)) {
+        const RowView r = row_view(a.logits + rowi * (long long)a.V, a.V);
+        const int per = kBatch * 32 * NW, batches = max(1, (r.nv + per - 1) / per);
+        // Slots of this warp: one a group of 8 where all the row's fit, else one for every `wide` batches.
+        const bool fine = NW * batches * kBatch <= kSlots;
+        const int wide = (NW * batches + kSlots - 1) / kSlots, ns = fine ? batches * kBatch : (batches + wide - 1) / wide;
+        const int v0 = wrow * 32 + lane;                                                  // group u of batch t: v0 + (t * kBatch + u) * 32 * NW
+        auto load = [&](int t, uint4 (&q)[kBatch]) {
+            const uint4* p = r.body + v0 + t * per;
+            if ((t + 1) * per <= r.nv) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) q[u] = ldg_stream(p + u * 32 * NW);
+            } else {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) q[u] = v0 + t * per + u * 32 * NW < r.nv ? ldg_stream(p + u * 32 * NW) : all4(kNegInf2);
             }
-            if (tid == 0 && (!select || handed)) {                      // a row that is left over gets these from the general kernel
-                const float lse = lmax_row + logf(sum_row);
-                if (a.lse) a.lse[rowi] = lse;
-                if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) {
-                    const int tk = a.tokens[rowi];
-                    const float v = (tk >= 0 && tk < Vrow) ? (__half2float(a.logits[rowi * (long long)Vrow + tk]) - lse) * 1.44269504088896341f
-                                                           : __int_as_float(0x7fc00000);
-                    if (a.logp2) a.logp2[rowi] = v;
-                    if (a.step_exp || a.bits_out) {
-                        // Def. 7: b = max(1, floor(b0 h / hbar)), capped at b0 + extra; decided in binary32
-                        const float r = __fmul_rn((float)a.b0, __fdiv_rn(-v, a.hbar));
-                        int b = (r >= 1.0f) ? (int)floorf(r) : 1;
-                        b = min(b, a.b0 + a.extra);
-                        if (a.step_exp) a.step_exp[rowi] = a.b0 - b;
-                        if (a.bits_out) a.bits_out[rowi] = b;
+        };
+        uint4 cur[kBatch], nxt[kBatch];
+        load(0, cur);
+        load(1, nxt);
+        const bool has_ends = wrow == 0 && (r.head > 0 || r.head + 8 * r.nv < r.V);
+        const uint4 ends = has_ends ? row_ends(r, lane) : all4(kNoValue2);
+        uint32_t m2 = kNegInf2;
+        if (has_ends) m2 = hmax2_bits(m2, top2_of(ends));
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) m2 = hmax2_bits(m2, top2_of(cur[u]));
+        float ref = fmaxf(val_of_key(__reduce_max_sync(kFull, top_key(m2))), -65504.0f);
+        // A logit more than 4 above the reference moves it, so that no exponent is large (its rounding would
+        // show in the sum).
+        auto lim_of = [](float rf) { const uint32_t b = (uint32_t)__half_as_ushort(__float2half_ru(rf + 4.0f)); return b | (b << 16); };
+        uint32_t lim2 = lim_of(ref);
+        float nb = -ref * 1.44269504088896341f;
+        unsigned long long s0 = 0ull, s1 = 0ull;
+        auto add_group = [&](const uint4& q) {
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+            const unsigned long long l2e = both(1.44269504088896341f, 1.44269504088896341f), nb2 = both(nb, nb);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 f = __half22float2(as_half2(w[j]));
+                float x, y, ex, ey;
+                parts(fma2(both(f.x, f.y), l2e, nb2), x, y);
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
+                if (j & 1) s1 = add2(s1, both(ex, ey)); else s0 = add2(s0, both(ex, ey));
+            }
+        };
+        if (has_ends) {
+            auto real = [](uint32_t w) { const uint32_t m = __vcmpeq2(w, kNoValue2); return (w & ~m) | (kNegInf2 & m); };
+            add_group(make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)));
+        }
+        // slot s of a lane: half s & 1 of word (s / 2, lane)
+        auto put_slot = [&](int slot, uint32_t top2) {
+            const int sl = wrow * ns + slot;
+            my_slots[(sl >> 1) * 64 + lane * 2 + (sl & 1)] = (uint16_t)hmax2_bits(top2, top2 >> 16);   // the low half: of both
+        };
+        auto batch = [&](const uint4 (&q)[kBatch], uint32_t (&top)[kBatch]) {             // returns the maximum
+            uint32_t top4 = kNegInf2;
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) { top[u] = top2_of(q[u]); top4 = hmax2_bits(top4, top[u]); }
+            m2 = hmax2_bits(m2, top4);
+            if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
+                const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
+                const float f = expf(ref - to);
+                const unsigned long long ff = both(f, f), z = 0ull;
+                s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
+                ref = to; nb = -ref * 1.44269504088896341f; lim2 = lim_of(ref);
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) add_group(q[u]);
+            return top4;
+        };
+        uint32_t top[kBatch];
+        if (SELECT && fine) {
+#pragma unroll 1
+            for (int t = 0; t < batches; ++t) {
+                batch(cur, top);
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) { put_slot(t * kBatch + u, top[u]); cur[u] = nxt[u]; }
+                load(t + 2, nxt);
+            }
+        } else {
+            uint32_t group2 = kNegInf2;                                                   // of the slot being filled
+            int left = wide, slot = 0;
+            auto filled = [&](uint32_t top4) {
+                group2 = hmax2_bits(group2, top4);
+                if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = wide; }
+            };
+#pragma unroll 1
+            for (int t = 0; t < batches; t += 2) {
+                const uint32_t t0 = batch(cur, top);
+                if (SELECT) filled(t0);
+                load(t + 2, cur);
+                if (t + 1 < batches) {
+                    const uint32_t t1 = batch(nxt, top);
+                    if (SELECT) filled(t1);
+                }
+                load(t + 3, nxt);
+            }
+            if (SELECT && left != wide) put_slot(slot, group2);
+        }
+
+        // Row maximum and sum.
+        uint32_t kmax = __reduce_max_sync(kFull, top_key(m2));
+        float x0, x1, x2, x3;
+        parts(s0, x0, x1); parts(s1, x2, x3);
+        float sum_all = warp_sum((x0 + x1) + (x2 + x3)), lmax;
+        if (SHARE) {
+            if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
+            if (SELECT && wrow == 0 && lane < 19) sh.cnt[lane] = 0;
+            meet();
+            for (int w = 0; w < NW; ++w) kmax = max(kmax, sh.key[w]);
+            lmax = val_of_key(kmax);
+            sum_all = 0.f;
+            for (int w = 0; w < NW; ++w) sum_all += sh.sum[w] * expf(sh.ref[w] - lmax);
+        } else {
+            lmax = val_of_key(kmax);
+            sum_all *= expf(ref - lmax);
+        }
+
+        if (SELECT && (!SHARE || wrow < nwarps)) {
+            // The row's own warp, or all warps of the first block.
+            const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
+            auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
+            // The bound: the K-th largest group maximum (any value that exactly K of them reach will do).
+            const int S = NW * ns, words = (S + 1) >> 1;
+            if ((S & 1) && tw == 0) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
+            sync();
+            uint32_t mx[kSlots / 2];                                                      // this warp's words, two maxima each
+#pragma unroll
+            for (int i = 0; i < kSlots / 2; ++i) mx[i] = tw + i * tws < words ? slots[(tw + i * tws) * 32 + lane] : kNoValue2;
+            uint32_t theta = kKeyNegInf, hi = kmax + 1, down = 256;                       // first downwards from the maximum, then between
+#pragma unroll 1
+            for (int it = 0; hi - theta > 1; ++it) {
+                const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
+                __half2 c2 = __float2half2_rn(0.f);
+#pragma unroll
+                for (int i = 0; i < kSlots / 2; i += 4) {
+                    if (tw + i * tws < words) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) c2 = __hadd2(c2, __hge2(as_half2(mx[i + k]), as_half2(h2)));
+                    }
+                }
+                int c = __reduce_add_sync(kFull, __half2int_rn(__hadd(__low2half(c2), __high2half(c2))));
+                if (SHARE) {
+                    if (lane == 0) atomicAdd(&local_sh.cnt[it], c);
+                    sync();
+                    c = local_sh.cnt[it];
+                }
+                if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
+                if (c == K) break;
+            }
+            // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
+            auto place = [&](int mine, int* shared_total, int& total) {
+                int all;
+                int at = warp_excl_scan(mine, lane, all);
+                int base = total;
+                if (SHARE) {
+                    if (lane == 0) base = atomicAdd(shared_total, all);
+                    base = __shfl_sync(kFull, base, 0);
+                }
+                total += all;                                                             // SHARE: of this warp only
+                return base + at;
+            };
+            // The groups that reach it.
+            const uint32_t th2 = bits_of_key(theta) * 0x10001u;
+            int n_codes = 0, n = 0;
+            uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
+#pragma unroll
+            for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= __hge2_mask(as_half2(mx[i]), as_half2(th2)) & (0x10001u << (i & 15));
+            int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.cnt[kCntCodes], n_codes);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                for (uint32_t m = hits[h]; m; m &= m - 1) {
+                    const int b = __ffs(m) - 1, i = tw + (16 * h + (b & 15)) * tws;
+                    if (at < kCodes) codes[at] = (uint16_t)((2 * i + (b >> 4)) * 32 + lane);
+                    ++at;
+                }
+            sync();
+            if (SHARE) n_codes = local_sh.cnt[kCntCodes];
+            if (n_codes <= kCodes) {
+                // their logits at or above the bound; head and tail of the row are a turn of their own
+#pragma unroll 1
+                for (int i0 = tw * 32 - (has_ends ? 32 : 0); i0 < n_codes; i0 += i0 < 0 ? 32 : 32 * tws) {
+                    const bool mine = i0 >= 0 && i0 + lane < n_codes;
+                    const int code = mine ? codes[i0 + lane] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
+                    const int steps = i0 < 0 || fine ? 1 : wide;
+#pragma unroll 1
+                    for (int st = 0; st < steps; ++st) {
+                        const int t = fine ? ls >> 2 : ls * wide + st;
+                        const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
+                        uint4 q[kBatch];
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const int v = vb + u * 32 * NW;
+                            q[u] = mine && v < r.nv && !(fine && u) ? __ldg(r.body + v) : all4(kNoValue2);
+                        }
+                        if (i0 < 0) q[0] = row_ends(r, lane);
+                        uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) {
+                            const uint32_t w4[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
+                        }
+                        for (int to = place(__popc(m), &local_sh.cnt[kCntList], n); m; m &= m - 1, ++to) {
+                            const int b = __ffs(m) - 1, u = (b >> 2) & 3;
+                            const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
+                            const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
+                            if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(__ldg(r.row + e))), e);   // a first-level hit
+                        }
                     }
                 }
             }
-        }
-        __syncthreads();                                                 // sm.list, sm.nlist are free again
-        rowi = next; c = next_c;
-    }
-}
-
-// One compare-exchange step of a bitonic network on 256 order words held 8 per lane: word e = r * 32 +
-// lane sits in v[r].  K2 = the size of the bitonic blocks being merged, J = the distance.  The
-// network sorts descending overall.
-template <class W, int K2, int J>
-__device__ __forceinline__ void bitonic_step(W (&v)[8], int lane) {
-    if constexpr (J >= 32) {
-        constexpr int RJ = J >> 5;
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            if ((r & RJ) == 0) {
-                const bool desc = (((r * 32) & K2) == 0) || K2 == 256;       // K2 >= 64 here: the bit of e lies in r
-                const W x = v[r], y = v[r | RJ];
-                const bool sw = desc ? (x < y) : (x > y);
-                v[r] = sw ? y : x; v[r | RJ] = sw ? x : y;
+            sync();
+            if (SHARE) n = local_sh.cnt[kCntList];
+            if (n_codes > kCodes || n > kListCap) {
+                if (tw == 0) slow_select<W>(r.row, r.V, K, theta, kmax, list, lane);
+                n = K;
+                sync();
             }
+            W* sorted = reinterpret_cast<W*>(slots);                                      // the maxima are done with
+            order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);
+            if (tw == 0) emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
         }
-    } else {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const W p = __shfl_xor_sync(kFull, v[r], J);
-            const int e = r * 32 + lane;
-            const bool lower = (lane & J) == 0;
-            const bool desc = K2 == 256 || (e & K2) == 0;
-            const bool keep_max = lower == desc;
-            const W mx = v[r] > p ? v[r] : p, mn = v[r] > p ? p : v[r];
-            v[r] = keep_max ? mx : mn;
+        if (lane == 0 && wrow == 0) {
+            const float lse = lmax + logf(sum_all);
+            if (a.lse) a.lse[rowi] = lse;
+            if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) put_surprisal(a, rowi, r.row, lse);
         }
-    }
-}
-template <class W, int K2, int J>
-__device__ __forceinline__ void bitonic_merge(W (&v)[8], int lane) {
-    bitonic_step<W, K2, J>(v, lane);
-    if constexpr (J > 1) bitonic_merge<W, K2, J / 2>(v, lane);
-}
-template <class W, int K2>
-__device__ __forceinline__ void bitonic_sort256(W (&v)[8], int lane) {
-    if constexpr (K2 > 2) bitonic_sort256<W, K2 / 2>(v, lane);
-    bitonic_merge<W, K2, K2 / 2>(v, lane);
-}
-
-// Second kernel of the two-kernel selection: one warp per row sorts the row's candidate list (at
-// most 256 order words, larger = earlier in (logit descending, index ascending)) in registers and
-// writes what the streaming kernel would have written for the first K: order, renormalised weights
-// (the same sums in the same order), Z_k.  Rows the streaming kernel finished itself carry -1.
-template <bool NARROW>
-__global__ void __launch_bounds__(256) topk_rank_kernel(TopkArgs a) {
-    using W = std::conditional_t<NARROW, uint32_t, unsigned long long>;
-    const int lane = threadIdx.x & 31, K = a.K;
-    const long long warp = (long long)blockIdx.x * 8 + (threadIdx.x >> 5), nw = (long long)gridDim.x * 8;
-    for (long long rowi = warp; rowi < a.N; rowi += nw) {
-        if (a.pos_begin || a.pos_end) {
-            int s = (int)(rowi / a.n_per_session), i = (int)(rowi % a.n_per_session);
-            int b = a.pos_begin ? a.pos_begin[s] : 0, e = a.pos_end ? a.pos_end[s] : a.n_per_session;
-            if (i < b || i >= e) continue;
-        }
-        const float4 hdr = a.cand_hdr[rowi];
-        const int nlist = __float_as_int(hdr.z);
-        if (nlist < 0) continue;
-        const W* src = static_cast<const W*>(a.cand) + rowi * kTopkListCap;
-        W v[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = r * 32 + lane < nlist ? src[r * 32 + lane] : (W)0;   // 0 orders after everything
-        bitonic_sort256<W, 256>(v, lane);
-        const float lmax = hdr.x;
-        float ek[4];
-        int idx[4];
-        float p = 0.f;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {                   // K <= 128: the first K words sit in v[0..3]
-            const uint32_t key = NARROW ? (uint32_t)(v[r] >> 16) : (uint32_t)((unsigned long long)v[r] >> 32);
-            idx[r] = NARROW ? (int)(0xffffu - ((uint32_t)v[r] & 0xffffu)) : (int)(0xffffffffu - (uint32_t)v[r]);
-            ek[r] = r * 32 + lane < K ? expf(val_of_key(key) - lmax) : 0.f;
-            if (r * 32 + lane < K) p += ek[r];
-        }
-        const float sum_k = warp_sum(p);
-        const int idx0 = __shfl_sync(kFull, idx[0], 0);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int k = r * 32 + lane;
-            if (k < K) {
-                const float w = ek[r] / sum_k;
-                if (a.pairs) a.pairs[rowi * a.Kp + k] = make_int2(idx[r], __float_as_int(w));
-                if (a.idx) a.idx[rowi * K + k] = idx[r];
-                if (a.w) a.w[rowi * K + k] = w;
-            }
-        }
-        if (a.pairs)
-            for (int k = K + lane; k < a.Kp; k += 32) a.pairs[rowi * a.Kp + k] = make_int2(idx0, 0);
-        if (a.zk && lane == 0) a.zk[rowi] = sum_k / hdr.y;
+        __syncwarp();
+        if (SHARE) meet();                                                                // the row's shared state is free again
     }
 }
 
 }  // namespace
+
+template <bool SELECT, class W>
+static cudaError_t launch_stream(const TopkArgs& a, int sms, cudaStream_t st) {
+    // Warps a row, in powers of two, each with at least 1024 logits of its own; one when rows alone fill the
+    // GPU.  Up to a block of eight: as many as the GPU holds for all rows (32 a SM).  Up to four blocks (a
+    // cluster): only while that is a quarter of the GPU, since a cluster's blocks are placed together
+    // (64 rows of 128256, 64 warps each: 51 us; 16 warps: 25; one row: 8 warps 24.6, 32 warps 20.5).
+    int warps = 1;
+    while (warps < kStreamWarps * kMaxCluster && 2ll * warps * 1024 <= a.V &&
+           2ll * warps * a.N <= (warps < kStreamWarps ? 32ll : 8ll) * sms) warps *= 2;
+    const bool share = warps > 1;
+    const int per_block = share ? std::min(warps, kStreamWarps) : kStreamWarps, cluster = share ? warps / per_block : 1;
+    const size_t smem = !SELECT ? 0 : stream_smem_per_row<W>() * (share ? 1 : per_block);
+    auto kern = share ? topk_stream_kernel<SELECT, true, W> : topk_stream_kernel<SELECT, false, W>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    int occ = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, per_block * 32, smem) != cudaSuccess || occ < 1) occ = 1;
+    const long long want = share ? a.N * cluster : (a.N + per_block - 1) / per_block;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster));
+    cfg.blockDim = dim3(per_block * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cluster; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    e = cudaLaunchKernelEx(&cfg, kern, a);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
 
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
     if (a.N <= 0) return cudaSuccess;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
+    const bool select = a.pairs || a.idx || a.w || a.zk;
+    if (!select) return launch_stream<false, uint32_t>(a, sms, st);
+    if (a.K <= kFinal) return a.V <= 65536 ? launch_stream<true, uint32_t>(a, sms, st) : launch_stream<true, unsigned long long>(a, sms, st);
     // The second pass over a row should find it in L2: rows of up to 128 KB are read by 256 threads
     // with five blocks per SM, longer rows by 512 threads with two blocks per SM (two, so that one
     // block streams while the other sits at the barrier between its passes).
+    const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     const bool wide = (long long)a.V * 2 > 128 * 1024;
-    TopkArgs g = a;                                           // what the general kernel is launched with
     auto launch = [&](auto kern, int threads, int cap) {
         int occ = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0) != cudaSuccess || occ < 1) occ = 1;
         const long long per_sm = occ < cap ? occ : cap;       // the rows in flight stay within L2
         const long long blocks = a.N < sms * per_sm ? a.N : sms * per_sm;
-        kern<<<(unsigned)blocks, threads, 0, st>>>(g);
+        kern<<<(unsigned)blocks, threads, 0, st>>>(a);
     };
-    const bool select = a.pairs || a.idx || a.w || a.zk;
-    // The staged kernel takes what it can finish: calls without a selection (rows of any length, in
-    // chunks), and rows that fit in its buffer when the selection can be handed to the ranking
-    // kernel (K <= 128 and the scratch for it).
-    const bool staged = vec && (select ? (long long)a.V * 2 <= kStageBytes && a.K <= 128 && a.cand && a.cand_hdr && a.redo
-                                       : a.V < (1 << 30));
-    cudaError_t e = cudaSuccess;
-    if (staged) {
-        const size_t smem = stage_buf_bytes(a.V) + sizeof(StageSm);
-        e = cudaFuncSetAttribute(topk_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (select) {
-            e = cudaMemsetAsync(a.redo, 0, sizeof(unsigned int), st);
-            if (e != cudaSuccess) return e;
-        }
-        int occ = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, topk_staged_kernel, kStageThreads, smem) != cudaSuccess || occ < 1) occ = 1;
-        const long long blocks = a.N < (long long)sms * occ ? a.N : (long long)sms * occ;
-        topk_staged_kernel<<<(unsigned)blocks, kStageThreads, smem, st>>>(a);
-        count_launch();
-        e = cudaGetLastError();
-        if (e != cudaSuccess || !select) return e;
-        g.redo_only = 1;                                      // then only what the staged kernel left over
-    }
     if (wide) {
         if (vec) launch(topk_softmax_kernel<true, 512>, 512, 2);
         else launch(topk_softmax_kernel<false, 512>, 512, 2);
@@ -906,17 +933,7 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
         else launch(topk_softmax_kernel<false, 256>, 256, 5);
     }
     count_launch();
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (a.cand && a.cand_hdr && select && a.K <= 128) {
-        const long long want = (a.N + 7) / 8, cap = (long long)sms * 8;
-        const unsigned blocks = (unsigned)(want < cap ? want : cap);
-        if (a.V <= 65536) topk_rank_kernel<true><<<blocks, 256, 0, st>>>(a);
-        else topk_rank_kernel<false><<<blocks, 256, 0, st>>>(a);
-        count_launch();
-        e = cudaGetLastError();
-    }
-    return e;
+    return cudaGetLastError();
 }
 
 }  // namespace plc
