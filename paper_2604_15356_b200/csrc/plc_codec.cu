@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const Co
             if (lane == 0 && !FROM_OPEN) { a.st.chunk_offset[it.slot] = 0; a.st.chunk_bytes[it.slot] = 0; }
             continue;
         }
-        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
         const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         uint32_t x = kRansL;
         int wp = cap_words;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const Co
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
                 int zero_q = ZR ? a.sh.zero_q : 0;
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const Co
         const int last = nwords - 1;                 // -1 for a chunk of states only: words[-1] is inside the chunk
         auto read_word = [&](int i) { return (uint32_t)__ldg(words + min(i, last)); };   // past the end: the last word
         int rp = 0;
-        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
         const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
         __syncwarp();
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const Co
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
             int zero_q = ZR ? a.sh.zero_q : 0;
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) rotq_kernel(const Code
     for (unsigned item = next_queued(a, qc, per_table, Wt, lane); item < total; item = next_queued(a, qc, per_table, Wt, lane)) {
         const Item it = bulk_item(a, item);
         if (it.P <= 0) continue;
-        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+        const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
         const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
         __syncwarp();
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) rotq_kernel(const Code
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -434,8 +434,8 @@ __global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_k
                 floor2 = a.sh.sigma_floor * a.sh.sigma_floor;
     const int c0 = first_comp<D>(lane);
     for (long long item = gw; item < (long long)Wt * a.S; item += nw) {
-        const int t = (int)(item / a.S), b = (int)(item % a.S);
-        const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+        const int t = (int)from_lane0((unsigned)(item / a.S), lane), b = (int)(item % a.S);
+        const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D);
         const int2* gp = a.pairs + (long long)b * Kp;
         __syncwarp();
         prefetch_pairs(sp, gp, Kp, lane);
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_k
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;
@@ -464,7 +464,7 @@ cudaError_t pair_smem_bytes(Kern kern, int Kp, size_t& bytes) {
 
 int codec_grid_warps(int) { return sm_count() * kBlocksPerSM * kWarpsPerBlock; }
 
-static void set_queues(CodecArgs& a, int n_tables);
+static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kBlocksPerSM * kWarpsPerBlock);
 
 #include <cstdlib>
 static bool use_coop(const CodecArgs& a) {
@@ -485,8 +485,8 @@ void codec_schedule(const CodecArgs& a0, int n_tables, int* nq, int* g) {
     *nq = a.sched_nq; *g = a.sched_g;
 }
 
-static void set_queues(CodecArgs& a, int n_tables) {
-    const int sms = sm_count(), warps_per_sm = kBlocksPerSM * kWarpsPerBlock;
+static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
+    const int sms = sm_count(), warps_per_sm = items_per_sm;
     const long long per_table = std::max(1LL, (long long)a.S * a.st.max_chunks);
     const long long spanned = ((long long)sms * warps_per_sm + per_table - 1) / per_table + 1;
     const double table_bytes = 2.0 * a.sh.V * a.sh.d;
@@ -516,6 +516,7 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
     set_queues(a, 2 * a.sh.L * a.sh.H);
     cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
     if (e != cudaSuccess) return e;
+    if (use_coop(a)) set_queues(a, 2 * a.sh.L * a.sh.H, 4);
     if (use_coop(a)) return launch_coop(a, true, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.dbg.ideal || a.step_exp;
@@ -558,6 +559,7 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
     set_queues(a, 2 * a.sh.L * a.sh.H);
     cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
     if (e != cudaSuccess) return e;
+    if (use_coop(a)) set_queues(a, 2 * a.sh.L * a.sh.H, 4);
     if (use_coop(a)) return launch_coop(a, false, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.step_exp;

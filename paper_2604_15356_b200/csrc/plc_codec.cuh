@@ -51,34 +51,53 @@ __device__ __forceinline__ void ffma2(unsigned long long& acc, unsigned long lon
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-// Mixture of one position for one table.  sp: the position's Kp {idx, w} entries in shared memory,
-// Kp = K rounded up to a multiple of ROWS (the padding has weight 0 and a valid index).
+// acc2 += w * (8 components of a row): four pairs.
+__device__ __forceinline__ void add_row(const char* p, float w, unsigned long long (&acc2)[4]) {
+    const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
+    const unsigned long long ww = pack2(w, w);
+    const __half2* hp = reinterpret_cast<const __half2*>(&r);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(hp[j]);
+        ffma2(acc2[j], ww, pack2(f.x, f.y));
+    }
+}
+// Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
+// offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
+// multiple of 2 ROWS (the padding has weight 0 and a valid offset).  table, n2: the table's rows and
+// their squared norms, the same pointers in every lane.
+// What bounds it: issue slots (per row and lane 8 conversions, 4 packed FMAs, a load), with the rows'
+// latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
+// beside its load.
 template <int D>
-__device__ __forceinline__ void predict(const char* __restrict__ col, const float* __restrict__ n2,
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, bool pair_index,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
-    const int h = lane / R;
+    const int h = lane / R, iters = Kp / ROWS;
+    const uint32_t lane_off = 16u * (lane % R);
     // variance term first: its row-norm loads are in flight while the rows are gathered
     float s1 = 0.f;
     for (int k = lane; k < Kp; k += 32) {
-        const int2 pr = sp[k];
-        s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + pr.x), s1);
+        const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
+        const uint32_t at = pair_index ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
+        s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
-    const int2* pl = sp + h;
-    const int iters = Kp / ROWS;
-#pragma unroll kGatherUnroll
-    for (int it = 0; it < iters; ++it) {
-        const int2 pr = pl[it * ROWS];
-        const float w = __int_as_float(pr.y);
-        const uint4 r = __ldg(reinterpret_cast<const uint4*>(col + (long long)pr.x * (D * 2)));
-        const unsigned long long ww = pack2(w, w);
-        const __half2* hp = reinterpret_cast<const __half2*>(&r);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __half22float2(hp[j]);
-            ffma2(acc2[j], ww, pack2(f.x, f.y));
+    if (!pair_index) {
+        const int4* pl = reinterpret_cast<const int4*>(sp + h * iters);
+        constexpr int kUnroll = kGatherUnroll / 2;
+#pragma unroll kUnroll
+        for (int it = 0; it < iters / 2; ++it) {
+            const int4 pr = pl[it];
+            add_row(table + ((uint32_t)pr.x + lane_off), __int_as_float(pr.y), acc2);
+            add_row(table + ((uint32_t)pr.z + lane_off), __int_as_float(pr.w), acc2);
+        }
+    } else {                                                 // tables of 4 GB or more: 64-bit offsets
+#pragma unroll 1
+        for (int it = 0; it < iters; ++it) {
+            const int2 pr = sp[h * iters + it];
+            add_row(table + ((size_t)(uint32_t)pr.x * (2 * D) + lane_off), __int_as_float(pr.y), acc2);
         }
     }
     float acc[8];
@@ -100,27 +119,27 @@ __device__ __forceinline__ void predict(const char* __restrict__ col, const floa
         }
         cnt = half;
     }
+    float s2 = 0.f;
 #pragma unroll
-    for (int g = 0; g < G; ++g) mu[g] = acc[g];
-    // variance: (sum_k w_k ||T_k||^2 - ||mu||^2) / d
-    s1 = warp_sum(s1);
-    float s2 = warp_norm2<G>(mu);
-    sigma2 = fmaxf(0.f, (s1 - s2) * inv_d);
+    for (int g = 0; g < G; ++g) { mu[g] = acc[g]; s2 = __fmaf_rn(mu[g], mu[g], s2); }
+    // variance: (sum_k w_k ||T_k||^2 - ||mu||^2) / d.  Both sums over the warp in one butterfly: after the
+    // first exchange the lower half-warp carries s1 and the upper s2 (the additions are warp_sum's, so a
+    // point-mass mixture has exactly zero variance).
+    const bool up = (lane & 16) != 0;
+    float v = (up ? s2 : s1) + __shfl_xor_sync(kFull, up ? s1 : s2, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    const float other = __shfl_xor_sync(kFull, v, 16);
+    sigma2 = fmaxf(0.f, (up ? other - v : v - other) * inv_d);
 }
 
 // The pairs of a position are brought into the warp's shared-memory slot with cp.async, one
-// position ahead of their use and without passing through registers (two slots per warp).
+// position ahead of their use and without passing through registers (two slots per warp): two entries
+// (16 bytes) per copy, Kp is even.
 __device__ __forceinline__ void prefetch_pairs(int2* sp, const int2* __restrict__ gp, int Kp, int lane) {
-    if ((Kp & 1) == 0) {                            // two entries (16 bytes) per copy: the slots and the rows of `pairs` are 16-byte aligned
-        for (int k = 2 * lane; k < Kp; k += 64) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(sp + k);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gp + k) : "memory");
-        }
-    } else {
-        for (int k = lane; k < Kp; k += 32) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(sp + k);
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(gp + k) : "memory");
-        }
+    for (int k = 2 * lane; k < Kp; k += 64) {
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(sp + k);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(gp + k) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -343,9 +362,8 @@ __device__ __forceinline__ void commit_chunk(const CodecArgs& a, long long slot,
 
 // Quantiser decision in binary32: sym = rint((kv - mu) * fl(1/delta)), clamped to +-2^30.
 __device__ __forceinline__ int quantise(float kv, float mu, float inv_delta) {
-    float n = rintf(__fmul_rn(__fsub_rn(kv, mu), inv_delta));
-    n = fminf(fmaxf(n, -(float)kSymLimit), (float)kSymLimit);
-    return (int)n;
+    const float n = __fmul_rn(__fsub_rn(kv, mu), inv_delta);
+    return __float2int_rn(fminf(fmaxf(n, -(float)kSymLimit), (float)kSymLimit));   // the limits are whole numbers: as if rounded first
 }
 
 extern __shared__ __align__(16) int2 g_pair_smem[];   // per warp: two slots of Kp entries

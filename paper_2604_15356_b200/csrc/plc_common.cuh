@@ -126,8 +126,8 @@ void count_launch(int n = 1);
 // Internal launchers (one per .cu file).
 struct TopkArgs {
     const __half* logits; const int32_t* tokens; int64_t N; int V, K;
-    int2* pairs;            // [N][Kp] {idx, float bits of w}, or null; entries K..Kp-1 get {idx_0, 0}
-    int Kp;
+    int2* pairs;            // [N][Kp], or null: see put_pair; entries K..Kp-1 get candidate 0 with weight 0
+    int Kp, pair_rows, pair_mul;   // log2 of the rows a warp-wide load fetches; bytes of a table row (1: pairs hold indices)
     int32_t* idx; float* w; float* lse; float* zk; float* logp2;   // optional user outputs
     // Adaptive step (needs tokens): step_exp[row] = b0 - b_i, bits_out[row] = b_i (both optional).
     int* step_exp; int* bits_out; int b0, extra; float hbar;
@@ -145,7 +145,7 @@ cudaError_t launch_prefix_clusters(const int32_t* lcp, const float* dT, int S, f
 constexpr int kZeroOff = -1000000;
 
 struct CodecShape {
-    int L, H, d, V, K, Kp, chunk_pos, out_dtype;   // Kp: K rounded up to the rows one warp-wide load fetches
+    int L, H, d, V, K, Kp, chunk_pos, out_dtype;   // Kp: K rounded up to twice the rows one warp-wide load fetches
     float delta, sigma_floor;
     float inv_delta, inv_delta2;   // fl(1/delta), fl(1/(delta*delta)), rounded once on the host
     int zero_q;                    // zero-rate rule (Thm. 3): positions of class <= zero_q carry no symbols (kZeroOff = never)
@@ -171,7 +171,8 @@ struct CodecArgs {
     CodecShape sh;
     const CoderTables* tables;                     // frequency tables of the coder
     const __half* T; const float* rownorm2;        // [tables][V][d], [tables][V]
-    const int2* pairs;                             // [S*n][Kp]
+    const int2* pairs;                             // [S*n][Kp] (written by the top-K kernels, put_pair)
+    bool pair_index;                               // pairs hold row indices instead of byte offsets (tables of 4 GB or more)
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
     KvView kv;                                     // encode: input f16; decode: output
     int S, n; const int32_t* pos_begin; const int32_t* pos_end;

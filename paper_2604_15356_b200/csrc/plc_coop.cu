@@ -136,10 +136,10 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
     const int P = sh.item.it.P, Kp = DENSE ? 0 : a.sh.Kp, n_batches = (P + NP - 1) / NP, c0 = first_comp<D>(lane);
-    const int t = sh.item.it.t, t0 = DENSE ? a.dense_t0 : 0;
+    const int t = (int)from_lane0((unsigned)sh.item.it.t, lane), t0 = DENSE ? a.dense_t0 : 0;
     const int first = ENC ? P - 1 : 0, dir = ENC ? -1 : 1;
     const long long row0 = sh.item.row0;
-    const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D + 8 * (lane % Geo<D>::R));
+    const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D);
     const float* n2 = a.rownorm2 + (size_t)t * a.sh.V;
     const bool zr = a.sh.zero_q != kZeroOff;
     int buf = 0;
@@ -211,7 +211,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                 if (k + NP < P) { fetch(k + NP, buf ^ 1); pairs_ready<1>(); }
                 else pairs_ready<0>();
                 buf ^= 1;
-                predict<D>(col, n2, sp, Kp, lane, 1.0f / D, mu, sigma2);
+                predict<D>(col, n2, a.pair_index, sp, Kp, lane, 1.0f / D, mu, sigma2);
             }
             float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
             int zero_q = a.sh.zero_q;
