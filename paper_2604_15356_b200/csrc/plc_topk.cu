@@ -571,11 +571,14 @@ __device__ __forceinline__ void emit_selected(const TopkArgs& a, long long rowi,
     if (a.zk && lane == 0) a.zk[rowi] = sum_k / sum_all;
 }
 
-constexpr int kCntCodes = 17, kCntList = 18;        // places of the running totals behind the bound's 17 counters
+// Counters of the end of a row: one a step of the search for the bound (at most 4 downwards and 16 between),
+// and the running totals of the groups and the list.
+constexpr int kBoundSteps = 20, kCntCodes = 30, kCntList = 31;
+static_assert(kBoundSteps < kCntCodes, "the search must not reach the totals");
 struct StreamShared {                               // of the warps that share a row (the first block's copy counts)
     float ref[kStreamWarps * kMaxCluster], sum[kStreamWarps * kMaxCluster];
     uint32_t key[kStreamWarps * kMaxCluster];
-    int cnt[19];                                    // of the end of the row, which the first block's warps share: see kCntCodes
+    int cnt[32];                                    // of the end of the row, which the first block's warps share
 };
 
 // The row after `rowi` (stride: the rows in work at a time) inside its session's position range, or N.
@@ -747,7 +750,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
         float sum_all = warp_sum((x0 + x1) + (x2 + x3)), lmax;
         if (SHARE) {
             if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
-            if (SELECT && wrow == 0 && lane < 19) sh.cnt[lane] = 0;
+            if (SELECT && wrow == 0) sh.cnt[lane] = 0;
             meet();
             for (int w = 0; w < NW; ++w) kmax = max(kmax, sh.key[w]);
             lmax = val_of_key(kmax);
