@@ -927,3 +927,36 @@ def test_adaptive_quantiser_parity(dev, orc):
     plain = plc.Context(T.to(dev), K, delta, chunk_pos=CP)
     with pytest.raises(plc.PlcError):
         plain.encode(kvd, lgd, st, tokens=tkd)
+
+
+# (rows, V, K, first element of the rows in their buffer): one row over the blocks of a cluster, a few rows a
+# block each, rows of a warp; one group of 8 and less, the last vocabulary whose groups of 8 all have a slot
+# and the next, several batches a slot; heads and tails of every length; K at the ordering's limit
+@pytest.mark.parametrize("N,V,K,off", [(1, 128256, 64, 0), (3, 131071, 128, 5), (40, 33000, 64, 1), (300, 9001, 50, 3),
+                                       (2500, 4099, 33, 7), (9, 16384, 128, 0), (9, 16392, 100, 2), (70, 7, 3, 1),
+                                       (5, 8, 8, 0), (11, 1031, 128, 4), (4800, 257, 16, 0)])
+def test_topk_rows_of_every_layout(dev, orc, N, V, K, off):
+    """Selection exact, sums in binary32: tolerances as in test_topk_softmax_parity.  Rows: ordinary, from nearly
+    uniform to point masses (the K-th logit far below the maximum), ties across the K-th place, ascending."""
+    rng = np.random.default_rng(N + V)
+    lg = (rng.standard_normal((N, V)) * np.exp(rng.uniform(-1.0, 3.0, (N, 1)))).astype(np.float16)
+    lg[0] = -np.abs(lg[0])
+    lg[0, :K // 2 + 1] = np.float16(30.0)                           # half of the selected far above the rest, which are negative
+    if N > 2:
+        lg[1] = np.round(lg[1].astype(np.float32)).astype(np.float16)   # many ties everywhere
+        lg[2] = np.sort(lg[2])
+    tok = rng.integers(0, V, N).astype(np.int32)
+    buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
+    rows = buf[off:off + N * V].view(N, V)
+    rows.copy_(torch.from_numpy(lg))
+    ctx = plc.Context(torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02)
+    out = ctx.topk_softmax(rows, torch.from_numpy(tok).to(dev))
+    assert ctx.sync_status() == plc.OK
+    idx, w, lse, zk, lp = orc.topk_softmax(lg, tok, K)
+    assert np.array_equal(out["idx"].cpu().numpy(), idx)
+    np.testing.assert_allclose(out["w"].cpu().numpy(), w, rtol=2e-5, atol=1e-9)
+    np.testing.assert_allclose(out["lse"].cpu().numpy(), lse, atol=2e-5, rtol=1e-6)
+    np.testing.assert_allclose(out["zk"].cpu().numpy(), zk, rtol=2e-5)
+    np.testing.assert_allclose(out["logp2"].cpu().numpy(), lp, atol=1e-4, rtol=1e-6)
+    only = ctx.topk_softmax(rows, torch.from_numpy(tok).to(dev), want=("lse", "logp2"))
+    np.testing.assert_allclose(only["lse"].cpu().numpy(), lse, atol=2e-5, rtol=1e-6)
