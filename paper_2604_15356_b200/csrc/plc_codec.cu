@@ -20,15 +20,15 @@
 namespace plc {
 namespace {
 
-#ifndef PLC_BLOCKS_PER_SM
-#define PLC_BLOCKS_PER_SM 5
-#endif
-#ifndef PLC_WARPS_PER_BLOCK
-#define PLC_WARPS_PER_BLOCK 8
-#endif
-constexpr int kWarpsPerBlock = PLC_WARPS_PER_BLOCK;
+constexpr int kWarpsPerBlock = 8;
 constexpr int kThreads = kWarpsPerBlock * 32;
-constexpr int kBlocksPerSM = PLC_BLOCKS_PER_SM;
+// Blocks per SM.  The coder alone (symbols or predictions read from memory) wants warps: 5, 48 registers.
+// The gather wants row loads in flight more than warps: 4 blocks at 64 registers hold a stretch of 32
+// rows' loads where 5 held 8 (256 streams x 16384 positions, skewed candidates: 6.18 + 6.46 -> 5.49 +
+// 5.79 ms), and where the rows come from L2 (one queue for the whole GPU) 3 at 80 are better still:
+// fewer tables in flight, more L1 (131072 positions x 32 streams, uniform candidates: decode 7.7 ->
+// 6.8 ms).
+constexpr int kBlocksPerSM = 5, kGatherBlocks = 4, kFarBlocks = 3;
 
 template <int D>
 __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows) {
@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__
 // ZR: the zero-rate rule (Thm. 3) is on; a separate instantiation keeps the plain coder's loop free of it.
 // FLEX: the call exports intermediate values or statistics, or uses a per-position step; the plain
 // instantiation carries none of those branches in its position loop.
-template <int D, int SRC, bool ZR, bool FLEX>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const CodecArgs a) {
+template <int D, int SRC, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
+__global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     constexpr bool FROM_OPEN = SRC == kSrcOpen;
     constexpr bool DENSE = SRC == kSrcDense;
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) encode_kernel(const Co
     }
 }
 
-template <int D, bool DENSE, bool ZR, bool FLEX>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSM) decode_kernel(const CodecArgs a) {
+template <int D, bool DENSE, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
+__global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     __shared__ DecTables tb;
     load_tables(&tb, &a.tables->dec);
@@ -330,7 +330,7 @@ __device__ __forceinline__ void hadamard(float (&v)[Geo<D>::G], int lane) {
 // record is s followed by one ballot word per (register, code bit).  ENC: KV -> records;
 // otherwise records -> KV' = KV^ + eps * H y^.  One warp per (stream, chunk of positions).
 template <int D, bool ENC>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSM) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
+__global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp, B = rq.bits;
@@ -464,14 +464,16 @@ cudaError_t pair_smem_bytes(Kern kern, int Kp, size_t& bytes) {
 
 int codec_grid_warps(int) { return sm_count() * kBlocksPerSM * kWarpsPerBlock; }
 
-static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kBlocksPerSM * kWarpsPerBlock);
+static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kGatherBlocks * kWarpsPerBlock);
 
-#include <cstdlib>
+// A block per chunk (plc_coop.cu) while the chunks would not fill the GPU with a warp each: below that a
+// warp's own chain is what the call waits for; above it the kernels here do more work per instruction
+// (65536 chunks: 12.6 ms a layer group against 11.3).
 static bool use_coop(const CodecArgs& a) {
     const long long items = (long long)(a.mu_dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
-    static const char* e = getenv("PLC_COOP");
-    return items <= (e ? atoll(e) : 5920);
+    return items <= (long long)sm_count() * kWarpsPerBlock * (a.mu_dense ? kBlocksPerSM : kGatherBlocks);
 }
+constexpr int kCoopItems = 4;                    // chunks an SM works on at a time there
 
 // Queue layout of a gather launch.  With one queue for the whole GPU the resident warps span
 // about (resident warps / chunks per table) + 1 consecutive tables; if those tables fit in L2 that
@@ -481,7 +483,7 @@ static bool use_coop(const CodecArgs& a) {
 // so that the warps of an SM gather from one or two tables and shared rows stay in that SM's L1.
 void codec_schedule(const CodecArgs& a0, int n_tables, int* nq, int* g) {
     CodecArgs a = a0;
-    set_queues(a, n_tables);
+    set_queues(a, n_tables, use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock);
     *nq = a.sched_nq; *g = a.sched_g;
 }
 
@@ -513,10 +515,10 @@ cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, c
 
 cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
-    set_queues(a, 2 * a.sh.L * a.sh.H);
+    const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
+    set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
     cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
     if (e != cudaSuccess) return e;
-    if (use_coop(a)) set_queues(a, 2 * a.sh.L * a.sh.H, 4);
     if (use_coop(a)) return launch_coop(a, true, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.dbg.ideal || a.step_exp;
@@ -529,12 +531,17 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
             count_launch();
             return cudaGetLastError();
         }
-        auto kern = zr ? (flex ? encode_kernel<d, kSrcGather, true, true> : encode_kernel<d, kSrcGather, true, false>)
-                       : (flex ? encode_kernel<d, kSrcGather, false, true> : encode_kernel<d, kSrcGather, false, false>);
+        auto pick = [&](auto blocks) {
+            constexpr int B = decltype(blocks)::value;
+            return zr ? (flex ? encode_kernel<d, kSrcGather, true, true, B> : encode_kernel<d, kSrcGather, true, false, B>)
+                      : (flex ? encode_kernel<d, kSrcGather, false, true, B> : encode_kernel<d, kSrcGather, false, false, B>);
+        };
+        const int blocks = a.sched_nq == 1 ? kFarBlocks : kGatherBlocks;
+        auto kern = a.sched_nq == 1 ? pick(std::integral_constant<int, kFarBlocks>{}) : pick(std::integral_constant<int, kGatherBlocks>{});
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * kBlocksPerSM, kThreads, sm, st>>>(a);
+        kern<<<sm_count() * blocks, kThreads, sm, st>>>(a);
         count_launch();
         return cudaGetLastError();
     });
@@ -556,10 +563,10 @@ cudaError_t launch_append_seal(const CodecArgs& a, cudaStream_t st) {
 
 cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
-    set_queues(a, 2 * a.sh.L * a.sh.H);
+    const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
+    set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
     cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
     if (e != cudaSuccess) return e;
-    if (use_coop(a)) set_queues(a, 2 * a.sh.L * a.sh.H, 4);
     if (use_coop(a)) return launch_coop(a, false, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.step_exp;
@@ -572,12 +579,17 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
             count_launch();
             return cudaGetLastError();
         }
-        auto kern = zr ? (flex ? decode_kernel<d, false, true, true> : decode_kernel<d, false, true, false>)
-                       : (flex ? decode_kernel<d, false, false, true> : decode_kernel<d, false, false, false>);
+        auto pick = [&](auto blocks) {
+            constexpr int B = decltype(blocks)::value;
+            return zr ? (flex ? decode_kernel<d, false, true, true, B> : decode_kernel<d, false, true, false, B>)
+                      : (flex ? decode_kernel<d, false, false, true, B> : decode_kernel<d, false, false, false, B>);
+        };
+        const int blocks = a.sched_nq == 1 ? kFarBlocks : kGatherBlocks;
+        auto kern = a.sched_nq == 1 ? pick(std::integral_constant<int, kFarBlocks>{}) : pick(std::integral_constant<int, kGatherBlocks>{});
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * kBlocksPerSM, kThreads, sm, st>>>(a);
+        kern<<<sm_count() * blocks, kThreads, sm, st>>>(a);
         count_launch();
         return cudaGetLastError();
     });
@@ -593,7 +605,7 @@ cudaError_t launch_rotq(const CodecArgs& a0, const RotqArgs& r, bool encode, cud
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * kBlocksPerSM, kThreads, sm, st>>>(a, r);
+        kern<<<sm_count() * kGatherBlocks, kThreads, sm, st>>>(a, r);
         count_launch();
         return cudaGetLastError();
     });

@@ -13,14 +13,13 @@
 // The decoder's words come through a ring in shared memory filled by asynchronous copies, so no
 // refill waits for global memory.
 #include <algorithm>
-#include <cstdlib>
 
 #include "plc_codec.cuh"
 
 namespace plc {
 namespace {
 
-constexpr int kCoopMaxWarps = 16;
+constexpr int kCoopWarps = 8;
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
 // Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; about four such are held.
 __host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 8192 : 4096; }
@@ -123,7 +122,7 @@ struct CoopItem {
 };
 struct CoopShared {
     CoopItem item;
-    SlotMeta meta[2][kCoopMaxWarps];
+    SlotMeta meta[2][kCoopWarps];
     uint8_t* dst;                        // encoding: where the finished chunk's words go (null: nowhere)
     int wp;
 };
@@ -370,7 +369,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
 
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
 template <int D, bool DENSE, bool ENC>
-__global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
+__global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel(const CodecArgs a) {
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
     __shared__ CoopShared sh;
@@ -431,9 +430,9 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         auto kern = dense ? (encode ? coop_kernel<d, true, true> : coop_kernel<d, true, false>)
                           : (encode ? coop_kernel<d, false, true> : coop_kernel<d, false, false>);
         const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
-        int warps = items <= 2ll * sm_count() ? kCoopMaxWarps : kCoopMaxWarps / 2;
-        { static const char* e = getenv(dense ? "PLC_NWD" : "PLC_NW"); if (e) warps = atoi(e); }
-        if (coop_smem(warps, a.sh.Kp, d, dense, encode) > 96 * 1024) warps = kCoopMaxWarps / 2;
+        // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
+        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).
+        const int warps = kCoopWarps;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
