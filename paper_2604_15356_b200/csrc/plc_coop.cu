@@ -6,10 +6,10 @@
 // load, the coder), about 1.8 us a position however little work there is.  Only the coder is serial
 // in a chunk, and of the coder only the state and the word cursor; the rest is independent from
 // position to position.  Here warp 0 of a block carries the chunk's state and the other warps do
-// everything else, one position each at a time, handed over in slots of shared memory (two a warp, an
-// mbarrier each way): encoding, they predict, quantise, look the table entries up and transpose the bit planes, so
+// everything else, one position each and batch, two batches deep in shared memory with one barrier a
+// batch: encoding, they predict, quantise, look the table entries up and transpose the bit planes, so
 // that the coder's chain per step is one state update; decoding, they predict (the coder needs the
-// class) and, a turn later, fetch the planes whose places the coder has found and write the vectors.
+// class) and, a batch later, fetch the planes whose places the coder has found and write the vectors.
 // The decoder's words come through a ring in shared memory filled by asynchronous copies, so no
 // refill waits for global memory.
 #include <algorithm>
@@ -109,8 +109,8 @@ size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
     return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G));
 }
 
-constexpr int kCoopSlots = 2 * (kCoopWarps - 1);         // two positions a predicting warp
-constexpr uint32_t kCoopSpin = 1u << 22;
+// All warps of the block meet here; the two roles reach it from different places in the code.
+__device__ __forceinline__ void block_barrier() { asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)blockDim.x) : "memory"); }
 
 // The block's current chunk.
 struct CoopItem {
@@ -121,57 +121,20 @@ struct CoopItem {
     int go;                              // 0: nothing to do for this chunk, -1: no chunks left
 };
 struct CoopShared {
-    unsigned long long full[kCoopSlots], done[kCoopSlots];   // mbarriers: a slot is filled, the coder is done with it
     CoopItem item;
-    SlotMeta meta[kCoopSlots];
+    SlotMeta meta[2][kCoopWarps];
     uint8_t* dst;                        // encoding: where the finished chunk's words go (null: nowhere)
     int wp;
-    unsigned failed;                     // a wait ran out: no further waits, nothing is committed
 };
 
-// Slots are used in turns: in turn T (counted over all chunks of the block, the same in all warps) warp w
-// fills slot (T & 1) NP + w for the T/2-th time.  A predicting warp runs up to two positions ahead of the
-// coder and the coder takes slots as they fill, so neither waits for the slowest of a batch.  Every wait
-// is bounded.
-__device__ __forceinline__ uint32_t bar_addr(const unsigned long long* b) { return (uint32_t)__cvta_generic_to_shared(b); }
-__device__ __forceinline__ void bar_arrive(unsigned long long* b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_addr(b)) : "memory");
-}
-__device__ __forceinline__ bool bar_try(const unsigned long long* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar_addr(b)), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool bar_test(const unsigned long long* b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar_addr(b)), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void bar_wait(CoopShared& sh, const unsigned long long* b, uint32_t parity, unsigned int* status) {
-    for (uint32_t i = 0; i < kCoopSpin; ++i) {
-        if (__all_sync(kFull, bar_try(b, parity))) return;
-        if (__any_sync(kFull, *(volatile unsigned*)&sh.failed != 0)) return;
-    }
-    sh.failed = 1u;
-    atomicOr(status, kStTimeout);
-}
-
-// Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a turn; the inputs
-// of the next are fetched while it works on one.  turn0: turns of the block so far.
+// Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a batch; the inputs
+// of the next are fetched while it works on one.
 template <int D, bool DENSE, bool ENC, class Tab>
 __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
-                                             unsigned turn0, const LaneCode& lc) {
+                                             const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
-    const int P = sh.item.it.P, Kp = DENSE ? 0 : a.sh.Kp, n_turns = (P + NP - 1) / NP, c0 = first_comp<D>(lane);
+    const int P = sh.item.it.P, Kp = DENSE ? 0 : a.sh.Kp, n_batches = (P + NP - 1) / NP, c0 = first_comp<D>(lane);
     const int t = (int)from_lane0((unsigned)sh.item.it.t, lane), t0 = DENSE ? a.dense_t0 : 0;
     const int first = ENC ? P - 1 : 0, dir = ENC ? -1 : 1;
     const long long row0 = sh.item.row0;
@@ -190,22 +153,19 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
         else prefetch_pairs(sp0 + into * Kp, a.pairs + (row0 + p) * Kp, Kp, lane);
         if (ENC) load_half_raw<G>(reinterpret_cast<const __half*>(a.kv.base) + sh.item.kv0 + c0 + p * a.kv.sp, kv_next);
     };
-    auto slot_at = [&](int b) { return (int)((turn0 + b) & 1u) * NP + w; };
-    auto use_at = [&](int b) { return (turn0 + b) >> 1; };
-    auto finish = [&](int b) {                                                 // decoding: position of turn b
+    auto finish = [&](int b) {                                                 // decoding: position of batch b
         const int p = b * NP + w;
         if (b < 0 || p >= P) return;
-        bar_wait(sh, &sh.done[slot_at(b)], use_at(b) & 1u, a.status);
         int sym[G];
         float out[G];
         if (old.q == kSkipped) {                                               // zero-rate position: KV' = KV^
 #pragma unroll
             for (int g = 0; g < G; ++g) { sym[g] = 0; out[g] = mu_old[g]; }
         } else {
-            const int* slot = slots + slot_at(b) * SW;
+            const int* slot = slots + ((b & 1) * NP + w) * SW;
             int hi[G];
             slot_get_ints<G>(slot, lane, hi);
-            if (sh.meta[slot_at(b)].escaped) {
+            if (sh.meta[b & 1][w].escaped) {
 #pragma unroll
                 for (int g = 0; g < G; ++g) sym[g] = hi[g];
             } else {
@@ -229,7 +189,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
         }
     };
     if (w < P) fetch(w, 0);
-    for (int b = 0; b < n_turns; ++b) {
+    for (int b = 0; b < n_batches; ++b) {
         const int k = b * NP + w, p = first + dir * k;
         float mu[G] = {};
         SlotMeta sm{kSkipped, 0, 0, 0};
@@ -271,8 +231,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
 #pragma unroll
                 for (int g = 0; g < G; ++g) sym[g] = quantise(kvv[g], mu[g], inv_delta);
                 class_params(q, s, qp);
-                int* slot = slots + slot_at(b) * SW;
-                bar_wait(sh, &sh.done[slot_at(b)], (use_at(b) & 1u) ^ 1u, a.status);   // its last position has been coded
+                int* slot = slots + ((b & 1) * NP + w) * SW;
                 if (split_symbols<G>(sym, s, u, at)) {
                     Prepared<G> pr;
                     prepare_position<G>(u, at, s, tb.enc[qp - kQMin], lc, pr);
@@ -301,13 +260,10 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                 for (int g = 0; g < G; ++g)
                     if (a.dbg.mu) a.dbg.mu[o * D + c0 + g] = mu[g];
             }
-            if (!ENC) bar_wait(sh, &sh.done[slot_at(b)], (use_at(b) & 1u) ^ 1u, a.status);
-            if (lane == 0) sh.meta[slot_at(b)] = sm;
-        } else {
-            bar_wait(sh, &sh.done[slot_at(b)], (use_at(b) & 1u) ^ 1u, a.status);
+            if (lane == 0) sh.meta[b & 1][w] = sm;
+            __syncwarp();                                                      // readers of the pair slot are done
         }
-        __syncwarp();                                                          // the slot is written; readers of the pair slot are done
-        if (lane == 0) bar_arrive(&sh.full[slot_at(b)]);
+        block_barrier();
         if constexpr (!ENC) {
             finish(b - 1);
 #pragma unroll
@@ -315,72 +271,51 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
             old = sm;
         }
     }
-    if constexpr (!ENC) finish(n_turns - 1);
+    block_barrier();
+    if constexpr (!ENC) finish(n_batches - 1);
     if (ENC && a.dbg.ideal) {
         ideal = warp_sum(ideal);
         if (lane == 0) atomicAdd(&a.counters->ideal_bits, (double)ideal);
     }
 }
 
-// Coder of the block's chunk.
+// Coder of the block's chunk, one batch behind the predictions.
 template <int D, bool ENC, class Tab>
-__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, unsigned turn0,
-                                          const LaneCode& lc) {
+__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
-    const int P = sh.item.it.P, n_turns = (P + NP - 1) / NP;
+    const int P = sh.item.it.P, n_batches = (P + NP - 1) / NP;
     uint32_t x = kRansL;
-    // slot of the k-th position (turn k / NP, warp k mod NP), walked without divisions
-    struct Walk { int j; uint32_t turn; };
-    auto step_to_next = [&](Walk& k) { if (++k.j == NP) { k.j = 0; ++k.turn; } };
-    auto slot_of = [&](const Walk& k) { return (int)(k.turn & 1u) * NP + k.j; };
-    auto parity_of = [&](const Walk& k) { return (k.turn >> 1) & 1u; };
-    Walk at{0, turn0};
-    auto wait_full = [&](const Walk& k) { bar_wait(sh, &sh.full[slot_of(k)], parity_of(k), a.status); };
-    auto release = [&](const Walk& k) {
-        __syncwarp();
-        if (lane == 0) bar_arrive(&sh.done[slot_of(k)]);
-    };
     if constexpr (ENC) {
         uint16_t* stage = a.staging + (long long)blockIdx.x * a.staging_words_per_warp;
         const int cap_words = (int)a.staging_words_per_warp;
         int wp = cap_words, n_skipped = 0;
         unsigned n_escapes = 0;
-        Prepared<G> next;
-        SlotMeta next_meta;
-        auto fetch = [&](const Walk& k) {
-            slot_get<G>(slots + slot_of(k) * SW, lane, next);
-            next_meta = sh.meta[slot_of(k)];
-        };
-        wait_full(at);
-        fetch(at);
-        for (int k = 0; k < P; ++k) {
-            const Prepared<G> pr = next;
-            const SlotMeta m = next_meta;
-            const Walk here = at;
-            step_to_next(at);
-            // the next position is fetched beside this one's chain if it is there already
-            const bool ready = k + 1 < P && __all_sync(kFull, bar_test(&sh.full[slot_of(at)], parity_of(at)));
-            if (ready) fetch(at);
-            if (m.q == kSkipped) {
-                ++n_skipped;
-            } else {
+        for (int b = 0; b < n_batches; ++b) {
+            block_barrier();                                                   // batch b is there
+            const int cnt = min(NP, P - b * NP);
+            const int* slot = slots + (b & 1) * NP * SW;
+            Prepared<G> next;
+            slot_get<G>(slot, lane, next);
+            SlotMeta sm = sh.meta[b & 1][0];
+            for (int j = 0; j < cnt; ++j, slot += SW) {
+                const Prepared<G> pr = next;
+                const SlotMeta m = sm;
+                if (j + 1 < cnt) { slot_get<G>(slot + SW, lane, next); sm = sh.meta[b & 1][j + 1]; }
+                if (m.q == kSkipped) { ++n_skipped; continue; }
                 int s, qp;
                 class_params(m.q, s, qp);
                 if (!m.escaped) {
                     wp = push_position<G>(pr, s, x, stage, wp, lc);
                 } else {
                     int u[G];
-                    slot_get_ints<G>(slots + slot_of(here) * SW, lane, u);
+                    slot_get_ints<G>(slot, lane, u);
                     wp = encode_position_escapes<G>(u, s, tb.enc[qp - kQMin], x, stage, wp, lane, n_escapes);
                 }
             }
-            release(here);
-            if (!ready && k + 1 < P) { wait_full(at); fetch(at); }
         }
-        uint8_t* dst = nullptr;
-        if (!__any_sync(kFull, *(volatile unsigned*)&sh.failed != 0))
-            dst = reserve_chunk(a, sh.item.it.slot, x, cap_words - wp, lane, P, n_escapes, n_skipped);
+        block_barrier();
+        uint8_t* dst = reserve_chunk(a, sh.item.it.slot, x, cap_words - wp, lane, P, n_escapes, n_skipped);
         if (lane == 0) { sh.dst = dst; sh.wp = wp; }
     } else {
         const uint8_t* src = a.st.payload + sh.item.off;
@@ -391,11 +326,15 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         int rp = 0, fetched = 0, ready = 0;
         ring_fetch<G>(ring, src, 2 * nwords, 0, fetched, lane);
         const RingWords<G> words{ring};
-        for (int k = 0; k < P; ++k, step_to_next(at)) {
-            wait_full(at);
-            const int q = sh.meta[slot_of(at)].q;
-            int* slot = slots + slot_of(at) * SW;
-            if (q != kSkipped) {
+        for (int b = 0; b < n_batches; ++b) {
+            block_barrier();                                                   // the classes of batch b are there
+            const int cnt = min(NP, P - b * NP);
+            int* slot = slots + (b & 1) * NP * SW;
+            int q = sh.meta[b & 1][0].q;
+            for (int j = 0; j < cnt; ++j, slot += SW) {
+                const int qj = q;
+                if (j + 1 < cnt) q = sh.meta[b & 1][j + 1].q;
+                if (qj == kSkipped) continue;
                 // a position's words, and the last refill window
                 if (min(2 * rp + 252 * G + 64, 2 * nwords) > ready) {
                     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -403,7 +342,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                     ready = fetched;
                 }
                 int s, qp, base[G], hi[G];
-                class_params(q, s, qp);
+                class_params(qj, s, qp);
                 auto step = [&](const auto& find) {
                     if (pull_position<G>(s, find, x, words, rp, lc, base, hi)) {
 #pragma unroll
@@ -411,23 +350,20 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                             if (lane == g) slot[32 * G + g] = base[g];
                     } else {
                         decode_position_escapes<G>(hi, s, find, x, words, rp, lane);
-                        if (lane == 0) sh.meta[slot_of(at)].escaped = 1;
+                        if (lane == 0) sh.meta[b & 1][j].escaped = 1;
                     }
                 };
                 if (qp - kQMin >= kWideFrom) step(WideLookup{tb.wide[qp - kQMin - kWideFrom]});
                 else step(Lookup{tb.first[qp - kQMin], tb.fc[qp - kQMin]});
                 slot_put_ints<G>(slot, lane, hi);
+                __syncwarp();                                                  // readers of the ring are done
+                ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
             }
-            release(at);                                                       // also: readers of the ring are done
-            ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
         }
+        block_barrier();
         bad = bad || x != kRansL || rp != nwords;
         if (__any_sync(kFull, bad) && lane == 0) atomicOr(a.status, kStCorrupt);
         asm volatile("cp.async.wait_all;" ::: "memory");                       // of a damaged chunk: nothing may land later
-    }
-    for (; at.turn != turn0 + (unsigned)n_turns; step_to_next(at)) {           // places without a position in the last turn
-        wait_full(at);
-        release(at);
     }
 }
 
@@ -442,12 +378,6 @@ __global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel
     int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
     const LaneCode lc = lane_code(lane);
-    if (threadIdx.x < kCoopSlots) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_addr(&sh.full[threadIdx.x])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_addr(&sh.done[threadIdx.x])) : "memory");
-        if (threadIdx.x == 0) sh.failed = 0u;
-    }
-    unsigned turn0 = 0;                                                                      // turns of the block so far
     load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->wide));
     const int Wl = DENSE ? a.dense_nt : 2 * a.sh.L * a.sh.H;
     const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks, total = (unsigned)Wl * per_table;
@@ -481,9 +411,8 @@ __global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel
         const int go = sh.item.go;
         if (go < 0) break;
         if (go > 0) {
-            if (warp == 0) coop_code<D, ENC>(a, sh, tb, slots, ring, NP, turn0, lc);
-            else coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, turn0, lc);
-            turn0 += (unsigned)((sh.item.it.P + NP - 1) / NP);
+            if (warp == 0) coop_code<D, ENC>(a, sh, tb, slots, ring, NP, lc);
+            else coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
         }
         __syncthreads();                                                       // the chunk is coded; its item has been read
         if (ENC && go > 0 && sh.dst)
