@@ -179,7 +179,6 @@ struct CodecArgs {
     StreamsDev st; DebugDev dbg;
     uint16_t* staging; unsigned long long staging_words_per_warp;   // encoder scratch
     unsigned int* ticket;                          // kTicketWords work counters (zeroed by the launcher)
-    int sms;                                       // SMs of the device (plc_coop.cu)
     int sched_nq, sched_g;                         // gather kernels: work queues, SMs that share one (set by the launcher)
     unsigned int* status; Counters* counters;
     // dense variant: prediction read from buffers; one launch covers tables [dense_t0, dense_t0 + dense_nt)

@@ -373,10 +373,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
     __shared__ CoopShared sh;
-    // Role 0 is the coder.  Warps go to an SM's four schedulers in turn, so the coders of the blocks that
-    // share an SM (blocks one grid row of SMs apart) are put on different ones.
-    const int lane = threadIdx.x & 31, NP = (blockDim.x >> 5) - 1;                           // NP predicting warps
-    const int warp = ((threadIdx.x >> 5) + (blockIdx.x / a.sms)) & NP;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NP = (blockDim.x >> 5) - 1;   // NP predicting warps
     const int Kp = DENSE ? 0 : a.sh.Kp;
     int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
@@ -442,9 +439,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         int occ = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem) != cudaSuccess || occ < 1) occ = 1;
         const long long blocks = std::min<long long>(items, (long long)sm_count() * occ);
-        CodecArgs b = a;
-        b.sms = sm_count();
-        kern<<<(unsigned)blocks, warps * 32, smem, st>>>(b);
+        kern<<<(unsigned)blocks, warps * 32, smem, st>>>(a);
         count_launch();
         return cudaGetLastError();
     });
