@@ -19,7 +19,9 @@
 namespace plc {
 namespace {
 
-constexpr int kCoopWarps = 8;
+constexpr int kCoopMaxWarps = 16;
+// Predicting warps of a block.
+__host__ __device__ constexpr int coop_predictors(int warps) { return warps == kCoopMaxWarps ? 3 * warps / 4 : warps - 1; }
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
 // Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; about four such are held.
 __host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 8192 : 4096; }
@@ -104,13 +106,13 @@ __device__ __forceinline__ void slot_get(const int* slot, int lane, Prepared<G>&
 }
 
 size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
-    const int NP = warps - 1, G = d / 32, planes = G <= 2 ? 1 : G / 2;
+    const int NP = coop_predictors(warps), G = d / 32, planes = G <= 2 ? 1 : G / 2;
     const int slot = enc ? 32 * (2 * G + planes) : 32 * G + 8;
     return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G));
 }
 
 // All warps of the block meet here; the two roles reach it from different places in the code.
-__device__ __forceinline__ void block_barrier() { asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)blockDim.x) : "memory"); }
+__device__ __forceinline__ void block_barrier() { asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)(32 + 32 * coop_predictors(blockDim.x >> 5))) : "memory"); }
 
 // The block's current chunk.
 struct CoopItem {
@@ -122,7 +124,7 @@ struct CoopItem {
 };
 struct CoopShared {
     CoopItem item;
-    SlotMeta meta[2][kCoopWarps];
+    SlotMeta meta[2][kCoopMaxWarps];
     uint8_t* dst;                        // encoding: where the finished chunk's words go (null: nowhere)
     int wp;
 };
@@ -369,11 +371,14 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
 
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
 template <int D, bool DENSE, bool ENC>
-__global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel(const CodecArgs a) {
+__global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
     __shared__ CoopShared sh;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NP = (blockDim.x >> 5) - 1;   // NP predicting warps
+    // Warps go to an SM's four schedulers in turn.  A block that has its SM to itself (16 warps) leaves the
+    // coder's scheduler to the coder: the warps that would share it stay idle.
+    const int lane = threadIdx.x & 31, hw = threadIdx.x >> 5, NP = coop_predictors(blockDim.x >> 5);   // NP predicting warps
+    const int warp = NP < (int)(blockDim.x >> 5) - 1 ? ((hw & 3) == 0 ? (hw == 0 ? 0 : -1) : hw - (hw >> 2)) : hw;
     const int Kp = DENSE ? 0 : a.sh.Kp;
     int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
@@ -412,7 +417,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32, D == 256 ? 2 : 4) coop_kernel
         if (go < 0) break;
         if (go > 0) {
             if (warp == 0) coop_code<D, ENC>(a, sh, tb, slots, ring, NP, lc);
-            else coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
+            else if (warp > 0) coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
         }
         __syncthreads();                                                       // the chunk is coded; its item has been read
         if (ENC && go > 0 && sh.dst)
@@ -431,8 +436,9 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
                           : (encode ? coop_kernel<d, false, true> : coop_kernel<d, false, false>);
         const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
         // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
-        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).
-        const int warps = kCoopWarps;
+        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  Fifteen where there is
+        // a chunk an SM at most: then a prediction's latency is what the coder waits for.
+        const int warps = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode) <= 160 * 1024 ? kCoopMaxWarps : kCoopMaxWarps / 2;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
