@@ -156,29 +156,39 @@ __device__ __forceinline__ bool split_symbols(const int (&sym)[G], int S, int (&
     return !__any_sync(kFull, worst > 2u * kHiMax);
 }
 
-// Words of the stream are written back to front: stage[wp - 1], stage[wp - 2], ...  In decoder order a
-// step is: 2S plane words, the refill words of the lanes that renormalise (lanes ascending), the raw
-// high parts of escaped lanes (lanes ascending, low half first).  Last component first; returns the
-// new wp.
+// The serial part of coding a position: the state through its steps, last component first.  low[g], emask[g]:
+// the state before step g and the lanes whose low half goes into the stream there.
 template <int G>
-__device__ __forceinline__ int push_position(const Prepared<G>& pr, int S, uint32_t& x, uint16_t* __restrict__ stage, int wp, const LaneCode& lc) {
-    // the state's chain first, the words' places (votes and counts) after it, so that no step waits for them
-    uint32_t low[G], emask[G];
-    bool emit[G];
+__device__ __forceinline__ void chain_position(const EncEntry (&e)[G], uint32_t& x, uint32_t (&low)[G], uint32_t (&emask)[G], bool (&emit)[G]) {
 #pragma unroll
     for (int g = G - 1; g >= 0; --g) {
-        emit[g] = x >= (pr.e[g].fc << 17);                 // f << 17: the count above f is shifted out
+        emit[g] = x >= (e[g].fc << 17);                    // f << 17: the count above f is shifted out
         emask[g] = __ballot_sync(kFull, emit[g]);
         low[g] = x;
-        x = push_state(x, emit[g], pr.e[g]);
+        x = push_state(x, emit[g], e[g]);
     }
-    int base[G];
+}
+// Words a position takes.
+template <int G>
+__device__ __forceinline__ int words_of(const uint32_t (&emask)[G], int S) {
+    int n = 2 * S * G;
 #pragma unroll
-    for (int g = G - 1; g >= 0; --g) {
-        wp -= __popc(emask[g]);
-        if (emit[g]) stage[wp + __popc(emask[g] & lc.lt)] = (uint16_t)low[g];
-        wp -= 2 * S;
-        base[g] = wp - 2 * S * g;                          // lane j = g S + b of a group: halfword base + 2 j
+    for (int g = 0; g < G; ++g) n += __popc(emask[g]);
+    return n;
+}
+// The rest: its words to stage[base ...].  In decoder order a step is: 2S plane words, the refill words of the
+// lanes that renormalise (lanes ascending), the raw high parts of escaped lanes (lanes ascending, low
+// half first).
+template <int G>
+__device__ __forceinline__ void place_position(const uint32_t (&plane)[kPlaneWords<G>], const uint32_t (&low)[G], const uint32_t (&emask)[G],
+                                               const bool (&emit)[G], int S, uint16_t* __restrict__ stage, int base, const LaneCode& lc) {
+    int first[G];                                          // lane j = g S + b of a group: halfword first + 2 j
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        first[g] = base - 2 * S * g;
+        base += 2 * S;
+        if (emit[g]) stage[base + __popc(emask[g] & lc.lt)] = (uint16_t)low[g];
+        base += __popc(emask[g]);
     }
     if (S > 0)
         by_plane_group<G>(S, [&](auto gp) {
@@ -186,13 +196,12 @@ __device__ __forceinline__ int push_position(const Prepared<G>& pr, int S, uint3
 #pragma unroll
             for (int i = 0; i < G / GP; ++i) {
                 if (lc.lane < GP * S) {
-                    uint16_t* p = stage + (of_my_step<GP>(base + i * GP, lc.lane, S) + 2 * (i * GP * S + lc.lane));
-                    p[0] = (uint16_t)pr.plane[i];
-                    p[1] = (uint16_t)(pr.plane[i] >> 16);
+                    uint16_t* p = stage + (of_my_step<GP>(first + i * GP, lc.lane, S) + 2 * (i * GP * S + lc.lane));
+                    p[0] = (uint16_t)plane[i];
+                    p[1] = (uint16_t)(plane[i] >> 16);
                 }
             }
         });
-    return wp;
 }
 
 // Positions with an escaped component, one step at a time.
@@ -238,7 +247,12 @@ __device__ __forceinline__ int encode_position(const int (&sym)[G], int S, const
     if (!split_symbols<G>(sym, S, u, at)) return encode_position_escapes<G>(u, S, tbl, x, stage, wp, lc.lane, n_escapes);
     Prepared<G> pr;
     prepare_position<G>(u, at, S, tbl, lc, pr);
-    return push_position<G>(pr, S, x, stage, wp, lc);
+    uint32_t low[G], emask[G];
+    bool emit[G];
+    chain_position<G>(pr.e, x, low, emask, emit);
+    wp -= words_of<G>(emask, S);
+    place_position<G>(pr.plane, low, emask, emit, S, stage, wp, lc);
+    return wp;
 }
 
 // One decoder step before its refill: the symbol (place in the alphabet) of state x and the next state.
@@ -311,41 +325,39 @@ __device__ __forceinline__ void decode_position_escapes(int (&sym)[G], int S, co
 }
 
 // The serial part of decoding a position: advances x and rp, gives every step's place in the word
-// stream and high part; false if a component escaped (x and rp are then as before the call).
+// stream and symbol (place in the alphabet); false if a component escaped (x and rp are then as before the call).
 // words(i) reads 16-bit word i of the chunk (any i: the reader keeps the access in bounds; rp advances
 // regardless, so the caller's final check of rp reports a short chunk).
 template <int G, class Find, class Words>
 __device__ __forceinline__ bool pull_position(int S, const Find& find, uint32_t& x, const Words& words, int& rp, const LaneCode& lc,
-                                              int (&base)[G], int (&hi)[G]) {
+                                              int (&base)[G], int (&zz)[G]) {
     const uint32_t x0 = x;
     const int rp0 = rp;
-    bool esc = false;
+    int top = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         base[g] = rp;
         rp += 2 * S;
         const uint32_t window = words(rp + lc.lane);       // the step's refill words, fetched beside the look-up
-        int zz;
-        x = find(x, zz);
+        x = find(x, zz[g]);
         const bool need = x < kRansL;
         const uint32_t nmask = __ballot_sync(kFull, need);
         const uint32_t word = __shfl_sync(kFull, window, __popc(nmask & lc.lt));
         x = need ? (x << 16) | word : x;
         rp += __popc(nmask);
-        esc = esc || zz == kEsc;
-        hi[g] = hi_of(zz);
+        top = max(top, zz[g]);
     }
-    if (!__any_sync(kFull, esc)) return true;
+    if (!__any_sync(kFull, top == kEsc)) return true;
     x = x0; rp = rp0;                                      // the words after the first escape were read wrongly
     return false;
 }
 
 // The rest: a position's planes from the word stream, and its symbols.
 template <int G, class Words>
-__device__ __forceinline__ void join_position(const int (&base)[G], const int (&hi)[G], int S, const Words& words, const LaneCode& lc, int (&sym)[G]) {
+__device__ __forceinline__ void join_position(const int (&base)[G], const int (&zz)[G], int S, const Words& words, const LaneCode& lc, int (&sym)[G]) {
     if (S == 0) {
 #pragma unroll
-        for (int g = 0; g < G; ++g) sym[g] = hi[g];
+        for (int g = 0; g < G; ++g) sym[g] = hi_of(zz[g]);
         return;
     }
     const uint32_t mask = (1u << S) - 1u, half = (1u << S) >> 1;
@@ -363,7 +375,7 @@ __device__ __forceinline__ void join_position(const int (&base)[G], const int (&
             }
             const uint32_t v = transpose32(plane, lc);
 #pragma unroll
-            for (int k = 0; k < GP; ++k) sym[i * GP + k] = (int)(((uint32_t)hi[i * GP + k] << S) + ((v >> (k * S)) & mask) - half);
+            for (int k = 0; k < GP; ++k) sym[i * GP + k] = (int)(((uint32_t)hi_of(zz[i * GP + k]) << S) + ((v >> (k * S)) & mask) - half);
         }
     });
 }
@@ -372,8 +384,8 @@ __device__ __forceinline__ void join_position(const int (&base)[G], const int (&
 template <int G, class Find, class Words>
 __device__ __forceinline__ void decode_position(int (&sym)[G], int S, const Find& find, uint32_t& x, const Words& words, int& rp,
                                                 const LaneCode& lc) {
-    int base[G], hi[G];
-    if (pull_position<G>(S, find, x, words, rp, lc, base, hi)) join_position<G>(base, hi, S, words, lc, sym);
+    int base[G], zz[G];
+    if (pull_position<G>(S, find, x, words, rp, lc, base, zz)) join_position<G>(base, zz, S, words, lc, sym);
     else decode_position_escapes<G>(sym, S, find, x, words, rp, lc.lane);
 }
 

@@ -7,9 +7,11 @@
 // in a chunk, and of the coder only the state and the word cursor; the rest is independent from
 // position to position.  Here warp 0 of a block carries the chunk's state and the other warps do
 // everything else, one position each and batch, two batches deep in shared memory with one barrier a
-// batch: encoding, they predict, quantise, look the table entries up and transpose the bit planes, so
-// that the coder's chain per step is one state update; decoding, they predict (the coder needs the
-// class) and, a batch later, fetch the planes whose places the coder has found and write the vectors.
+// batch: encoding, they predict, quantise, look the table entries up and transpose the bit planes, and a
+// batch later put the words where the coder has found their places; decoding, they predict (the coder
+// needs the class) and, a batch later, fetch the planes whose places the coder has found and write the
+// vectors.  The coder itself is the bottleneck of a block (it never waits at the barrier), and every
+// instruction of it counts: 940 cycles a position of 128 components when it also placed the words.
 // The decoder's words come through a ring in shared memory filled by asynchronous copies, so no
 // refill waits for global memory.
 #include <algorithm>
@@ -25,9 +27,10 @@ __host__ __device__ constexpr int coop_predictors(int warps) { return warps == k
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
 // Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; about four such are held.
 __host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 8192 : 4096; }
-constexpr int kSkipped = -1000000;                       // class mark of a zero-rate position
 
-struct SlotMeta { int q, e, escaped, pad; };             // class (or kSkipped), step exponent, whether a component escapes
+// What a predicting warp tells the coder about a position (one 16-byte word): bit planes (-1: nothing is
+// coded), table id - kQMin, whether a component escapes (encoding; decoding: the coder's answer).
+struct __align__(16) SlotMeta { int planes, table, escaped, pad; };
 
 // The words of a chunk, read through the ring.  `ready` bytes have landed, `fetched` are on their way.
 template <int G>
@@ -47,13 +50,31 @@ __device__ __forceinline__ void ring_fetch(uint16_t* ring, const uint8_t* src, i
     }
 }
 
-// A position's slot, 16 (or 8) bytes a lane at a time.  Encoding: the table entries and planes of a
-// Prepared position (u itself where a component escapes); decoding: the steps' high parts (the symbols
-// themselves where one escapes) and, behind them, the steps' places in the word stream.
+// A position's slot.  Encoding: in, the table entries of its steps (u itself where a component escapes);
+// out, over them, the state before each step, and behind them the lanes that emit at each step and the
+// place of the position's words.  Decoding, out: the steps' symbols (the position's symbols themselves
+// where one escapes) and behind them the steps' places in the word stream.
+constexpr int kTailWords = 12;                           // 8 words, one a step, and the place; padded to 16 bytes
 template <int G>
-constexpr int kEncSlotWords = 32 * (2 * G + kPlaneWords<G>);
+constexpr int kEncSlotWords = 64 * G + kTailWords;
 template <int G>
-constexpr int kDecSlotWords = 32 * G + 8;
+constexpr int kDecSlotWords = 32 * G + kTailWords;
+// v[0 .. G) for all lanes, the same value in every lane.
+template <int G, class V>
+__device__ __forceinline__ void tail_put(int* tail, const V (&v)[G]) {
+    if constexpr (G >= 4) {
+#pragma unroll
+        for (int i = 0; i < G / 4; ++i) reinterpret_cast<int4*>(tail)[i] = make_int4((int)v[4 * i], (int)v[4 * i + 1], (int)v[4 * i + 2], (int)v[4 * i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < G; ++i) tail[i] = (int)v[i];
+    }
+}
+template <int G, class V>
+__device__ __forceinline__ void tail_get(const int* tail, V (&v)[G]) {
+#pragma unroll
+    for (int i = 0; i < G; ++i) v[i] = (V)tail[i];
+}
 template <int G>
 __device__ __forceinline__ void slot_put_ints(int* slot, int lane, const int (&v)[G]) {
     if constexpr (G >= 4) {
@@ -78,36 +99,31 @@ __device__ __forceinline__ void slot_get_ints(const int* slot, int lane, int (&v
     }
 }
 template <int G>
-__device__ __forceinline__ void slot_put(int* slot, int lane, const Prepared<G>& pr) {
+__device__ __forceinline__ void slot_put_entries(int* slot, int lane, const EncEntry (&e)[G]) {
     if constexpr (G >= 2) {
 #pragma unroll
         for (int i = 0; i < G / 2; ++i)
-            reinterpret_cast<uint4*>(slot)[i * 32 + lane] = make_uint4(pr.e[2 * i].rcp, pr.e[2 * i].fc, pr.e[2 * i + 1].rcp, pr.e[2 * i + 1].fc);
+            reinterpret_cast<uint4*>(slot)[i * 32 + lane] = make_uint4(e[2 * i].rcp, e[2 * i].fc, e[2 * i + 1].rcp, e[2 * i + 1].fc);
     } else {
-        reinterpret_cast<uint2*>(slot)[lane] = make_uint2(pr.e[0].rcp, pr.e[0].fc);
+        reinterpret_cast<uint2*>(slot)[lane] = make_uint2(e[0].rcp, e[0].fc);
     }
-#pragma unroll
-    for (int i = 0; i < kPlaneWords<G>; ++i) slot[64 * G + i * 32 + lane] = (int)pr.plane[i];
 }
 template <int G>
-__device__ __forceinline__ void slot_get(const int* slot, int lane, Prepared<G>& pr) {
+__device__ __forceinline__ void slot_get_entries(const int* slot, int lane, EncEntry (&e)[G]) {
     if constexpr (G >= 2) {
 #pragma unroll
         for (int i = 0; i < G / 2; ++i) {
             const uint4 w = reinterpret_cast<const uint4*>(slot)[i * 32 + lane];
-            pr.e[2 * i] = EncEntry{w.x, w.y}; pr.e[2 * i + 1] = EncEntry{w.z, w.w};
+            e[2 * i] = EncEntry{w.x, w.y}; e[2 * i + 1] = EncEntry{w.z, w.w};
         }
     } else {
         const uint2 w = reinterpret_cast<const uint2*>(slot)[lane];
-        pr.e[0] = EncEntry{w.x, w.y};
+        e[0] = EncEntry{w.x, w.y};
     }
-#pragma unroll
-    for (int i = 0; i < kPlaneWords<G>; ++i) pr.plane[i] = (uint32_t)slot[64 * G + i * 32 + lane];
 }
 
 size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
-    const int NP = coop_predictors(warps), G = d / 32, planes = G <= 2 ? 1 : G / 2;
-    const int slot = enc ? 32 * (2 * G + planes) : 32 * G + 8;
+    const int NP = coop_predictors(warps), G = d / 32, slot = (enc ? 64 : 32) * G + kTailWords;
     return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G));
 }
 
@@ -146,55 +162,71 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
     int buf = 0;
     float m_next[G] = {}, s1_next = 0.f, ideal = 0.f;
     uint32_t kv_next[(G + 1) / 2] = {};
-    // decoding: the position predicted a batch ago, whose vector is written when the coder has passed it
+    // what finishing the position of the batch before takes, once the coder has passed it: encoding, its bit
+    // planes; decoding, its prediction and step
     float mu_old[G] = {};
-    SlotMeta old{kSkipped, 0, 0, 0};
+    uint32_t planes_old[kPlaneWords<G>] = {};
+    int s_old = -1, e_old = 0;
+    bool esc_old = false;
     auto fetch = [&](int k, int into) {
         const int p = first + dir * k;
         if (DENSE) dense_fetch<D>(a, row0 + p, t - t0, c0, m_next, s1_next);
         else prefetch_pairs(sp0 + into * Kp, a.pairs + (row0 + p) * Kp, Kp, lane);
         if (ENC) load_half_raw<G>(reinterpret_cast<const __half*>(a.kv.base) + sh.item.kv0 + c0 + p * a.kv.sp, kv_next);
     };
-    auto finish = [&](int b) {                                                 // decoding: position of batch b
-        const int p = b * NP + w;
-        if (b < 0 || p >= P) return;
-        int sym[G];
-        float out[G];
-        if (old.q == kSkipped) {                                               // zero-rate position: KV' = KV^
+    auto finish = [&](int b) {                                                 // the position of batch b
+        if (b < 0 || b * NP + w >= P) return;
+        const int* slot = slots + ((b & 1) * NP + w) * SW;
+        if constexpr (ENC) {
+            if (s_old < 0 || esc_old) return;                                  // nothing to write, or written by the coder
+            int low[G];
+            uint32_t lows[G], emask[G];
+            bool emit[G];
+            slot_get_ints<G>(slot, lane, low);
+            tail_get<G>(slot + 64 * G, emask);
 #pragma unroll
-            for (int g = 0; g < G; ++g) { sym[g] = 0; out[g] = mu_old[g]; }
+            for (int g = 0; g < G; ++g) { lows[g] = (uint32_t)low[g]; emit[g] = (emask[g] >> lane) & 1u; }
+            place_position<G>(planes_old, lows, emask, emit, s_old, a.staging + (long long)blockIdx.x * a.staging_words_per_warp,
+                              slot[64 * G + 8], lc);
         } else {
-            const int* slot = slots + ((b & 1) * NP + w) * SW;
-            int hi[G];
-            slot_get_ints<G>(slot, lane, hi);
-            if (sh.meta[b & 1][w].escaped) {
+            const int p = b * NP + w;
+            int sym[G];
+            float out[G];
+            if (s_old < 0) {                                                   // zero-rate position: KV' = KV^
 #pragma unroll
-                for (int g = 0; g < G; ++g) sym[g] = hi[g];
+                for (int g = 0; g < G; ++g) { sym[g] = 0; out[g] = mu_old[g]; }
             } else {
-                int base[G], s, qp;
+                int zz[G];
+                slot_get_ints<G>(slot, lane, zz);
+                if (sh.meta[b & 1][w].escaped) {
 #pragma unroll
-                for (int g = 0; g < G; ++g) base[g] = slot[32 * G + g];
-                class_params(old.q, s, qp);
-                const uint16_t* words = reinterpret_cast<const uint16_t*>(a.st.payload + sh.item.off + 128);
-                const int last = (int)((sh.item.nbytes - 128u) >> 1) - 1;      // past the end: the last word
-                join_position<G>(base, hi, s, [&](int i) { return (uint32_t)__ldg(words + min(i, last)); }, lc, sym);
+                    for (int g = 0; g < G; ++g) sym[g] = zz[g];
+                } else {
+                    int base[G];
+                    tail_get<G>(slot + 32 * G, base);
+                    const uint16_t* words = reinterpret_cast<const uint16_t*>(a.st.payload + sh.item.off + 128);
+                    const int last = (int)((sh.item.nbytes - 128u) >> 1) - 1;  // past the end: the last word
+                    join_position<G>(base, zz, s_old, [&](int i) { return (uint32_t)__ldg(words + min(i, last)); }, lc, sym);
+                }
+                const float delta = a.step_exp ? ldexpf(a.sh.delta, e_old) : a.sh.delta;
+#pragma unroll
+                for (int g = 0; g < G; ++g) out[g] = __fmaf_rn((float)sym[g], delta, mu_old[g]);
             }
-            const float delta = a.step_exp ? ldexpf(a.sh.delta, old.e) : a.sh.delta;
+            store_vec<G>(a.kv.base, sh.item.kv0 + c0 + p * a.kv.sp, out, a.sh.out_dtype);
+            if (a.dbg.sym) {
+                const long long o = (row0 + p) * (2 * a.sh.L * a.sh.H) + t;
 #pragma unroll
-            for (int g = 0; g < G; ++g) out[g] = __fmaf_rn((float)sym[g], delta, mu_old[g]);
-        }
-        store_vec<G>(a.kv.base, sh.item.kv0 + c0 + p * a.kv.sp, out, a.sh.out_dtype);
-        if (a.dbg.sym) {
-            const long long o = (row0 + p) * (2 * a.sh.L * a.sh.H) + t;
-#pragma unroll
-            for (int g = 0; g < G; ++g) a.dbg.sym[o * D + c0 + g] = sym[g];
+                for (int g = 0; g < G; ++g) a.dbg.sym[o * D + c0 + g] = sym[g];
+            }
         }
     };
     if (w < P) fetch(w, 0);
     for (int b = 0; b < n_batches; ++b) {
         const int k = b * NP + w, p = first + dir * k;
         float mu[G] = {};
-        SlotMeta sm{kSkipped, 0, 0, 0};
+        uint32_t planes[kPlaneWords<G>] = {};
+        int s = -1, qp = 0, e = 0;
+        bool esc = false;
         if (k < P) {
             float sigma2;
             uint32_t kv_raw[(G + 1) / 2];
@@ -217,29 +249,30 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
             float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
             int zero_q = a.sh.zero_q;
             if (a.step_exp) {                                                  // adaptive step delta * 2^e
-                sm.e = __ldg(a.step_exp + row0 + p);
-                inv_delta = ldexpf(inv_delta, -sm.e);
-                inv_delta2 = ldexpf(inv_delta2, -2 * sm.e);
-                if (zr) zero_q -= 8 * sm.e;
+                e = __ldg(a.step_exp + row0 + p);
+                inv_delta = ldexpf(inv_delta, -e);
+                inv_delta2 = ldexpf(inv_delta2, -2 * e);
+                if (zr) zero_q -= 8 * e;
             }
             const int q = __reduce_max_sync(kFull, scale_class(sigma2, a.sh.sigma_floor * a.sh.sigma_floor, inv_delta2));   // same in all lanes
             const bool skip = zr && q <= zero_q;
-            sm.q = skip ? kSkipped : q;
+            class_params(q, s, qp);
             if constexpr (ENC) {
                 float kvv[G];
                 half_raw_to_float<G>(kv_raw, kvv);
-                int sym[G], u[G], s, qp;
+                int sym[G], u[G];
                 uint32_t at[G];
 #pragma unroll
                 for (int g = 0; g < G; ++g) sym[g] = quantise(kvv[g], mu[g], inv_delta);
-                class_params(q, s, qp);
                 int* slot = slots + ((b & 1) * NP + w) * SW;
                 if (split_symbols<G>(sym, s, u, at)) {
                     Prepared<G> pr;
                     prepare_position<G>(u, at, s, tb.enc[qp - kQMin], lc, pr);
-                    slot_put<G>(slot, lane, pr);
+                    slot_put_entries<G>(slot, lane, pr.e);
+#pragma unroll
+                    for (int i = 0; i < kPlaneWords<G>; ++i) planes[i] = pr.plane[i];
                 } else {
-                    sm.escaped = 1;
+                    esc = true;
                     slot_put_ints<G>(slot, lane, u);
                 }
                 if (a.dbg.sym) {
@@ -262,19 +295,21 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                 for (int g = 0; g < G; ++g)
                     if (a.dbg.mu) a.dbg.mu[o * D + c0 + g] = mu[g];
             }
-            if (lane == 0) sh.meta[b & 1][w] = sm;
+            if (skip) s = -1;
+            if (lane == 0) sh.meta[b & 1][w] = SlotMeta{s, qp - kQMin, esc, 0};
             __syncwarp();                                                      // readers of the pair slot are done
         }
         block_barrier();
-        if constexpr (!ENC) {
-            finish(b - 1);
+        finish(b - 1);
 #pragma unroll
-            for (int g = 0; g < G; ++g) mu_old[g] = mu[g];
-            old = sm;
-        }
+        for (int g = 0; g < G; ++g) mu_old[g] = mu[g];
+#pragma unroll
+        for (int i = 0; i < kPlaneWords<G>; ++i) planes_old[i] = planes[i];
+        s_old = s; e_old = e; esc_old = esc;
+        __syncwarp();                                                          // the slot's readers are done before it is filled again
     }
     block_barrier();
-    if constexpr (!ENC) finish(n_batches - 1);
+    finish(n_batches - 1);
     if (ENC && a.dbg.ideal) {
         ideal = warp_sum(ideal);
         if (lane == 0) atomicAdd(&a.counters->ideal_bits, (double)ideal);
@@ -296,23 +331,32 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         for (int b = 0; b < n_batches; ++b) {
             block_barrier();                                                   // batch b is there
             const int cnt = min(NP, P - b * NP);
-            const int* slot = slots + (b & 1) * NP * SW;
-            Prepared<G> next;
-            slot_get<G>(slot, lane, next);
+            int* slot = slots + (b & 1) * NP * SW;
+            EncEntry next[G];
+            slot_get_entries<G>(slot, lane, next);
             SlotMeta sm = sh.meta[b & 1][0];
             for (int j = 0; j < cnt; ++j, slot += SW) {
-                const Prepared<G> pr = next;
+                EncEntry ent[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) ent[g] = next[g];
                 const SlotMeta m = sm;
-                if (j + 1 < cnt) { slot_get<G>(slot + SW, lane, next); sm = sh.meta[b & 1][j + 1]; }
-                if (m.q == kSkipped) { ++n_skipped; continue; }
-                int s, qp;
-                class_params(m.q, s, qp);
+                if (j + 1 < cnt) { slot_get_entries<G>(slot + SW, lane, next); sm = sh.meta[b & 1][j + 1]; }
+                if (m.planes < 0) { ++n_skipped; continue; }
                 if (!m.escaped) {
-                    wp = push_position<G>(pr, s, x, stage, wp, lc);
+                    uint32_t low[G], emask[G];
+                    bool emit[G];
+                    int lows[G];
+                    chain_position<G>(ent, x, low, emask, emit);
+                    wp -= words_of<G>(emask, m.planes);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) lows[g] = (int)low[g];
+                    slot_put_ints<G>(slot, lane, lows);
+                    tail_put<G>(slot + 64 * G, emask);
+                    slot[64 * G + 8] = wp;
                 } else {
                     int u[G];
                     slot_get_ints<G>(slot, lane, u);
-                    wp = encode_position_escapes<G>(u, s, tb.enc[qp - kQMin], x, stage, wp, lane, n_escapes);
+                    wp = encode_position_escapes<G>(u, m.planes, tb.enc[m.table], x, stage, wp, lane, n_escapes);
                 }
             }
         }
@@ -325,41 +369,46 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         bool bad = x < kRansL;
         src += 128;
         const int nwords = (int)((sh.item.nbytes - 128u) >> 1);
-        int rp = 0, fetched = 0, ready = 0;
+        int rp = 0, fetched = 0;
         ring_fetch<G>(ring, src, 2 * nwords, 0, fetched, lane);
         const RingWords<G> words{ring};
+        // rp from which on copies in flight are needed, and from which on more are asked for.  A position and its
+        // last refill window take at most 252 G + 64 bytes; copies are asked for at least every kFetchStep
+        // words and a position, so at least ring - 512 - 2 kFetchStep - 252 G bytes ahead of rp are asked for.
+        constexpr int kNeed = 252 * G + 64, kFetchStep = 512;
+        static_assert(ring_bytes(G) - kRingBlock - 2 * kFetchStep - 252 * G >= kNeed, "a wait has to cover the next position");
+        int wait_at = 0, fetch_at = kFetchStep;
         for (int b = 0; b < n_batches; ++b) {
             block_barrier();                                                   // the classes of batch b are there
             const int cnt = min(NP, P - b * NP);
             int* slot = slots + (b & 1) * NP * SW;
-            int q = sh.meta[b & 1][0].q;
+            SlotMeta sm = sh.meta[b & 1][0];
             for (int j = 0; j < cnt; ++j, slot += SW) {
-                const int qj = q;
-                if (j + 1 < cnt) q = sh.meta[b & 1][j + 1].q;
-                if (qj == kSkipped) continue;
-                // a position's words, and the last refill window
-                if (min(2 * rp + 252 * G + 64, 2 * nwords) > ready) {
+                const SlotMeta m = sm;
+                if (j + 1 < cnt) sm = sh.meta[b & 1][j + 1];
+                if (m.planes < 0) continue;
+                if (rp >= wait_at) {
                     asm volatile("cp.async.wait_all;" ::: "memory");
                     __syncwarp();
-                    ready = fetched;
+                    wait_at = fetched >= 2 * nwords ? 0x7fffffff : (fetched - kNeed) / 2 + 1;
                 }
-                int s, qp, base[G], hi[G];
-                class_params(qj, s, qp);
+                if (rp >= fetch_at) {
+                    __syncwarp();                                              // readers of what is overwritten are done
+                    ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
+                    fetch_at = rp + kFetchStep;
+                }
+                int base[G], zz[G];
                 auto step = [&](const auto& find) {
-                    if (pull_position<G>(s, find, x, words, rp, lc, base, hi)) {
-#pragma unroll
-                        for (int g = 0; g < G; ++g)
-                            if (lane == g) slot[32 * G + g] = base[g];
+                    if (pull_position<G>(m.planes, find, x, words, rp, lc, base, zz)) {
+                        tail_put<G>(slot + 32 * G, base);
                     } else {
-                        decode_position_escapes<G>(hi, s, find, x, words, rp, lane);
+                        decode_position_escapes<G>(zz, m.planes, find, x, words, rp, lane);
                         if (lane == 0) sh.meta[b & 1][j].escaped = 1;
                     }
                 };
-                if (qp - kQMin >= kWideFrom) step(WideLookup{tb.wide[qp - kQMin - kWideFrom]});
-                else step(Lookup{tb.first[qp - kQMin], tb.fc[qp - kQMin]});
-                slot_put_ints<G>(slot, lane, hi);
-                __syncwarp();                                                  // readers of the ring are done
-                ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
+                if (m.table >= kWideFrom) step(WideLookup{tb.wide[m.table - kWideFrom]});
+                else step(Lookup{tb.first[m.table], tb.fc[m.table]});
+                slot_put_ints<G>(slot, lane, zz);
             }
         }
         block_barrier();
