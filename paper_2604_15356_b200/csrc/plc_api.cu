@@ -369,6 +369,7 @@ static plc_status run_topk_for(plc_ctx* c, const void* logits_dev, int S, int n,
     TopkArgs a{};
     a.logits = static_cast<const __half*>(logits_dev); a.N = (long long)S * n; a.V = c->cfg.vocab; a.K = c->cfg.top_k;
     a.pairs = c->pairs; a.Kp = padded_k(c->cfg); a.n_per_session = n; a.pos_begin = pb; a.pos_end = pe;
+    a.tickets = c->ticket;
     a.pair_mul = pair_index(c->cfg) ? 1 : c->cfg.head_dim * 2;
     for (a.pair_rows = 0; (c->cfg.head_dim << a.pair_rows) < 256; ++a.pair_rows) {}
     if (tokens) {

@@ -55,7 +55,9 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
     constexpr bool FROM_OPEN = SRC == kSrcOpen;
     constexpr bool DENSE = SRC == kSrcDense;
     __shared__ EncTables tb;
+    chain_next();
     load_tables(&tb, &a.tables->enc);
+    chain_wait();
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -195,7 +197,9 @@ template <int D, bool DENSE, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
 __global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     __shared__ DecTables tb;
+    chain_next();
     load_tables(&tb, &a.tables->dec);
+    chain_wait();
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -332,6 +336,8 @@ __device__ __forceinline__ void hadamard(float (&v)[Geo<D>::G], int lane) {
 template <int D, bool ENC>
 __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
     constexpr int G = Geo<D>::G;
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp, B = rq.bits;
     int2* sp0 = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
@@ -425,6 +431,8 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
 template <int D>
 __global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp;
     int2* sp = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
@@ -517,8 +525,10 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
     const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
     set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
-    cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
-    if (e != cudaSuccess) return e;
+    if (a.mu_dense) {
+        const cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int), st);
+        if (e != cudaSuccess) return e;
+    }
     if (use_coop(a)) return launch_coop(a, true, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.dbg.ideal || a.step_exp;
@@ -541,9 +551,8 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * blocks, kThreads, sm, st>>>(a);
         count_launch();
-        return cudaGetLastError();
+        return launch_chained(kern, sm_count() * blocks, kThreads, sm, st, 1, a);
     });
 }
 
@@ -565,8 +574,10 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
     const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
     set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
-    cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
-    if (e != cudaSuccess) return e;
+    if (a.mu_dense) {
+        const cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int), st);
+        if (e != cudaSuccess) return e;
+    }
     if (use_coop(a)) return launch_coop(a, false, st);
     const bool zr = a.sh.zero_q != kZeroOff;
     const bool flex = a.dbg.sym || a.dbg.q || a.dbg.mu || a.step_exp;
@@ -589,25 +600,21 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * blocks, kThreads, sm, st>>>(a);
         count_launch();
-        return cudaGetLastError();
+        return launch_chained(kern, sm_count() * blocks, kThreads, sm, st, 1, a);
     });
 }
 
 cudaError_t launch_rotq(const CodecArgs& a0, const RotqArgs& r, bool encode, cudaStream_t st) {
     CodecArgs a = a0;
     set_queues(a, 2 * a.sh.L * a.sh.H);
-    cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int) * kTicketWords, st);
-    if (e != cudaSuccess) return e;
     return dispatch_d(a.sh.d, [&](auto D) {
         auto kern = encode ? rotq_kernel<decltype(D)::value, true> : rotq_kernel<decltype(D)::value, false>;
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<sm_count() * kGatherBlocks, kThreads, sm, st>>>(a, r);
         count_launch();
-        return cudaGetLastError();
+        return launch_chained(kern, sm_count() * kGatherBlocks, kThreads, sm, st, 1, a, r);
     });
 }
 
@@ -623,9 +630,8 @@ cudaError_t launch_append_quantise(const CodecArgs& a, cudaStream_t st) {
         int occ = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, sm) != cudaSuccess || occ < 1) occ = 1;
         if (blocks > (long long)sm_count() * occ) blocks = (long long)sm_count() * occ;
-        kern<<<(unsigned)blocks, kThreads, sm, st>>>(a);
         count_launch();
-        return cudaGetLastError();
+        return launch_chained(kern, (unsigned)blocks, kThreads, sm, st, 1, a);
     });
 }
 

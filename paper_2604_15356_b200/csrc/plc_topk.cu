@@ -283,6 +283,11 @@ __device__ __forceinline__ void put_surprisal(const TopkArgs& a, long long rowi,
     }
 }
 
+__device__ __forceinline__ void zero_tickets(const TopkArgs& a) {
+    if (a.tickets && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < kTicketWords; i += blockDim.x) a.tickets[i] = 0u;
+}
+
 template <bool VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     constexpr int NW = THREADS / 32;
@@ -290,6 +295,9 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int V = a.V, K = a.K;
     const int ntiles = (V + THREADS * 8 - 1) / (THREADS * 8);
+    chain_next();
+    chain_wait();
+    zero_tickets(a);
     for (long long rowi = blockIdx.x; rowi < a.N; rowi += gridDim.x) {
         if (a.pos_begin || a.pos_end) {
             int s = (int)(rowi / a.n_per_session), i = (int)(rowi % a.n_per_session);
@@ -638,6 +646,9 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
     W* list = reinterpret_cast<W*>(codes + kCodes);
     uint16_t* my_slots = reinterpret_cast<uint16_t*>(SHARE && blocks > 1 ? at_first_block(slots) : slots);
     if (SHARE && blocks > 1) meet();                                                      // all blocks of the cluster have started
+    chain_next();
+    chain_wait();
+    zero_tickets(a);
     const int K = a.K;
     const long long group = SHARE ? blockIdx.x / blocks : (long long)blockIdx.x * nwarps + warp;
     const long long stride = SHARE ? gridDim.x / blocks : (long long)gridDim.x * nwarps;
@@ -896,19 +907,8 @@ static cudaError_t launch_stream(const TopkArgs& a, int sms, cudaStream_t st) {
     int occ = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, per_block * 32, smem) != cudaSuccess || occ < 1) occ = 1;
     const long long want = share ? a.N * cluster : (a.N + per_block - 1) / per_block;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster));
-    cfg.blockDim = dim3(per_block * 32);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cluster; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = cluster > 1 ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, a);
     count_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return launch_chained(kern, (unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster), per_block * 32, smem, st, cluster, a);
 }
 
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
@@ -929,17 +929,11 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0) != cudaSuccess || occ < 1) occ = 1;
         const long long per_sm = occ < cap ? occ : cap;       // the rows in flight stay within L2
         const long long blocks = a.N < sms * per_sm ? a.N : sms * per_sm;
-        kern<<<(unsigned)blocks, threads, 0, st>>>(a);
+        count_launch();
+        return launch_chained(kern, (unsigned)blocks, threads, 0, st, 1, a);
     };
-    if (wide) {
-        if (vec) launch(topk_softmax_kernel<true, 512>, 512, 2);
-        else launch(topk_softmax_kernel<false, 512>, 512, 2);
-    } else {
-        if (vec) launch(topk_softmax_kernel<true, 256>, 256, 5);
-        else launch(topk_softmax_kernel<false, 256>, 256, 5);
-    }
-    count_launch();
-    return cudaGetLastError();
+    if (wide) return vec ? launch(topk_softmax_kernel<true, 512>, 512, 2) : launch(topk_softmax_kernel<false, 512>, 512, 2);
+    return vec ? launch(topk_softmax_kernel<true, 256>, 256, 5) : launch(topk_softmax_kernel<false, 256>, 256, 5);
 }
 
 }  // namespace plc
