@@ -960,3 +960,31 @@ def test_topk_rows_of_every_layout(dev, orc, N, V, K, off):
     np.testing.assert_allclose(out["logp2"].cpu().numpy(), lp, atol=1e-4, rtol=1e-6)
     only = ctx.topk_softmax(rows, torch.from_numpy(tok).to(dev), want=("lse", "logp2"))
     np.testing.assert_allclose(only["lse"].cpu().numpy(), lse, atol=2e-5, rtol=1e-6)
+
+
+@pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
+def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
+    """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
+    (fewer chunks get a block each); candidate counts that leave remainders of the gather's stretches."""
+    S, n, L, H = 3, 50 * CP, 2, 8
+    tokens, logits, T, kv = make_workload(3000 + d, S, n, L, H, d, V, K, pp=10.0)
+    pb, pe = ([0, 3, n // 2], [n, n - 1, n]) if ranges else (None, None)
+    g = gpu_encode(dev, T, kv, logits, K, 0.02, CP, pb, pe)
+    assert g["rc"] == plc.OK and g["W"] * S * g["mc"] > 32 * torch.cuda.get_device_properties(dev).multi_processor_count
+    check_against_oracle(orc, g, T, kv, logits, K, 0.02, CP, pb, pe)
+    gpu_decode_check(g, kv, 0.02, n, pb, pe)
+
+
+def test_long_chunks_with_escapes_and_wide_planes(dev, orc):
+    """A block per chunk over positions of very different classes: chunks long enough for the decoder's word ring
+    to turn several times, with escapes (which send a position through the step-by-step route) among them."""
+    S, n, L, H, d, V, K, CP, delta = 1, 700, 1, 2, 128, 512, 24, 700, 1.0 / 512
+    tokens, logits, T, kv = make_workload(4711, S, n, L, H, d, V, K, pp=6.0, sigma=0.2)
+    lg = logits.numpy().copy()
+    for i in range(0, n, 3):                                        # every third position: a point mass
+        lg[0, i] = np.float16(-40.0); lg[0, i, int(tokens[0, i])] = np.float16(40.0)
+    logits = torch.from_numpy(lg)
+    g = gpu_encode(dev, T, kv, logits, K, delta, CP, capacity=9 * n * 4 * d + 4096)
+    assert g["rc"] == plc.OK and g["ctx"].stats().n_escapes > 0
+    check_against_oracle(orc, g, T, kv, logits, K, delta, CP)
+    gpu_decode_check(g, kv, delta, n)
