@@ -332,31 +332,49 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
             block_barrier();                                                   // batch b is there
             const int cnt = min(NP, P - b * NP);
             int* slot = slots + (b & 1) * NP * SW;
+            const SlotMeta* meta = sh.meta[b & 1];
             EncEntry next[G];
             slot_get_entries<G>(slot, lane, next);
-            SlotMeta sm = sh.meta[b & 1][0];
-            for (int j = 0; j < cnt; ++j, slot += SW) {
-                EncEntry ent[G];
+            int next_planes = meta[0].planes;
+            auto code = [&](const EncEntry (&ent)[G], int planes, int* to) {
+                uint32_t low[G], emask[G];
+                bool emit[G];
+                int lows[G];
+                chain_position<G>(ent, x, low, emask, emit);
+                wp -= words_of<G>(emask, planes);
 #pragma unroll
-                for (int g = 0; g < G; ++g) ent[g] = next[g];
-                const SlotMeta m = sm;
-                if (j + 1 < cnt) { slot_get_entries<G>(slot + SW, lane, next); sm = sh.meta[b & 1][j + 1]; }
-                if (m.planes < 0) { ++n_skipped; continue; }
-                if (!m.escaped) {
-                    uint32_t low[G], emask[G];
-                    bool emit[G];
-                    int lows[G];
-                    chain_position<G>(ent, x, low, emask, emit);
-                    wp -= words_of<G>(emask, m.planes);
+                for (int g = 0; g < G; ++g) lows[g] = (int)low[g];
+                slot_put_ints<G>(to, lane, lows);
+                tail_put<G>(to + 64 * G, emask);
+                to[64 * G + 8] = wp;
+            };
+            // One vote a batch: without a position that is skipped or escapes the loop has no branches, and the
+            // independent work of neighbouring positions fills the gaps of the state's chain.
+            if (!__any_sync(kFull, lane < cnt && (meta[lane].planes < 0 || meta[lane].escaped))) {
+#pragma unroll 4
+                for (int j = 0; j < cnt; ++j, slot += SW) {
+                    EncEntry ent[G];
 #pragma unroll
-                    for (int g = 0; g < G; ++g) lows[g] = (int)low[g];
-                    slot_put_ints<G>(slot, lane, lows);
-                    tail_put<G>(slot + 64 * G, emask);
-                    slot[64 * G + 8] = wp;
-                } else {
-                    int u[G];
-                    slot_get_ints<G>(slot, lane, u);
-                    wp = encode_position_escapes<G>(u, m.planes, tb.enc[m.table], x, stage, wp, lane, n_escapes);
+                    for (int g = 0; g < G; ++g) ent[g] = next[g];
+                    const int planes = next_planes, ahead = j + 1 < cnt ? 1 : 0;         // the last one is fetched again
+                    slot_get_entries<G>(slot + ahead * SW, lane, next);
+                    next_planes = meta[j + ahead].planes;
+                    code(ent, planes, slot);
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < cnt; ++j, slot += SW) {
+                    const SlotMeta m = meta[j];
+                    if (m.planes < 0) { ++n_skipped; continue; }
+                    if (!m.escaped) {
+                        EncEntry ent[G];
+                        slot_get_entries<G>(slot, lane, ent);
+                        code(ent, m.planes, slot);
+                    } else {
+                        int u[G];
+                        slot_get_ints<G>(slot, lane, u);
+                        wp = encode_position_escapes<G>(u, m.planes, tb.enc[m.table], x, stage, wp, lane, n_escapes);
+                    }
                 }
             }
         }
