@@ -25,8 +25,8 @@ constexpr int kCoopMaxWarps = 16;
 // Predicting warps of a block.
 __host__ __device__ constexpr int coop_predictors(int warps) { return warps == kCoopMaxWarps ? 3 * warps / 4 : warps - 1; }
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
-// Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; about four such are held.
-__host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 8192 : 4096; }
+// Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; eight such and more are held.
+__host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 16384 : 8192; }
 
 // What a predicting warp tells the coder about a position (one 16-byte word): bit planes (-1: nothing is
 // coded), table id - kQMin, whether a component escapes (encoding; decoding: the coder's answer).
@@ -390,43 +390,59 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         int rp = 0, fetched = 0;
         ring_fetch<G>(ring, src, 2 * nwords, 0, fetched, lane);
         const RingWords<G> words{ring};
-        // rp from which on copies in flight are needed, and from which on more are asked for.  A position and its
-        // last refill window take at most 252 G + 64 bytes; copies are asked for at least every kFetchStep
-        // words and a position, so at least ring - 512 - 2 kFetchStep - 252 G bytes ahead of rp are asked for.
-        constexpr int kNeed = 252 * G + 64, kFetchStep = 512;
-        static_assert(ring_bytes(G) - kRingBlock - 2 * kFetchStep - 252 * G >= kNeed, "a wait has to cover the next position");
+        // rp from which on copies in flight are needed, and from which on more are asked for.  Two positions and
+        // their last refill window take at most 504 G + 64 bytes; copies are asked for at least every
+        // kFetchStep words and two positions, so at least ring - 512 - 2 kFetchStep - 504 G bytes ahead of rp
+        // are asked for.
+        constexpr int kNeed = 504 * G + 64, kFetchStep = 512;
+        static_assert(ring_bytes(G) - kRingBlock - 2 * kFetchStep - 504 * G >= kNeed, "a wait has to cover the next positions");
         int wait_at = 0, fetch_at = kFetchStep;
+        auto keep_filled = [&]() {
+            if (rp >= wait_at) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+                wait_at = fetched >= 2 * nwords ? 0x7fffffff : (fetched - kNeed) / 2 + 1;
+            }
+            if (rp >= fetch_at) {
+                __syncwarp();                                                  // readers of what is overwritten are done
+                ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
+                fetch_at = rp + kFetchStep;
+            }
+        };
         for (int b = 0; b < n_batches; ++b) {
             block_barrier();                                                   // the classes of batch b are there
             const int cnt = min(NP, P - b * NP);
             int* slot = slots + (b & 1) * NP * SW;
-            SlotMeta sm = sh.meta[b & 1][0];
-            for (int j = 0; j < cnt; ++j, slot += SW) {
-                const SlotMeta m = sm;
-                if (j + 1 < cnt) sm = sh.meta[b & 1][j + 1];
-                if (m.planes < 0) continue;
-                if (rp >= wait_at) {
-                    asm volatile("cp.async.wait_all;" ::: "memory");
-                    __syncwarp();
-                    wait_at = fetched >= 2 * nwords ? 0x7fffffff : (fetched - kNeed) / 2 + 1;
-                }
-                if (rp >= fetch_at) {
-                    __syncwarp();                                              // readers of what is overwritten are done
-                    ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
-                    fetch_at = rp + kFetchStep;
-                }
+            SlotMeta* meta = sh.meta[b & 1];
+            auto code = [&](const auto& find, int planes, int j) {
                 int base[G], zz[G];
-                auto step = [&](const auto& find) {
-                    if (pull_position<G>(m.planes, find, x, words, rp, lc, base, zz)) {
-                        tail_put<G>(slot + 32 * G, base);
-                    } else {
-                        decode_position_escapes<G>(zz, m.planes, find, x, words, rp, lane);
-                        if (lane == 0) sh.meta[b & 1][j].escaped = 1;
-                    }
-                };
-                if (m.table >= kWideFrom) step(WideLookup{tb.wide[m.table - kWideFrom]});
-                else step(Lookup{tb.first[m.table], tb.fc[m.table]});
-                slot_put_ints<G>(slot, lane, zz);
+                if (pull_position<G>(planes, find, x, words, rp, lc, base, zz)) {
+                    tail_put<G>(slot + j * SW + 32 * G, base);
+                } else {
+                    decode_position_escapes<G>(zz, planes, find, x, words, rp, lane);
+                    if (lane == 0) meta[j].escaped = 1;
+                }
+                slot_put_ints<G>(slot + j * SW, lane, zz);
+            };
+            // One vote a batch: where all positions have wide tables, the loop has no other case, and two
+            // positions share the check of the ring.
+            if (!__any_sync(kFull, lane < cnt && (meta[lane].planes < 0 || meta[lane].table < kWideFrom))) {
+#pragma unroll 1
+                for (int j = 0; j < cnt; j += 2) {
+                    const SlotMeta m0 = meta[j], m1 = meta[min(j + 1, cnt - 1)];
+                    keep_filled();
+                    code(WideLookup{tb.wide[m0.table - kWideFrom]}, m0.planes, j);
+                    if (j + 1 < cnt) code(WideLookup{tb.wide[m1.table - kWideFrom]}, m1.planes, j + 1);
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < cnt; ++j) {
+                    const SlotMeta m = meta[j];
+                    if (m.planes < 0) continue;
+                    keep_filled();
+                    if (m.table >= kWideFrom) code(WideLookup{tb.wide[m.table - kWideFrom]}, m.planes, j);
+                    else code(Lookup{tb.first[m.table], tb.fc[m.table]}, m.planes, j);
+                }
             }
         }
         block_barrier();
