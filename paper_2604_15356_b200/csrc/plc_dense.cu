@@ -270,65 +270,51 @@ dense_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     }
 }
 
-// P[row][v] = bf16(exp(l_v - lse)), columns V..ldp-1 = 0.  One block per row; 8 logits per thread
-// and step when the row is 16-byte aligned.  exp is the fast intrinsic: its relative error (~1e-6)
-// is far below the 2^-9 of the bfloat16 result.
+// P[row][v] = bf16(exp(l_v - lse)), columns V..ldp-1 = 0.  One block per row; 8 logits per thread and step when
+// the row is 16-byte aligned.  Two passes: maximum and sum together (a thread rescales its sum when it
+// meets a larger logit), then the exponentials (the row is in L2 by then); HBM bound, the logits once and
+// P once.  exp is the fast intrinsic: its relative error (~1e-6) is far below the 2^-9 of the bfloat16
+// result.
 template <bool VEC>
 __global__ void __launch_bounds__(256) softmax_bf16_kernel(const __half* __restrict__ logits, long long rows, int V, int ldp,
                                                            __nv_bfloat16* __restrict__ P) {
     __shared__ float red_m[8], red_s[8];
-    __shared__ float sh_max, sh_lse;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
         const __half* lr = logits + row * V;
-        // pass 1: maximum
-        float m = -INFINITY;
+        float m = -65504.0f, s = 0.f;                                   // not -inf: exp(-inf - m) stays 0
+        auto raise = [&](float to) {                                    // a larger logit: the sum so far is scaled to it
+            if (to > m) { s *= __expf(m - to); m = to; }
+        };
         if (VEC) {
+#pragma unroll 4
             for (int v = tid * 8; v < V; v += 256 * 8) {
                 const uint4 r = *reinterpret_cast<const uint4*>(lr + v);
                 const __half2* hp = reinterpret_cast<const __half2*>(&r);
+                const __half2 top = __hmax2(__hmax2(hp[0], hp[1]), __hmax2(hp[2], hp[3]));
+                raise(fmaxf(__low2float(top), __high2float(top)));
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); m = fmaxf(m, fmaxf(f.x, f.y)); }
+                for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); s += __expf(f.x - m) + __expf(f.y - m); }
             }
         } else {
-            for (int v = tid; v < V; v += 256) m = fmaxf(m, __half2float(lr[v]));
+            for (int v = tid; v < V; v += 256) { const float x = __half2float(lr[v]); raise(x); s += __expf(x - m); }
         }
+        float mx = m;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+        s = warp_sum(s * __expf(m - mx));
+        if (lane == 0) { red_m[wid] = mx; red_s[wid] = s; }
         __syncthreads();
-        if (lane == 0) red_m[wid] = m;
-        __syncthreads();
-        if (tid == 0) {
-            float mm = red_m[0];
-            for (int w = 1; w < 8; ++w) mm = fmaxf(mm, red_m[w]);
-            sh_max = mm;
-        }
-        __syncthreads();
-        const float mx = sh_max;
-        // pass 2: sum of exponentials (row is in L2 now)
-        float s = 0.f;
-        if (VEC) {
-            for (int v = tid * 8; v < V; v += 256 * 8) {
-                const uint4 r = *reinterpret_cast<const uint4*>(lr + v);
-                const __half2* hp = reinterpret_cast<const __half2*>(&r);
+        mx = red_m[0];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); s += __expf(f.x - mx) + __expf(f.y - mx); }
-            }
-        } else {
-            for (int v = tid; v < V; v += 256) s += __expf(__half2float(lr[v]) - mx);
-        }
-        s = warp_sum(s);
-        if (lane == 0) red_s[wid] = s;
-        __syncthreads();
-        if (tid == 0) {
-            float ss = 0.f;
-            for (int w = 0; w < 8; ++w) ss += red_s[w];
-            sh_lse = mx + __logf(ss);
-        }
-        __syncthreads();
-        const float lse = sh_lse;
+        for (int w = 1; w < 8; ++w) mx = fmaxf(mx, red_m[w]);
+        s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += red_s[w] * __expf(red_m[w] - mx);
+        const float lse = mx + __logf(s);
         __nv_bfloat16* pr = P + row * ldp;
         if (VEC) {
+#pragma unroll 4
             for (int v = tid * 8; v < ldp; v += 256 * 8) {          // ldp is a multiple of 64
                 __nv_bfloat162 o[4];
                 if (v < V) {
