@@ -25,25 +25,27 @@ constexpr int kCoopMaxWarps = 16;
 // Predicting warps of a block.
 __host__ __device__ constexpr int coop_predictors(int warps) { return warps == kCoopMaxWarps ? 3 * warps / 4 : warps - 1; }
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
-// Ring size: a position takes at most G * (2 * 15 + 32 + 64) words; eight such and more are held.
-__host__ __device__ constexpr int ring_bytes(int G) { return G == 8 ? 16384 : 8192; }
+// Ring size: a position takes at most G * (2 * 15 + 32 + 64) words.  The roomy ring holds two positions at a
+// time for the coder (of blocks whose predictions come from memory, or that have an SM to themselves);
+// where blocks gather rows beside each other the 4 KB more a block cost more L1 than the coder gains.
+__host__ __device__ constexpr int ring_bytes(int G, bool roomy) { return (G == 8 ? 8192 : 4096) * (roomy ? 2 : 1); }
 
 // What a predicting warp tells the coder about a position (one 16-byte word): bit planes (-1: nothing is
 // coded), table id - kQMin, whether a component escapes (encoding; decoding: the coder's answer).
 struct __align__(16) SlotMeta { int planes, table, escaped, pad; };
 
 // The words of a chunk, read through the ring.  `ready` bytes have landed, `fetched` are on their way.
-template <int G>
+template <int BYTES>
 struct RingWords {
     const uint16_t* ring;
-    __device__ __forceinline__ uint32_t operator()(int i) const { return ring[i & (ring_bytes(G) / 2 - 1)]; }
+    __device__ __forceinline__ uint32_t operator()(int i) const { return ring[i & (BYTES / 2 - 1)]; }
 };
-template <int G>
+template <int BYTES>
 __device__ __forceinline__ void ring_fetch(uint16_t* ring, const uint8_t* src, int total, int rp, int& fetched, int lane) {
-    while (fetched < total && fetched + kRingBlock <= 2 * rp + ring_bytes(G)) {
+    while (fetched < total && fetched + kRingBlock <= 2 * rp + BYTES) {
         const int at = fetched + 16 * lane;
         if (at < total) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(ring) + (at & (ring_bytes(G) - 1)));
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(ring) + (at & (BYTES - 1)));
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src + at), "r"(min(16, total - at)) : "memory");
         }
         fetched += kRingBlock;
@@ -122,9 +124,9 @@ __device__ __forceinline__ void slot_get_entries(const int* slot, int lane, EncE
     }
 }
 
-size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc) {
+size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc, bool roomy) {
     const int NP = coop_predictors(warps), G = d / 32, slot = (enc ? 64 : 32) * G + kTailWords;
-    return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G));
+    return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G, roomy));
 }
 
 // All warps of the block meet here; the two roles reach it from different places in the code.
@@ -317,11 +319,12 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
 }
 
 // Coder of the block's chunk, one batch behind the predictions.
-template <int D, bool ENC, class Tab>
+template <int D, bool ENC, bool ROOMY, class Tab>
 __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
     const int P = sh.item.it.P, n_batches = (P + NP - 1) / NP;
+    constexpr int kRing = ring_bytes(G, ROOMY);
     uint32_t x = kRansL;
     if constexpr (ENC) {
         uint16_t* stage = a.staging + (long long)blockIdx.x * a.staging_words_per_warp;
@@ -348,10 +351,11 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                 tail_put<G>(to + 64 * G, emask);
                 to[64 * G + 8] = wp;
             };
+            constexpr int kAhead = ROOMY ? 4 : 1;                              // (beside gathering warps the longer code costs more)
             // One vote a batch: without a position that is skipped or escapes the loop has no branches, and the
             // independent work of neighbouring positions fills the gaps of the state's chain.
             if (!__any_sync(kFull, lane < cnt && (meta[lane].planes < 0 || meta[lane].escaped))) {
-#pragma unroll 4
+#pragma unroll kAhead
                 for (int j = 0; j < cnt; ++j, slot += SW) {
                     EncEntry ent[G];
 #pragma unroll
@@ -388,14 +392,14 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         src += 128;
         const int nwords = (int)((sh.item.nbytes - 128u) >> 1);
         int rp = 0, fetched = 0;
-        ring_fetch<G>(ring, src, 2 * nwords, 0, fetched, lane);
-        const RingWords<G> words{ring};
-        // rp from which on copies in flight are needed, and from which on more are asked for.  Two positions and
-        // their last refill window take at most 504 G + 64 bytes; copies are asked for at least every
-        // kFetchStep words and two positions, so at least ring - 512 - 2 kFetchStep - 504 G bytes ahead of rp
-        // are asked for.
-        constexpr int kNeed = 504 * G + 64, kFetchStep = 512;
-        static_assert(ring_bytes(G) - kRingBlock - 2 * kFetchStep - 504 * G >= kNeed, "a wait has to cover the next positions");
+        ring_fetch<kRing>(ring, src, 2 * nwords, 0, fetched, lane);
+        const RingWords<kRing> words{ring};
+        // rp from which on copies in flight are needed, and from which on more are asked for.  A stretch (two
+        // positions in a roomy ring, else one) and its last refill window take at most kStretch + 64 bytes;
+        // copies are asked for at least every kFetchStep words and a stretch, so at least ring - 512 -
+        // 2 kFetchStep - kStretch bytes ahead of rp are asked for.
+        constexpr int kStretch = (ROOMY ? 504 : 252) * G, kNeed = kStretch + 64, kFetchStep = 512;
+        static_assert(kRing - kRingBlock - 2 * kFetchStep - kStretch >= kNeed, "a wait has to cover the next positions");
         int wait_at = 0, fetch_at = kFetchStep;
         auto keep_filled = [&]() {
             if (rp >= wait_at) {
@@ -405,7 +409,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
             }
             if (rp >= fetch_at) {
                 __syncwarp();                                                  // readers of what is overwritten are done
-                ring_fetch<G>(ring, src, 2 * nwords, rp, fetched, lane);
+                ring_fetch<kRing>(ring, src, 2 * nwords, rp, fetched, lane);
                 fetch_at = rp + kFetchStep;
             }
         };
@@ -424,9 +428,13 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                 }
                 slot_put_ints<G>(slot + j * SW, lane, zz);
             };
+            auto any_code = [&](const SlotMeta& m, int j) {
+                if (m.table >= kWideFrom) code(WideLookup{tb.wide[m.table - kWideFrom]}, m.planes, j);
+                else code(Lookup{tb.first[m.table], tb.fc[m.table]}, m.planes, j);
+            };
             // One vote a batch: where all positions have wide tables, the loop has no other case, and two
             // positions share the check of the ring.
-            if (!__any_sync(kFull, lane < cnt && (meta[lane].planes < 0 || meta[lane].table < kWideFrom))) {
+            if (ROOMY && !__any_sync(kFull, lane < cnt && (meta[lane].planes < 0 || meta[lane].table < kWideFrom))) {
 #pragma unroll 1
                 for (int j = 0; j < cnt; j += 2) {
                     const SlotMeta m0 = meta[j], m1 = meta[min(j + 1, cnt - 1)];
@@ -435,13 +443,14 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                     if (j + 1 < cnt) code(WideLookup{tb.wide[m1.table - kWideFrom]}, m1.planes, j + 1);
                 }
             } else {
+                SlotMeta next = meta[0];
 #pragma unroll 1
                 for (int j = 0; j < cnt; ++j) {
-                    const SlotMeta m = meta[j];
+                    const SlotMeta m = next;
+                    if (j + 1 < cnt) next = meta[j + 1];
                     if (m.planes < 0) continue;
                     keep_filled();
-                    if (m.table >= kWideFrom) code(WideLookup{tb.wide[m.table - kWideFrom]}, m.planes, j);
-                    else code(Lookup{tb.first[m.table], tb.fc[m.table]}, m.planes, j);
+                    any_code(m, j);
                 }
             }
         }
@@ -453,7 +462,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
 }
 
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
-template <int D, bool DENSE, bool ENC>
+template <int D, bool DENSE, bool ENC, bool ROOMY>
 __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
@@ -501,7 +510,7 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
         const int go = sh.item.go;
         if (go < 0) break;
         if (go > 0) {
-            if (warp == 0) coop_code<D, ENC>(a, sh, tb, slots, ring, NP, lc);
+            if (warp == 0) coop_code<D, ENC, ROOMY>(a, sh, tb, slots, ring, NP, lc);
             else if (warp > 0) coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
         }
         __syncthreads();                                                       // the chunk is coded; its item has been read
@@ -517,14 +526,17 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
     return dispatch_d(a.sh.d, [&](auto D) {
         constexpr int d = decltype(D)::value;
         const bool dense = a.mu_dense != nullptr;
-        auto kern = dense ? (encode ? coop_kernel<d, true, true> : coop_kernel<d, true, false>)
-                          : (encode ? coop_kernel<d, false, true> : coop_kernel<d, false, false>);
         const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
         // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
-        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  Fifteen where there is
-        // a chunk an SM at most: then a prediction's latency is what the coder waits for.
-        const int warps = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode) <= 160 * 1024 ? kCoopMaxWarps : kCoopMaxWarps / 2;
-        const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode);
+        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  A block of sixteen where
+        // there is a chunk an SM at most.
+        const bool alone = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode, true) <= 160 * 1024;
+        const bool roomy = dense || alone;
+        auto kern = dense ? (encode ? coop_kernel<d, true, true, true> : coop_kernel<d, true, false, true>)
+                  : roomy ? (encode ? coop_kernel<d, false, true, true> : coop_kernel<d, false, false, true>)
+                          : (encode ? coop_kernel<d, false, true, false> : coop_kernel<d, false, false, false>);
+        const int warps = alone ? kCoopMaxWarps : kCoopMaxWarps / 2;
+        const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode, roomy);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int occ = 1;
