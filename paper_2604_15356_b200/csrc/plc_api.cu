@@ -152,6 +152,7 @@ int padded_k(const plc_config& cfg) {
     const int rows = 2 * 256 / cfg.head_dim;  // rows of T that two warp-wide 16-byte-per-lane loads fetch (lanes read two pairs at a time)
     return (cfg.top_k + rows - 1) / rows * rows;
 }
+bool pair_index(const plc_config& cfg) { return (long long)cfg.vocab * cfg.head_dim * 2 >= (1ll << 32); }
 
 plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (positions <= c->pairs_cap) return PLC_OK;
@@ -176,7 +177,7 @@ CodecArgs base_args(const plc_ctx* c) {
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
     a.tables = c->tables;
-    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs;
+    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs; a.pair_index = pair_index(c->cfg);
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
     return a;
@@ -369,6 +370,7 @@ static plc_status run_topk_for(plc_ctx* c, const void* logits_dev, int S, int n,
     a.logits = static_cast<const __half*>(logits_dev); a.N = (long long)S * n; a.V = c->cfg.vocab; a.K = c->cfg.top_k;
     a.pairs = c->pairs; a.Kp = padded_k(c->cfg); a.n_per_session = n; a.pos_begin = pb; a.pos_end = pe;
     a.tickets = c->ticket;
+    a.pair_mul = pair_index(c->cfg) ? 1 : c->cfg.head_dim * 2;
     for (a.pair_rows = 0; (c->cfg.head_dim << a.pair_rows) < 256; ++a.pair_rows) {}
     if (tokens) {
         a.tokens = tokens; a.step_exp = c->step_exp; a.bits_out = bits_out;

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
                 int zero_q = ZR ? a.sh.zero_q : 0;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArg
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
             int zero_q = ZR ? a.sh.zero_q : 0;
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D>(col, n2, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_k
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;

@@ -57,49 +57,58 @@ __device__ __forceinline__ void add_row(const char* p, float w, unsigned long lo
         ffma2(acc2[j], ww, pack2(f.x, f.y));
     }
 }
-// Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: the
-// candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a multiple of 2 ROWS
-// (the padding has weight 0 and a valid row).  table, n2: the table's rows and their squared norms, the
-// same pointers in every lane.
+// Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
+// offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
+// multiple of 2 ROWS (the padding has weight 0 and a valid offset).  table, n2: the table's rows and
+// their squared norms, the same pointers in every lane.
 // What bounds it: issue slots (per row and lane 8 conversions, 4 packed FMAs, a load), with the rows'
-// latency on top; pairs are read two at a time, and a row's address is one wide multiply-add (byte offsets
-// in the pairs cost three additions in its place).
+// latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
+// beside its load.
 template <int D>
-__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2,
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, bool pair_index,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
     const int h = lane / R, iters = Kp / ROWS;
-    const char* mine = table + 16 * (lane % R);
+    const uint32_t lane_off = 16u * (lane % R);
     // variance term first: its row-norm loads are in flight while the rows are gathered
     float s1 = 0.f;
     for (int k = lane; k < Kp; k += 32) {
         const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
-        s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + (uint32_t)pr.x), s1);
+        const uint32_t at = pair_index ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
+        s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
-    // Straight-line stretches of 32, 16 and 8 rows: the loads of a stretch are issued as far ahead as the
-    // kernel's registers allow (64 rows of 128 components, uniform candidates, 24 warps an SM: 8.0 ms
-    // with stretches of 8 only, 6.4 ms with 32).
-    const int4* pl = reinterpret_cast<const int4*>(sp + h * iters);
-    int left = iters >> 1;
-    auto rows = [&](auto count) {
-        constexpr int N = decltype(count)::value;
+    if (!pair_index) {
+        // Straight-line stretches of 32, 16 and 8 rows: the loads of a stretch are issued as far ahead as the
+        // kernel's registers allow (64 rows of 128 components, uniform candidates, 24 warps an SM: 8.0 ms
+        // with stretches of 8 only, 6.4 ms with 32).
+        const int4* pl = reinterpret_cast<const int4*>(sp + h * iters);
+        int left = iters >> 1;
+        auto rows = [&](auto count) {
+            constexpr int N = decltype(count)::value;
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const int4 pr = pl[i];
-            add_row(mine + (unsigned long long)(uint32_t)pr.x * (2 * D), __int_as_float(pr.y), acc2);
-            add_row(mine + (unsigned long long)(uint32_t)pr.z * (2 * D), __int_as_float(pr.w), acc2);
+            for (int i = 0; i < N; ++i) {
+                const int4 pr = pl[i];
+                add_row(table + ((uint32_t)pr.x + lane_off), __int_as_float(pr.y), acc2);
+                add_row(table + ((uint32_t)pr.z + lane_off), __int_as_float(pr.w), acc2);
+            }
+            pl += N;
+            left -= N;
+        };
+#pragma unroll 1
+        while (left >= 16) rows(std::integral_constant<int, 16>{});
+        if (left >= 8) rows(std::integral_constant<int, 8>{});
+        if (left >= 4) rows(std::integral_constant<int, 4>{});
+#pragma unroll 1
+        while (left > 0) rows(std::integral_constant<int, 1>{});
+    } else {                                                 // tables of 4 GB or more: 64-bit offsets
+#pragma unroll 1
+        for (int it = 0; it < iters; ++it) {
+            const int2 pr = sp[h * iters + it];
+            add_row(table + ((size_t)(uint32_t)pr.x * (2 * D) + lane_off), __int_as_float(pr.y), acc2);
         }
-        pl += N;
-        left -= N;
-    };
-#pragma unroll 1
-    while (left >= 16) rows(std::integral_constant<int, 16>{});
-    if (left >= 8) rows(std::integral_constant<int, 8>{});
-    if (left >= 4) rows(std::integral_constant<int, 4>{});
-#pragma unroll 1
-    while (left > 0) rows(std::integral_constant<int, 1>{});
+    }
     float acc[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) unpack2(acc2[j], acc[2 * j], acc[2 * j + 1]);

@@ -153,7 +153,7 @@ constexpr int kTicketWords = 1024;               // one counter per work queue (
 struct TopkArgs {
     const __half* logits; const int32_t* tokens; int64_t N; int V, K;
     int2* pairs;            // [N][Kp], or null: see put_pair; entries K..Kp-1 get candidate 0 with weight 0
-    int Kp, pair_rows;      // pair_rows: log2 of the rows a warp-wide load fetches
+    int Kp, pair_rows, pair_mul;   // log2 of the rows a warp-wide load fetches; bytes of a table row (1: pairs hold indices)
     int32_t* idx; float* w; float* lse; float* zk; float* logp2;   // optional user outputs
     // Adaptive step (needs tokens): step_exp[row] = b0 - b_i, bits_out[row] = b_i (both optional).
     int* step_exp; int* bits_out; int b0, extra; float hbar;
@@ -199,6 +199,7 @@ struct CodecArgs {
     const CoderTables* tables;                     // frequency tables of the coder
     const __half* T; const float* rownorm2;        // [tables][V][d], [tables][V]
     const int2* pairs;                             // [S*n][Kp] (written by the top-K kernels, put_pair)
+    bool pair_index;                               // pairs hold row indices instead of byte offsets (tables of 4 GB or more)
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
     KvView kv;                                     // encode: input f16; decode: output
     int S, n; const int32_t* pos_begin; const int32_t* pos_end;

@@ -260,11 +260,12 @@ __device__ void select_by_histogram(Smem<THREADS>& sm, const __half* row, int V,
     __syncthreads();
 }
 
-// Entry k of a row's pairs: candidate and weight, in the order in which the gather's lanes read them: the
-// entries of one of the 1 << pair_rows row groups of a warp-wide load follow each other.
+// Entry k of a row's pairs: byte offset of the candidate's table row (its index where a table's rows span
+// 4 GB or more) and weight, in the order in which the gather's lanes read them: the entries of one of
+// the 1 << pair_rows row groups of a warp-wide load follow each other.
 __device__ __forceinline__ void put_pair(const TopkArgs& a, long long rowi, int k, int idx, float w) {
     const int at = (k & ((1 << a.pair_rows) - 1)) * (a.Kp >> a.pair_rows) + (k >> a.pair_rows);
-    a.pairs[rowi * a.Kp + at] = make_int2(idx, __float_as_int(w));
+    a.pairs[rowi * a.Kp + at] = make_int2((int)((unsigned)idx * (unsigned)a.pair_mul), __float_as_int(w));
 }
 
 // log2 P of the row's token and, for the adaptive step (Def. 7), b = max(1, floor(b0 h / hbar)) capped at
