@@ -723,7 +723,7 @@ def dedup_arm(args, torch, plc, workloads, dev):
                          "peak_kind": kind, "ms_per_launch": max(mean["encode"], mean["decode"]) / (S // Sb),
                          "accounting": "K*d*2 B of random T rows + 2*d B of KV per coded vector + the coded bytes, over the slower "
                                        "of encode / decode (top-K of the coded positions included)"},
-            "logp2_stage": {"kernel": "topk_staged_kernel", "bound": "hbm", "achieved": logits_bytes / (mean["logp2"] / 1e3) / 1e9,
+            "logp2_stage": {"kernel": "topk_stream_kernel", "bound": "hbm", "achieved": logits_bytes / (mean["logp2"] / 1e3) / 1e9,
                             "peak": peak, "unit": "GB/s", "frac": logits_bytes / (mean["logp2"] / 1e3) / 1e9 / peak,
                             "ms_per_launch": mean["logp2"] / (S // Sb),
                             "accounting": "logits read once (2*S*n*V bytes) over the summed log2 P launches; the encode and "
@@ -769,7 +769,7 @@ def topk_arm(args, torch, plc, workloads, dev):
             "n_gpus": 1, "steps": args.steps, "warmup": max(args.warmup, 3), "ms_per_step": sel["ms_per_call"],
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": "top-K softmax alone", "rows": N, "V": V, "K": K, "l2": "input of %.2f GB, larger than L2" % (N * V * 2 / 1e9)},
-            "roofline": {"kernel": "topk_staged_kernel" if V * 2 <= 65536 else "topk_softmax_kernel", "bound": "hbm",
+            "roofline": {"kernel": "topk_stream_kernel" if K <= 128 else "topk_softmax_kernel", "bound": "hbm",
                          "achieved": sel["achieved"], "peak": peak, "unit": "GB/s", "frac": sel["frac"], "traffic": None,
                          "peak_kind": kind, "accounting": "the logits once (rows * V * 2 bytes) over the whole call (all its kernels)"},
             "modes": out, "gpu_launches": plc.launch_count() - launches0, "clocks": clocks}

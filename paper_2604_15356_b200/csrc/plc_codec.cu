@@ -472,7 +472,11 @@ cudaError_t pair_smem_bytes(Kern kern, int Kp, size_t& bytes) {
 
 int codec_grid_warps(int) { return sm_count() * kBlocksPerSM * kWarpsPerBlock; }
 
-static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kGatherBlocks * kWarpsPerBlock);
+// Chunks an SM is counted to take from a queue: a quarter more than its resident warps, so that the SMs of a
+// queue finish a table at about the same time.
+constexpr int kQueueItems = 40;
+static_assert(kQueueItems >= kGatherBlocks * kWarpsPerBlock, "a queue must keep its SMs busy");
+static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kQueueItems);
 
 // A block per chunk (plc_coop.cu) while the chunks would not fill the GPU with a warp each: below that a
 // warp's own chain is what the call waits for; above it the kernels here do more work per instruction
@@ -491,7 +495,7 @@ constexpr int kCoopItems = 4;                    // chunks an SM works on at a t
 // so that the warps of an SM gather from one or two tables and shared rows stay in that SM's L1.
 void codec_schedule(const CodecArgs& a0, int n_tables, int* nq, int* g) {
     CodecArgs a = a0;
-    set_queues(a, n_tables, use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock);
+    set_queues(a, n_tables, use_coop(a) ? kCoopItems : kQueueItems);
     *nq = a.sched_nq; *g = a.sched_g;
 }
 
@@ -523,7 +527,7 @@ cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, c
 
 cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
-    const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
+    const int items_per_sm = use_coop(a) ? kCoopItems : kQueueItems;
     set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
     if (a.mu_dense) {
         const cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int), st);
@@ -572,7 +576,7 @@ cudaError_t launch_append_seal(const CodecArgs& a, cudaStream_t st) {
 
 cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
     CodecArgs a = a0;
-    const int items_per_sm = use_coop(a) ? kCoopItems : kGatherBlocks * kWarpsPerBlock;
+    const int items_per_sm = use_coop(a) ? kCoopItems : kQueueItems;
     set_queues(a, 2 * a.sh.L * a.sh.H, items_per_sm);
     if (a.mu_dense) {
         const cudaError_t e = cudaMemsetAsync(a.ticket, 0, sizeof(unsigned int), st);
