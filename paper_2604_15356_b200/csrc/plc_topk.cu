@@ -7,6 +7,7 @@
 // refinement finds the key itself, and equal keys are taken in index order.
 // Reductions use warp shuffles in a fixed order, so results are bit-reproducible from run to run.
 #include <algorithm>
+#include <type_traits>
 
 #include "plc_common.cuh"
 
@@ -579,15 +580,13 @@ __device__ __forceinline__ void emit_selected(const TopkArgs& a, long long rowi,
     if (a.zk && lane == 0) a.zk[rowi] = sum_k / sum_all;
 }
 
-// Counters of the end of a row: one a step of the search for the bound (at most 4 downwards and 16 between),
-// and the running totals of the groups and the list.
-constexpr int kBoundSteps = 20, kCntCodes = 30, kCntList = 31;
-static_assert(kBoundSteps < kCntCodes, "the search must not reach the totals");
 struct StreamShared {                               // of the warps that share a row (the first block's copy counts)
     float ref[kStreamWarps * kMaxCluster], sum[kStreamWarps * kMaxCluster];
     uint32_t key[kStreamWarps * kMaxCluster];
-    int cnt[32];                                    // of the end of the row, which the first block's warps share
+    int n_codes, n_list;                            // running totals of the end of the row, which the first block's warps share
+    uint32_t theta;                                 // its bound
 };
+static_assert(kStreamWarps * kMaxCluster <= 32, "a lane for every warp of a row");
 
 // The row after `rowi` (stride: the rows in work at a time) inside its session's position range, or N.
 __device__ __forceinline__ long long next_row(const TopkArgs& a, long long rowi, long long stride) {
@@ -761,12 +760,12 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
         float sum_all = warp_sum((x0 + x1) + (x2 + x3)), lmax;
         if (SHARE) {
             if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
-            if (SELECT && wrow == 0) sh.cnt[lane] = 0;
+            if (SELECT && wrow == 0 && lane == 0) sh.n_codes = sh.n_list = 0;
             meet();
-            for (int w = 0; w < NW; ++w) kmax = max(kmax, sh.key[w]);
+            const bool on = lane < NW;                                                    // a lane a warp of the row
+            kmax = __reduce_max_sync(kFull, on ? sh.key[lane] : 0u);
             lmax = val_of_key(kmax);
-            sum_all = 0.f;
-            for (int w = 0; w < NW; ++w) sum_all += sh.sum[w] * expf(sh.ref[w] - lmax);
+            sum_all = warp_sum(on ? sh.sum[lane] * expf(sh.ref[lane] - lmax) : 0.f);
         } else {
             lmax = val_of_key(kmax);
             sum_all *= expf(ref - lmax);
@@ -776,34 +775,41 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             // The row's own warp, or all warps of the first block.
             const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
             auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
-            // The bound: the K-th largest group maximum (any value that exactly K of them reach will do).
+            // The bound: the K-th largest group maximum (any value that exactly K of them reach will do), searched
+            // by one warp with all maxima in its registers.  The search is a chain of ten steps or so: shared among
+            // eight warps a step cost 1300 cycles (guards, a shared counter, a barrier), 14400 of the 34000 cycles of a
+            // row of 128256 logits by itself; now 5350 of 22000.
             const int S = NW * ns, words = (S + 1) >> 1;
-            if ((S & 1) && tw == 0) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
-            sync();
-            uint32_t mx[kSlots / 2];                                                      // this warp's words, two maxima each
+            uint32_t mx[kSlots / 2];                                                      // two maxima each
+            uint32_t theta = kKeyNegInf;
+            if (tw == 0) {
+                if (S & 1) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
+                __syncwarp();
 #pragma unroll
-            for (int i = 0; i < kSlots / 2; ++i) mx[i] = tw + i * tws < words ? slots[(tw + i * tws) * 32 + lane] : kNoValue2;
-            uint32_t theta = kKeyNegInf, hi = kmax + 1, down = 256;                       // first downwards from the maximum, then between
+                for (int i = 0; i < kSlots / 2; ++i) mx[i] = i < words ? slots[i * 32 + lane] : kNoValue2;
+                auto reach = [&](uint32_t h2, auto first) {                               // of this lane's first words
+                    constexpr int A = SHARE ? 4 : 1;                                      // one sum where other rows fill the gaps
+                    __half2 c[A];
+#pragma unroll
+                    for (int i = 0; i < A; ++i) c[i] = __float2half2_rn(0.f);
+#pragma unroll
+                    for (int i = 0; i < decltype(first)::value; ++i) c[i % A] = __hadd2(c[i % A], __hge2(as_half2(mx[i]), as_half2(h2)));
+                    if constexpr (A > 1) c[0] = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
+                    return __half2int_rn(__hadd(__low2half(c[0]), __high2half(c[0])));
+                };
+                uint32_t hi = kmax + 1, down = 256;                                       // first downwards from the maximum, then between
 #pragma unroll 1
-            for (int it = 0; hi - theta > 1; ++it) {
-                const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
-                __half2 c2 = __float2half2_rn(0.f);
-#pragma unroll
-                for (int i = 0; i < kSlots / 2; i += 4) {
-                    if (tw + i * tws < words) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) c2 = __hadd2(c2, __hge2(as_half2(mx[i + k]), as_half2(h2)));
-                    }
+                while (hi - theta > 1) {
+                    const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
+                    const int c = __reduce_add_sync(kFull, words <= 8 ? reach(h2, std::integral_constant<int, 8>{})
+                                                                      : reach(h2, std::integral_constant<int, kSlots / 2>{}));
+                    if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
+                    if (c == K) break;
                 }
-                int c = __reduce_add_sync(kFull, __half2int_rn(__hadd(__low2half(c2), __high2half(c2))));
-                if (SHARE) {
-                    if (lane == 0) atomicAdd(&local_sh.cnt[it], c);
-                    sync();
-                    c = local_sh.cnt[it];
-                }
-                if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
-                if (c == K) break;
+                if (SHARE && lane == 0) local_sh.theta = theta;
             }
+            sync();
+            if (SHARE) theta = local_sh.theta;
             // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
             auto place = [&](int mine, int* shared_total, int& total) {
                 int all;
@@ -820,9 +826,15 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             const uint32_t th2 = bits_of_key(theta) * 0x10001u;
             int n_codes = 0, n = 0;
             uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
+            auto hit = [&](uint32_t w, int i) { return __hge2_mask(as_half2(w), as_half2(th2)) & (0x10001u << (i & 15)); };
+            if (SHARE) {                                                                  // two warps at least: 16 words at most
+#pragma unroll 4
+                for (int i = 0; tw + i * tws < words; ++i) hits[0] |= hit(slots[(tw + i * tws) * 32 + lane], i);
+            } else {
 #pragma unroll
-            for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= __hge2_mask(as_half2(mx[i]), as_half2(th2)) & (0x10001u << (i & 15));
-            int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.cnt[kCntCodes], n_codes);
+                for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= hit(mx[i], i);
+            }
+            int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.n_codes, n_codes);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
                 for (uint32_t m = hits[h]; m; m &= m - 1) {
@@ -831,16 +843,21 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                     ++at;
                 }
             sync();
-            if (SHARE) n_codes = local_sh.cnt[kCntCodes];
+            if (SHARE) n_codes = local_sh.n_codes;
             if (n_codes <= kCodes) {
-                // their logits at or above the bound; head and tail of the row are a turn of their own
+                // their logits at or above the bound; head and tail of the row are a turn of the last warp's own.  A
+                // lane takes one batch of a group where warps share the row (turns are memory latencies: 1700 cycles
+                // each), else all of a group (where rows fill the GPU the lanes' divisions cost more than a turn).
+                const int steps = fine ? 1 : wide, items = SHARE ? n_codes * steps : n_codes;
+                const bool ends_turn = tw == tws - 1 && (r.head > 0 || r.head + 8 * r.nv < r.V);
 #pragma unroll 1
-                for (int i0 = tw * 32 - (has_ends ? 32 : 0); i0 < n_codes; i0 += i0 < 0 ? 32 : 32 * tws) {
-                    const bool mine = i0 >= 0 && i0 + lane < n_codes;
-                    const int code = mine ? codes[i0 + lane] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
-                    const int steps = i0 < 0 || fine ? 1 : wide;
+                for (int i0 = tw * 32 - (ends_turn ? 32 * tws : 0); i0 < items; i0 += 32 * tws) {
+                    const bool mine = i0 >= 0 && i0 + lane < items;
+                    const int ci = !mine ? 0 : SHARE ? (i0 + lane) / steps : i0 + lane, first = SHARE && mine ? i0 + lane - ci * steps : 0;
+                    const int code = mine ? codes[ci] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
+                    const int turns = SHARE || i0 < 0 ? 1 : steps;
 #pragma unroll 1
-                    for (int st = 0; st < steps; ++st) {
+                    for (int st = first; st < first + turns; ++st) {
                         const int t = fine ? ls >> 2 : ls * wide + st;
                         const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
                         uint4 q[kBatch];
@@ -857,7 +874,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 #pragma unroll
                             for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
                         }
-                        for (int to = place(__popc(m), &local_sh.cnt[kCntList], n); m; m &= m - 1, ++to) {
+                        for (int to = place(__popc(m), &local_sh.n_list, n); m; m &= m - 1, ++to) {
                             const int b = __ffs(m) - 1, u = (b >> 2) & 3;
                             const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
                             const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
@@ -867,7 +884,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                 }
             }
             sync();
-            if (SHARE) n = local_sh.cnt[kCntList];
+            if (SHARE) n = local_sh.n_list;
             if (n_codes > kCodes || n > kListCap) {
                 if (tw == 0) slow_select<W>(r.row, r.V, K, theta, kmax, list, lane);
                 n = K;
