@@ -56,8 +56,8 @@ def parse_over(pairs):
 
 
 # Issue-slot use of the fused kernels (smsp__issue_active) from the ncu capture summarised in
-# profiles/fused_kernels_mid_L4.md; quoted beside the roofline fraction, not part of it.
-NCU_ISSUE_SLOT_USE = {"encode_kernel": 0.637, "decode_kernel": 0.638}
+# profiles/gather_and_topk_after_rework.md; quoted beside the roofline fraction, not part of it.
+NCU_ISSUE_SLOT_USE = {"encode_kernel": 0.684, "decode_kernel": 0.654}
 
 
 def fused_roofline(vecs, K, d, t_bytes, kv_bytes, payload, ek, dk, sm_mhz, sms, peak, peak_kind, traffic_per_vector=None):
@@ -84,8 +84,8 @@ def fused_roofline(vecs, K, d, t_bytes, kv_bytes, payload, ek, dk, sm_mhz, sms, 
          "fp32_fma": {"achieved": flop_ach, "peak": flop_peak, "unit": "TFLOP/s", "frac": alu_frac,
                       "peak_kind": "SMs x 128 lanes x 2 flop x sampled SM clock (%d x %.0f MHz)" % (sms, sm_mhz)},
          "issue_slot_use_ncu": NCU_ISSUE_SLOT_USE.get(name),
-         "busiest_units_ncu": "heavy half of the FMA pipe 67 %, L1 data pipe 60 %, issue slots 64 % "
-                              "(profiles/fused_kernels_mid_L4.md: no single unit saturated)",
+         "busiest_units_ncu": "issue slots 65-68 % (profiles/gather_and_topk_after_rework.md); heavy half of the FMA pipe "
+                              "and L1 data pipe level behind them (profiles/fused_kernels_mid_L4.md): no single unit saturated",
          "gathered_row_bytes_frac": bytes_ns / sec / 1e9 / peak,
          "gathered_row_note": "KV + K*d*2 B of gathered rows per vector + bitstream over the HBM copy peak; the rows are "
                            "L1 / L2 hits, so this is an on-chip gather rate, not an HBM utilisation",
