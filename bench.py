@@ -138,10 +138,10 @@ class ClockSampler:
 
 
 # DRAM bytes per vector of the fused kernels, from the ncu capture summarised in
-# profiles/fused_kernels_mid_L4.md (dram__bytes_read.sum + dram__bytes_write.sum over 4.19 M vectors;
+# profiles/gather_and_topk_after_rework.md (dram__bytes_read.sum + dram__bytes_write.sum over 4.19 M vectors;
 # traffic grows in proportion to the vectors).  Valid for the default workload and chunk size only.
-NCU_DRAM_BYTES_PER_VECTOR = {"encode_kernel": 671.0, "decode_kernel": 433.1}
-NCU_TRAFFIC_NOTE = ("dram__bytes_read + dram__bytes_write of a 4-layer ncu capture (profiles/fused_kernels_mid_L4.md) "
+NCU_DRAM_BYTES_PER_VECTOR = {"encode_kernel": 664.9, "decode_kernel": 423.5}
+NCU_TRAFFIC_NOTE = ("dram__bytes_read + dram__bytes_write of a 4-layer ncu capture (profiles/gather_and_topk_after_rework.md) "
                     "scaled by the vectors of a launch")
 
 
