@@ -159,6 +159,7 @@ struct TopkArgs {
     int* step_exp; int* bits_out; int b0, extra; float hbar;
     // Rows are skipped (nothing written) when pos ranges are given and the row is outside them.
     int n_per_session; const int32_t* pos_begin; const int32_t* pos_end;
+    int parts;              // parts of a row where its sum must not depend on the call (set by the launcher)
     unsigned int* tickets;  // kTicketWords work counters that the launch zeroes for the kernel behind it, or null
 };
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st);

@@ -437,19 +437,44 @@ __device__ __forceinline__ int warp_excl_scan(int mine, int lane, int& total) {
     return inc - mine;
 }
 
-// A row as head logits up to the first 16-byte boundary, nv whole 16-byte groups, and a tail.
+// A row as head logits up to the first 16-byte boundary, nv whole 16-byte groups, and a tail; with FIXED
+// the groups are counted from the row's first logit wherever it lies (no head; `phase` logits behind a
+// boundary).
 struct RowView {
     const __half* row;
     const uint4* body;
-    int V, head, nv;
+    int V, head, nv, phase;
 };
+template <bool FIXED = false>
 __device__ __forceinline__ RowView row_view(const __half* row, int V) {
     RowView r;
+    const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(row) & 15u) >> 1;
     r.row = row; r.V = V;
-    r.head = min((int)((16u - (uint32_t)(reinterpret_cast<uintptr_t>(row) & 15u)) & 15u) >> 1, V);
+    r.head = FIXED ? 0 : min((int)((8u - off) & 7u), V);
+    r.phase = FIXED ? (int)off : 0;
     r.nv = (V - r.head) >> 3;
     r.body = reinterpret_cast<const uint4*>(row + r.head);
     return r;
+}
+// Group v of a row whose groups do not start on 16-byte boundaries: out of the two aligned vectors that hold
+// it (never outside the row), or logit by logit where one of them reaches beyond the row.
+__device__ __forceinline__ uint4 group_across(const RowView& r, int v) {
+    uint32_t w[8];
+    if (v == 0 || 8 * v + 16 > r.V) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            w[j] = (uint32_t)__half_as_ushort(r.row[8 * v + 2 * j]) | ((uint32_t)__half_as_ushort(r.row[8 * v + 2 * j + 1]) << 16);
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    const uint4* p = reinterpret_cast<const uint4*>(r.row + (8 * v - r.phase));
+    const uint4 lo = p[0], hi = p[1];
+    w[0] = lo.x; w[1] = lo.y; w[2] = lo.z; w[3] = lo.w; w[4] = hi.x; w[5] = hi.y; w[6] = hi.z; w[7] = hi.w;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) w[i] = (r.phase & 2) ? w[i + 1] : w[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = (r.phase & 4) ? w[i + 2] : w[i];
+    const uint32_t sh = (r.phase & 1) ? 16u : 0u;
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh), __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
 }
 // The ends of the row as groups -1 (lane 0: the head) and nv (lane 1: the tail) of 8, kNoValue where the
 // row is not.
@@ -623,13 +648,19 @@ __device__ __forceinline__ T* at_first_block(T* p) {
 
 // SHARE: the warps of a cluster of blocks (of a block, if it is alone) share a row; otherwise every warp
 // has a row of its own.
-template <bool SELECT, bool SHARE, class W>
+// FIXED: the order in which a row's exponentials are added depends on V alone, not on how many rows the call
+// has or where the row lies in memory.  The adaptive step (Def. 7) floors a multiple of the row's
+// log-sum-exp, so a batch encoded at once and restored a session at a time must find the same bits.  The
+// row is cut into parts of its own (row_parts), a warp takes one after another, and groups are counted
+// from the row's first logit.
+template <bool SELECT, bool SHARE, bool FIXED, class W>
 __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const TopkArgs a) {
     extern __shared__ __align__(16) unsigned char stream_raw[];
     __shared__ StreamShared local_sh;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int blocks = SHARE ? (int)cluster_blocks() : 1;
-    const int NW = SHARE ? nwarps * blocks : 1, wrow = SHARE ? (int)cluster_rank() * nwarps + warp : 0;   // warps of the row, this one's number
+    const int warps = SHARE ? nwarps * blocks : 1, wfirst = SHARE ? (int)cluster_rank() * nwarps + warp : 0;   // warps of the row, this one's number
+    const int NW = FIXED ? a.parts : warps;                                              // parts of the row: one a warp, or several
     StreamShared& sh = *(SHARE && blocks > 1 ? at_first_block(&local_sh) : &local_sh);
     auto meet = [&]() {
         if (blocks > 1) {
@@ -653,125 +684,151 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
     const long long stride = SHARE ? gridDim.x / blocks : (long long)gridDim.x * nwarps;
 
     for (long long rowi = next_row(a, group, stride); rowi < a.N; rowi = next_row(a, rowi + stride, stride)) {
-        const RowView r = row_view(a.logits + rowi * (long long)a.V, a.V);
+        const RowView r = row_view<FIXED>(a.logits + rowi * (long long)a.V, a.V);
+        auto fetch = [&](int v) { return FIXED && r.phase ? group_across(r, v) : ldg_stream(r.body + v); };
         const int per = kBatch * 32 * NW, batches = max(1, (r.nv + per - 1) / per);
         // Slots of this warp: one a group of 8 where all the row's fit, else one for every `wide` batches.
         const bool fine = NW * batches * kBatch <= kSlots;
         const int wide = (NW * batches + kSlots - 1) / kSlots, ns = fine ? batches * kBatch : (batches + wide - 1) / wide;
-        const int v0 = wrow * 32 + lane;                                                  // group u of batch t: v0 + (t * kBatch + u) * 32 * NW
-        auto load = [&](int t, uint4 (&q)[kBatch]) {
-            const uint4* p = r.body + v0 + t * per;
+        uint32_t part_key = 0;                                                            // FIXED: lane p holds part p
+        float part_ref = 0.f, part_sum = 0.f;
+        uint32_t kmax = 0;
+        float ref = 0.f, sum_all = 0.f;
+        auto load = [&](int w, int t, uint4 (&q)[kBatch]) {                               // group u of batch t of part w
+            const int at = w * 32 + lane + t * per;
             if ((t + 1) * per <= r.nv) {
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) q[u] = ldg_stream(p + u * 32 * NW);
+                for (int u = 0; u < kBatch; ++u) q[u] = fetch(at + u * 32 * NW);
             } else {
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) q[u] = v0 + t * per + u * 32 * NW < r.nv ? ldg_stream(p + u * 32 * NW) : all4(kNegInf2);
+                for (int u = 0; u < kBatch; ++u) q[u] = at + u * 32 * NW < r.nv ? fetch(at + u * 32 * NW) : all4(kNegInf2);
             }
+        };
+        int wrow = wfirst, wload = wfirst, tload = 0;
+        auto load_next = [&](uint4 (&q)[kBatch]) {                                        // FIXED: on into the next part of this warp
+            load(wload, tload, q);
+            if (++tload == batches && wload + warps < NW) { tload = 0; wload += warps; }
         };
         uint4 cur[kBatch], nxt[kBatch];
-        load(0, cur);
-        load(1, nxt);
-        const bool has_ends = wrow == 0 && (r.head > 0 || r.head + 8 * r.nv < r.V);
-        const uint4 ends = has_ends ? row_ends(r, lane) : all4(kNoValue2);
-        uint32_t m2 = kNegInf2;
-        if (has_ends) m2 = hmax2_bits(m2, top2_of(ends));
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) m2 = hmax2_bits(m2, top2_of(cur[u]));
-        float ref = fmaxf(val_of_key(__reduce_max_sync(kFull, top_key(m2))), -65504.0f);
-        // A logit more than 4 above the reference moves it, so that no exponent is large (its rounding would
-        // show in the sum).
-        auto lim_of = [](float rf) { const uint32_t b = (uint32_t)__half_as_ushort(__float2half_ru(rf + 4.0f)); return b | (b << 16); };
-        uint32_t lim2 = lim_of(ref);
-        float nb = -ref * 1.44269504088896341f;
-        unsigned long long s0 = 0ull, s1 = 0ull;
-        auto add_group = [&](const uint4& q) {
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-            const unsigned long long l2e = both(1.44269504088896341f, 1.44269504088896341f), nb2 = both(nb, nb);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __half22float2(as_half2(w[j]));
-                float x, y, ex, ey;
-                parts(fma2(both(f.x, f.y), l2e, nb2), x, y);
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
-                if (j & 1) s1 = add2(s1, both(ex, ey)); else s0 = add2(s0, both(ex, ey));
-            }
-        };
-        if (has_ends) {
-            auto real = [](uint32_t w) { const uint32_t m = __vcmpeq2(w, kNoValue2); return (w & ~m) | (kNegInf2 & m); };
-            add_group(make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)));
-        }
-        // slot s of a lane: half s & 1 of word (s / 2, lane)
-        auto put_slot = [&](int slot, uint32_t top2) {
-            const int sl = wrow * ns + slot;
-            my_slots[(sl >> 1) * 64 + lane * 2 + (sl & 1)] = (uint16_t)hmax2_bits(top2, top2 >> 16);   // the low half: of both
-        };
-        auto batch = [&](const uint4 (&q)[kBatch], uint32_t (&top)[kBatch]) {             // returns the maximum
-            uint32_t top4 = kNegInf2;
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) { top[u] = top2_of(q[u]); top4 = hmax2_bits(top4, top[u]); }
-            m2 = hmax2_bits(m2, top4);
-            if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
-                const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
-                const float f = expf(ref - to);
-                const unsigned long long ff = both(f, f), z = 0ull;
-                s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
-                ref = to; nb = -ref * 1.44269504088896341f; lim2 = lim_of(ref);
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) add_group(q[u]);
-            return top4;
-        };
-        uint32_t top[kBatch];
-        if (SELECT && fine) {
+        if (FIXED) { load_next(cur); load_next(nxt); }
+        else { load(wrow, 0, cur); load(wrow, 1, nxt); }
 #pragma unroll 1
-            for (int t = 0; t < batches; ++t) {
-                batch(cur, top);
+        do {
+            const bool has_ends = wrow == 0 && (r.head > 0 || r.head + 8 * r.nv < r.V);
+            const uint4 ends = has_ends ? row_ends(r, lane) : all4(kNoValue2);
+            uint32_t m2 = kNegInf2;
+            if (has_ends) m2 = hmax2_bits(m2, top2_of(ends));
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) { put_slot(t * kBatch + u, top[u]); cur[u] = nxt[u]; }
-                load(t + 2, nxt);
+            for (int u = 0; u < kBatch; ++u) m2 = hmax2_bits(m2, top2_of(cur[u]));
+            ref = fmaxf(val_of_key(__reduce_max_sync(kFull, top_key(m2))), -65504.0f);
+            // A logit more than 4 above the reference moves it, so that no exponent is large (its rounding would
+            // show in the sum).
+            auto lim_of = [](float rf) { const uint32_t b = (uint32_t)__half_as_ushort(__float2half_ru(rf + 4.0f)); return b | (b << 16); };
+            uint32_t lim2 = lim_of(ref);
+            float nb = -ref * 1.44269504088896341f;
+            unsigned long long s0 = 0ull, s1 = 0ull;
+            auto add_group = [&](const uint4& q) {
+                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+                const unsigned long long l2e = both(1.44269504088896341f, 1.44269504088896341f), nb2 = both(nb, nb);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __half22float2(as_half2(w[j]));
+                    float x, y, ex, ey;
+                    parts(fma2(both(f.x, f.y), l2e, nb2), x, y);
+                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
+                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
+                    if (j & 1) s1 = add2(s1, both(ex, ey)); else s0 = add2(s0, both(ex, ey));
+                }
+            };
+            if (has_ends) {
+                auto real = [](uint32_t w) { const uint32_t m = __vcmpeq2(w, kNoValue2); return (w & ~m) | (kNegInf2 & m); };
+                add_group(make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)));
             }
-        } else {
-            uint32_t group2 = kNegInf2;                                                   // of the slot being filled
+            // slot s of a lane: half s & 1 of word (s / 2, lane)
+            auto put_slot = [&](int slot, uint32_t top2) {
+                const int sl = wrow * ns + slot;
+                my_slots[(sl >> 1) * 64 + lane * 2 + (sl & 1)] = (uint16_t)hmax2_bits(top2, top2 >> 16);   // the low half: of both
+            };
+            auto batch = [&](const uint4 (&q)[kBatch], uint32_t (&top)[kBatch]) {             // returns the maximum
+                uint32_t top4 = kNegInf2;
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) { top[u] = top2_of(q[u]); top4 = hmax2_bits(top4, top[u]); }
+                m2 = hmax2_bits(m2, top4);
+                if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
+                    const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
+                    const float f = expf(ref - to);
+                    const unsigned long long ff = both(f, f), z = 0ull;
+                    s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
+                    ref = to; nb = -ref * 1.44269504088896341f; lim2 = lim_of(ref);
+                }
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) add_group(q[u]);
+                return top4;
+            };
+            uint32_t top[kBatch];
+            uint32_t group2 = kNegInf2;                                                       // of the slot being filled
             int left = wide, slot = 0;
             auto filled = [&](uint32_t top4) {
                 group2 = hmax2_bits(group2, top4);
                 if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = wide; }
             };
+            if (SELECT && (fine || FIXED)) {
 #pragma unroll 1
-            for (int t = 0; t < batches; t += 2) {
-                const uint32_t t0 = batch(cur, top);
-                if (SELECT) filled(t0);
-                load(t + 2, cur);
-                if (t + 1 < batches) {
-                    const uint32_t t1 = batch(nxt, top);
-                    if (SELECT) filled(t1);
+                for (int t = 0; t < batches; ++t) {
+                    const uint32_t top4 = batch(cur, top);
+                    if (FIXED && !fine) filled(top4);
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        if (!FIXED || fine) put_slot(t * kBatch + u, top[u]);
+                        cur[u] = nxt[u];
+                    }
+                    if (FIXED) load_next(nxt);
+                    else load(wrow, t + 2, nxt);
                 }
-                load(t + 3, nxt);
+                if (FIXED && !fine && left != wide) put_slot(slot, group2);
+            } else {
+#pragma unroll 1
+                for (int t = 0; t < batches; t += 2) {
+                    const uint32_t t0 = batch(cur, top);
+                    if (SELECT) filled(t0);
+                    load(wrow, t + 2, cur);
+                    if (t + 1 < batches) {
+                        const uint32_t t1 = batch(nxt, top);
+                        if (SELECT) filled(t1);
+                    }
+                    load(wrow, t + 3, nxt);
+                }
+                if (SELECT && left != wide) put_slot(slot, group2);
             }
-            if (SELECT && left != wide) put_slot(slot, group2);
-        }
 
-        // Row maximum and sum.
-        uint32_t kmax = __reduce_max_sync(kFull, top_key(m2));
-        float x0, x1, x2, x3;
-        parts(s0, x0, x1); parts(s1, x2, x3);
-        float sum_all = warp_sum((x0 + x1) + (x2 + x3)), lmax;
-        if (SHARE) {
-            if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
-            if (SELECT && wrow == 0 && lane == 0) sh.n_codes = sh.n_list = 0;
-            meet();
-            const bool on = lane < NW;                                                    // a lane a warp of the row
-            kmax = __reduce_max_sync(kFull, on ? sh.key[lane] : 0u);
+            // Maximum and sum of the part, then of the row.
+            kmax = __reduce_max_sync(kFull, top_key(m2));
+            float x0, x1, x2, x3;
+            parts(s0, x0, x1); parts(s1, x2, x3);
+            sum_all = warp_sum((x0 + x1) + (x2 + x3));
+            if (SHARE) {
+                if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
+            } else if (FIXED && lane == wrow) {
+                part_key = kmax; part_ref = ref; part_sum = sum_all;
+            }
+        } while (FIXED && (wrow += warps) < NW);
+        float lmax;
+        if (SHARE || FIXED) {
+            const bool on = lane < NW;                                                    // a lane a part of the row
+            if (SHARE) {
+                if (SELECT && wfirst == 0 && lane == 0) sh.n_codes = sh.n_list = 0;
+                meet();
+                if (on) { part_key = sh.key[lane]; part_ref = sh.ref[lane]; part_sum = sh.sum[lane]; }
+            }
+            kmax = __reduce_max_sync(kFull, on ? part_key : 0u);
             lmax = val_of_key(kmax);
-            sum_all = warp_sum(on ? sh.sum[lane] * expf(sh.ref[lane] - lmax) : 0.f);
+            sum_all = warp_sum(on ? part_sum * expf(part_ref - lmax) : 0.f);
         } else {
             lmax = val_of_key(kmax);
             sum_all *= expf(ref - lmax);
         }
 
-        if (SELECT && (!SHARE || wrow < nwarps)) {
+        if (SELECT && (!SHARE || wfirst < nwarps)) {
             // The row's own warp, or all warps of the first block.
             const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
             auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
@@ -864,7 +921,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
                             const int v = vb + u * 32 * NW;
-                            q[u] = mine && v < r.nv && !(fine && u) ? __ldg(r.body + v) : all4(kNoValue2);
+                            q[u] = mine && v < r.nv && !(fine && u) ? (FIXED && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
                         }
                         if (i0 < 0) q[0] = row_ends(r, lane);
                         uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
@@ -894,7 +951,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);
             if (tw == 0) emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
         }
-        if (lane == 0 && wrow == 0) {
+        if (lane == 0 && wfirst == 0) {
             const float lse = lmax + logf(sum_all);
             if (a.lse) a.lse[rowi] = lse;
             if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) put_surprisal(a, rowi, r.row, lse);
@@ -906,19 +963,29 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 
 }  // namespace
 
-template <bool SELECT, class W>
-static cudaError_t launch_stream(const TopkArgs& a, int sms, cudaStream_t st) {
+// Parts of a row whose sum must not depend on the call (FIXED): a power of two with at least 1024 logits
+// each, at most a warp of one block.
+static int row_parts(int V) {
+    int n = 1;
+    while (n < kStreamWarps && 2ll * n * 1024 <= V) n *= 2;
+    return n;
+}
+
+template <bool SELECT, bool FIXED, class W>
+static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st) {
     // Warps a row, in powers of two, each with at least 1024 logits of its own; one when rows alone fill the
     // GPU.  Up to a block of eight: as many as the GPU holds for all rows (32 a SM).  Up to four blocks (a
     // cluster): only while that is a quarter of the GPU, since a cluster's blocks are placed together
     // (64 rows of 128256, 64 warps each: 51 us; 16 warps: 25; one row: 8 warps 24.6, 32 warps 20.5).
+    a.parts = row_parts(a.V);
+    const int most = FIXED ? a.parts : kStreamWarps * kMaxCluster;
     int warps = 1;
-    while (warps < kStreamWarps * kMaxCluster && 2ll * warps * 1024 <= a.V &&
+    while (warps < most && 2ll * warps * 1024 <= a.V &&
            2ll * warps * a.N <= (warps < kStreamWarps ? 32ll : 8ll) * sms) warps *= 2;
     const bool share = warps > 1;
     const int per_block = share ? std::min(warps, kStreamWarps) : kStreamWarps, cluster = share ? warps / per_block : 1;
     const size_t smem = !SELECT ? 0 : stream_smem_per_row<W>() * (share ? 1 : per_block);
-    auto kern = share ? topk_stream_kernel<SELECT, true, W> : topk_stream_kernel<SELECT, false, W>;
+    auto kern = share ? topk_stream_kernel<SELECT, true, FIXED, W> : topk_stream_kernel<SELECT, false, FIXED, W>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int occ = 1;
@@ -934,8 +1001,12 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool select = a.pairs || a.idx || a.w || a.zk;
-    if (!select) return launch_stream<false, uint32_t>(a, sms, st);
-    if (a.K <= kFinal) return a.V <= 65536 ? launch_stream<true, uint32_t>(a, sms, st) : launch_stream<true, unsigned long long>(a, sms, st);
+    if (!select) return launch_stream<false, false, uint32_t>(a, sms, st);
+    if (a.K <= kFinal) {
+        if (a.step_exp || a.bits_out)
+            return a.V <= 65536 ? launch_stream<true, true, uint32_t>(a, sms, st) : launch_stream<true, true, unsigned long long>(a, sms, st);
+        return a.V <= 65536 ? launch_stream<true, false, uint32_t>(a, sms, st) : launch_stream<true, false, unsigned long long>(a, sms, st);
+    }
     // The second pass over a row should find it in L2: rows of up to 128 KB are read by 256 threads
     // with five blocks per SM, longer rows by 512 threads with two blocks per SM (two, so that one
     // block streams while the other sits at the barrier between its passes).

@@ -988,3 +988,96 @@ def test_long_chunks_with_escapes_and_wide_planes(dev, orc):
     assert g["rc"] == plc.OK and g["ctx"].stats().n_escapes > 0
     check_against_oracle(orc, g, T, kv, logits, K, delta, CP)
     gpu_decode_check(g, kv, delta, n)
+
+
+class _SessionStreams:
+    """The streams of one session of a coded batch (same payload, its part of the index)."""
+
+    def __init__(self, st, W, s):
+        self.st, self.W, self.s = st, W, s
+
+    def c(self):
+        st, at = self.st, self.s * self.W * self.st.max_chunks
+        return plc.Streams(st.payload.data_ptr(), st.capacity, st.chunk_offset.data_ptr() + 8 * at,
+                           st.chunk_bytes.data_ptr() + 4 * at, st.total_bytes.data_ptr(), st.max_chunks)
+
+
+@pytest.mark.parametrize("kind,floor,V", [("topk", 0.0, 2000), ("topk", 0.3, 2001), ("adaptive", 0.0, 4003), ("adaptive", 0.3, 4000),
+                                          ("dense", 0.0, 520), ("linear", 0.0, 520)])
+def test_sessions_of_a_batch_decode_alone(dev, kind, floor, V):
+    """A batch encoded in one call is restored one session at a time: prediction, class and step of a position do
+    not depend on what else a call holds.  The batch has a warp per chunk (more than 32 chunks an SM; dense and
+    linear 40), a session alone a block per chunk."""
+    S, n, L, H, d, K, CP, delta = 5, 160, 4, 16, 64, 50, 16, 0.02
+    tokens, logits, T, kv = make_workload(8800 + V, S, n, L, H, d, V, K, pp=15.0)
+    ad = (6, 4, math.log2(15.0)) if kind == "adaptive" else None
+    if kind == "linear":
+        E, A, c = synth.make_linear_model(L, H, V, d, 128, 5)
+        kv = synth.make_kv_linear(E, A, c, tokens, 0.05, 6)
+        ctx = plc.Context.linear(E.to(dev), A.to(dev), c.to(dev), delta, chunk_pos=CP)
+    else:
+        ctx = plc.Context(T.to(dev), K, delta, chunk_pos=CP, sigma_floor=floor, adaptive=ad,
+                          variant=plc.PRED_DENSE if kind == "dense" else plc.PRED_TOPK)
+    W, mc = ctx.W, ctx.max_chunks(n)
+    assert S * W * mc > 40 * torch.cuda.get_device_properties(dev).multi_processor_count
+    st = plc.StreamSet(S * W, mc, S * W * mc * 160 + 3 * S * n * W * d, dev)
+    sym = torch.zeros(S, n, W, d, dtype=torch.int32, device=dev)
+    kvd, lgd, tkd = kv.to(dev), logits.to(dev), tokens.to(dev)
+    ctx.encode(kvd, lgd, st, debug=plc.DebugBuffers(sym.data_ptr(), None, None), tokens=tkd if ad else None)
+    assert ctx.sync_status() == plc.OK
+    out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+    for s in range(S):
+        back = torch.zeros(1, n, W, d, dtype=torch.int32, device=dev)
+        ctx.decode(_SessionStreams(st, W, s), lgd[s:s + 1].clone(), out[:, :, s:s + 1],
+                   debug=plc.DebugBuffers(back.data_ptr(), None, None), tokens=tkd[s:s + 1] if ad else None)
+        assert ctx.sync_status() == plc.OK, s
+        assert torch.equal(back[0], sym[s]), s
+    bound = delta / 2 * (2.0 ** 5 if ad else 1.0) + 1e-3          # adaptive: one bit at least, 2^(6 - 1) steps
+    assert float((out - kvd.float()).abs().max()) <= bound
+
+
+@pytest.mark.parametrize("V", [32000, 32003])
+def test_adaptive_depth_does_not_depend_on_the_call(dev, V):
+    """Def. 7 floors b0 h / hbar: the depth of a row must be the same whether the row is alone in a call or one of
+    many, on a 16-byte boundary or not.  hbar is laid so that the last bit of h decides: the two log2 P that the
+    plain top-K call gives for a row alone and in the batch (sums in another order) fall on different sides."""
+    N, K, b0, extra, n_tried = 512, 64, 16, 12, 0
+    g = torch.Generator(device=dev).manual_seed(V)
+    lg = torch.randn(N, V, generator=g, device=dev).mul_(2.5).half()
+    tok = torch.randint(0, V, (N,), generator=g, device=dev, dtype=torch.int32)
+    T = torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev)
+    plain = plc.Context(T, K, 0.02)
+    many = plain.topk_softmax(lg, tok)["logp2"].cpu().numpy()
+
+    def depths(ctx, rows, toks):
+        m = rows.shape[0]
+        bits = torch.zeros(m, dtype=torch.int32, device=dev)
+        st = plc.StreamSet(ctx.W, ctx.max_chunks(m), 1 << 22, dev)
+        ctx.encode(torch.zeros(1, 2, 1, 1, m, 32, dtype=torch.float16, device=dev), rows.view(1, m, V), st, tokens=toks,
+                   debug=plc.DebugBuffers(None, None, None, bits.data_ptr()))
+        assert ctx.sync_status() == plc.OK
+        return bits.cpu().numpy()
+
+    for i in range(N):
+        one = plain.topk_softmax(lg[i:i + 1].clone(), tok[i:i + 1])["logp2"].cpu().numpy()[0]
+        if one == many[i] or n_tried == 8:
+            continue
+        ha, hb, k = -many[i], -one, np.float32(20)
+        hbar = np.float32(b0) * ha / k
+        for _ in range(40):
+            hbar = np.nextafter(hbar, np.float32(0))
+        for _ in range(80):
+            r = [np.floor(np.float32(b0) * np.float32(h / hbar)) for h in (ha, hb)]
+            if r[0] != r[1]:
+                break
+            hbar = np.nextafter(hbar, np.float32(np.inf))
+        else:
+            continue
+        n_tried += 1
+        ctx = plc.Context(T, K, 0.02, adaptive=(b0, extra, float(hbar)))
+        batch = depths(ctx, lg, tok)
+        buf = torch.zeros(V + 8, dtype=torch.float16, device=dev)
+        for off in (0, 3, 6):
+            buf[off:off + V] = lg[i]
+            assert depths(ctx, buf[off:off + V].view(1, V), tok[i:i + 1])[0] == batch[i], (i, off)
+        ctx.close()
