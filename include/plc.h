@@ -18,7 +18,8 @@
  *   - Problems found on the host (shapes, alignment) are returned at once and nothing is launched.
  *     Problems found on the device (output capacity, damaged streams) are OR-ed into a device status
  *     word that plc_sync_status reads; kernels never read or write outside the stated extents.
- *   - Floating-point inputs are IEEE binary16 ("f16").  NaN logits are not supported.
+ *   - Floating-point inputs are IEEE binary16 ("f16").  NaN logits are not supported: the results of
+ *     their rows are unspecified (selected indices stay inside the vocabulary), those of others are not.
  *
  * Notation: S sessions, n positions per session, L layers, H KV heads, d head dimension
  * (32, 64, 128 or 256), V vocabulary, K candidates, W = 2*L*H streams per position.

@@ -497,13 +497,13 @@ __device__ __forceinline__ uint4 row_ends(const RowView& r, int lane) {
 
 // Exact selection by one warp reading the row from memory: bisection of the K-th largest key between `lo`
 // (at least K logits reach it) and the maximum by counting passes, then the K elements, equal keys in
-// index order, into the list (packed).  For rows whose ties overflow the lists.
+// index order, into the list (packed); returns how many there are.  For rows whose ties overflow the lists.
 template <class W>
-__device__ __noinline__ void slow_select(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, int lane) {
+__device__ __noinline__ int slow_select(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, int lane) {
     const RowView r = row_view(row, V);
     const uint32_t lt = lanemask_lt();
     const uint4 ends = row_ends(r, lane);
-    auto key_at = [&](const uint4& q, int j) { const uint32_t h = half_at(q, j); return h == 0xffffu ? 0u : key_of(h); };   // 0: no value
+    auto key_at = [&](const uint4& q, int j) { const uint32_t h = half_at(q, j); return (h & 0x7fffu) > 0x7c00u ? 0u : key_of(h); };   // NaN: no value, 0
     auto count = [&](uint32_t t) {
         int c = 0;
 #pragma unroll
@@ -540,12 +540,14 @@ __device__ __noinline__ void slow_select(const __half* row, int V, int K, uint32
             const bool ok = key > lo || (key == lo && before < need);
             before += key == lo;
             const uint32_t m = __ballot_sync(kFull, ok);
-            if (ok) list[n + __popc(m & lt)] = order_word<W>(key, r.head + 8 * v + j);
+            const int at = n + __popc(m & lt);
+            if (ok && at < K) list[at] = order_word<W>(key, r.head + 8 * v + j);
             n += __popc(m);
         }
         need = max(0, need - all);
     }
     __syncwarp();
+    return min(n, K);
 }
 
 // Orders a list of n words into `sorted`: a word's place is the number of larger ones, which the team's
@@ -943,13 +945,22 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             sync();
             if (SHARE) n = local_sh.n_list;
             if (n_codes > kCodes || n > kListCap) {
-                if (tw == 0) slow_select<W>(r.row, r.V, K, theta, kmax, list, lane);
-                n = K;
+                sync();                                                                   // all have read the total
+                if (tw == 0) {
+                    n = slow_select<W>(r.row, r.V, K, theta, kmax, list, lane);
+                    if (SHARE && lane == 0) local_sh.n_list = n;
+                }
                 sync();
+                if (SHARE) n = local_sh.n_list;
             }
             W* sorted = reinterpret_cast<W*>(slots);                                      // the maxima are done with
             order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);
-            if (tw == 0) emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
+            if (tw == 0) {
+                // NaN logits reach no bound: a row with fewer than K others is filled up with candidate 0 at weight 0
+                for (int i = n + lane; i < K; i += 32) sorted[i] = order_word<W>(kKeyNegInf, 0);
+                __syncwarp();
+                emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
+            }
         }
         if (lane == 0 && wfirst == 0) {
             const float lse = lmax + logf(sum_all);

@@ -1081,3 +1081,45 @@ def test_adaptive_depth_does_not_depend_on_the_call(dev, V):
             buf[off:off + V] = lg[i]
             assert depths(ctx, buf[off:off + V].view(1, V), tok[i:i + 1])[0] == batch[i], (i, off)
         ctx.close()
+
+
+@pytest.mark.parametrize("N,V,K", [(1, 128256, 64), (40, 33000, 100), (9, 300, 128), (12, 37, 5), (5000, 2001, 64), (6, 70000, 256), (7, 8200, 300)])
+def test_rows_with_nan_logits_stay_inside_the_vocabulary(dev, orc, N, V, K):
+    """NaN logits are outside the contract, but every selected index is one of the vocabulary and the other rows of
+    the call are what they are without them: rows of NaNs only (of every kind), of fewer than K other logits, of
+    NaNs among ordinary logits, and a whole encode and decode over such rows."""
+    rng = np.random.default_rng(V)
+    lg = (rng.standard_normal((N, V)) * 2.5).astype(np.float16)
+    bits = lg.view(np.uint16)
+    kinds = [0x7e00, 0xfe00, 0x7c01, 0xffff, 0x7fff]
+    bad = np.arange(0, N, 3)
+    for j, i in enumerate(bad):
+        if j % 3 == 0:
+            bits[i] = kinds[(j // 3) % 5]
+        elif j % 3 == 1:
+            bits[i, K // 2:] = kinds[j % 5]
+        else:
+            bits[i, rng.random(V) < 0.3] = kinds[j % 5]
+    good = np.setdiff1d(np.arange(N), bad)
+    tok = rng.integers(0, V, N).astype(np.int32)
+    ctx = plc.Context(torch.ones(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02, chunk_pos=16)
+    lgd = torch.from_numpy(lg).to(dev)
+    out = ctx.topk_softmax(lgd, torch.from_numpy(tok).to(dev))
+    assert ctx.sync_status() == plc.OK
+    idx = out["idx"].cpu().numpy()
+    assert idx.min() >= 0 and idx.max() < V
+    if len(good):
+        want, w, lse, _, _ = orc.topk_softmax(lg[good], tok[good], K)
+        assert np.array_equal(idx[good], want)
+        np.testing.assert_allclose(out["w"].cpu().numpy()[good], w, rtol=2e-5, atol=1e-9)
+        np.testing.assert_allclose(out["lse"].cpu().numpy()[good], lse, atol=2e-5)
+    n = min(N, 64)
+    kv = torch.randn(1, 2, 1, 1, n, 32, device=dev).half()
+    st = plc.StreamSet(ctx.W, ctx.max_chunks(n), 1 << 22, dev)
+    ctx.encode(kv, lgd[:n].view(1, n, V), st)
+    res = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+    ctx.decode(st, lgd[:n].view(1, n, V), res)
+    assert ctx.sync_status() == plc.OK
+    ok = torch.from_numpy(good[good < n]).to(dev)
+    if len(ok):
+        assert float((res - kv.float())[..., ok, :].abs().max()) <= 0.01 + 1e-3
