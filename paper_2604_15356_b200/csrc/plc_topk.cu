@@ -469,12 +469,32 @@ __device__ __forceinline__ uint4 group_across(const RowView& r, int v) {
     const uint4* p = reinterpret_cast<const uint4*>(r.row + (8 * v - r.phase));
     const uint4 lo = p[0], hi = p[1];
     w[0] = lo.x; w[1] = lo.y; w[2] = lo.z; w[3] = lo.w; w[4] = hi.x; w[5] = hi.y; w[6] = hi.z; w[7] = hi.w;
-#pragma unroll
-    for (int i = 0; i < 7; ++i) w[i] = (r.phase & 2) ? w[i + 1] : w[i];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) w[i] = (r.phase & 4) ? w[i + 2] : w[i];
     const uint32_t sh = (r.phase & 1) ? 16u : 0u;
-    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh), __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+    auto at = [&](int i) { return make_uint4(__funnelshift_r(w[i], w[i + 1], sh), __funnelshift_r(w[i + 1], w[i + 2], sh),
+                                             __funnelshift_r(w[i + 2], w[i + 3], sh), __funnelshift_r(w[i + 3], w[i + 4], sh)); };
+    return r.phase < 4 ? (r.phase < 2 ? at(0) : at(1)) : (r.phase < 6 ? at(2) : at(3));
+}
+// Four groups that lie `step` apart, all with both their vectors inside the row: the phase, the same in all
+// lanes, is looked at once.
+__device__ __forceinline__ void groups_across(const RowView& r, int v, int step, uint4 (&q)[4]) {
+    const uint4* p = reinterpret_cast<const uint4*>(r.row + (8 * v - r.phase));
+    const uint32_t sh = (r.phase & 1) ? 16u : 0u;
+    auto fetch = [&](auto word) {
+        constexpr int A = decltype(word)::value;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint4 lo = p[u * step], hi = p[u * step + 1];
+            const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+            q[u] = make_uint4(__funnelshift_r(w[A], w[A + 1], sh), __funnelshift_r(w[A + 1], w[A + 2], sh),
+                              __funnelshift_r(w[A + 2], w[A + 3], sh), __funnelshift_r(w[A + 3], w[A + 4], sh));
+        }
+    };
+    switch (r.phase >> 1) {
+        case 0: fetch(std::integral_constant<int, 0>{}); break;
+        case 1: fetch(std::integral_constant<int, 1>{}); break;
+        case 2: fetch(std::integral_constant<int, 2>{}); break;
+        default: fetch(std::integral_constant<int, 3>{});
+    }
 }
 // The ends of the row as groups -1 (lane 0: the head) and nv (lane 1: the tail) of 8, kNoValue where the
 // row is not.
@@ -655,7 +675,8 @@ __device__ __forceinline__ T* at_first_block(T* p) {
 // log-sum-exp, so a batch encoded at once and restored a session at a time must find the same bits.  The
 // row is cut into parts of its own (row_parts), a warp takes one after another, and groups are counted
 // from the row's first logit.
-template <bool SELECT, bool SHARE, bool FIXED, class W>
+// (1: all rows start on a 16-byte boundary; 2: any rows; the same sums.)
+template <bool SELECT, bool SHARE, int FIXED, class W>
 __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const TopkArgs a) {
     extern __shared__ __align__(16) unsigned char stream_raw[];
     __shared__ StreamShared local_sh;
@@ -686,8 +707,8 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
     const long long stride = SHARE ? gridDim.x / blocks : (long long)gridDim.x * nwarps;
 
     for (long long rowi = next_row(a, group, stride); rowi < a.N; rowi = next_row(a, rowi + stride, stride)) {
-        const RowView r = row_view<FIXED>(a.logits + rowi * (long long)a.V, a.V);
-        auto fetch = [&](int v) { return FIXED && r.phase ? group_across(r, v) : ldg_stream(r.body + v); };
+        const RowView r = row_view<FIXED != 0>(a.logits + rowi * (long long)a.V, a.V);
+        auto fetch = [&](int v) { return FIXED == 2 && r.phase ? group_across(r, v) : ldg_stream(r.body + v); };
         const int per = kBatch * 32 * NW, batches = max(1, (r.nv + per - 1) / per);
         // Slots of this warp: one a group of 8 where all the row's fit, else one for every `wide` batches.
         const bool fine = NW * batches * kBatch <= kSlots;
@@ -698,9 +719,11 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
         float ref = 0.f, sum_all = 0.f;
         auto load = [&](int w, int t, uint4 (&q)[kBatch]) {                               // group u of batch t of part w
             const int at = w * 32 + lane + t * per;
-            if ((t + 1) * per <= r.nv) {
+            if (FIXED == 2 && r.phase && w + t > 0 && (t + 1) * per < r.nv) {
+                groups_across(r, at, 32 * NW, q);
+            } else if ((FIXED != 2 || !r.phase) && (t + 1) * per <= r.nv) {
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) q[u] = fetch(at + u * 32 * NW);
+                for (int u = 0; u < kBatch; ++u) q[u] = ldg_stream(r.body + at + u * 32 * NW);
             } else {
 #pragma unroll
                 for (int u = 0; u < kBatch; ++u) q[u] = at + u * 32 * NW < r.nv ? fetch(at + u * 32 * NW) : all4(kNegInf2);
@@ -774,31 +797,36 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                 group2 = hmax2_bits(group2, top4);
                 if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = wide; }
             };
-            if (SELECT && (fine || FIXED)) {
+            if (FIXED == 2 || (SELECT && fine)) {
 #pragma unroll 1
                 for (int t = 0; t < batches; ++t) {
                     const uint32_t top4 = batch(cur, top);
-                    if (FIXED && !fine) filled(top4);
+                    if (FIXED == 2 && !fine) filled(top4);
 #pragma unroll
                     for (int u = 0; u < kBatch; ++u) {
-                        if (!FIXED || fine) put_slot(t * kBatch + u, top[u]);
+                        if (FIXED != 2 || fine) put_slot(t * kBatch + u, top[u]);
                         cur[u] = nxt[u];
                     }
                     if (FIXED) load_next(nxt);
                     else load(wrow, t + 2, nxt);
                 }
-                if (FIXED && !fine && left != wide) put_slot(slot, group2);
+                if (FIXED == 2 && !fine && left != wide) put_slot(slot, group2);
             } else {
 #pragma unroll 1
                 for (int t = 0; t < batches; t += 2) {
                     const uint32_t t0 = batch(cur, top);
                     if (SELECT) filled(t0);
-                    load(wrow, t + 2, cur);
+                    if (FIXED) load_next(cur);
+                    else load(wrow, t + 2, cur);
                     if (t + 1 < batches) {
                         const uint32_t t1 = batch(nxt, top);
                         if (SELECT) filled(t1);
+                        if (FIXED) load_next(nxt);
+                    } else if (FIXED) {                                                       // the next part begins with what lies in nxt
+#pragma unroll
+                        for (int u = 0; u < kBatch; ++u) { const uint4 q = cur[u]; cur[u] = nxt[u]; nxt[u] = q; }
                     }
-                    load(wrow, t + 3, nxt);
+                    if (!FIXED) load(wrow, t + 3, nxt);
                 }
                 if (SELECT && left != wide) put_slot(slot, group2);
             }
@@ -923,7 +951,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
                             const int v = vb + u * 32 * NW;
-                            q[u] = mine && v < r.nv && !(fine && u) ? (FIXED && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
+                            q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
                         }
                         if (i0 < 0) q[0] = row_ends(r, lane);
                         uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
@@ -982,7 +1010,7 @@ static int row_parts(int V) {
     return n;
 }
 
-template <bool SELECT, bool FIXED, class W>
+template <bool SELECT, int FIXED, class W>
 static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st) {
     // Warps a row, in powers of two, each with at least 1024 logits of its own; one when rows alone fill the
     // GPU.  Up to a block of eight: as many as the GPU holds for all rows (32 a SM).  Up to four blocks (a
@@ -1012,16 +1040,18 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool select = a.pairs || a.idx || a.w || a.zk;
-    if (!select) return launch_stream<false, false, uint32_t>(a, sms, st);
+    if (!select) return launch_stream<false, 0, uint32_t>(a, sms, st);
+    const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     if (a.K <= kFinal) {
-        if (a.step_exp || a.bits_out)
-            return a.V <= 65536 ? launch_stream<true, true, uint32_t>(a, sms, st) : launch_stream<true, true, unsigned long long>(a, sms, st);
-        return a.V <= 65536 ? launch_stream<true, false, uint32_t>(a, sms, st) : launch_stream<true, false, unsigned long long>(a, sms, st);
+        const int fixed = !(a.step_exp || a.bits_out) ? 0 : vec ? 1 : 2;
+        if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st)
+                               : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st) : launch_stream<true, 2, uint32_t>(a, sms, st);
+        return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st)
+             : fixed == 1 ? launch_stream<true, 1, unsigned long long>(a, sms, st) : launch_stream<true, 2, unsigned long long>(a, sms, st);
     }
     // The second pass over a row should find it in L2: rows of up to 128 KB are read by 256 threads
     // with five blocks per SM, longer rows by 512 threads with two blocks per SM (two, so that one
     // block streams while the other sits at the barrier between its passes).
-    const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     const bool wide = (long long)a.V * 2 > 128 * 1024;
     auto launch = [&](auto kern, int threads, int cap) {
         int occ = 1;
