@@ -340,8 +340,9 @@ plc_status plc_topk_softmax(plc_ctx* c, const void* logits_dev, const int32_t* t
     a.logits = static_cast<const __half*>(logits_dev); a.tokens = tokens_dev; a.N = N;
     a.V = c->cfg.vocab; a.K = c->cfg.top_k;
     a.idx = idx_dev; a.w = w_dev; a.lse = lse_dev; a.zk = zk_dev; a.logp2 = logp2_dev;
-    a.n_per_session = 1;
-    return launch_topk(a, static_cast<cudaStream_t>(stream)) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
+    a.n_per_session = 1; a.chained = true;
+    int few = 0;
+    return launch_topk(a, static_cast<cudaStream_t>(stream), &few) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
 }
 
 plc_status plc_prefix_dedup(plc_ctx* c, const int32_t* tokens_dev, const int32_t* lens_dev, const float* logp2_dev,
@@ -362,21 +363,22 @@ plc_status plc_prefix_clusters(plc_ctx* c, const int32_t* lcp_dev, const float* 
                                   static_cast<cudaStream_t>(stream)) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
 }
 
+// `chained`: the launch ahead is this context's own and short (append steps); *few: see launch_topk.
 static plc_status run_topk_for(plc_ctx* c, const void* logits_dev, int S, int n, const int32_t* pb, const int32_t* pe,
-                               cudaStream_t st, const int32_t* tokens = nullptr, int32_t* bits_out = nullptr) {
+                               cudaStream_t st, bool chained, int* few, const int32_t* tokens = nullptr, int32_t* bits_out = nullptr) {
     plc_status rc = ensure_pairs(c, (long long)S * n);
     if (rc) return rc;
     TopkArgs a{};
     a.logits = static_cast<const __half*>(logits_dev); a.N = (long long)S * n; a.V = c->cfg.vocab; a.K = c->cfg.top_k;
     a.pairs = c->pairs; a.Kp = padded_k(c->cfg); a.n_per_session = n; a.pos_begin = pb; a.pos_end = pe;
-    a.tickets = c->ticket;
+    a.tickets = c->ticket; a.chained = chained;
     a.pair_mul = pair_index(c->cfg) ? 1 : c->cfg.head_dim * 2;
     for (a.pair_rows = 0; (c->cfg.head_dim << a.pair_rows) < 256; ++a.pair_rows) {}
     if (tokens) {
         a.tokens = tokens; a.step_exp = c->step_exp; a.bits_out = bits_out;
         a.b0 = c->cfg.adaptive_b0; a.extra = c->cfg.adaptive_extra; a.hbar = c->cfg.adaptive_hbar;
     }
-    return launch_topk(a, st) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
+    return launch_topk(a, st, few) == cudaSuccess ? PLC_OK : PLC_E_CUDA;
 }
 
 // Dense variant: softmax once, then per group of layers the bf16 contraction and the coding of its tables.
@@ -451,7 +453,7 @@ static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* log
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, true, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, true, st);
-    rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, tokens_dev, dbg ? dbg->bits_dev : nullptr);
+    rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, false, &a.behind, tokens_dev, dbg ? dbg->bits_dev : nullptr);
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
@@ -496,7 +498,7 @@ static plc_status decode_impl(plc_ctx* c, const plc_streams* in, const void* log
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, false, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, false, st);
-    rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, tokens_dev, dbg ? dbg->bits_dev : nullptr);
+    rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, false, &a.behind, tokens_dev, dbg ? dbg->bits_dev : nullptr);
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
@@ -550,7 +552,8 @@ static plc_status rotq_impl(plc_ctx* c, const plc_kv_view* kv, int elem_bytes, c
     const int mc = (n + cp - 1) / cp;
     if ((long long)W * S * mc >= (1ll << 32)) return PLC_E_SHAPE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    rc = run_topk_for(c, logits_dev, S, n, pb, pe, st);
+    int few = 0;
+    rc = run_topk_for(c, logits_dev, S, n, pb, pe, st, false, &few);
     if (rc) return rc;
     CodecArgs a = base_args(c);
     a.kv = to_dev(kv); a.S = S; a.n = n; a.pos_begin = pb; a.pos_end = pe; a.pairs = c->pairs;
@@ -633,9 +636,13 @@ plc_status plc_append_step(plc_ctx* c, plc_session_batch* sb, const void* kv_ste
         if (rc) return rc;
         if (cudaEventRecord(c->side_ev[1], c->side_stream) != cudaSuccess) return PLC_E_CUDA;
     }
-    rc = run_topk_for(c, logits_step_dev, sb->B, 1, nullptr, nullptr, st);
+    // Both kernels of a step are short and chained while rows are few (one session, V = 128256: 24.9 -> 22.0 us a
+    // step; 3000 sessions, a warp a row: 349 -> 366, and not).
+    int few = 0;
+    rc = run_topk_for(c, logits_step_dev, sb->B, 1, nullptr, nullptr, st, true, &few);
     if (rc) return rc;
     CodecArgs a = base_args(c);
+    a.behind = few;
     const size_t per_buf = (size_t)n_streams * CP;
     const int chunk = sb->steps / CP;
     a.kv = KvView{const_cast<void*>(kv_step_dev), 2 * B * H * d, B * H * d, H * d, d, 0};

@@ -55,9 +55,8 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
     constexpr bool FROM_OPEN = SRC == kSrcOpen;
     constexpr bool DENSE = SRC == kSrcDense;
     __shared__ EncTables tb;
-    chain_next();
+    if (FROM_OPEN) chain_next();                             // an append step's first launch may follow
     load_tables(&tb, &a.tables->enc);
-    chain_wait();
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -197,9 +196,7 @@ template <int D, bool DENSE, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
 __global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     __shared__ DecTables tb;
-    chain_next();
     load_tables(&tb, &a.tables->dec);
-    chain_wait();
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
@@ -336,8 +333,6 @@ __device__ __forceinline__ void hadamard(float (&v)[Geo<D>::G], int lane) {
 template <int D, bool ENC>
 __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
     constexpr int G = Geo<D>::G;
-    chain_next();
-    chain_wait();
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp, B = rq.bits;
     int2* sp0 = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
@@ -556,7 +551,7 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
         count_launch();
-        return launch_chained(kern, sm_count() * blocks, kThreads, sm, st, 1, a);
+        return launch_kernel(kern, sm_count() * blocks, kThreads, sm, st, false, 1, a);
     });
 }
 
@@ -605,7 +600,7 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
         count_launch();
-        return launch_chained(kern, sm_count() * blocks, kThreads, sm, st, 1, a);
+        return launch_kernel(kern, sm_count() * blocks, kThreads, sm, st, false, 1, a);
     });
 }
 
@@ -618,7 +613,7 @@ cudaError_t launch_rotq(const CodecArgs& a0, const RotqArgs& r, bool encode, cud
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
         count_launch();
-        return launch_chained(kern, sm_count() * kGatherBlocks, kThreads, sm, st, 1, a, r);
+        return launch_kernel(kern, sm_count() * kGatherBlocks, kThreads, sm, st, false, 1, a, r);
     });
 }
 
@@ -635,7 +630,7 @@ cudaError_t launch_append_quantise(const CodecArgs& a, cudaStream_t st) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kThreads, sm) != cudaSuccess || occ < 1) occ = 1;
         if (blocks > (long long)sm_count() * occ) blocks = (long long)sm_count() * occ;
         count_launch();
-        return launch_chained(kern, (unsigned)blocks, kThreads, sm, st, 1, a);
+        return launch_kernel(kern, (unsigned)blocks, kThreads, sm, st, a.behind > 0, 1, a);
     });
 }
 

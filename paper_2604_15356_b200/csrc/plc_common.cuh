@@ -89,26 +89,36 @@ __host__ __device__ inline void class_params(int q, int& s, int& qp) {
 }
 
 #ifdef __CUDACC__
-// Programmatic dependent launch: a kernel launched with launch_chained may start before the kernel ahead of
+// Programmatic dependent launch: a kernel launched with `chained` set may start before the kernel ahead of
 // it in the stream has finished; it calls chain_wait before it touches anything another kernel wrote or
 // still reads, and chain_next as soon as its own successor may be started.  What it saves is the launch
-// gap between the short kernels of a call (3 to 4 us each).
+// gap between short kernels (1 to 3 us).  What it can cost: blocks that become resident beside those of the
+// kernel ahead take over their SM's division of L1 and shared memory for as long as they run (the coder
+// behind a top-K of many rows, which holds up to 213 KB of shared memory an SM: 64 sessions' tails, rows from
+// HBM, 18.3 -> 29.0 ms), and crowd on the SMs that are free first (128 chunks, a block each: 355 -> 447 us).
+// So a kernel is chained only where neither can happen: see launch_coop and plc_append_step's launches.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
-inline cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, unsigned cluster, A... args) {
+inline cudaError_t launch_kernel(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, bool chained, unsigned cluster,
+                                 A... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[2]{};
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    if (chained) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = cluster;
+        at[cfg.numAttrs].val.clusterDim.y = at[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -161,8 +171,10 @@ struct TopkArgs {
     int n_per_session; const int32_t* pos_begin; const int32_t* pos_end;
     int parts;              // parts of a row where its sum must not depend on the call (set by the launcher)
     unsigned int* tickets;  // kTicketWords work counters that the launch zeroes for the kernel behind it, or null
+    bool chained;           // where rows are few, the launch may start while the kernel ahead of it ends
 };
-cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st);
+// *few_blocks: the blocks launched where rows are few (several warps a row, little shared memory), else 0.
+cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks);
 
 cudaError_t launch_prefix_dedup(const int32_t* tokens, const int32_t* lens, const float* logp2, int S, int64_t stride,
                                 int32_t* lcp, float* dT, int32_t* parent, int32_t* shared_len, cudaStream_t st);
@@ -207,6 +219,7 @@ struct CodecArgs {
     StreamsDev st; DebugDev dbg;
     uint16_t* staging; unsigned long long staging_words_per_warp;   // encoder scratch
     unsigned int* ticket;                          // kTicketWords work counters (zeroed by the top-K launch, or by the launcher where none precedes)
+    int behind;                                    // blocks of the top-K launch ahead that this one may be chained to, or 0
     int sched_nq, sched_g;                         // gather kernels: work queues, SMs that share one (set by the launcher)
     unsigned int* status; Counters* counters;
     // dense variant: prediction read from buffers; one launch covers tables [dense_t0, dense_t0 + dense_nt)

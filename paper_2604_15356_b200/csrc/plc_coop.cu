@@ -475,7 +475,6 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
     int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
     const LaneCode lc = lane_code(lane);
-    chain_next();
     load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->wide));
     chain_wait();
     const int Wl = DENSE ? a.dense_nt : 2 * a.sh.L * a.sh.H;
@@ -542,8 +541,10 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         int occ = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem) != cudaSuccess || occ < 1) occ = 1;
         const long long blocks = std::min<long long>(items, (long long)sm_count() * occ);
+        // chained where its blocks and the top-K's fit beside each other, a block an SM
+        const bool chained = a.behind > 0 && a.behind + blocks <= sm_count();
         count_launch();
-        return launch_chained(kern, (unsigned)blocks, warps * 32, smem, st, 1, a);
+        return launch_kernel(kern, (unsigned)blocks, warps * 32, smem, st, chained, 1, a);
     });
 }
 

@@ -1011,7 +1011,7 @@ static int row_parts(int V) {
 }
 
 template <bool SELECT, int FIXED, class W>
-static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st) {
+static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st, int* few_blocks) {
     // Warps a row, in powers of two, each with at least 1024 logits of its own; one when rows alone fill the
     // GPU.  Up to a block of eight: as many as the GPU holds for all rows (32 a SM).  Up to four blocks (a
     // cluster): only while that is a quarter of the GPU, since a cluster's blocks are placed together
@@ -1030,24 +1030,27 @@ static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st) {
     int occ = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, per_block * 32, smem) != cudaSuccess || occ < 1) occ = 1;
     const long long want = share ? a.N * cluster : (a.N + per_block - 1) / per_block;
+    const unsigned blocks = (unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster);
+    *few_blocks = share ? (int)blocks : 0;
     count_launch();
-    return launch_chained(kern, (unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster), per_block * 32, smem, st, cluster, a);
+    return launch_kernel(kern, blocks, per_block * 32, smem, st, a.chained && share, cluster, a);
 }
 
-cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
+cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
+    *few_blocks = 0;
     if (a.N <= 0) return cudaSuccess;
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool select = a.pairs || a.idx || a.w || a.zk;
-    if (!select) return launch_stream<false, 0, uint32_t>(a, sms, st);
+    if (!select) return launch_stream<false, 0, uint32_t>(a, sms, st, few_blocks);
     const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     if (a.K <= kFinal) {
         const int fixed = !(a.step_exp || a.bits_out) ? 0 : vec ? 1 : 2;
-        if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st)
-                               : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st) : launch_stream<true, 2, uint32_t>(a, sms, st);
-        return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st)
-             : fixed == 1 ? launch_stream<true, 1, unsigned long long>(a, sms, st) : launch_stream<true, 2, unsigned long long>(a, sms, st);
+        if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st, few_blocks)
+                               : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st, few_blocks) : launch_stream<true, 2, uint32_t>(a, sms, st, few_blocks);
+        return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st, few_blocks)
+             : fixed == 1 ? launch_stream<true, 1, unsigned long long>(a, sms, st, few_blocks) : launch_stream<true, 2, unsigned long long>(a, sms, st, few_blocks);
     }
     // The second pass over a row should find it in L2: rows of up to 128 KB are read by 256 threads
     // with five blocks per SM, longer rows by 512 threads with two blocks per SM (two, so that one
@@ -1058,8 +1061,10 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0) != cudaSuccess || occ < 1) occ = 1;
         const long long per_sm = occ < cap ? occ : cap;       // the rows in flight stay within L2
         const long long blocks = a.N < sms * per_sm ? a.N : sms * per_sm;
+        const bool few = a.N <= sms;
+        *few_blocks = few ? (int)blocks : 0;
         count_launch();
-        return launch_chained(kern, (unsigned)blocks, threads, 0, st, 1, a);
+        return launch_kernel(kern, (unsigned)blocks, threads, 0, st, a.chained && few, 1, a);
     };
     if (wide) return vec ? launch(topk_softmax_kernel<true, 512>, 512, 2) : launch(topk_softmax_kernel<false, 512>, 512, 2);
     return vec ? launch(topk_softmax_kernel<true, 256>, 256, 5) : launch(topk_softmax_kernel<false, 256>, 256, 5);
