@@ -449,7 +449,7 @@ static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* log
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     CodecArgs a = base_args(c);
     a.kv = to_dev(kv); a.S = S; a.n = n; a.pos_begin = pos_begin_dev; a.pos_end = pos_end_dev;
-    a.st = to_dev(out);
+    a.st = to_dev(out); a.chunks = need;
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, true, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, true, st);
@@ -494,7 +494,7 @@ static plc_status decode_impl(plc_ctx* c, const plc_streams* in, const void* log
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     CodecArgs a = base_args(c);
     a.kv = to_dev(kv_out); a.S = S; a.n = n; a.pos_begin = pos_begin_dev; a.pos_end = pos_end_dev;
-    a.st = to_dev(in);
+    a.st = to_dev(in); a.chunks = need;
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, false, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, false, st);
@@ -557,7 +557,7 @@ static plc_status rotq_impl(plc_ctx* c, const plc_kv_view* kv, int elem_bytes, c
     if (rc) return rc;
     CodecArgs a = base_args(c);
     a.kv = to_dev(kv); a.S = S; a.n = n; a.pos_begin = pb; a.pos_end = pe; a.pairs = c->pairs;
-    a.st.max_chunks = mc; a.sh.chunk_pos = cp;
+    a.chunks = mc; a.sh.chunk_pos = cp;
     RotqArgs r{};
     r.bits = p->bits; r.rec_words = rotq_words(c, p->bits);
     for (int i = 0; i < 8; ++i) r.sign_bits[i] = p->sign_bits[i];

@@ -66,14 +66,15 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp;
     int2* sp0 = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
     const int Wl = DENSE ? a.dense_nt : Wt;                  // tables this launch covers
-    const unsigned total = FROM_OPEN ? a.open_items : (unsigned)Wl * a.S * a.st.max_chunks;
+    const unsigned total = FROM_OPEN ? a.open_items : (unsigned)Wl * a.S * a.chunks;
+    if (!FROM_OPEN) clear_unused_slots(a, DENSE ? a.dense_t0 : 0, Wl);
     const float inv_d = 1.0f / D, inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2,
                 floor2 = a.sh.sigma_floor * a.sh.sigma_floor;
     const int c0 = first_comp<D>(lane);
 
     constexpr bool QUEUED = SRC == kSrcGather;
     QueueCursor qc = QUEUED ? queue_of_this_sm(a) : QueueCursor{0, 0};
-    const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks;
     auto next = [&]() { return QUEUED ? next_queued(a, qc, per_table, Wl, lane) : next_ticket(a.ticket, lane); };
     for (unsigned item = next(); item < total; item = next()) {
         Item it;
@@ -203,13 +204,13 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArg
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp;
     int2* sp0 = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
     const int Wl = DENSE ? a.dense_nt : Wt;
-    const unsigned total = (unsigned)Wl * a.S * a.st.max_chunks;
+    const unsigned total = (unsigned)Wl * a.S * a.chunks;
     const float inv_d = 1.0f / D, delta = a.sh.delta, inv_delta2 = a.sh.inv_delta2,
                 floor2 = a.sh.sigma_floor * a.sh.sigma_floor;
     const int c0 = first_comp<D>(lane);
 
     QueueCursor qc = DENSE ? QueueCursor{0, 0} : queue_of_this_sm(a);
-    const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks;
     auto next = [&]() { return DENSE ? next_ticket(a.ticket, lane) : next_queued(a, qc, per_table, Wl, lane); };
     for (unsigned item = next(); item < total; item = next()) {
         const Item it = bulk_item(a, item, DENSE ? a.dense_t0 : 0);
@@ -336,14 +337,14 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp, B = rq.bits;
     int2* sp0 = g_pair_smem + (threadIdx.x >> 5) * 2 * Kp;
-    const unsigned total = (unsigned)Wt * a.S * a.st.max_chunks;
+    const unsigned total = (unsigned)Wt * a.S * a.chunks;
     const float inv_d = 1.0f / D, half_levels = 0.5f * (float)(1 << B), cell = 2.0f / (float)(1 << B);
     const int c0 = first_comp<D>(lane);
     float sgn[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) sgn[g] = (rq.sign_bits[(c0 + g) >> 5] >> ((c0 + g) & 31)) & 1u ? -1.0f : 1.0f;
     QueueCursor qc = queue_of_this_sm(a);
-    const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks;
     for (unsigned item = next_queued(a, qc, per_table, Wt, lane); item < total; item = next_queued(a, qc, per_table, Wt, lane)) {
         const Item it = bulk_item(a, item);
         if (it.P <= 0) continue;
@@ -477,7 +478,7 @@ static void set_queues(CodecArgs& a, int n_tables, int items_per_sm = kQueueItem
 // warp's own chain is what the call waits for; above it the kernels here do more work per instruction
 // (65536 chunks: 12.6 ms a layer group against 11.3).
 static bool use_coop(const CodecArgs& a) {
-    const long long items = (long long)(a.mu_dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
+    const long long items = (long long)(a.mu_dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.chunks;
     return items <= (long long)sm_count() * kWarpsPerBlock * (a.mu_dense ? kBlocksPerSM : kGatherBlocks);
 }
 constexpr int kCoopItems = 4;                    // chunks an SM works on at a time there
@@ -496,7 +497,7 @@ void codec_schedule(const CodecArgs& a0, int n_tables, int* nq, int* g) {
 
 static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
     const int sms = sm_count(), warps_per_sm = items_per_sm;
-    const long long per_table = std::max(1LL, (long long)a.S * a.st.max_chunks);
+    const long long per_table = std::max(1LL, (long long)a.S * a.chunks);
     const long long spanned = ((long long)sms * warps_per_sm + per_table - 1) / per_table + 1;
     const double table_bytes = 2.0 * a.sh.V * a.sh.d;
     int dev = 0, l2 = 0;

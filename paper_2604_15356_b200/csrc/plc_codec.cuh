@@ -292,20 +292,31 @@ struct Item {
 
 __device__ __forceinline__ Item bulk_item(const CodecArgs& a, unsigned item, int t_first = 0) {
     Item it;
-    const int MC = a.st.max_chunks;
-    const unsigned per_table = (unsigned)a.S * (unsigned)MC;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks;
     it.t = t_first + (int)(item / per_table);
     unsigned r = item % per_table;
-    it.s = (int)(r / MC);
-    it.c = (int)(r % MC);
+    it.s = (int)(r / a.chunks);
+    it.c = (int)(r % a.chunks);
     const int Wt = 2 * a.sh.L * a.sh.H;
-    it.slot = ((long long)it.s * Wt + it.t) * MC + it.c;
+    it.slot = ((long long)it.s * Wt + it.t) * a.st.max_chunks + it.c;
     int b = a.pos_begin ? a.pos_begin[it.s] : 0, e = a.pos_end ? a.pos_end[it.s] : a.n;
     b = max(b, 0); e = min(e, a.n);
     long long p0 = (long long)b + (long long)it.c * a.sh.chunk_pos;
     it.p0 = (int)min(p0, (long long)a.n);
     it.P = p0 < e ? min(a.sh.chunk_pos, e - (int)p0) : 0;
     return it;
+}
+
+// Encoders rewrite the whole index of the launch's tables: the entries behind the chunks that a session of
+// this call can have, by the whole grid.
+__device__ __forceinline__ void clear_unused_slots(const CodecArgs& a, int t_first, int n_tables) {
+    const int room = a.st.max_chunks - a.chunks, Wt = 2 * a.sh.L * a.sh.H;
+    const long long total = (long long)a.S * n_tables * room;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const long long stream = i / room;
+        const long long slot = (stream / n_tables * Wt + t_first + stream % n_tables) * a.st.max_chunks + a.chunks + i % room;
+        a.st.chunk_offset[slot] = 0; a.st.chunk_bytes[slot] = 0;
+    }
 }
 
 __device__ __forceinline__ long long kv_elem(const KvView& v, int t, int H, int s, int pos) {

@@ -216,6 +216,7 @@ struct CodecArgs {
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
     KvView kv;                                     // encode: input f16; decode: output
     int S, n; const int32_t* pos_begin; const int32_t* pos_end;
+    int chunks;                                    // chunks a session of the call can have, ceil(n / chunk_pos): the unit of work; st.max_chunks is the room of the index
     StreamsDev st; DebugDev dbg;
     uint16_t* staging; unsigned long long staging_words_per_warp;   // encoder scratch
     unsigned int* ticket;                          // kTicketWords work counters (zeroed by the top-K launch, or by the launcher where none precedes)

@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
     load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->wide));
     chain_wait();
     const int Wl = DENSE ? a.dense_nt : 2 * a.sh.L * a.sh.H;
-    const unsigned per_table = (unsigned)a.S * (unsigned)a.st.max_chunks, total = (unsigned)Wl * per_table;
+    const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks, total = (unsigned)Wl * per_table;
+    if (ENC) clear_unused_slots(a, DENSE ? a.dense_t0 : 0, Wl);
     QueueCursor qc = DENSE ? QueueCursor{0, 0} : queue_of_this_sm(a);
 
     for (;;) {
@@ -525,7 +526,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
     return dispatch_d(a.sh.d, [&](auto D) {
         constexpr int d = decltype(D)::value;
         const bool dense = a.mu_dense != nullptr;
-        const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.st.max_chunks;
+        const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.chunks;
         // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
         // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  A block of sixteen where
         // there is a chunk an SM at most.

@@ -1123,3 +1123,29 @@ def test_rows_with_nan_logits_stay_inside_the_vocabulary(dev, orc, N, V, K):
     ok = torch.from_numpy(good[good < n]).to(dev)
     if len(ok):
         assert float((res - kv.float())[..., ok, :].abs().max()) <= 0.01 + 1e-3
+
+
+@pytest.mark.parametrize("kind,S,n", [("topk", 1, 200), ("topk", 8, 1300), ("dense", 2, 100)])
+def test_index_with_room_to_grow(dev, kind, S, n):
+    """An index larger than the call needs: the work and its layout are those of the chunks that exist (few chunks
+    take a block each whatever the room), the chunks are the same, and the entries behind them are rewritten to 0."""
+    L, H, d, V, K, CP, delta = 2, 4, 64, 1000, 24, 32, 0.02
+    tokens, logits, T, kv = make_workload(900 + S, S, n, L, H, d, V, K)
+    ctx = plc.Context(T.to(dev), K, delta, chunk_pos=CP, variant=plc.PRED_DENSE if kind == "dense" else plc.PRED_TOPK)
+    W, need = ctx.W, ctx.max_chunks(n)
+    kvd, lgd = kv.to(dev), logits.to(dev)
+    seen = []
+    for mc in (need, need + 3, 40 * need):
+        st = plc.StreamSet(S * W, mc, S * W * need * 160 + 3 * S * n * W * d, dev)
+        st.chunk_offset.fill_(77); st.chunk_bytes.fill_(77)
+        ctx.encode(kvd, lgd, st)
+        out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+        ctx.decode(st, lgd, out)
+        assert ctx.sync_status() == plc.OK
+        assert float((out - kvd.float()).abs().max()) <= delta / 2 + 1e-3
+        nb, off = st.chunk_bytes.view(S * W, mc), st.chunk_offset.view(S * W, mc)
+        assert not nb[:, need:].any() and not off[:, need:].any() and (nb[:, :need] >= 128).all()
+        seen.append((nb[:, :need].clone(), ctx.last_schedule() if kind == "topk" else None,
+                     [st.chunk((S * W - 1) * mc + c).tobytes() for c in range(need)]))
+    for s_ in seen[1:]:
+        assert torch.equal(s_[0], seen[0][0]) and s_[1:] == seen[0][1:]
