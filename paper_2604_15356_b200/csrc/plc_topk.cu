@@ -515,59 +515,110 @@ __device__ __forceinline__ uint4 row_ends(const RowView& r, int lane) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Exact selection by one warp reading the row from memory: bisection of the K-th largest key between `lo`
-// (at least K logits reach it) and the maximum by counting passes, then the K elements, equal keys in
-// index order, into the list (packed); returns how many there are.  For rows whose ties overflow the lists.
-template <class W>
-__device__ __noinline__ int slow_select(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, int lane) {
+// Logits of a group that reach h2 (one value in both halves): bits p and 16 + p, the halves of word p.
+__device__ __forceinline__ uint32_t reach_mask(const uint4& q, uint32_t h2) {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+    uint32_t m = 0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) m |= __hge2_mask(as_half2(w[p]), as_half2(h2)) & (0x10001u << p);
+    return m;
+}
+
+struct CountShared {                                // of the warps that select a row together
+    int count[3], eq[kStreamWarps], n;
+};
+// Exact selection by counting passes over the row in memory, by the warps of a row's first block (SHARE) or
+// one warp: bisection of the K-th largest key between `lo` (at least K logits reach it) and the maximum, then
+// the K elements, equal keys in index order, into the list (packed); returns how many there are.  For rows
+// whose ties overflow the lists (few finite logits, quantised logits) and rows with few more groups than
+// K.  A pass costs ten instructions per 8 logits; NaN reaches nothing.
+template <bool SHARE, class W>
+__device__ __noinline__ int select_by_count(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, CountShared& sh, int tw, int tws,
+                                            int lane) {
     const RowView r = row_view(row, V);
-    const uint32_t lt = lanemask_lt();
     const uint4 ends = row_ends(r, lane);
-    auto key_at = [&](const uint4& q, int j) { const uint32_t h = half_at(q, j); return (h & 0x7fffu) > 0x7c00u ? 0u : key_of(h); };   // NaN: no value, 0
-    auto count = [&](uint32_t t) {
-        int c = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) c += key_at(ends, j) >= t;
-#pragma unroll 2
-        for (int v = lane; v < r.nv; v += 32) {
-            const uint4 q = r.body[v];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) c += key_at(q, j) >= t;
+    auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
+    if (SHARE) {
+        if (tw == 0 && lane < 3) sh.count[lane] = 0;
+        if (tw == 0 && lane == 0) sh.n = 0;
+        __syncthreads();
+    }
+    int phase = 0;
+    auto count = [&](uint32_t key) {
+        const uint32_t h2 = bits_of_key(key) * 0x10001u;
+        int c = tw == 0 ? __popc(reach_mask(ends, h2)) : 0;
+#pragma unroll 4
+        for (int v = tw * 32 + lane; v < r.nv; v += 32 * tws) c += __popc(reach_mask(r.body[v], h2));
+        c = __reduce_add_sync(kFull, c);
+        if (SHARE) {                                                     // three counters in turn: the one read last is zeroed for the pass after the next
+            if (lane == 0) atomicAdd(&sh.count[phase], c);
+            __syncthreads();
+            c = sh.count[phase];
+            phase = phase == 2 ? 0 : phase + 1;
+            if (tw == 0 && lane == 0) sh.count[phase == 2 ? 0 : phase + 1] = 0;
         }
-        return (int)__reduce_add_sync(kFull, c);
+        return c;
     };
     uint32_t hi = kmax + 1;                                              // nothing reaches it
+    int at_lo = -1, at_hi = 0;                                           // logits that reach lo (-1: not counted), hi
 #pragma unroll 1
     for (bool first = true; hi - lo > 1; first = false) {
         const uint32_t mid = first ? lo + 1 : lo + ((hi - lo) >> 1);     // most often the bound itself is the key
-        if (count(mid) >= K) lo = mid; else hi = mid;
+        const int c = count(mid);
+        if (c >= K) { lo = mid; at_lo = c; } else { hi = mid; at_hi = c; }
     }
-    int need = K - count(lo + 1), n = 0;
-    const int last = (r.nv + 31) >> 5;
-#pragma unroll 1
-    for (int s = -1; s <= last; ++s) {                                   // head, body, tail: index order over the lanes
-        const int v = s < 0 ? -1 : s < last ? s * 32 + lane : r.nv;
-        const bool body = s >= 0 && s < last;
-        const bool have = body ? v < r.nv : lane == (s < 0 ? 0 : 1);
-        const uint4 q = !have ? all4(kNoValue2) : body ? r.body[v] : ends;
-        int eq = 0, all;
+    const uint32_t ge2 = bits_of_key(lo) * 0x10001u, gt2 = bits_of_key(lo + 1) * 0x10001u;   // hi = lo + 1 (past +inf: a NaN, which nothing reaches)
+    const int need = K - at_hi;                                          // of those equal to lo, in index order
+    const bool ranked = at_lo != K;                                      // else all of them
+    // a warp takes consecutive groups, the first the head of the row, the last its tail
+    const int seg = ((r.nv + tws - 1) / tws + 31) & ~31, v0 = min(tw * seg, r.nv), v1 = min(v0 + seg, r.nv);
+    int before = 0, n = 0;                                               // equal ones ahead; elements written (not SHARE)
+    if (SHARE && ranked) {
+        int e = tw == 0 && lane == 0 ? __popc(reach_mask(ends, ge2) & ~reach_mask(ends, gt2)) : 0;
+#pragma unroll 4
+        for (int v = v0 + lane; v < v1; v += 32) { const uint4 q = r.body[v]; e += __popc(reach_mask(q, ge2) & ~reach_mask(q, gt2)); }
+        e = __reduce_add_sync(kFull, e);
+        if (lane == 0) sh.eq[tw] = e;
+        __syncthreads();
+        for (int w = 0; w < tw; ++w) before += sh.eq[w];
+    }
+    auto take = [&](const uint4& q, int v) {                             // a group a lane, in index order over the lanes
+        const uint32_t ge = reach_mask(q, ge2);
+        if (!__any_sync(kFull, ge != 0)) return;
+        uint32_t got = reach_mask(q, gt2), eq = ge & ~got;
+        if (ranked) {
+            int all;
+            int rank = before + warp_excl_scan(__popc(eq), lane, all);
+            before += all;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) eq += key_at(q, j) == lo;
-        int before = warp_excl_scan(eq, lane, all);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const uint32_t key = key_at(q, j);
-            const bool ok = key > lo || (key == lo && before < need);
-            before += key == lo;
-            const uint32_t m = __ballot_sync(kFull, ok);
-            const int at = n + __popc(m & lt);
-            if (ok && at < K) list[at] = order_word<W>(key, r.head + 8 * v + j);
-            n += __popc(m);
+            for (int j = 0; j < 8; ++j) {                                // word j / 2, half j & 1: index order
+                const uint32_t bit = 1u << ((j >> 1) + 16 * (j & 1));
+                if (eq & bit) { if (rank < need) got |= bit; ++rank; }
+            }
+        } else {
+            got |= eq;
         }
-        need = max(0, need - all);
-    }
-    __syncwarp();
-    return min(n, K);
+        int all;
+        int at = warp_excl_scan(__popc(got), lane, all);
+        int base = n;
+        if (SHARE) {
+            if (lane == 0) base = atomicAdd(&sh.n, all);
+            base = __shfl_sync(kFull, base, 0);
+        }
+        n += all; at += base;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (got & (1u << ((j >> 1) + 16 * (j & 1)))) {
+                if (at < K) list[at] = order_word<W>(key_of(half_at(q, j)), r.head + 8 * v + j);
+                ++at;
+            }
+    };
+    if (tw == 0 && r.head > 0) take(lane == 0 ? ends : all4(kNoValue2), -1);
+#pragma unroll 1
+    for (int v = v0; v < v1; v += 32) take(v + lane < v1 ? r.body[v + lane] : all4(kNoValue2), v + lane);
+    if (tw == tws - 1) take(lane == 1 ? ends : all4(kNoValue2), r.nv);
+    sync();
+    return min(SHARE ? sh.n : n, K);
 }
 
 // Orders a list of n words into `sorted`: a word's place is the number of larger ones, which the team's
@@ -632,6 +683,7 @@ struct StreamShared {                               // of the warps that share a
     uint32_t key[kStreamWarps * kMaxCluster];
     int n_codes, n_list;                            // running totals of the end of the row, which the first block's warps share
     uint32_t theta;                                 // its bound
+    CountShared by_count;
 };
 static_assert(kStreamWarps * kMaxCluster <= 32, "a lane for every warp of a row");
 
@@ -862,124 +914,127 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             // The row's own warp, or all warps of the first block.
             const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
             auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
-            // The bound: the K-th largest group maximum (any value that exactly K of them reach will do), searched
-            // by one warp with all maxima in its registers.  The search is a chain of ten steps or so: shared among
-            // eight warps a step cost 1300 cycles (guards, a shared counter, a barrier), 14400 of the 34000 cycles of a
-            // row of 128256 logits by itself; now 5350 of 22000.
-            const int S = NW * ns, words = (S + 1) >> 1;
-            uint32_t mx[kSlots / 2];                                                      // two maxima each
+            // With three quarters as many selected as there are groups the bound holds back little: the logits are
+            // counted instead.
+            const bool few_groups = fine && 4 * K > 3 * r.nv;
             uint32_t theta = kKeyNegInf;
-            if (tw == 0) {
-                if (S & 1) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
-                __syncwarp();
+            int n = 0;
+            bool counted = few_groups;
+            if (!few_groups) {
+                // The bound: the K-th largest group maximum (any value that exactly K of them reach will do), searched
+                // by one warp with all maxima in its registers.  The search is a chain of ten steps or so: shared among
+                // eight warps a step cost 1300 cycles (guards, a shared counter, a barrier), 14400 of the 34000 cycles of a
+                // row of 128256 logits by itself; now 5350 of 22000.
+                const int S = NW * ns, words = (S + 1) >> 1;
+                uint32_t mx[kSlots / 2];                                                      // two maxima each
+                if (tw == 0) {
+                    if (S & 1) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
+                    __syncwarp();
 #pragma unroll
-                for (int i = 0; i < kSlots / 2; ++i) mx[i] = i < words ? slots[i * 32 + lane] : kNoValue2;
-                auto reach = [&](uint32_t h2, auto first) {                               // of this lane's first words
-                    constexpr int A = SHARE ? 4 : 1;                                      // one sum where other rows fill the gaps
-                    __half2 c[A];
+                    for (int i = 0; i < kSlots / 2; ++i) mx[i] = i < words ? slots[i * 32 + lane] : kNoValue2;
+                    auto reach = [&](uint32_t h2, auto first) {                               // of this lane's first words
+                        constexpr int A = SHARE ? 4 : 1;                                      // one sum where other rows fill the gaps
+                        __half2 c[A];
 #pragma unroll
-                    for (int i = 0; i < A; ++i) c[i] = __float2half2_rn(0.f);
+                        for (int i = 0; i < A; ++i) c[i] = __float2half2_rn(0.f);
 #pragma unroll
-                    for (int i = 0; i < decltype(first)::value; ++i) c[i % A] = __hadd2(c[i % A], __hge2(as_half2(mx[i]), as_half2(h2)));
-                    if constexpr (A > 1) c[0] = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
-                    return __half2int_rn(__hadd(__low2half(c[0]), __high2half(c[0])));
+                        for (int i = 0; i < decltype(first)::value; ++i) c[i % A] = __hadd2(c[i % A], __hge2(as_half2(mx[i]), as_half2(h2)));
+                        if constexpr (A > 1) c[0] = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
+                        return __half2int_rn(__hadd(__low2half(c[0]), __high2half(c[0])));
+                    };
+                    uint32_t hi = kmax + 1, down = 256;                                       // first downwards from the maximum, then between
+#pragma unroll 1
+                    while (hi - theta > 1) {
+                        const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
+                        const int c = __reduce_add_sync(kFull, words <= 8 ? reach(h2, std::integral_constant<int, 8>{})
+                                                                          : reach(h2, std::integral_constant<int, kSlots / 2>{}));
+                        if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
+                        if (c == K) break;
+                    }
+                    if (SHARE && lane == 0) local_sh.theta = theta;
+                }
+                sync();
+                if (SHARE) theta = local_sh.theta;
+                // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
+                auto place = [&](int mine, int* shared_total, int& total) {
+                    int all;
+                    int at = warp_excl_scan(mine, lane, all);
+                    int base = total;
+                    if (SHARE) {
+                        if (lane == 0) base = atomicAdd(shared_total, all);
+                        base = __shfl_sync(kFull, base, 0);
+                    }
+                    total += all;                                                             // SHARE: of this warp only
+                    return base + at;
                 };
-                uint32_t hi = kmax + 1, down = 256;                                       // first downwards from the maximum, then between
-#pragma unroll 1
-                while (hi - theta > 1) {
-                    const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
-                    const int c = __reduce_add_sync(kFull, words <= 8 ? reach(h2, std::integral_constant<int, 8>{})
-                                                                      : reach(h2, std::integral_constant<int, kSlots / 2>{}));
-                    if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
-                    if (c == K) break;
-                }
-                if (SHARE && lane == 0) local_sh.theta = theta;
-            }
-            sync();
-            if (SHARE) theta = local_sh.theta;
-            // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
-            auto place = [&](int mine, int* shared_total, int& total) {
-                int all;
-                int at = warp_excl_scan(mine, lane, all);
-                int base = total;
-                if (SHARE) {
-                    if (lane == 0) base = atomicAdd(shared_total, all);
-                    base = __shfl_sync(kFull, base, 0);
-                }
-                total += all;                                                             // SHARE: of this warp only
-                return base + at;
-            };
-            // The groups that reach it.
-            const uint32_t th2 = bits_of_key(theta) * 0x10001u;
-            int n_codes = 0, n = 0;
-            uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
-            auto hit = [&](uint32_t w, int i) { return __hge2_mask(as_half2(w), as_half2(th2)) & (0x10001u << (i & 15)); };
-            if (SHARE) {                                                                  // two warps at least: 16 words at most
+                // The groups that reach it.
+                const uint32_t th2 = bits_of_key(theta) * 0x10001u;
+                int n_codes = 0;
+                uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
+                auto hit = [&](uint32_t w, int i) { return __hge2_mask(as_half2(w), as_half2(th2)) & (0x10001u << (i & 15)); };
+                if (SHARE) {                                                                  // two warps at least: 16 words at most
 #pragma unroll 4
-                for (int i = 0; tw + i * tws < words; ++i) hits[0] |= hit(slots[(tw + i * tws) * 32 + lane], i);
-            } else {
+                    for (int i = 0; tw + i * tws < words; ++i) hits[0] |= hit(slots[(tw + i * tws) * 32 + lane], i);
+                } else {
 #pragma unroll
-                for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= hit(mx[i], i);
-            }
-            int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.n_codes, n_codes);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                for (uint32_t m = hits[h]; m; m &= m - 1) {
-                    const int b = __ffs(m) - 1, i = tw + (16 * h + (b & 15)) * tws;
-                    if (at < kCodes) codes[at] = (uint16_t)((2 * i + (b >> 4)) * 32 + lane);
-                    ++at;
+                    for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= hit(mx[i], i);
                 }
-            sync();
-            if (SHARE) n_codes = local_sh.n_codes;
-            if (n_codes <= kCodes) {
-                // their logits at or above the bound; head and tail of the row are a turn of the last warp's own.  A
-                // lane takes one batch of a group where warps share the row (turns are memory latencies: 1700 cycles
-                // each), else all of a group (where rows fill the GPU the lanes' divisions cost more than a turn).
-                const int steps = fine ? 1 : wide, items = SHARE ? n_codes * steps : n_codes;
-                const bool ends_turn = tw == tws - 1 && (r.head > 0 || r.head + 8 * r.nv < r.V);
+                int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.n_codes, n_codes);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    for (uint32_t m = hits[h]; m; m &= m - 1) {
+                        const int b = __ffs(m) - 1, i = tw + (16 * h + (b & 15)) * tws;
+                        if (at < kCodes) codes[at] = (uint16_t)((2 * i + (b >> 4)) * 32 + lane);
+                        ++at;
+                    }
+                sync();
+                if (SHARE) n_codes = local_sh.n_codes;
+                if (n_codes <= kCodes) {
+                    // their logits at or above the bound; head and tail of the row are a turn of the last warp's own.  A
+                    // lane takes one batch of a group where warps share the row (turns are memory latencies: 1700 cycles
+                    // each), else all of a group (where rows fill the GPU the lanes' divisions cost more than a turn).
+                    const int steps = fine ? 1 : wide, items = SHARE ? n_codes * steps : n_codes;
+                    const bool ends_turn = tw == tws - 1 && (r.head > 0 || r.head + 8 * r.nv < r.V);
 #pragma unroll 1
-                for (int i0 = tw * 32 - (ends_turn ? 32 * tws : 0); i0 < items; i0 += 32 * tws) {
-                    const bool mine = i0 >= 0 && i0 + lane < items;
-                    const int ci = !mine ? 0 : SHARE ? (i0 + lane) / steps : i0 + lane, first = SHARE && mine ? i0 + lane - ci * steps : 0;
-                    const int code = mine ? codes[ci] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
-                    const int turns = SHARE || i0 < 0 ? 1 : steps;
+                    for (int i0 = tw * 32 - (ends_turn ? 32 * tws : 0); i0 < items; i0 += 32 * tws) {
+                        const bool mine = i0 >= 0 && i0 + lane < items;
+                        const int ci = !mine ? 0 : SHARE ? (i0 + lane) / steps : i0 + lane, first = SHARE && mine ? i0 + lane - ci * steps : 0;
+                        const int code = mine ? codes[ci] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
+                        const int turns = SHARE || i0 < 0 ? 1 : steps;
 #pragma unroll 1
-                    for (int st = first; st < first + turns; ++st) {
-                        const int t = fine ? ls >> 2 : ls * wide + st;
-                        const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
-                        uint4 q[kBatch];
+                        for (int st = first; st < first + turns; ++st) {
+                            const int t = fine ? ls >> 2 : ls * wide + st;
+                            const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
+                            uint4 q[kBatch];
 #pragma unroll
-                        for (int u = 0; u < kBatch; ++u) {
-                            const int v = vb + u * 32 * NW;
-                            q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
-                        }
-                        if (i0 < 0) q[0] = row_ends(r, lane);
-                        uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
+                            for (int u = 0; u < kBatch; ++u) {
+                                const int v = vb + u * 32 * NW;
+                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
+                            }
+                            if (i0 < 0) q[0] = row_ends(r, lane);
+                            uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
 #pragma unroll
-                        for (int u = 0; u < kBatch; ++u) {
-                            const uint32_t w4[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+                            for (int u = 0; u < kBatch; ++u) {
+                                const uint32_t w4[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
-                        }
-                        for (int to = place(__popc(m), &local_sh.n_list, n); m; m &= m - 1, ++to) {
-                            const int b = __ffs(m) - 1, u = (b >> 2) & 3;
-                            const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
-                            const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
-                            if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(__ldg(r.row + e))), e);   // a first-level hit
+                                for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
+                            }
+                            for (int to = place(__popc(m), &local_sh.n_list, n); m; m &= m - 1, ++to) {
+                                const int b = __ffs(m) - 1, u = (b >> 2) & 3;
+                                const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
+                                const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
+                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(__ldg(r.row + e))), e);   // a first-level hit
+                            }
                         }
                     }
                 }
-            }
-            sync();
-            if (SHARE) n = local_sh.n_list;
-            if (n_codes > kCodes || n > kListCap) {
-                sync();                                                                   // all have read the total
-                if (tw == 0) {
-                    n = slow_select<W>(r.row, r.V, K, theta, kmax, list, lane);
-                    if (SHARE && lane == 0) local_sh.n_list = n;
-                }
                 sync();
                 if (SHARE) n = local_sh.n_list;
+                counted = n_codes > kCodes || n > kListCap;
+            }
+            if (counted) {
+                sync();                                                                   // all have read the totals
+                n = select_by_count<SHARE, W>(r.row, r.V, K, theta, kmax, list, local_sh.by_count, tw, tws, lane);
             }
             W* sorted = reinterpret_cast<W*>(slots);                                      // the maxima are done with
             order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);

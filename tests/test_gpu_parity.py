@@ -1149,3 +1149,41 @@ def test_index_with_room_to_grow(dev, kind, S, n):
                      [st.chunk((S * W - 1) * mc + c).tobytes() for c in range(need)]))
     for s_ in seen[1:]:
         assert torch.equal(s_[0], seen[0][0]) and s_[1:] == seen[0][1:]
+
+
+@pytest.mark.parametrize("N,V,K,off", [(1, 128256, 64, 0), (700, 128257, 64, 0), (1, 32000, 128, 3), (60, 33001, 100, 1), (5000, 4099, 64, 0),
+                                       (64, 256, 64, 0), (5000, 256, 64, 5), (64, 777, 128, 0), (64, 1024, 128, 0), (33, 129, 128, 2),
+                                       (9, 128, 128, 0), (4800, 37, 5, 1), (6, 9, 9, 3), (3, 262144, 64, 0)])
+def test_topk_rows_selected_by_counting(dev, orc, N, V, K, off):
+    """Rows that no bound from group maxima narrows down: fewer finite logits than K, equal logits, few values that
+    repeat, ties across the K-th place, few groups for K; a warp, a block or a cluster a row, rows on and off
+    16-byte boundaries.  The selection is exact: order, indices and weights are the oracle's."""
+    rng = np.random.default_rng(N * 7 + V)
+    lg = (rng.standard_normal((N, V)) * 2.5).astype(np.float16)
+    for i in range(0, N, 2):
+        k = (i // 2) % 6
+        if k == 0:
+            lg[i, rng.permutation(V)[max(1, K // 2):]] = -np.inf
+        elif k == 1:
+            lg[i] = np.float16(1.5)
+        elif k == 2:
+            lg[i] = np.float16(rng.integers(-2, 3)) * (rng.random(V) < 0.5)          # two values, +0 and -0 among them
+        elif k == 3:
+            lg[i] = np.round(lg[i].astype(np.float32))
+        elif k == 4:
+            lg[i, :] = np.float16(-65504.0); lg[i, V // 3] = np.float16(20.0)        # one logit, the rest the lowest value (the maximum is moderate: l_max log2(e) is rounded to binary32, which moves Z_k by |l_max| 2^-24)
+        else:
+            lg[i] = np.sort(lg[i]); lg[i, -max(1, K // 3):] = lg[i, -1]
+    tok = rng.integers(0, V, N).astype(np.int32)
+    buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
+    rows = buf[off:off + N * V].view(N, V)
+    rows.copy_(torch.from_numpy(lg))
+    ctx = plc.Context(torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02)
+    out = ctx.topk_softmax(rows, torch.from_numpy(tok).to(dev))
+    assert ctx.sync_status() == plc.OK
+    some = np.unique(np.concatenate([np.arange(min(N, 40)), rng.integers(0, N, 60), [N - 1]]))
+    idx, w, lse, zk, _ = orc.topk_softmax(lg[some], tok[some], K)
+    assert np.array_equal(out["idx"].cpu().numpy()[some], idx)
+    np.testing.assert_allclose(out["w"].cpu().numpy()[some], w, rtol=2e-5, atol=1e-9)
+    np.testing.assert_allclose(out["lse"].cpu().numpy()[some], lse, atol=2e-5, rtol=1e-6)
+    np.testing.assert_allclose(out["zk"].cpu().numpy()[some], zk, rtol=2e-5)
