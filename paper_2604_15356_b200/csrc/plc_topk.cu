@@ -2,9 +2,10 @@
 // ascending, -0 = +0).
 //
 // K <= 128, and calls that ask for no selected set (only lse / log2 P): topk_stream_kernel, which reads
-// a row once, any alignment (see there).  K > 128: topk_softmax_kernel, one block a row: a 4096-bin
-// histogram of the order-preserving 16-bit key finds the bin that holds the K-th largest, a 16-way
-// refinement finds the key itself, and equal keys are taken in index order.
+// a row once, any alignment (see there).  K > 128: topk_softmax_kernel, one block a row: thread maxima bound
+// the K-th logit where K allows it; else a 4096-bin histogram of the order-preserving 16-bit key finds the
+// bin that holds the K-th largest, a 16-way refinement finds the key itself, and equal keys are taken in
+// index order.
 // Reductions use warp shuffles in a fixed order, so results are bit-reproducible from run to run.
 #include <algorithm>
 #include <type_traits>
@@ -39,10 +40,10 @@ struct __align__(16) Smem {
     uint32_t cand_key[kCandCap];
     int32_t cand_idx[kCandCap];
     float ek[kCandCap];
-    uint32_t red_k[THREADS / 32];
+    uint32_t red_k[THREADS / 32], red_t[THREADS / 32];
     float red_s[THREADS / 32];
     int scan[THREADS / 32];
-    int nsel, ncand, bstar, count_above, cstar, thr, need, neq, running;
+    int nsel, ncand, bstar, count_above, cstar, thr, need, neq, running, nlist, nhit;
     float sum_k;
 };
 
@@ -289,6 +290,11 @@ __device__ __forceinline__ void zero_tickets(const TopkArgs& a) {
         for (int i = threadIdx.x; i < kTicketWords; i += blockDim.x) a.tickets[i] = 0u;
 }
 
+// K > 128: a block a row, two passes over it.  The first takes a maximum per thread.  Where a warp's share of K
+// is at most half of its lanes (K <= 256 with 16 warps: rows of more than 65536 logits) the per_warp-th largest
+// of a warp's maxima, the smallest over the warps, bounds the K-th logit from below; the second pass, the
+// sum, then notes the groups of 8 that reach it, and their logits, a few more than K, are sorted.
+// Otherwise, and where ties overflow the list, select_by_histogram reads the row again.
 template <bool VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     constexpr int NW = THREADS / 32;
@@ -296,6 +302,10 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int V = a.V, K = a.K;
     const int ntiles = (V + THREADS * 8 - 1) / (THREADS * 8);
+    const int per_warp = (K + NW - 1) / NW;
+    const bool bounded = per_warp <= 16;
+    unsigned long long* list = reinterpret_cast<unsigned long long*>(sm.hist);           // idle until the histograms
+    static_assert(kCandCap * sizeof(unsigned long long) <= sizeof(sm.hist), "the list lives there");
     chain_next();
     chain_wait();
     zero_tickets(a);
@@ -306,29 +316,120 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
             if (i < b || i >= e) continue;
         }
         const __half* row = a.logits + rowi * (long long)V;
+        if (tid == 0) { sm.nlist = 0; sm.nhit = 0; }
         // Pass 0 (HBM): the maximum.
         uint32_t tkey = 0;
-        for (int t = 0; t < ntiles; ++t)
-            for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { tkey = max(tkey, key_of(bits)); });
-        tkey = __reduce_max_sync(kFull, tkey);
-        if (lane == 0) sm.red_k[wid] = tkey;
+        if (VEC) {
+            uint32_t m2 = 0xfc00fc00u;                               // (-inf, -inf)
+#pragma unroll 4
+            for (int t = 0; t < ntiles; ++t) {
+                const int i0 = t * (THREADS * 8) + tid * 8;
+                if (i0 < V) {
+                    const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
+                    m2 = hmax2_bits(m2, hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w)));
+                }
+            }
+            if (tid * 8 < V) tkey = max(key_of(m2 & 0xffffu), key_of(m2 >> 16));
+        } else {
+            for (int t = 0; t < ntiles; ++t)
+                for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) {
+                    if ((bits & 0x7fffu) <= 0x7c00u) tkey = max(tkey, key_of(bits));       // not NaN, as above
+                });
+        }
+        const uint32_t wmax = __reduce_max_sync(kFull, tkey);
+        uint32_t wth = 0;
+        if (bounded) {
+            uint32_t v = tkey;
+            for (int r = 0; r < per_warp; ++r) {
+                wth = __reduce_max_sync(kFull, v);
+                const uint32_t eq = __ballot_sync(kFull, v == wth);
+                if (lane == __ffs(eq) - 1) v = 0;
+            }
+        }
+        if (lane == 0) { sm.red_k[wid] = wmax; sm.red_t[wid] = wth; }
         __syncthreads();
-        uint32_t km = sm.red_k[0];
+        uint32_t km = sm.red_k[0], theta = sm.red_t[0];
 #pragma unroll
-        for (int w = 1; w < NW; ++w) km = max(km, sm.red_k[w]);
-        const float lmax = val_of_key(km);
-        // Pass 1 (L2): sum of exp(l - l_max).
+        for (int w = 1; w < NW; ++w) { km = max(km, sm.red_k[w]); theta = min(theta, sm.red_t[w]); }
+        theta = max(theta, kKeyNegInf);
+        const float lmax = val_of_key(max(km, kKeyNegInf));
+        // Pass 1 (L2): sum of exp(l - l_max), and what reaches the bound.
         const float nb = -lmax * 1.44269504088896341f;
+        const uint32_t th2 = bits_of_key(theta) * 0x10001u;
         float s = 0.f;
-        for (int t = 0; t < ntiles; ++t)
-            for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { s += exp_rel(__half2float(__ushort_as_half((unsigned short)bits)), nb); });
+        if (VEC) {
+#pragma unroll 2
+            for (int t = 0; t < ntiles; ++t) {
+                const int i0 = t * (THREADS * 8) + tid * 8;
+                if (i0 < V) {
+                    const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
+                    const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
+                    const uint32_t top = hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&wds[j]));
+                        s += exp_rel(f.x, nb);
+                        s += exp_rel(f.y, nb);
+                    }
+                    // a group is only noted here (few lanes get here); the noted ones are taken apart after the pass
+                    if (bounded && __hge2_mask(*reinterpret_cast<const __half2*>(&top), *reinterpret_cast<const __half2*>(&th2))) {
+                        const int slot = atomicAdd(&sm.nhit, 1);
+                        if (slot < kCandCap) sm.sel_idx[slot] = i0;              // sel_idx is idle until the histograms
+                    }
+                }
+            }
+        } else {
+            for (int t = 0; t < ntiles; ++t)
+                for_tile<VEC, THREADS>(row, V, t, [&](int i, uint32_t bits) {
+                    s += exp_rel(__half2float(__ushort_as_half((unsigned short)bits)), nb);
+                    const uint32_t key = key_of(bits);
+                    if (bounded && key >= theta) {
+                        const int slot = atomicAdd(&sm.nlist, 1);
+                        if (slot < kCandCap) list[slot] = ((unsigned long long)key << 32) | (0xffffffffu - (uint32_t)i);
+                    }
+                });
+        }
         s = warp_sum(s);
         if (lane == 0) sm.red_s[wid] = s;
         __syncthreads();
         float sum_all = 0.f;
 #pragma unroll
         for (int w = 0; w < NW; ++w) sum_all += sm.red_s[w];
-        select_by_histogram<VEC, THREADS>(sm, row, V, K, ntiles);
+        if (VEC && bounded) {
+            const int nhit = sm.nhit;
+            for (int t = tid; t < min(nhit, kCandCap); t += THREADS) {
+                const int i0 = sm.sel_idx[t];
+                const uint4 r = *reinterpret_cast<const uint4*>(row + i0);
+                const uint32_t wds[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t ge = __hge2_mask(*reinterpret_cast<const __half2*>(&wds[j]), *reinterpret_cast<const __half2*>(&th2));
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        if ((ge >> (16 * h)) & 1u) {
+                            const int slot = atomicAdd(&sm.nlist, 1);
+                            if (slot < kCandCap) list[slot] = ((unsigned long long)key_of(wds[j] >> (16 * h)) << 32) | (0xffffffffu - (uint32_t)(i0 + 2 * j + h));
+                        }
+                }
+            }
+            if (tid == 0 && nhit > kCandCap) atomicAdd(&sm.nlist, kCandCap + 1);       // too many
+            __syncthreads();
+        }
+        const int nlist = sm.nlist;
+        if (bounded && nlist >= K && nlist <= kCandCap) {
+            int n_pad = 256;
+            while (n_pad < nlist) n_pad <<= 1;
+            for (int k = nlist + tid; k < n_pad; k += THREADS) list[k] = 0;              // orders after everything
+            __syncthreads();
+            bitonic_desc<THREADS>(list, n_pad);
+            for (int k = tid; k < K; k += THREADS) {
+                sm.cand_key[k] = (uint32_t)(list[k] >> 32); sm.cand_idx[k] = (int)(0xffffffffu - (uint32_t)list[k]);
+            }
+            __syncthreads();
+        } else {
+            __syncthreads();
+            select_by_histogram<VEC, THREADS>(sm, row, V, K, ntiles);
+        }
         for (int k = tid; k < K; k += THREADS) sm.ek[k] = expf(val_of_key(sm.cand_key[k]) - lmax);
         __syncthreads();
         if (wid == 0) {

@@ -1187,3 +1187,31 @@ def test_topk_rows_selected_by_counting(dev, orc, N, V, K, off):
     np.testing.assert_allclose(out["w"].cpu().numpy()[some], w, rtol=2e-5, atol=1e-9)
     np.testing.assert_allclose(out["lse"].cpu().numpy()[some], lse, atol=2e-5, rtol=1e-6)
     np.testing.assert_allclose(out["zk"].cpu().numpy()[some], zk, rtol=2e-5)
+
+
+@pytest.mark.parametrize("N,V,K,off", [(5, 100003, 200, 3), (3, 65544, 129, 0), (4, 128256, 256, 1), (400, 70000, 256, 0), (2, 128256, 257, 0),
+                                       (4, 40000, 256, 0), (3, 33001, 1024, 1)])
+def test_topk_of_more_than_128(dev, orc, N, V, K, off):
+    """K above 128: bounded by thread maxima (K <= 256 and rows of more than 65536 logits) or by histograms; rows
+    with ties across the K-th place, with fewer finite logits than K, sorted rows, aligned and not."""
+    rng = np.random.default_rng(V + K)
+    lg = (rng.standard_normal((N, V)) * 2.5).astype(np.float16)
+    lg[0] = np.round(lg[0].astype(np.float32) * 2) / 2
+    lg[1] = -np.sort(-lg[1])
+    if N > 2:
+        lg[2, K // 2:] = -np.inf
+    if N > 3:
+        lg[3] = np.float16(0.25)
+    tok = rng.integers(0, V, N).astype(np.int32)
+    buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
+    rows = buf[off:off + N * V].view(N, V)
+    rows.copy_(torch.from_numpy(lg))
+    ctx = plc.Context(torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02)
+    out = ctx.topk_softmax(rows, torch.from_numpy(tok).to(dev))
+    assert ctx.sync_status() == plc.OK
+    some = np.unique(np.concatenate([np.arange(min(N, 8)), rng.integers(0, N, 8)]))
+    idx, w, lse, zk, _ = orc.topk_softmax(lg[some], tok[some], K)
+    assert np.array_equal(out["idx"].cpu().numpy()[some], idx)
+    np.testing.assert_allclose(out["w"].cpu().numpy()[some], w, rtol=2e-5, atol=1e-9)
+    np.testing.assert_allclose(out["lse"].cpu().numpy()[some], lse, atol=2e-5, rtol=1e-6)
+    np.testing.assert_allclose(out["zk"].cpu().numpy()[some], zk, rtol=2e-5)
