@@ -482,7 +482,7 @@ constexpr int kMaxCluster = 4;
 
 __device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
     uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
 }
 __device__ __forceinline__ __half2 as_half2(uint32_t w) { return *reinterpret_cast<const __half2*>(&w); }
@@ -1110,7 +1110,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 #pragma unroll
                             for (int u = 0; u < kBatch; ++u) {
                                 const int v = vb + u * 32 * NW;
-                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : __ldg(r.body + v)) : all4(kNoValue2);
+                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : r.body[v]) : all4(kNoValue2);
                             }
                             if (i0 < 0) q[0] = row_ends(r, lane);
                             uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
@@ -1124,7 +1124,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                                 const int b = __ffs(m) - 1, u = (b >> 2) & 3;
                                 const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
                                 const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
-                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(__ldg(r.row + e))), e);   // a first-level hit
+                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(r.row[e])), e);   // a first-level hit
                             }
                         }
                     }
