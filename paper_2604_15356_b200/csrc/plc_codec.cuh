@@ -426,6 +426,20 @@ inline cudaError_t dispatch_d(int d, F&& f) {
     return cudaErrorInvalidValue;
 }
 
+// Lets a kernel take as much dynamic shared memory as a block of this device has beside the kernel's own static
+// share.  The limit belongs to the function, for all contexts and threads of the process: it is only ever
+// raised, always to the same value, so that no thread's launch falls between another's set and launch.
+template <class... P>
+cudaError_t allow_smem(void (*kern)(P...), size_t bytes) {
+    cudaFuncAttributes fa{};
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+    int dev = 0, most = 0;
+    cudaGetDevice(&dev);
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+}
+
 inline int sm_count() {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);

@@ -537,7 +537,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
                           : (encode ? coop_kernel<d, false, true, false> : coop_kernel<d, false, false, false>);
         const int warps = alone ? kCoopMaxWarps : kCoopMaxWarps / 2;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode, roomy);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
         int occ = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, smem) != cudaSuccess || occ < 1) occ = 1;

@@ -1215,3 +1215,34 @@ def test_topk_of_more_than_128(dev, orc, N, V, K, off):
     np.testing.assert_allclose(out["w"].cpu().numpy()[some], w, rtol=2e-5, atol=1e-9)
     np.testing.assert_allclose(out["lse"].cpu().numpy()[some], lse, atol=2e-5, rtol=1e-6)
     np.testing.assert_allclose(out["zk"].cpu().numpy()[some], zk, rtol=2e-5)
+
+
+def test_contexts_of_different_top_k_on_two_threads(dev):
+    """Two host threads, each with a context and a stream of its own; the two sizes of top_k need different amounts
+    of shared memory from the same kernels, and every launch of either succeeds."""
+    import threading
+    n, V, d, errors = 64, 2048, 64, []
+    tokens, logits, T, kv = make_workload(51, 1, n, 1, 2, d, V, 32)
+    Td, kvd, lgd = T.to(dev), kv.to(dev), logits.to(dev)
+    torch.cuda.synchronize()
+
+    def work(K):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                ctx = plc.Context(Td, K, 0.02, chunk_pos=16)
+                st = plc.StreamSet(ctx.W, ctx.max_chunks(n), 1 << 20, dev)
+                out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+                for _ in range(1500):
+                    st.total_bytes.zero_()
+                    ctx.encode(kvd, lgd, st)
+                    ctx.decode(st, lgd, out)
+                assert ctx.sync_status() == plc.OK
+                assert float((out - kvd.float()).abs().max()) <= 0.01 + 1e-3
+        except Exception as e:                                     # a thread's failure is the test's
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(K,)) for K in (32, 1024)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not errors, errors
