@@ -82,6 +82,7 @@ struct plc_ctx {
     uint8_t* model;                 // linear: E transposed, the candidate-norm table of every (layer, table), A (all bf16);
                                     // dense: the candidate-norm table and T transposed (bf16)
     size_t model_off[3];
+    int group_cap;                  // most layers a contraction forms at once (0: no limit): set when the memory for more was not to be had
     bool resident;                  // the model holds A / the transposed T of every layer (otherwise converted a layer at a time per call)
     int last_nq, last_g;            // work-queue layout of the most recent top-K encode / decode launch
     int profiling;                  // record events around the codec kernels
@@ -159,8 +160,11 @@ plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (c->pairs) cudaFree(c->pairs);
     if (c->step_exp) cudaFree(c->step_exp);
     c->pairs = nullptr; c->step_exp = nullptr; c->pairs_cap = 0;
-    if (cudaMalloc(&c->pairs, sizeof(int2) * (size_t)positions * padded_k(c->cfg)) != cudaSuccess) return PLC_E_CUDA;
-    if (cudaMalloc(&c->step_exp, sizeof(int) * (size_t)positions) != cudaSuccess) return PLC_E_CUDA;
+    if (cudaMalloc(&c->pairs, sizeof(int2) * (size_t)positions * padded_k(c->cfg)) != cudaSuccess ||
+        cudaMalloc(&c->step_exp, sizeof(int) * (size_t)positions) != cudaSuccess) {
+        cudaGetLastError();                     // the launches that follow ask for the last error
+        return PLC_E_CUDA;
+    }
     c->pairs_cap = positions;
     return PLC_OK;
 }
@@ -183,13 +187,19 @@ CodecArgs base_args(const plc_ctx* c) {
     return a;
 }
 
+int layer_group(const plc_ctx* c, long long rows, int ncols) {
+    if (!c->resident) return 1;
+    const int n = layers_per_group(c->cfg.n_layers, rows, ncols);
+    return c->group_cap > 0 ? std::min(n, c->group_cap) : n;
+}
+
 DenseShape dense_shape(const plc_ctx* c, long long rows) {
     DenseShape sh;
     sh.rows = rows; sh.V = c->cfg.vocab; sh.d = c->cfg.head_dim; sh.tables = 2 * c->cfg.n_kv_heads;
     sh.ldv = (sh.V + 63) / 64 * 64;
     sh.ncols = sh.tables * sh.d; sh.nt_all = c->cfg.n_layers * sh.tables;
     sh.resident = c->resident;
-    sh.group = sh.resident ? layers_per_group(c->cfg.n_layers, rows, sh.ncols) : 1;
+    sh.group = layer_group(c, rows, sh.ncols);
     return sh;
 }
 
@@ -199,7 +209,7 @@ LinearShape linear_shape(const plc_ctx* c, long long rows) {
     sh.ldv = (sh.V + 63) / 64 * 64;
     sh.ncols = sh.tables * sh.d; sh.nt_all = sh.L * sh.tables;
     sh.resident = c->resident;
-    sh.group = sh.resident ? layers_per_group(sh.L, rows, sh.ncols) : 1;
+    sh.group = layer_group(c, rows, sh.ncols);
     return sh;
 }
 
@@ -210,13 +220,39 @@ bool keep_weights(size_t bytes) {
     return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4;
 }
 
+// Builds a context's model with the kept weights where there is memory for them and for what building them
+// takes, else without.
+template <class Build>
+bool with_or_without_weights(plc_ctx* c, Build&& build) {
+    if (build()) return true;
+    if (!c->resident) return false;
+    cudaGetLastError();
+    if (c->model) cudaFree(c->model);
+    c->model = nullptr; c->resident = false;
+    return build();
+}
+
 plc_status ensure_scratch(plc_ctx* c, size_t need) {
     if (need <= c->dense_bytes) return PLC_OK;
     if (c->dense_scratch) cudaFree(c->dense_scratch);
     c->dense_scratch = nullptr; c->dense_bytes = 0;
-    if (cudaMalloc(&c->dense_scratch, need) != cudaSuccess) return PLC_E_CUDA;
+    if (cudaMalloc(&c->dense_scratch, need) != cudaSuccess) {
+        cudaGetLastError();                     // the launches that follow ask for the last error
+        c->dense_scratch = nullptr;
+        return PLC_E_CUDA;
+    }
     c->dense_bytes = need;
     return PLC_OK;
+}
+// Scratch of a dense or linear call; with fewer layers a contraction where the memory for a group's
+// predictions (up to 1 GB) is not there.
+template <class Shape>
+plc_status ensure_group_scratch(plc_ctx* c, Shape& sh, size_t* off, size_t (*bytes)(const Shape&, size_t*)) {
+    for (;;) {
+        const plc_status rc = ensure_scratch(c, bytes(sh, off));
+        if (rc == PLC_OK || sh.group == 1) return rc;
+        sh.group = c->group_cap = sh.group / 2;
+    }
 }
 
 StreamsDev to_dev(const plc_streams* s) {
@@ -294,18 +330,21 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
                           cudaDeviceSynchronize() == cudaSuccess;
     if (ok && T_dev && cfg->variant == PLC_PRED_DENSE) {     // operands of every layer, once
         c->resident = keep_weights((size_t)rows * cfg->head_dim * 2);
-        const DenseShape sh = dense_shape(c, 0);
-        ok = sh.nt_all <= 65536 && cudaMalloc(&c->model, dense_model_bytes(sh, c->model_off)) == cudaSuccess &&
-             dense_prepare(c->T, sh, c->model, c->model_off, 0) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+        ok = with_or_without_weights(c, [&]() {
+            const DenseShape sh = dense_shape(c, 0);
+            return sh.nt_all <= 65536 && cudaMalloc(&c->model, dense_model_bytes(sh, c->model_off)) == cudaSuccess &&
+                   dense_prepare(c->T, sh, c->model, c->model_off, 0) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+        });
     }
     if (ok && lin) {
         c->lin_E = static_cast<const __half*>(lin->E_dev); c->lin_A = static_cast<const __half*>(lin->A_dev);
         c->lin_c = static_cast<const __half*>(lin->c_dev); c->lin_dm = lin->d_model;
         c->resident = keep_weights((size_t)cfg->n_layers * 2 * cfg->n_kv_heads * cfg->head_dim * lin->d_model * 2);
-        const LinearShape sh = linear_shape(c, 0);
-        const size_t bytes = linear_model_bytes(sh, c->model_off);
-        ok = cudaMalloc(&c->model, bytes) == cudaSuccess &&
-             linear_prepare(c->lin_E, c->lin_A, c->lin_c, sh, c->model, c->model_off, c->status, 0) == cudaSuccess;
+        ok = with_or_without_weights(c, [&]() {
+            const LinearShape sh = linear_shape(c, 0);
+            return cudaMalloc(&c->model, linear_model_bytes(sh, c->model_off)) == cudaSuccess &&
+                   linear_prepare(c->lin_E, c->lin_A, c->lin_c, sh, c->model, c->model_off, c->status, 0) == cudaSuccess;
+        });
     }
     if (!ok) { plc_destroy(c); return PLC_E_CUDA; }
     *out = c;
@@ -383,10 +422,10 @@ static plc_status run_topk_for(plc_ctx* c, const void* logits_dev, int S, int n,
 
 // Dense variant: softmax once, then per group of layers the bf16 contraction and the coding of its tables.
 static plc_status run_dense(plc_ctx* c, CodecArgs a, const void* logits_dev, bool encode, cudaStream_t st) {
-    const DenseShape sh = dense_shape(c, (long long)a.S * a.n);
+    DenseShape sh = dense_shape(c, (long long)a.S * a.n);
     if (sh.tables > 256) return PLC_E_SHAPE;              // one norm column per table, at most 256 per layer
     size_t off[4];
-    plc_status rc = ensure_scratch(c, dense_scratch_bytes(sh, off));
+    plc_status rc = ensure_group_scratch(c, sh, off, dense_scratch_bytes);
     if (rc) return rc;
     if (dense_softmax(static_cast<const __half*>(logits_dev), sh, c->dense_scratch, off, st) != cudaSuccess) return PLC_E_CUDA;
     a.mu_dense = reinterpret_cast<const float*>(c->dense_scratch + off[2]);
@@ -408,9 +447,9 @@ static plc_status run_dense(plc_ctx* c, CodecArgs a, const void* logits_dev, boo
 
 // Linear-embedding variant (Sec. 7.1): Ebar and the variance term once, then per group of layers mu = Ebar A^T and the coding.
 static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bool encode, cudaStream_t st) {
-    const LinearShape sh = linear_shape(c, (long long)a.S * a.n);
+    LinearShape sh = linear_shape(c, (long long)a.S * a.n);
     size_t off[5];
-    plc_status rc = ensure_scratch(c, linear_scratch_bytes(sh, off));
+    plc_status rc = ensure_group_scratch(c, sh, off, linear_scratch_bytes);
     if (rc) return rc;
     if (linear_begin(static_cast<const __half*>(logits_dev), sh, c->model, c->model_off, c->dense_scratch, off, c->status, st) !=
         cudaSuccess) return PLC_E_CUDA;

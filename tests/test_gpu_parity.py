@@ -1246,3 +1246,42 @@ def test_contexts_of_different_top_k_on_two_threads(dev):
     [t.start() for t in threads]
     [t.join() for t in threads]
     assert not errors, errors
+
+
+@pytest.mark.parametrize("kind", ["dense", "linear"])
+def test_contraction_in_little_memory(dev, kind):
+    """A call whose layers' predictions do not all fit in the memory that is left forms fewer layers at a time and
+    gives the same chunks, and the calls after it work too."""
+    S, n, L, H, d, V, K, CP = 1, 2048, 8, 8, 128, 4096, 16, 64
+    tokens, logits, T, kv = make_workload(61, S, n, L, H, d, V, K)
+    if kind == "linear":
+        E, A, c = synth.make_linear_model(L, H, V, d, 128, 5)
+        kv = synth.make_kv_linear(E, A, c, tokens, 0.05, 6)
+        model = [t.to(dev) for t in (E, A, c)]
+        make = lambda: plc.Context.linear(*model, 0.02, chunk_pos=CP)
+    else:
+        Td = T.to(dev)
+        make = lambda: plc.Context(Td, K, 0.02, chunk_pos=CP, variant=plc.PRED_DENSE)
+    kvd, lgd = kv.to(dev), logits.to(dev)
+    sizes, hold = [], []
+    try:
+        for tight in (False, True):
+            ctx = make()
+            st = plc.StreamSet(ctx.W, ctx.max_chunks(n), 3 * n * ctx.W * d, dev)
+            if tight:
+                # P 16 MB, a layer's prediction 16 MB, all layers' 128 MB, the rest a few: leave 80 MB
+                torch.cuda.synchronize(); torch.cuda.empty_cache()
+                free = torch.cuda.mem_get_info()[0] - (80 << 20)
+                hold.append(torch.empty(free - (64 << 20), dtype=torch.uint8, device=dev))
+                while torch.cuda.mem_get_info()[0] > (82 << 20):
+                    hold.append(torch.empty(2 << 20, dtype=torch.uint8, device=dev))
+            for _ in range(2):
+                st.total_bytes.zero_()
+                ctx.encode(kvd, lgd, st)
+            assert ctx.sync_status() == plc.OK
+            sizes.append(st.chunk_bytes.clone())
+            ctx.close()
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+    assert torch.equal(sizes[0], sizes[1])
