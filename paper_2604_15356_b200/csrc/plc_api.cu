@@ -25,16 +25,19 @@ bool build_coder_tables(CoderTables* t) {
         t->dec.fc[id][kNumSym] = c[kNumSym] << 16;
         uint8_t* first = t->dec.first[id];
         memset(first, 0xff, sizeof(t->dec.first[id]));
-        int z = 0;
-        for (uint32_t slot = 0; slot < kProbM; ++slot) {               // r = 2^15 - slot falls: an interval's first slot comes first
-            while (c[z + 1] <= slot) ++z;
-            const uint32_t r = kProbM - slot;
-            int e = 0;
-            while ((r >> e) > 1) ++e;
-            const int at = e * 16 + (int)(((r << 4) >> e) - 16);
-            if (first[at] == 0xff) first[at] = (uint8_t)z;
-            if (z > first[at] + 1) return false;
-        }
+        // Interval (e, i): the r = 2^15 - slot with exponent e and top four mantissa bits i, i.e. r in
+        // [(16 + i) 2^e / 16, (17 + i) 2^e / 16); its first slot is the one of its largest r.
+        for (int e = 0; e <= kProbBits; ++e)
+            for (int i = 0; i < 16; ++i) {
+                const uint32_t r0 = (((16u + i) << e) + 15u) >> 4, r1 = std::min(((((17u + i) << e) + 15u) >> 4) - 1u, kProbM);
+                if (r0 > r1) continue;
+                int z0 = 0;                                            // symbol of the first slot
+                while (c[z0 + 1] <= kProbM - r1) ++z0;
+                int z1 = z0;                                           // and of the last
+                while (c[z1 + 1] <= kProbM - r0) ++z1;
+                first[e * 16 + i] = (uint8_t)z0;
+                if (z1 > z0 + 1) return false;
+            }
         if (id < kWideFrom) {
             memcpy(t->wide.first[id], first, sizeof(t->wide.first[id]));
             memcpy(t->wide.fc[id], t->dec.fc[id], sizeof(t->wide.fc[id]));
