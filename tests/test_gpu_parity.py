@@ -1285,3 +1285,57 @@ def test_contraction_in_little_memory(dev, kind):
         hold.clear()
         torch.cuda.empty_cache()
     assert torch.equal(sizes[0], sizes[1])
+
+
+@pytest.mark.parametrize("d,K,CP,n,kind", [(32, 40, 128, 500, "plain"), (64, 50, 128, 380, "ranges"), (128, 64, 200, 600, "escapes"),
+                                           (256, 33, 96, 290, "escapes"), (128, 64, 64, 200, "zero"), (64, 24, 256, 700, "adaptive"), (128, 48, 16, 200, "many")])
+def test_block_per_chunk_with_several_chunks_an_sm(dev, orc, d, K, CP, n, kind):
+    """Calls of more chunks than SMs and at most 32 an SM: a block of eight warps a chunk, several blocks an SM, the
+    small word ring.  Chunks several ring lengths long, blocks that code several chunks, position ranges, escapes,
+    the zero-rate rule, the adaptive step, more chunks than resident blocks."""
+    S, L, H, V = (10, 2, 4, 600) if kind == "many" else (6, 4, 2, 600)
+    delta = 0.02 if kind in ("zero", "adaptive", "many") else 1.0 / 512
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    tokens, logits, T, kv = make_workload(7000 + d + n, S, n, L, H, d, V, K, pp=10.0, sigma=0.2)
+    if kind in ("escapes", "zero"):
+        lg = logits.numpy().copy()
+        for i in range(0, n, 3):                                   # every third position: a point mass
+            for s in range(S):
+                lg[s, i] = np.float16(-40.0); lg[s, i, int(tokens[s, i])] = np.float16(40.0)
+        logits = torch.from_numpy(lg)
+    if kind not in ("zero", "adaptive"):
+        pb, pe = ([0, 1, 7, n // 2, n - 1, n], [n, n - 5, n, n, n, n]) if kind == "ranges" else (None, None)
+        g = gpu_encode(dev, T, kv, logits, K, delta, CP, pb, pe, capacity=9 * S * n * 2 * L * H * d + (1 << 20))
+        assert g["rc"] == plc.OK and sms < S * g["W"] * g["mc"] <= 32 * sms
+        if kind == "escapes":
+            assert g["ctx"].stats().n_escapes > 0
+        if kind == "many":
+            assert S * g["W"] * g["mc"] > 4 * sms                   # at most four such blocks are resident on an SM
+        check_against_oracle(orc, g, T, kv, logits, K, delta, CP, pb, pe)
+        gpu_decode_check(g, kv, delta, n, pb, pe)
+        return
+    # per-position step / skipped positions: the bitstream of what the call exports, and back
+    ad = (6, 4, math.log2(10.0)) if kind == "adaptive" else None
+    zero = 0.02 if kind == "zero" else 0.0
+    ctx = plc.Context(T.to(dev), K, delta, chunk_pos=CP, adaptive=ad, zero_rate_D=zero)
+    W, mc = ctx.W, ctx.max_chunks(n)
+    assert sms < S * W * mc <= 32 * sms
+    st = plc.StreamSet(S * W, mc, 4 * S * n * W * d + (1 << 20), dev)
+    sym = torch.zeros(S, n, W, d, dtype=torch.int32, device=dev)
+    q = torch.zeros(S, n, W, dtype=torch.int32, device=dev)
+    tk = tokens.to(dev) if ad else None
+    ctx.encode(kv.to(dev), logits.to(dev), st, debug=plc.DebugBuffers(sym.data_ptr(), q.data_ptr(), None), tokens=tk)
+    back, out = torch.zeros_like(sym), torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+    ctx.decode(st, logits.to(dev), out, debug=plc.DebugBuffers(back.data_ptr(), None, None), tokens=tk)
+    assert ctx.sync_status() == plc.OK and torch.equal(back, sym)
+    qlim = math.floor(4 * math.log2(zero / delta ** 2) - 0.5) if zero else -10 ** 6
+    sn, qn = sym.cpu().numpy(), q.cpu().numpy()
+    if kind == "zero":
+        assert 0 < ctx.stats().skipped_vectors < S * n * W and ctx.stats().skipped_vectors == (qn <= qlim).sum()
+    for s in range(S):
+        for t in range(0, W, 3):
+            for c in range(mc):
+                kept = qn[s, c * CP:(c + 1) * CP, t] > qlim
+                ref, _, _ = orc.rans_encode_chunk(np.ascontiguousarray(sn[s, c * CP:(c + 1) * CP, t][kept]),
+                                                  np.ascontiguousarray(qn[s, c * CP:(c + 1) * CP, t][kept]))
+                assert np.array_equal(st.chunk((s * W + t) * mc + c), ref), (s, t, c)
