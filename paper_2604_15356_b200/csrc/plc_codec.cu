@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_k
 template <class Kern>
 cudaError_t pair_smem_bytes(Kern kern, int Kp, size_t& bytes) {
     bytes = (size_t)kWarpsPerBlock * 2 * Kp * sizeof(int2);
-    return allow_smem(kern, bytes);
+    return bytes > 24 * 1024 ? allow_smem(kern, bytes) : cudaSuccess;
 }
 
 }  // namespace

@@ -426,18 +426,14 @@ inline cudaError_t dispatch_d(int d, F&& f) {
     return cudaErrorInvalidValue;
 }
 
-// Lets a kernel take as much dynamic shared memory as a block of this device has beside the kernel's own static
-// share.  The limit belongs to the function, for all contexts and threads of the process: it is only ever
-// raised, always to the same value, so that no thread's launch falls between another's set and launch.
+// Dynamic shared memory that the kernels are let take: K = 1024 is the most pairs, 144 KB with the slots of a
+// block of eight warps; 34 KB of tables are static.  The limit belongs to the function, for all contexts and
+// threads of the process, so it is set to this value always: no thread's launch falls between another's
+// set and launch.
+constexpr size_t kMostSmem = 160 * 1024;
 template <class... P>
 cudaError_t allow_smem(void (*kern)(P...), size_t bytes) {
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
-    int dev = 0, most = 0;
-    cudaGetDevice(&dev);
-    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    return bytes > kMostSmem ? cudaErrorInvalidValue : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostSmem);
 }
 
 inline int sm_count() {

@@ -530,7 +530,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
         // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  A block of sixteen where
         // there is a chunk an SM at most.
-        const bool alone = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode, true) <= 160 * 1024;
+        const bool alone = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode, true) <= kMostSmem;
         const bool roomy = dense || alone;
         auto kern = dense ? (encode ? coop_kernel<d, true, true, true> : coop_kernel<d, true, false, true>)
                   : roomy ? (encode ? coop_kernel<d, false, true, true> : coop_kernel<d, false, false, true>)
