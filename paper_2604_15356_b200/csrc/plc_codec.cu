@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArg
         const uint16_t* words = reinterpret_cast<const uint16_t*>(src + 128);
         const int nwords = (int)((nbytes - 128u) >> 1);
         const int last = nwords - 1;                 // -1 for a chunk of states only: words[-1] is inside the chunk
-        auto read_word = [&](int i) { return (uint32_t)words[min(i, last)]; };   // past the end: the last word
+        auto read_word = [&](int i) { return (uint32_t)__ldg(words + min(i, last)); };   // past the end: the last word
         int rp = 0;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
         const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
@@ -394,8 +394,8 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
                 if (lane < rq.rec_words) rec[lane] = mine0;                         // rec_words <= 64
                 if (lane + 32 < rq.rec_words) rec[lane + 32] = mine1;
             } else {
-                const uint32_t w0 = lane < rq.rec_words ? rec[lane] : 0u;
-                const uint32_t w1 = lane + 32 < rq.rec_words ? rec[lane + 32] : 0u;
+                const uint32_t w0 = lane < rq.rec_words ? __ldg(rec + lane) : 0u;
+                const uint32_t w1 = lane + 32 < rq.rec_words ? __ldg(rec + lane + 32) : 0u;
                 const float scale = __uint_as_float(__shfl_sync(kFull, w0, 0));
 #pragma unroll
                 for (int g = 0; g < G; ++g) {

@@ -98,7 +98,8 @@ __host__ __device__ inline void class_params(int q, int& s, int& qp) {
 // HBM, 18.3 -> 29.0 ms), and crowd on the SMs that are free first (128 chunks, a block each: 355 -> 447 us).
 // A chained kernel is resident while the kernel ahead writes, so what that kernel (or the caller's own, whose
 // logits a chained top-K reads) may write is read with ordinary loads: the non-coherent path (__ldg) asks for
-// data that does not change while the kernel lives.  T, row norms and coder tables may take it.
+// data that does not change while the kernel lives.  T, row norms and coder tables may take it, and payload
+// words and records, since no kernel is chained to an encoder or decoder.
 // So a kernel is chained only where neither can happen: see launch_coop and plc_append_step's launches.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

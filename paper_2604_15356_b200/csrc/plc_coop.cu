@@ -208,7 +208,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                     tail_get<G>(slot + 32 * G, base);
                     const uint16_t* words = reinterpret_cast<const uint16_t*>(a.st.payload + sh.item.off + 128);
                     const int last = (int)((sh.item.nbytes - 128u) >> 1) - 1;  // past the end: the last word
-                    join_position<G>(base, zz, s_old, [&](int i) { return (uint32_t)words[min(i, last)]; }, lc, sym);
+                    join_position<G>(base, zz, s_old, [&](int i) { return (uint32_t)__ldg(words + min(i, last)); }, lc, sym);
                 }
                 const float delta = a.step_exp ? ldexpf(a.sh.delta, e_old) : a.sh.delta;
 #pragma unroll

@@ -480,9 +480,12 @@ constexpr int kBatch = 4;                           // 16-byte loads a lane has 
 constexpr int kStreamWarps = 8;                     // most warps of a block
 constexpr int kMaxCluster = 4;
 
-__device__ __forceinline__ uint4 ldg_stream(const uint4* p) {
+// CHAINED: the kernel may be resident while the logits are being written.
+template <bool CHAINED>
+__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 r;
-    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    else asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
     return r;
 }
 __device__ __forceinline__ __half2 as_half2(uint32_t w) { return *reinterpret_cast<const __half2*>(&w); }
@@ -861,7 +864,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 
     for (long long rowi = next_row(a, group, stride); rowi < a.N; rowi = next_row(a, rowi + stride, stride)) {
         const RowView r = row_view<FIXED != 0>(a.logits + rowi * (long long)a.V, a.V);
-        auto fetch = [&](int v) { return FIXED == 2 && r.phase ? group_across(r, v) : ldg_stream(r.body + v); };
+        auto fetch = [&](int v) { return FIXED == 2 && r.phase ? group_across(r, v) : ld_stream<SHARE>(r.body + v); };
         const int per = kBatch * 32 * NW, batches = max(1, (r.nv + per - 1) / per);
         // Slots of this warp: one a group of 8 where all the row's fit, else one for every `wide` batches.
         const bool fine = NW * batches * kBatch <= kSlots;
@@ -876,7 +879,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                 groups_across(r, at, 32 * NW, q);
             } else if ((FIXED != 2 || !r.phase) && (t + 1) * per <= r.nv) {
 #pragma unroll
-                for (int u = 0; u < kBatch; ++u) q[u] = ldg_stream(r.body + at + u * 32 * NW);
+                for (int u = 0; u < kBatch; ++u) q[u] = ld_stream<SHARE>(r.body + at + u * 32 * NW);
             } else {
 #pragma unroll
                 for (int u = 0; u < kBatch; ++u) q[u] = at + u * 32 * NW < r.nv ? fetch(at + u * 32 * NW) : all4(kNegInf2);
@@ -1110,7 +1113,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 #pragma unroll
                             for (int u = 0; u < kBatch; ++u) {
                                 const int v = vb + u * 32 * NW;
-                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : r.body[v]) : all4(kNoValue2);
+                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : SHARE ? r.body[v] : __ldg(r.body + v)) : all4(kNoValue2);
                             }
                             if (i0 < 0) q[0] = row_ends(r, lane);
                             uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
@@ -1124,7 +1127,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                                 const int b = __ffs(m) - 1, u = (b >> 2) & 3;
                                 const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
                                 const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
-                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(r.row[e])), e);   // a first-level hit
+                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(SHARE ? r.row[e] : __ldg(r.row + e))), e);   // a first-level hit
                             }
                         }
                     }
