@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     const int V = a.V, K = a.K;
     const int ntiles = (V + THREADS * 8 - 1) / (THREADS * 8);
     const int per_warp = (K + NW - 1) / NW;
-    const bool bounded = per_warp <= 16;
+    const bool bounded = THREADS == 512 && per_warp <= 16;              // K <= 256
     unsigned long long* list = reinterpret_cast<unsigned long long*>(sm.hist);           // idle until the histograms
     static_assert(kCandCap * sizeof(unsigned long long) <= sizeof(sm.hist), "the list lives there");
     chain_next();
@@ -318,9 +318,8 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
         const __half* row = a.logits + rowi * (long long)V;
         if (tid == 0) { sm.nlist = 0; sm.nhit = 0; }
         // Pass 0 (HBM): the maximum.
-        uint32_t tkey = 0;
+        uint32_t m2 = 0xfc00fc00u;                                   // (-inf, -inf); NaN loses every maximum
         if (VEC) {
-            uint32_t m2 = 0xfc00fc00u;                               // (-inf, -inf)
 #pragma unroll 4
             for (int t = 0; t < ntiles; ++t) {
                 const int i0 = t * (THREADS * 8) + tid * 8;
@@ -329,13 +328,11 @@ __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
                     m2 = hmax2_bits(m2, hmax2_bits(hmax2_bits(r.x, r.y), hmax2_bits(r.z, r.w)));
                 }
             }
-            if (tid * 8 < V) tkey = max(key_of(m2 & 0xffffu), key_of(m2 >> 16));
         } else {
             for (int t = 0; t < ntiles; ++t)
-                for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) {
-                    if ((bits & 0x7fffu) <= 0x7c00u) tkey = max(tkey, key_of(bits));       // not NaN, as above
-                });
+                for_tile<VEC, THREADS>(row, V, t, [&](int, uint32_t bits) { m2 = hmax2_bits(m2, bits * 0x10001u); });
         }
+        const uint32_t tkey = tid * 8 < V ? max(key_of(m2 & 0xffffu), key_of(m2 >> 16)) : 0u;
         const uint32_t wmax = __reduce_max_sync(kFull, tkey);
         uint32_t wth = 0;
         if (bounded) {
