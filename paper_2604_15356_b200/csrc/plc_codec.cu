@@ -421,11 +421,8 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
 // symbols and class in slot a.open_slot of the stream's open chunk.  The rows come from HBM at
 // random, so what counts is row loads in flight: four blocks per SM (64 registers, the whole
 // unrolled batch of row loads issued before the first use) measured best.
-#ifndef PLC_APPEND_BLOCKS
-#define PLC_APPEND_BLOCKS 4
-#endif
 template <int D>
-__global__ void __launch_bounds__(kThreads, PLC_APPEND_BLOCKS) append_quantise_kernel(const CodecArgs a) {
+__global__ void __launch_bounds__(kThreads, kGatherBlocks) append_quantise_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     chain_next();
     chain_wait();

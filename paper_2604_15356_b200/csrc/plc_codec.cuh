@@ -31,21 +31,6 @@ __device__ __forceinline__ float warp_norm2(const float (&v)[G]) {
     return warp_sum(p);
 }
 
-// Two binary32 fused multiply-adds in one instruction (sm_100 packed f32x2) on register pairs that
-// stay packed across the gather loop; each half is an IEEE fma, so the result equals two scalar
-// __fmaf_rn.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1,%2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
-    asm("mov.b64 {%0,%1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void ffma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 // acc2 += w * (8 components of a row): four pairs.
 __device__ __forceinline__ void add_row(const char* p, float w, unsigned long long (&acc2)[4]) {
     const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
@@ -54,7 +39,7 @@ __device__ __forceinline__ void add_row(const char* p, float w, unsigned long lo
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const float2 f = __half22float2(hp[j]);
-        ffma2(acc2[j], ww, pack2(f.x, f.y));
+        acc2[j] = fma2(ww, pack2(f.x, f.y), acc2[j]);
     }
 }
 // Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
@@ -434,13 +419,6 @@ constexpr size_t kMostSmem = 160 * 1024;
 template <class... P>
 cudaError_t allow_smem(void (*kern)(P...), size_t bytes) {
     return bytes > kMostSmem ? cudaErrorInvalidValue : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostSmem);
-}
-
-inline int sm_count() {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
 }
 
 }  // namespace

@@ -23,13 +23,6 @@
 namespace plc {
 namespace {
 
-int dense_sm_count() {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        sms = 1;
-    return sms;
-}
-
 constexpr int kBM = 128, kBN = 256, kBK = 64, kStages = 4, kUmmaK = 16;
 constexpr int kABytes = kBM * kBK * 2, kBBytes = kBN * kBK * 2, kStageBytes = kABytes + kBBytes;
 constexpr int kGemmThreads = 192;
@@ -375,7 +368,7 @@ __global__ void __launch_bounds__(256) rownorm_bf16_kernel(const __half* __restr
 
 // Blocks of 256 threads for n work items, at most 16 per SM (grid-stride kernels).
 unsigned blocks_for(long long n) {
-    const long long b = (n + 255) / 256, cap = (long long)dense_sm_count() * 16;
+    const long long b = (n + 255) / 256, cap = (long long)sm_count() * 16;
     return (unsigned)(b < cap ? (b > 0 ? b : 1) : cap);
 }
 
@@ -433,7 +426,7 @@ cudaError_t launch_gemm(const __nv_bfloat16* A, long long rows, int ldk, const G
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)g.tiles_m * g.tiles_n;
     if (tiles >= (1ll << 31)) return cudaErrorInvalidValue;
-    const int sms = dense_sm_count();
+    const int sms = sm_count();
     dense_gemm_kernel<<<(unsigned)(tiles < sms ? tiles : sms), kGemmThreads, kGemmSmem, st>>>(ma, mb[0], mb[1], g);
     count_launch();
     return cudaGetLastError();
@@ -522,7 +515,7 @@ cudaError_t dense_prepare(const __half* T, const DenseShape& sh, uint8_t* model,
 }
 
 cudaError_t dense_softmax(const __half* logits, const DenseShape& sh, uint8_t* scratch, const size_t* off, cudaStream_t st) {
-    const long long cap_blocks = (long long)dense_sm_count() * 8;
+    const long long cap_blocks = (long long)sm_count() * 8;
     long long blocks = sh.rows < cap_blocks ? sh.rows : cap_blocks;
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(scratch + off[0]);
     if (sh.V % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15) == 0)

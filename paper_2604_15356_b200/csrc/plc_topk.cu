@@ -234,30 +234,16 @@ __device__ void select_by_histogram(Smem<THREADS>& sm, const __half* row, int V,
     }
     __syncthreads();
     // Order the K selected by (key descending, index ascending): a sort of packed order words in the
-    // histogram's memory for large K, rank by counting otherwise.
-    if (K > 128) {
-        unsigned long long* w = reinterpret_cast<unsigned long long*>(sm.hist);
-        int n_pad = 256;
-        while (n_pad < K) n_pad <<= 1;
-        for (int k = tid; k < n_pad; k += THREADS)
-            w[k] = k < K ? ((unsigned long long)sm.sel_key[k] << 32) | (0xffffffffu - (uint32_t)sm.sel_idx[k]) : 0ull;
-        __syncthreads();
-        bitonic_desc<THREADS>(w, n_pad);
-        for (int k = tid; k < K; k += THREADS) {
-            sm.cand_key[k] = (uint32_t)(w[k] >> 32); sm.cand_idx[k] = (int)(0xffffffffu - (uint32_t)w[k]);
-        }
-        __syncthreads();
-        return;
-    }
+    // histogram's memory.
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(sm.hist);
+    int n_pad = 256;
+    while (n_pad < K) n_pad <<= 1;
+    for (int k = tid; k < n_pad; k += THREADS)
+        w[k] = k < K ? ((unsigned long long)sm.sel_key[k] << 32) | (0xffffffffu - (uint32_t)sm.sel_idx[k]) : 0ull;
+    __syncthreads();
+    bitonic_desc<THREADS>(w, n_pad);
     for (int k = tid; k < K; k += THREADS) {
-        uint32_t key = sm.sel_key[k];
-        int idx = sm.sel_idx[k];
-        int rank = 0;
-        for (int j = 0; j < K; ++j) {
-            uint32_t kj = sm.sel_key[j];
-            rank += (kj > key) || (kj == key && sm.sel_idx[j] < idx);
-        }
-        sm.cand_key[rank] = key; sm.cand_idx[rank] = idx;
+        sm.cand_key[k] = (uint32_t)(w[k] >> 32); sm.cand_idx[k] = (int)(0xffffffffu - (uint32_t)w[k]);
     }
     __syncthreads();
 }
@@ -494,24 +480,6 @@ __device__ __forceinline__ uint32_t half_at(const uint4& r, int j) {       // j 
     const uint32_t w = j < 2 ? r.x : j < 4 ? r.y : j < 6 ? r.z : r.w;
     return (j & 1) ? w >> 16 : w & 0xffffu;
 }
-// Packed pairs of binary32 (sm_100 f32x2 instructions).
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ unsigned long long both(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1,%2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void parts(unsigned long long v, float& lo, float& hi) { asm("mov.b64 {%0,%1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-
 // Order words: larger = earlier in (key descending, index ascending); 32 bits while indices fit 16.
 template <class W>
 __device__ __forceinline__ W order_word(uint32_t key, int idx) {
@@ -907,15 +875,15 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             unsigned long long s0 = 0ull, s1 = 0ull;
             auto add_group = [&](const uint4& q) {
                 const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-                const unsigned long long l2e = both(1.44269504088896341f, 1.44269504088896341f), nb2 = both(nb, nb);
+                const unsigned long long l2e = pack2(1.44269504088896341f, 1.44269504088896341f), nb2 = pack2(nb, nb);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float2 f = __half22float2(as_half2(w[j]));
                     float x, y, ex, ey;
-                    parts(fma2(both(f.x, f.y), l2e, nb2), x, y);
+                    unpack2(fma2(pack2(f.x, f.y), l2e, nb2), x, y);
                     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
                     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
-                    if (j & 1) s1 = add2(s1, both(ex, ey)); else s0 = add2(s0, both(ex, ey));
+                    if (j & 1) s1 = add2(s1, pack2(ex, ey)); else s0 = add2(s0, pack2(ex, ey));
                 }
             };
             if (has_ends) {
@@ -935,7 +903,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
                 if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
                     const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
                     const float f = expf(ref - to);
-                    const unsigned long long ff = both(f, f), z = 0ull;
+                    const unsigned long long ff = pack2(f, f), z = 0ull;
                     s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
                     ref = to; nb = -ref * 1.44269504088896341f; lim2 = lim_of(ref);
                 }
@@ -987,7 +955,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             // Maximum and sum of the part, then of the row.
             kmax = __reduce_max_sync(kFull, top_key(m2));
             float x0, x1, x2, x3;
-            parts(s0, x0, x1); parts(s1, x2, x3);
+            unpack2(s0, x0, x1); unpack2(s1, x2, x3);
             sum_all = warp_sum((x0 + x1) + (x2 + x3));
             if (SHARE) {
                 if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
@@ -1195,9 +1163,7 @@ static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st, int* few_
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
     *few_blocks = 0;
     if (a.N <= 0) return cudaSuccess;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = sm_count();
     const bool select = a.pairs || a.idx || a.w || a.zk;
     if (!select) return launch_stream<false, 0, uint32_t>(a, sms, st, few_blocks);
     const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
