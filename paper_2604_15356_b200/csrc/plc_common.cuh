@@ -205,7 +205,8 @@ struct TopkArgs {
     unsigned int* tickets;  // kTicketWords work counters that the launch zeroes for the kernel behind it, or null
     bool chained;           // where rows are few, the launch may start while the kernel ahead of it ends
 };
-// *few_blocks: the blocks launched where rows are few (several warps a row, little shared memory), else 0.
+// *few_blocks: the blocks launched where rows are few (several warps a row, little shared memory; or at most a
+// block an SM), else 0.
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks);
 
 cudaError_t launch_prefix_dedup(const int32_t* tokens, const int32_t* lens, const float* logp2, int S, int64_t stride,

@@ -1155,9 +1155,9 @@ static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st, int* few_
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, per_block * 32, smem) != cudaSuccess || occ < 1) occ = 1;
     const long long want = share ? a.N * cluster : (a.N + per_block - 1) / per_block;
     const unsigned blocks = (unsigned)std::min<long long>(want, (long long)sms * occ / cluster * cluster);
-    *few_blocks = share ? (int)blocks : 0;
+    *few_blocks = share || (int)blocks <= sms ? (int)blocks : 0;
     count_launch();
-    return launch_kernel(kern, blocks, per_block * 32, smem, st, a.chained && share, cluster, a);
+    return launch_kernel(kern, blocks, per_block * 32, smem, st, a.chained && *few_blocks > 0, cluster, a);
 }
 
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {

@@ -1129,7 +1129,7 @@ def test_rows_with_nan_logits_stay_inside_the_vocabulary(dev, orc, N, V, K):
 def test_index_with_room_to_grow(dev, kind, S, n):
     """An index larger than the call needs: the work and its layout are those of the chunks that exist (few chunks
     take a block each whatever the room), the chunks are the same, and the entries behind them are rewritten to 0."""
-    L, H, d, V, K, CP, delta = 2, 4, 128, 32000 if kind == "topk" else 1000, 24, 32, 0.02   # topk: tables of 131 MB, several work queues
+    L, H, d, V, K, CP, delta = 3, 4, 128, 32000 if kind == "topk" else 1000, 24, 32, 0.02   # topk: 197 MB of tables, several work queues
     tokens, logits, T, kv = make_workload(900 + S, S, n, L, H, d, V, K)
     ctx = plc.Context(T.to(dev), K, delta, chunk_pos=CP, variant=plc.PRED_DENSE if kind == "dense" else plc.PRED_TOPK)
     W, need = ctx.W, ctx.max_chunks(n)
