@@ -281,6 +281,8 @@ __device__ __forceinline__ void zero_tickets(const TopkArgs& a) {
 // of a warp's maxima, the smallest over the warps, bounds the K-th logit from below; the second pass, the
 // sum, then notes the groups of 8 that reach it, and their logits, a few more than K, are sorted.
 // Otherwise, and where ties overflow the list, select_by_histogram reads the row again.
+// (4096 rows of 128256, K = 256: 1294 us by histograms, 510 so; K = 1024, 1024 rows: maxima key by key 425, packed
+// 370.)
 template <bool VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS) topk_softmax_kernel(TopkArgs a) {
     constexpr int NW = THREADS / 32;
@@ -600,7 +602,8 @@ struct CountShared {                                // of the warps that select 
 // one warp: bisection of the K-th largest key between `lo` (at least K logits reach it) and the maximum, then
 // the K elements, equal keys in index order, into the list (packed); returns how many there are.  For rows
 // whose ties overflow the lists (few finite logits, quantised logits) and rows with few more groups than
-// K.  A pass costs ten instructions per 8 logits; NaN reaches nothing.
+// K.  A pass costs ten instructions per 8 logits; NaN reaches nothing.  (40 finite logits of 128256, one row:
+// 875 us when one warp passed over it key by key, now 76; 1024 such rows: 1326, 311.)
 template <bool SHARE, class W>
 __device__ __noinline__ int select_by_count(const __half* row, int V, int K, uint32_t lo, uint32_t kmax, W* list, CountShared& sh, int tw, int tws,
                                             int lane) {
@@ -984,7 +987,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
             auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
             // With three quarters as many selected as there are groups the bound holds back little: the logits are
-            // counted instead.
+            // counted instead (V = 256, K = 64, 32768 rows: 438 -> 120 us).
             const bool few_groups = fine && 4 * K > 3 * r.nv;
             uint32_t theta = kKeyNegInf;
             int n = 0;

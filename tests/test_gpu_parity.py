@@ -166,9 +166,9 @@ def gpu_decode_check(g, kv, delta, n, pos_begin=None, pos_end=None, out_dtype=pl
 
 def test_topk_softmax_parity(dev, orc):
     rng = np.random.default_rng(0)
-    # the last three shapes have rows longer than 128 KB (the kernel's wide blocks), vectorised and not;
-    # K = 300 and K = 1024 are beyond the per-thread-maximum bound and take the radix-select path; K up to 128 on
-    # ordinary rows hands the candidate list to the ranking kernel (32-bit order words up to V = 65536, 64-bit beyond)
+    # rows of up to 128 KB and longer (K above 128: 256 or 512 threads a row), vectorised and not; K = 300 and 1024 are
+    # beyond the bound by thread maxima and take the histograms; K up to 128 is the row kernel's, with 32-bit order
+    # words up to V = 65536 and 64-bit ones beyond
     for V, K, N in [(256, 16, 40), (32000, 64, 24), (1000, 64, 16), (37, 5, 9), (4096, 1, 8), (2048, 1024, 4),
                     (32000, 256, 6), (8192, 300, 5), (70008, 64, 7), (65541, 40, 6), (128256, 256, 5),
                     (32000, 128, 9), (32000, 100, 9), (128256, 64, 6), (4096, 128, 8)]:
@@ -188,8 +188,7 @@ def test_topk_softmax_parity(dev, orc):
         np.testing.assert_allclose(out["lse"].cpu().numpy(), lse, atol=2e-5)
         np.testing.assert_allclose(out["zk"].cpu().numpy(), zk, rtol=2e-5)
         np.testing.assert_allclose(out["logp2"].cpu().numpy(), lp, atol=1e-4)
-        # a call that asks for no selected set takes its own route (rows staged in shared memory, rows
-        # longer than the buffer in chunks with a running maximum and sum): same lse and log2 P
+        # a call that asks for no selected set takes its own instantiation of the row kernel: same lse and log2 P
         only = ctx.topk_softmax(torch.from_numpy(lg).to(dev), torch.from_numpy(tok).to(dev), want=("lse", "logp2"))
         np.testing.assert_allclose(only["lse"].cpu().numpy(), lse, atol=2e-5)
         np.testing.assert_allclose(only["logp2"].cpu().numpy(), lp, atol=1e-4)
