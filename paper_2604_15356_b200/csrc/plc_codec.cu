@@ -23,12 +23,15 @@ namespace {
 constexpr int kWarpsPerBlock = 8;
 constexpr int kThreads = kWarpsPerBlock * 32;
 // Blocks per SM.  The coder alone (symbols or predictions read from memory) wants warps: 5, 48 registers.
-// The gather wants row loads in flight more than warps: 4 blocks at 64 registers hold a stretch of 32
-// rows' loads where 5 held 8 (256 streams x 16384 positions, skewed candidates: 6.18 + 6.46 -> 5.49 +
-// 5.79 ms), and where the rows come from L2 (one queue for the whole GPU) 3 at 80 are better still:
+// The gather wants row loads in flight more than warps: 32 warps at 64 registers hold a stretch of 32
+// rows' loads where 40 held 8 (256 streams x 16384 positions, skewed candidates: 6.18 + 6.46 -> 5.49 +
+// 5.79 ms), and where the rows come from L2 (one queue for the whole GPU) 24 at 80 are better still:
 // fewer tables in flight, more L1 (131072 positions x 32 streams, uniform candidates: decode 7.7 ->
-// 6.8 ms).
-constexpr int kBlocksPerSM = 5, kGatherBlocks = 4, kFarBlocks = 3;
+// 6.8 ms).  The gather kernels with a coder are one block an SM, so that its warps share one copy of the
+// coder's tables (20 KB) and the L1 is 60 KB larger than with blocks of eight (1024 streams x 16384
+// positions, skewed: 21.28 + 20.94 -> 20.51 + 20.21 ms; 131072 positions x 64 streams: decode 14.1 -> 13.6 ms).
+constexpr int kBlocksPerSM = 5, kGatherBlocks = 4;
+constexpr int kGatherWarps = kGatherBlocks * kWarpsPerBlock, kFarWarps = 24;
 
 template <int D>
 __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows) {
@@ -49,8 +52,8 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__
 // ZR: the zero-rate rule (Thm. 3) is on; a separate instantiation keeps the plain coder's loop free of it.
 // FLEX: the call exports intermediate values or statistics, or uses a per-position step; the plain
 // instantiation carries none of those branches in its position loop.
-template <int D, int SRC, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
-__global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArgs a) {
+template <int D, int SRC, bool ZR, bool FLEX, int WARPS = kWarpsPerBlock, int BLOCKS = kBlocksPerSM>
+__global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     constexpr bool FROM_OPEN = SRC == kSrcOpen;
     constexpr bool DENSE = SRC == kSrcDense;
@@ -60,7 +63,7 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const LaneCode lc = lane_code(lane);
-    const long long gw = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    const long long gw = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     uint16_t* stage = a.staging + gw * a.staging_words_per_warp;
     const int cap_words = (int)a.staging_words_per_warp;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp;
@@ -193,8 +196,8 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) encode_kernel(const CodecArg
     }
 }
 
-template <int D, bool DENSE, bool ZR, bool FLEX, int BLOCKS = kBlocksPerSM>
-__global__ void __launch_bounds__(kThreads, BLOCKS) decode_kernel(const CodecArgs a) {
+template <int D, bool DENSE, bool ZR, bool FLEX, int WARPS = kWarpsPerBlock, int BLOCKS = kBlocksPerSM>
+__global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecArgs a) {
     constexpr int G = Geo<D>::G;
     __shared__ DecTables tb;
     load_tables(&tb, &a.tables->dec);
@@ -460,6 +463,19 @@ cudaError_t pair_smem_bytes(Kern kern, int Kp, size_t& bytes) {
     return bytes > 24 * 1024 ? allow_smem(kern, bytes) : cudaSuccess;
 }
 
+// Gather kernels with a coder: one block an SM; where the pairs of that many warps do not fit beside each
+// other (K above 320, above 426 with 24 warps), blocks of eight, as many as fit.
+template <class Kern>
+cudaError_t launch_gather(const CodecArgs& a, Kern kern, int warps, cudaStream_t st) {
+    int blocks = sm_count();
+    size_t bytes = (size_t)warps * 2 * a.sh.Kp * sizeof(int2);
+    if (bytes > kMostSmem) { blocks *= warps / kWarpsPerBlock; bytes /= warps / kWarpsPerBlock; warps = kWarpsPerBlock; }
+    const cudaError_t e = allow_smem(kern, bytes);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return launch_kernel(kern, blocks, 32 * warps, bytes, st, false, 1, a);
+}
+
 }  // namespace
 
 int codec_grid_warps(int) { return sm_count() * kBlocksPerSM * kWarpsPerBlock; }
@@ -539,18 +555,13 @@ cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {
             count_launch();
             return cudaGetLastError();
         }
-        auto pick = [&](auto blocks) {
-            constexpr int B = decltype(blocks)::value;
-            return zr ? (flex ? encode_kernel<d, kSrcGather, true, true, B> : encode_kernel<d, kSrcGather, true, false, B>)
-                      : (flex ? encode_kernel<d, kSrcGather, false, true, B> : encode_kernel<d, kSrcGather, false, false, B>);
+        auto pick = [&](auto warps) {
+            constexpr int N = decltype(warps)::value;
+            return zr ? (flex ? encode_kernel<d, kSrcGather, true, true, N, 1> : encode_kernel<d, kSrcGather, true, false, N, 1>)
+                      : (flex ? encode_kernel<d, kSrcGather, false, true, N, 1> : encode_kernel<d, kSrcGather, false, false, N, 1>);
         };
-        const int blocks = a.sched_nq == 1 ? kFarBlocks : kGatherBlocks;
-        auto kern = a.sched_nq == 1 ? pick(std::integral_constant<int, kFarBlocks>{}) : pick(std::integral_constant<int, kGatherBlocks>{});
-        size_t sm = 0;
-        cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
-        if (e2 != cudaSuccess) return e2;
-        count_launch();
-        return launch_kernel(kern, sm_count() * blocks, kThreads, sm, st, false, 1, a);
+        return a.sched_nq == 1 ? launch_gather(a, pick(std::integral_constant<int, kFarWarps>{}), kFarWarps, st)
+                               : launch_gather(a, pick(std::integral_constant<int, kGatherWarps>{}), kGatherWarps, st);
     });
 }
 
@@ -588,18 +599,13 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
             count_launch();
             return cudaGetLastError();
         }
-        auto pick = [&](auto blocks) {
-            constexpr int B = decltype(blocks)::value;
-            return zr ? (flex ? decode_kernel<d, false, true, true, B> : decode_kernel<d, false, true, false, B>)
-                      : (flex ? decode_kernel<d, false, false, true, B> : decode_kernel<d, false, false, false, B>);
+        auto pick = [&](auto warps) {
+            constexpr int N = decltype(warps)::value;
+            return zr ? (flex ? decode_kernel<d, false, true, true, N, 1> : decode_kernel<d, false, true, false, N, 1>)
+                      : (flex ? decode_kernel<d, false, false, true, N, 1> : decode_kernel<d, false, false, false, N, 1>);
         };
-        const int blocks = a.sched_nq == 1 ? kFarBlocks : kGatherBlocks;
-        auto kern = a.sched_nq == 1 ? pick(std::integral_constant<int, kFarBlocks>{}) : pick(std::integral_constant<int, kGatherBlocks>{});
-        size_t sm = 0;
-        cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
-        if (e2 != cudaSuccess) return e2;
-        count_launch();
-        return launch_kernel(kern, sm_count() * blocks, kThreads, sm, st, false, 1, a);
+        return a.sched_nq == 1 ? launch_gather(a, pick(std::integral_constant<int, kFarWarps>{}), kFarWarps, st)
+                               : launch_gather(a, pick(std::integral_constant<int, kGatherWarps>{}), kGatherWarps, st);
     });
 }
 
