@@ -62,6 +62,7 @@ struct plc_ctx {
     plc_config cfg;
     const __half* T;
     float* rownorm2;
+    bool finite;                    // T holds neither infinities nor NaN
     int2* pairs;
     int* step_exp;                  // [positions] adaptive step exponents
     long long pairs_cap;            // positions
@@ -184,7 +185,8 @@ CodecArgs base_args(const plc_ctx* c) {
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
     a.tables = c->tables;
-    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs; a.pair_index = pair_index(c->cfg);
+    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs; 
+    a.row_form = pair_index(c->cfg) ? kRowIndices : c->finite ? kRowOffsets : kRowOffsetsPlain;
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
     return a;
@@ -329,8 +331,13 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
     if (ok) ok = tables && cudaMemcpy(c->tables, tables, sizeof(CoderTables), cudaMemcpyHostToDevice) == cudaSuccess;
     if (ok) ok = cudaMemset(c->status, 0, sizeof(unsigned int)) == cudaSuccess &&
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
-    if (ok && T_dev) ok = launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, 0) == cudaSuccess &&
-                          cudaDeviceSynchronize() == cudaSuccess;
+    if (ok && T_dev) {
+        unsigned int not_finite = 0;
+        ok = cudaMemset(c->ticket, 0, sizeof(unsigned int)) == cudaSuccess &&
+             launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
+             cudaMemcpy(&not_finite, c->ticket, sizeof(unsigned int), cudaMemcpyDeviceToHost) == cudaSuccess;
+        c->finite = not_finite == 0;
+    }
     if (ok && T_dev && cfg->variant == PLC_PRED_DENSE) {     // operands of every layer, once
         c->resident = keep_weights((size_t)rows * cfg->head_dim * 2);
         ok = with_or_without_weights(c, [&]() {

@@ -34,7 +34,8 @@ constexpr int kBlocksPerSM = 5, kGatherBlocks = 4;
 constexpr int kGatherWarps = kGatherBlocks * kWarpsPerBlock, kFarWarps = 24;
 
 template <int D>
-__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows) {
+__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows,
+                                                      unsigned int* not_finite) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
     const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -45,7 +46,10 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__
 #pragma unroll
         for (int g = 0; g < G; ++g) v[g] = __half2float(T[r * D + c0 + g]);
         float s = warp_norm2<G>(v);
-        if (lane == 0) out[r] = s;
+        if (lane == 0) {
+            out[r] = s;
+            if (!(s < __int_as_float(0x7f800000))) *not_finite = 1u;          // squares of finite binary16 values sum to less
+        }
     }
 }
 
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
                 int zero_q = ZR ? a.sh.zero_q : 0;
@@ -261,7 +265,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
             int zero_q = ZR ? a.sh.zero_q : 0;
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D>(col, n2, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D, true>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -447,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) append_quantise_kerne
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;
@@ -525,11 +529,11 @@ static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
     a.sched_g = (int)g; a.sched_nq = nq;
 }
 
-cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, cudaStream_t st) {
+cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, unsigned int* not_finite, cudaStream_t st) {
     return dispatch_d(d, [&](auto D) {
         long long blocks = (rows + 7) / 8;
         if (blocks > (long long)sm_count() * 16) blocks = (long long)sm_count() * 16;
-        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, rows);
+        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, rows, not_finite);
         count_launch();
         return cudaGetLastError();
     });

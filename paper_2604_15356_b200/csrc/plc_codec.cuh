@@ -31,16 +31,36 @@ __device__ __forceinline__ float warp_norm2(const float (&v)[G]) {
     return warp_sum(p);
 }
 
+// The values that a lane has loaded (two words of two), as binary32, through the tensor cores: in a product
+// with the 8 x 8 identity, a lane's share of the 16 x 8 operand and its share of the result are the same
+// elements, so the lanes need not hold anything that belongs together.  Every sum has one term that is not zero:
+// exact for finite values (zeros come out as +0), infinities and NaN would reach other lanes.
+__device__ __forceinline__ uint32_t widen_operand(int lane) {
+    const int row = 2 * (lane & 3), col = lane >> 2;         // elements (row, col), (row + 1, col) of the identity
+    return (row == col ? 0x3c00u : 0u) | (row + 1 == col ? 0x3c000000u : 0u);
+}
+__device__ __forceinline__ void widen(uint32_t lo, uint32_t hi, uint32_t operand, unsigned long long& a, unsigned long long& b) {
+    float f0, f1, f2, f3;
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%7,%7,%7};"
+        : "=f"(f0), "=f"(f1), "=f"(f2), "=f"(f3) : "r"(lo), "r"(hi), "r"(operand), "f"(0.f));
+    a = pack2(f0, f1); b = pack2(f2, f3);
+}
 // acc2 += w * (8 components of a row): four pairs.
-__device__ __forceinline__ void add_row(const char* p, float w, unsigned long long (&acc2)[4]) {
+template <bool WIDEN>
+__device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand, unsigned long long (&acc2)[4]) {
     const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
     const unsigned long long ww = pack2(w, w);
-    const __half2* hp = reinterpret_cast<const __half2*>(&r);
+    unsigned long long v[4];
+    if constexpr (WIDEN) {
+        widen(r.x, r.y, operand, v[0], v[1]);
+        widen(r.z, r.w, operand, v[2], v[3]);
+    } else {
+        const __half2* hp = reinterpret_cast<const __half2*>(&r);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float2 f = __half22float2(hp[j]);
-        acc2[j] = fma2(ww, pack2(f.x, f.y), acc2[j]);
+        for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); v[j] = pack2(f.x, f.y); }
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc2[j] = fma2(ww, v[j], acc2[j]);
 }
 // Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
 // offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
@@ -49,22 +69,33 @@ __device__ __forceinline__ void add_row(const char* p, float w, unsigned long lo
 // What bounds it: issue slots (per row and lane 8 conversions, 4 packed FMAs, a load), with the rows'
 // latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
 // beside its load.
-template <int D>
-__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, bool pair_index,
+// WIDEN: the conversions on the tensor cores, 2 instructions for 8 on the pipe that the packed FMAs need too (392
+// of the 570 instructions that 64 rows of 128 take), in stretches of 16 rows at most.  Right where a warp has
+// little else to do (rotated quantiser, 8 x 8 heads, 4000 positions: both calls 1700 -> 1500 us; stretches of 32 rows
+// 1530).  The coder's kernels lose more to the tensor instructions' latency than they gain (32 heads of 128, 8 layers,
+// 16384 positions: 20.6 -> 21.8 ms at 64 registers, 25.2 at 48 with more warps).
+// LANE_BASE: a row's address as the lane's own 64-bit base and the offset, one addition of three fewer, but two
+// registers more.  It pays in kernels with little state beside the gather (rotated quantiser 1500 -> 1475 us); the
+// others lose loads in flight (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
+template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN>
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, int row_form,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
     const int h = lane / R, iters = Kp / ROWS;
     const uint32_t lane_off = 16u * (lane % R);
+    const char* lane_table = table + lane_off;
+    auto row_at = [&](int off) { return LANE_BASE ? lane_table + (uint32_t)off : table + ((uint32_t)off + lane_off); };
     // variance term first: its row-norm loads are in flight while the rows are gathered
     float s1 = 0.f;
     for (int k = lane; k < Kp; k += 32) {
         const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
-        const uint32_t at = pair_index ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
+        const uint32_t at = row_form == kRowIndices ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
         s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
-    if (!pair_index) {
+    if (WIDEN ? row_form == kRowOffsets : row_form != kRowIndices) {
+        const uint32_t operand = WIDEN ? widen_operand(lane) : 0u;
         // Straight-line stretches of 32, 16 and 8 rows: the loads of a stretch are issued as far ahead as the
         // kernel's registers allow (64 rows of 128 components, uniform candidates, 24 warps an SM: 8.0 ms
         // with stretches of 8 only, 6.4 ms with 32).
@@ -75,23 +106,29 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
 #pragma unroll
             for (int i = 0; i < N; ++i) {
                 const int4 pr = pl[i];
-                add_row(table + ((uint32_t)pr.x + lane_off), __int_as_float(pr.y), acc2);
-                add_row(table + ((uint32_t)pr.z + lane_off), __int_as_float(pr.w), acc2);
+                add_row<WIDEN>(row_at(pr.x), __int_as_float(pr.y), operand, acc2);
+                add_row<WIDEN>(row_at(pr.z), __int_as_float(pr.w), operand, acc2);
             }
             pl += N;
             left -= N;
         };
+        if constexpr (WIDEN) {
 #pragma unroll 1
-        while (left >= 16) rows(std::integral_constant<int, 16>{});
-        if (left >= 8) rows(std::integral_constant<int, 8>{});
+            while (left >= 8) rows(std::integral_constant<int, 8>{});
+        } else {
+#pragma unroll 1
+            while (left >= 16) rows(std::integral_constant<int, 16>{});
+            if (left >= 8) rows(std::integral_constant<int, 8>{});
+        }
         if (left >= 4) rows(std::integral_constant<int, 4>{});
 #pragma unroll 1
         while (left > 0) rows(std::integral_constant<int, 1>{});
-    } else {                                                 // tables of 4 GB or more: 64-bit offsets
+    } else {                                                 // tables of 4 GB or more (64-bit offsets), values that are not finite
+        const uint32_t unit = row_form == kRowIndices ? 2 * D : 1;
 #pragma unroll 1
         for (int it = 0; it < iters; ++it) {
             const int2 pr = sp[h * iters + it];
-            add_row(table + ((size_t)(uint32_t)pr.x * (2 * D) + lane_off), __int_as_float(pr.y), acc2);
+            add_row<false>(lane_table + (size_t)(uint32_t)pr.x * unit, __int_as_float(pr.y), 0u, acc2);
         }
     }
     float acc[8];

@@ -240,12 +240,16 @@ struct DebugDev {
 
 struct CoderTables;                                // plc_coder.cuh
 
+// The pairs' candidates: byte offsets of rows; byte offsets where T holds infinities or NaN; row indices (tables of
+// 4 GB or more).
+enum { kRowOffsets = 0, kRowOffsetsPlain = 1, kRowIndices = 2 };
+
 struct CodecArgs {
     CodecShape sh;
     const CoderTables* tables;                     // frequency tables of the coder
     const __half* T; const float* rownorm2;        // [tables][V][d], [tables][V]
     const int2* pairs;                             // [S*n][Kp] (written by the top-K kernels, put_pair)
-    bool pair_index;                               // pairs hold row indices instead of byte offsets (tables of 4 GB or more)
+    int row_form;                                  // kRow...: what the pairs hold, and whether T may go through the tensor cores
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
     KvView kv;                                     // encode: input f16; decode: output
     int S, n; const int32_t* pos_begin; const int32_t* pos_end;
@@ -312,7 +316,8 @@ cudaError_t linear_begin(const __half* logits, const LinearShape& sh, const uint
                          uint8_t* scratch, const size_t* off, unsigned int* status, cudaStream_t st);
 cudaError_t linear_layers(const __half* A, int l0, int nl, const LinearShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
                           const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
-cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, cudaStream_t st);
+// Sets *not_finite where a row holds an infinity or NaN.
+cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, unsigned int* not_finite, cudaStream_t st);
 cudaError_t launch_encode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_decode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st);   // a block per chunk; queues set, tickets zeroed

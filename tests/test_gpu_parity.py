@@ -395,6 +395,37 @@ def test_rotated_quantiser_parity(dev, orc, d, bits, ranges):
     assert n_codes > 0 and n_diff <= 2e-3 * n_codes
 
 
+@pytest.mark.parametrize("d,K", [(128, 64), (128, 1), (128, 37), (64, 50), (64, 64), (32, 100), (256, 16), (256, 70)])
+def test_rows_widened_by_the_tensor_cores(dev, d, K):
+    """The rotated quantiser's rows go through the tensor cores while T is finite, value by value where it is not:
+    an infinity and a NaN in a row that is never a candidate must not change a bit.  T holds every kind of finite
+    value (both zeros, subnormal, largest); K covers stretches of 16, 8 and 2 rows and what remains."""
+    S, n, L, H, V, bits = 2, 40, 1, 2, 600, 6
+    _, logits, T, kv = make_workload(77 + d + K, S, n, L, H, d, V, K, pp=30.0)
+    rng = np.random.default_rng(d + K)
+    raw = rng.integers(0, 1 << 16, T.numel()).astype(np.uint16)
+    raw[(raw & 0x7c00) == 0x7c00] &= 0x83ff
+    T = torch.from_numpy(raw.view(np.float16)).reshape(T.shape).to(dev)
+    logits[..., V - 1] = -float("inf")
+    kvd, lgd = kv.to(dev), logits.to(dev)
+    got = []
+    for special in (False, True):
+        if special:
+            T = T.clone()
+            T[..., V - 1, 0], T[..., V - 1, 5] = float("inf"), float("nan")
+        ctx = plc.Context(T, K, 0.02)
+        params = ctx.rotq_params(bits, rng.integers(0, 2, d) if not special else neg)
+        neg = [(params.sign_bits[j >> 5] >> (j & 31)) & 1 for j in range(d)]
+        records = torch.zeros(S * ctx.W * n * ctx.rotq_record_bytes(bits), dtype=torch.uint8, device=dev)
+        out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+        ctx.encode_rotq(kvd, lgd, params, records)
+        ctx.decode_rotq(records, lgd, params, out)
+        assert ctx.sync_status() == plc.OK
+        got.append((records, out))
+    assert torch.isfinite(got[0][1]).all() and got[0][0].any()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
 def test_rotated_quantiser_argument_checks(dev):
     tokens, logits, T, kv = make_workload(5, 1, 8, 1, 1, 256, 64, 4)
     ctx = plc.Context(T.to(dev), 4, 0.02, chunk_pos=8)
