@@ -75,8 +75,9 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // 1530).  The coder's kernels lose more to the tensor instructions' latency than they gain (32 heads of 128, 8 layers,
 // 16384 positions: 20.6 -> 21.8 ms at 64 registers, 25.2 at 48 with more warps).
 // LANE_BASE: a row's address as the lane's own 64-bit base and the offset, one addition of three fewer, but two
-// registers more.  It pays in kernels with little state beside the gather (rotated quantiser 1500 -> 1475 us); the
-// others lose loads in flight (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
+// registers more.  It pays in kernels with little state beside the gather (rotated quantiser 1500 -> 1475 us,
+// block-per-chunk kernel, 128 streams x 4096 positions, both calls 2075 -> 2002); the others lose loads in flight
+// (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
 template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN>
 __device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, int row_form,
                                         const int2* sp, int Kp, int lane, float inv_d,
