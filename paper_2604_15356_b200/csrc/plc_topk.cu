@@ -2,7 +2,7 @@
 // ascending, -0 = +0).
 //
 // K <= 128, and calls that ask for no selected set (only lse / log2 P): topk_stream_kernel, which reads
-// a row once, any alignment (see there).  K > 128: topk_softmax_kernel, one block a row: thread maxima bound
+// a row once, any alignment (see there); topk_pipe_kernel where the rows are long and many.  K > 128: topk_softmax_kernel, one block a row: thread maxima bound
 // the K-th logit where K allows it; else a 4096-bin histogram of the order-preserving 16-bit key finds the
 // bin that holds the K-th largest, a 16-way refinement finds the key itself, and equal keys are taken in
 // index order.
@@ -269,6 +269,12 @@ __device__ __forceinline__ void put_surprisal(const TopkArgs& a, long long rowi,
         if (a.step_exp) a.step_exp[rowi] = a.b0 - b;
         if (a.bits_out) a.bits_out[rowi] = b;
     }
+}
+
+// What a row gives beside its selection.
+__device__ __forceinline__ void put_row(const TopkArgs& a, long long rowi, const __half* row, float lse) {
+    if (a.lse) a.lse[rowi] = lse;
+    if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) put_surprisal(a, rowi, row, lse);
 }
 
 __device__ __forceinline__ void zero_tickets(const TopkArgs& a) {
@@ -792,6 +798,211 @@ __device__ __forceinline__ T* at_first_block(T* p) {
     return r;
 }
 
+// Maximum and sum of exp(l - reference) of what a warp reads of a row.
+struct RowSum {
+    uint32_t m2, lim2;
+    float ref, nb;
+    unsigned long long s0, s1;
+    // A logit more than 4 above the reference moves it, so that no exponent is large (its rounding would
+    // show in the sum).
+    __device__ __forceinline__ void refer(float to) {
+        ref = to; nb = -to * 1.44269504088896341f;
+        const uint32_t b = (uint32_t)__half_as_ushort(__float2half_ru(to + 4.0f));
+        lim2 = b | (b << 16);
+    }
+    __device__ __forceinline__ void add_group(const uint4& q) {
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+        const unsigned long long l2e = pack2(1.44269504088896341f, 1.44269504088896341f), nb2 = pack2(nb, nb);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 f = __half22float2(as_half2(w[j]));
+            float x, y, ex, ey;
+            unpack2(fma2(pack2(f.x, f.y), l2e, nb2), x, y);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
+            if (j & 1) s1 = add2(s1, pack2(ex, ey)); else s0 = add2(s0, pack2(ex, ey));
+        }
+    }
+    // The first batch gives the reference; the row's ends are added.
+    __device__ __forceinline__ void begin(const uint4 (&first)[kBatch], const uint4& ends, bool has_ends) {
+        m2 = kNegInf2;
+        if (has_ends) m2 = hmax2_bits(m2, top2_of(ends));
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) m2 = hmax2_bits(m2, top2_of(first[u]));
+        refer(fmaxf(val_of_key(__reduce_max_sync(kFull, top_key(m2))), -65504.0f));
+        s0 = s1 = 0ull;
+        if (has_ends) {
+            auto real = [](uint32_t w) { const uint32_t m = __vcmpeq2(w, kNoValue2); return (w & ~m) | (kNegInf2 & m); };
+            add_group(make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)));
+        }
+    }
+    // Returns the batch's maximum, top[]: its groups'.
+    __device__ __forceinline__ uint32_t add(const uint4 (&q)[kBatch], uint32_t (&top)[kBatch]) {
+        uint32_t top4 = kNegInf2;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) { top[u] = top2_of(q[u]); top4 = hmax2_bits(top4, top[u]); }
+        m2 = hmax2_bits(m2, top4);
+        if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
+            const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
+            const float f = expf(ref - to);
+            const unsigned long long ff = pack2(f, f), z = 0ull;
+            s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
+            refer(to);
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) add_group(q[u]);
+        return top4;
+    }
+    __device__ __forceinline__ uint32_t max_key() const { return __reduce_max_sync(kFull, top_key(m2)); }
+    __device__ __forceinline__ float total() const {
+        float x0, x1, x2, x3;
+        unpack2(s0, x0, x1); unpack2(s1, x2, x3);
+        return warp_sum((x0 + x1) + (x2 + x3));
+    }
+};
+
+// The selected of a row whose maxima lie in `slots` (NW * ns a lane, `wide` batches each; 0: a group each), by the tws warps
+// of a block (SHARE) or by one.  ACROSS: rows may lie off 16-byte boundaries with their groups counted from the
+// first logit.
+template <bool SHARE, bool ACROSS, class W, class Read>
+__device__ __forceinline__ void select_row(const TopkArgs& a, long long rowi, const RowView& r, int NW, int ns, int wide, uint32_t* slots, uint16_t* codes, W* list,
+                                           W* sorted, StreamShared& local_sh, int tw, int tws, uint32_t kmax, float lmax, float sum_all, int lane, Read&& read) {
+    const int K = a.K;
+    const bool fine = wide == 0;
+    auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
+    // With three quarters as many selected as there are groups the bound holds back little: the logits are
+    // counted instead (V = 256, K = 64, 32768 rows: 438 -> 120 us).
+    const bool few_groups = fine && 4 * K > 3 * r.nv;
+    uint32_t theta = kKeyNegInf;
+    int n = 0;
+    bool counted = few_groups;
+    if (few_groups) read();
+    if (!few_groups) {
+        // The bound: the K-th largest group maximum (any value that exactly K of them reach will do), searched
+        // by one warp with all maxima in its registers.  The search is a chain of ten steps or so: shared among
+        // eight warps a step cost 1300 cycles (guards, a shared counter, a barrier), 14400 of the 34000 cycles of a
+        // row of 128256 logits by itself; now 5350 of 22000.
+        const int S = NW * ns, words = (S + 1) >> 1;
+        uint32_t mx[kSlots / 2];                                                      // two maxima each
+        if (tw == 0) {
+            if (S & 1) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kSlots / 2; ++i) mx[i] = i < words ? slots[i * 32 + lane] : kNoValue2;
+            read();
+            auto reach = [&](uint32_t h2, auto first) {                               // of this lane's first words
+                constexpr int A = SHARE ? 4 : 1;                                      // one sum where other rows fill the gaps
+                __half2 c[A];
+#pragma unroll
+                for (int i = 0; i < A; ++i) c[i] = __float2half2_rn(0.f);
+#pragma unroll
+                for (int i = 0; i < decltype(first)::value; ++i) c[i % A] = __hadd2(c[i % A], __hge2(as_half2(mx[i]), as_half2(h2)));
+                if constexpr (A > 1) c[0] = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
+                return __half2int_rn(__hadd(__low2half(c[0]), __high2half(c[0])));
+            };
+            uint32_t hi = kmax + 1, down = 256;                                       // first downwards from the maximum, then between
+#pragma unroll 1
+            while (hi - theta > 1) {
+                const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
+                const int c = __reduce_add_sync(kFull, words <= 8 ? reach(h2, std::integral_constant<int, 8>{})
+                                                                  : reach(h2, std::integral_constant<int, kSlots / 2>{}));
+                if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
+                if (c == K) break;
+            }
+            if (SHARE && lane == 0) local_sh.theta = theta;
+        }
+        sync();
+        if (SHARE) theta = local_sh.theta;
+        // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
+        auto place = [&](int mine, int* shared_total, int& total) {
+            int all;
+            int at = warp_excl_scan(mine, lane, all);
+            int base = total;
+            if (SHARE) {
+                if (lane == 0) base = atomicAdd(shared_total, all);
+                base = __shfl_sync(kFull, base, 0);
+            }
+            total += all;                                                             // SHARE: of this warp only
+            return base + at;
+        };
+        // The groups that reach it.
+        const uint32_t th2 = bits_of_key(theta) * 0x10001u;
+        int n_codes = 0;
+        uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
+        auto hit = [&](uint32_t w, int i) { return __hge2_mask(as_half2(w), as_half2(th2)) & (0x10001u << (i & 15)); };
+        if (SHARE) {                                                                  // two warps at least: 16 words at most
+#pragma unroll 4
+            for (int i = 0; tw + i * tws < words; ++i) hits[0] |= hit(slots[(tw + i * tws) * 32 + lane], i);
+        } else {
+#pragma unroll
+            for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= hit(mx[i], i);
+        }
+        int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.n_codes, n_codes);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            for (uint32_t m = hits[h]; m; m &= m - 1) {
+                const int b = __ffs(m) - 1, i = tw + (16 * h + (b & 15)) * tws;
+                if (at < kCodes) codes[at] = (uint16_t)((2 * i + (b >> 4)) * 32 + lane);
+                ++at;
+            }
+        sync();
+        if (SHARE) n_codes = local_sh.n_codes;
+        if (n_codes <= kCodes) {
+            // their logits at or above the bound; head and tail of the row are a turn of the last warp's own.  A
+            // lane takes one batch of a group where warps share the row (turns are memory latencies: 1700 cycles
+            // each), else all of a group (where rows fill the GPU the lanes' divisions cost more than a turn).
+            const int steps = fine ? 1 : wide, items = SHARE ? n_codes * steps : n_codes;
+            const bool ends_turn = tw == tws - 1 && (r.head > 0 || r.head + 8 * r.nv < r.V);
+#pragma unroll 1
+            for (int i0 = tw * 32 - (ends_turn ? 32 * tws : 0); i0 < items; i0 += 32 * tws) {
+                const bool mine = i0 >= 0 && i0 + lane < items;
+                const int ci = !mine ? 0 : SHARE ? (i0 + lane) / steps : i0 + lane, first = SHARE && mine ? i0 + lane - ci * steps : 0;
+                const int code = mine ? codes[ci] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
+                const int turns = SHARE || i0 < 0 ? 1 : steps;
+#pragma unroll 1
+                for (int st = first; st < first + turns; ++st) {
+                    const int t = fine ? ls >> 2 : ls * wide + st;
+                    const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
+                    uint4 q[kBatch];
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const int v = vb + u * 32 * NW;
+                        q[u] = mine && v < r.nv && !(fine && u) ? (ACROSS && r.phase ? group_across(r, v) : SHARE ? r.body[v] : __ldg(r.body + v)) : all4(kNoValue2);
+                    }
+                    if (i0 < 0) q[0] = row_ends(r, lane);
+                    uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const uint32_t w4[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
+                    }
+                    for (int to = place(__popc(m), &local_sh.n_list, n); m; m &= m - 1, ++to) {
+                        const int b = __ffs(m) - 1, u = (b >> 2) & 3;
+                        const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
+                        const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
+                        if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(SHARE ? r.row[e] : __ldg(r.row + e))), e);   // a first-level hit
+                    }
+                }
+            }
+        }
+        sync();
+        if (SHARE) n = local_sh.n_list;
+        counted = n_codes > kCodes || n > kListCap;
+    }
+    if (counted) {
+        sync();                                                                   // all have read the totals
+        n = select_by_count<SHARE, W>(r.row, r.V, K, theta, kmax, list, local_sh.by_count, tw, tws, lane);
+    }
+    order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);
+    if (tw == 0) {
+        // NaN logits reach no bound: a row with fewer than K others is filled up with candidate 0 at weight 0
+        for (int i = n + lane; i < K; i += 32) sorted[i] = order_word<W>(kKeyNegInf, 0);
+        __syncwarp();
+        emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
+    }
+}
+
 // SHARE: the warps of a cluster of blocks (of a block, if it is alone) share a row; otherwise every warp
 // has a row of its own.
 // FIXED: the order in which a row's exponentials are added depends on V alone, not on how many rows the call
@@ -826,7 +1037,6 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
     chain_next();
     chain_wait();
     zero_tickets(a);
-    const int K = a.K;
     const long long group = SHARE ? blockIdx.x / blocks : (long long)blockIdx.x * nwarps + warp;
     const long long stride = SHARE ? gridDim.x / blocks : (long long)gridDim.x * nwarps;
 
@@ -865,54 +1075,12 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
         do {
             const bool has_ends = wrow == 0 && (r.head > 0 || r.head + 8 * r.nv < r.V);
             const uint4 ends = has_ends ? row_ends(r, lane) : all4(kNoValue2);
-            uint32_t m2 = kNegInf2;
-            if (has_ends) m2 = hmax2_bits(m2, top2_of(ends));
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) m2 = hmax2_bits(m2, top2_of(cur[u]));
-            ref = fmaxf(val_of_key(__reduce_max_sync(kFull, top_key(m2))), -65504.0f);
-            // A logit more than 4 above the reference moves it, so that no exponent is large (its rounding would
-            // show in the sum).
-            auto lim_of = [](float rf) { const uint32_t b = (uint32_t)__half_as_ushort(__float2half_ru(rf + 4.0f)); return b | (b << 16); };
-            uint32_t lim2 = lim_of(ref);
-            float nb = -ref * 1.44269504088896341f;
-            unsigned long long s0 = 0ull, s1 = 0ull;
-            auto add_group = [&](const uint4& q) {
-                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-                const unsigned long long l2e = pack2(1.44269504088896341f, 1.44269504088896341f), nb2 = pack2(nb, nb);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 f = __half22float2(as_half2(w[j]));
-                    float x, y, ex, ey;
-                    unpack2(fma2(pack2(f.x, f.y), l2e, nb2), x, y);
-                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x));
-                    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(y));
-                    if (j & 1) s1 = add2(s1, pack2(ex, ey)); else s0 = add2(s0, pack2(ex, ey));
-                }
-            };
-            if (has_ends) {
-                auto real = [](uint32_t w) { const uint32_t m = __vcmpeq2(w, kNoValue2); return (w & ~m) | (kNegInf2 & m); };
-                add_group(make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)));
-            }
+            RowSum sum;
+            sum.begin(cur, ends, has_ends);
             // slot s of a lane: half s & 1 of word (s / 2, lane)
             auto put_slot = [&](int slot, uint32_t top2) {
                 const int sl = wrow * ns + slot;
                 my_slots[(sl >> 1) * 64 + lane * 2 + (sl & 1)] = (uint16_t)hmax2_bits(top2, top2 >> 16);   // the low half: of both
-            };
-            auto batch = [&](const uint4 (&q)[kBatch], uint32_t (&top)[kBatch]) {             // returns the maximum
-                uint32_t top4 = kNegInf2;
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) { top[u] = top2_of(q[u]); top4 = hmax2_bits(top4, top[u]); }
-                m2 = hmax2_bits(m2, top4);
-                if (__any_sync(kFull, !__hble2(as_half2(top4), as_half2(lim2)))) {             // a logit above the limit
-                    const float to = val_of_key(__reduce_max_sync(kFull, top_key(top4)));
-                    const float f = expf(ref - to);
-                    const unsigned long long ff = pack2(f, f), z = 0ull;
-                    s0 = fma2(s0, ff, z); s1 = fma2(s1, ff, z);
-                    ref = to; nb = -ref * 1.44269504088896341f; lim2 = lim_of(ref);
-                }
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) add_group(q[u]);
-                return top4;
             };
             uint32_t top[kBatch];
             uint32_t group2 = kNegInf2;                                                       // of the slot being filled
@@ -924,7 +1092,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             if (FIXED == 2 || (SELECT && fine)) {
 #pragma unroll 1
                 for (int t = 0; t < batches; ++t) {
-                    const uint32_t top4 = batch(cur, top);
+                    const uint32_t top4 = sum.add(cur, top);
                     if (FIXED == 2 && !fine) filled(top4);
 #pragma unroll
                     for (int u = 0; u < kBatch; ++u) {
@@ -938,12 +1106,12 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             } else {
 #pragma unroll 1
                 for (int t = 0; t < batches; t += 2) {
-                    const uint32_t t0 = batch(cur, top);
+                    const uint32_t t0 = sum.add(cur, top);
                     if (SELECT) filled(t0);
                     if (FIXED) load_next(cur);
                     else load(wrow, t + 2, cur);
                     if (t + 1 < batches) {
-                        const uint32_t t1 = batch(nxt, top);
+                        const uint32_t t1 = sum.add(nxt, top);
                         if (SELECT) filled(t1);
                         if (FIXED) load_next(nxt);
                     } else if (FIXED) {                                                       // the next part begins with what lies in nxt
@@ -956,10 +1124,9 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             }
 
             // Maximum and sum of the part, then of the row.
-            kmax = __reduce_max_sync(kFull, top_key(m2));
-            float x0, x1, x2, x3;
-            unpack2(s0, x0, x1); unpack2(s1, x2, x3);
-            sum_all = warp_sum((x0 + x1) + (x2 + x3));
+            kmax = sum.max_key();
+            ref = sum.ref;
+            sum_all = sum.total();
             if (SHARE) {
                 if (lane == 0) { sh.key[wrow] = kmax; sh.ref[wrow] = ref; sh.sum[wrow] = sum_all; }
             } else if (FIXED && lane == wrow) {
@@ -982,149 +1149,193 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
             sum_all *= expf(ref - lmax);
         }
 
-        if (SELECT && (!SHARE || wfirst < nwarps)) {
-            // The row's own warp, or all warps of the first block.
-            const int tw = SHARE ? warp : 0, tws = SHARE ? nwarps : 1;
-            auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
-            // With three quarters as many selected as there are groups the bound holds back little: the logits are
-            // counted instead (V = 256, K = 64, 32768 rows: 438 -> 120 us).
-            const bool few_groups = fine && 4 * K > 3 * r.nv;
-            uint32_t theta = kKeyNegInf;
-            int n = 0;
-            bool counted = few_groups;
-            if (!few_groups) {
-                // The bound: the K-th largest group maximum (any value that exactly K of them reach will do), searched
-                // by one warp with all maxima in its registers.  The search is a chain of ten steps or so: shared among
-                // eight warps a step cost 1300 cycles (guards, a shared counter, a barrier), 14400 of the 34000 cycles of a
-                // row of 128256 logits by itself; now 5350 of 22000.
-                const int S = NW * ns, words = (S + 1) >> 1;
-                uint32_t mx[kSlots / 2];                                                      // two maxima each
-                if (tw == 0) {
-                    if (S & 1) reinterpret_cast<uint16_t*>(slots)[(S >> 1) * 64 + lane * 2 + 1] = 0xffffu;   // reaches nothing
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < kSlots / 2; ++i) mx[i] = i < words ? slots[i * 32 + lane] : kNoValue2;
-                    auto reach = [&](uint32_t h2, auto first) {                               // of this lane's first words
-                        constexpr int A = SHARE ? 4 : 1;                                      // one sum where other rows fill the gaps
-                        __half2 c[A];
-#pragma unroll
-                        for (int i = 0; i < A; ++i) c[i] = __float2half2_rn(0.f);
-#pragma unroll
-                        for (int i = 0; i < decltype(first)::value; ++i) c[i % A] = __hadd2(c[i % A], __hge2(as_half2(mx[i]), as_half2(h2)));
-                        if constexpr (A > 1) c[0] = __hadd2(__hadd2(c[0], c[1]), __hadd2(c[2], c[3]));
-                        return __half2int_rn(__hadd(__low2half(c[0]), __high2half(c[0])));
-                    };
-                    uint32_t hi = kmax + 1, down = 256;                                       // first downwards from the maximum, then between
-#pragma unroll 1
-                    while (hi - theta > 1) {
-                        const uint32_t mid = down && kmax - theta > down ? kmax - down : theta + ((hi - theta) >> 1), h2 = bits_of_key(mid) * 0x10001u;
-                        const int c = __reduce_add_sync(kFull, words <= 8 ? reach(h2, std::integral_constant<int, 8>{})
-                                                                          : reach(h2, std::integral_constant<int, kSlots / 2>{}));
-                        if (c >= K) { theta = mid; down = 0; } else { hi = mid; down *= 4; }
-                        if (c == K) break;
-                    }
-                    if (SHARE && lane == 0) local_sh.theta = theta;
-                }
-                sync();
-                if (SHARE) theta = local_sh.theta;
-                // Places for a warp's items among the team's: `before` of this lane's first, from a running total.
-                auto place = [&](int mine, int* shared_total, int& total) {
-                    int all;
-                    int at = warp_excl_scan(mine, lane, all);
-                    int base = total;
-                    if (SHARE) {
-                        if (lane == 0) base = atomicAdd(shared_total, all);
-                        base = __shfl_sync(kFull, base, 0);
-                    }
-                    total += all;                                                             // SHARE: of this warp only
-                    return base + at;
-                };
-                // The groups that reach it.
-                const uint32_t th2 = bits_of_key(theta) * 0x10001u;
-                int n_codes = 0;
-                uint32_t hits[2] = {0u, 0u};                                                  // bits i, 16 + i: the maxima of word i (of 16 + i)
-                auto hit = [&](uint32_t w, int i) { return __hge2_mask(as_half2(w), as_half2(th2)) & (0x10001u << (i & 15)); };
-                if (SHARE) {                                                                  // two warps at least: 16 words at most
-#pragma unroll 4
-                    for (int i = 0; tw + i * tws < words; ++i) hits[0] |= hit(slots[(tw + i * tws) * 32 + lane], i);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < kSlots / 2; ++i) hits[i >> 4] |= hit(mx[i], i);
-                }
-                int at = place(__popc(hits[0]) + __popc(hits[1]), &local_sh.n_codes, n_codes);
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    for (uint32_t m = hits[h]; m; m &= m - 1) {
-                        const int b = __ffs(m) - 1, i = tw + (16 * h + (b & 15)) * tws;
-                        if (at < kCodes) codes[at] = (uint16_t)((2 * i + (b >> 4)) * 32 + lane);
-                        ++at;
-                    }
-                sync();
-                if (SHARE) n_codes = local_sh.n_codes;
-                if (n_codes <= kCodes) {
-                    // their logits at or above the bound; head and tail of the row are a turn of the last warp's own.  A
-                    // lane takes one batch of a group where warps share the row (turns are memory latencies: 1700 cycles
-                    // each), else all of a group (where rows fill the GPU the lanes' divisions cost more than a turn).
-                    const int steps = fine ? 1 : wide, items = SHARE ? n_codes * steps : n_codes;
-                    const bool ends_turn = tw == tws - 1 && (r.head > 0 || r.head + 8 * r.nv < r.V);
-#pragma unroll 1
-                    for (int i0 = tw * 32 - (ends_turn ? 32 * tws : 0); i0 < items; i0 += 32 * tws) {
-                        const bool mine = i0 >= 0 && i0 + lane < items;
-                        const int ci = !mine ? 0 : SHARE ? (i0 + lane) / steps : i0 + lane, first = SHARE && mine ? i0 + lane - ci * steps : 0;
-                        const int code = mine ? codes[ci] : 0, sl = code >> 5, w = sl / ns, ls = sl - w * ns;
-                        const int turns = SHARE || i0 < 0 ? 1 : steps;
-#pragma unroll 1
-                        for (int st = first; st < first + turns; ++st) {
-                            const int t = fine ? ls >> 2 : ls * wide + st;
-                            const int vb = w * 32 + (code & 31) + (t * kBatch + (fine ? ls & 3 : 0)) * 32 * NW;
-                            uint4 q[kBatch];
-#pragma unroll
-                            for (int u = 0; u < kBatch; ++u) {
-                                const int v = vb + u * 32 * NW;
-                                q[u] = mine && v < r.nv && !(fine && u) ? (FIXED == 2 && r.phase ? group_across(r, v) : SHARE ? r.body[v] : __ldg(r.body + v)) : all4(kNoValue2);
-                            }
-                            if (i0 < 0) q[0] = row_ends(r, lane);
-                            uint32_t m = 0;                                                    // bits p, 16 + p: the halves of word p
-#pragma unroll
-                            for (int u = 0; u < kBatch; ++u) {
-                                const uint32_t w4[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) m |= __hge2_mask(as_half2(w4[j]), as_half2(th2)) & (0x10001u << (4 * u + j));
-                            }
-                            for (int to = place(__popc(m), &local_sh.n_list, n); m; m &= m - 1, ++to) {
-                                const int b = __ffs(m) - 1, u = (b >> 2) & 3;
-                                const int v = i0 >= 0 ? vb + u * 32 * NW : lane == 0 ? -1 : r.nv;
-                                const int e = r.head + 8 * v + 2 * (b & 3) + (b >> 4);
-                                if (to < kListCap) list[to] = order_word<W>(key_of(__half_as_ushort(SHARE ? r.row[e] : __ldg(r.row + e))), e);   // a first-level hit
-                            }
-                        }
-                    }
-                }
-                sync();
-                if (SHARE) n = local_sh.n_list;
-                counted = n_codes > kCodes || n > kListCap;
-            }
-            if (counted) {
-                sync();                                                                   // all have read the totals
-                n = select_by_count<SHARE, W>(r.row, r.V, K, theta, kmax, list, local_sh.by_count, tw, tws, lane);
-            }
-            W* sorted = reinterpret_cast<W*>(slots);                                      // the maxima are done with
-            order_list<W>(list, n, sorted, SHARE ? (int)threadIdx.x : lane, tws * 32, sync);
-            if (tw == 0) {
-                // NaN logits reach no bound: a row with fewer than K others is filled up with candidate 0 at weight 0
-                for (int i = n + lane; i < K; i += 32) sorted[i] = order_word<W>(kKeyNegInf, 0);
-                __syncwarp();
-                emit_selected<W>(a, rowi, sorted, lmax, sum_all, lane);
-            }
-        }
-        if (lane == 0 && wfirst == 0) {
-            const float lse = lmax + logf(sum_all);
-            if (a.lse) a.lse[rowi] = lse;
-            if (a.tokens && (a.logp2 || a.step_exp || a.bits_out)) put_surprisal(a, rowi, r.row, lse);
-        }
+        if (SELECT && (!SHARE || wfirst < nwarps))                                        // the row's own warp, or all warps of the first block
+            select_row<SHARE, FIXED == 2, W>(a, rowi, r, NW, ns, fine ? 0 : wide, slots, codes, list,
+                                             reinterpret_cast<W*>(slots), local_sh, SHARE ? warp : 0, SHARE ? nwarps : 1, kmax, lmax, sum_all, lane, []() {});
+        if (lane == 0 && wfirst == 0) put_row(a, rowi, r.row, lmax + logf(sum_all));
         __syncwarp();
         if (SHARE) meet();                                                                // the row's shared state is free again
     }
+}
+
+// Long rows, many of them: a block an SM, in which teams of warps stream rows (a row's parts to a team's warps) and
+// other warps select from the rows that have passed, so that the end of a row (the bound's search, a second
+// look at a few groups, the ordering: 12000 cycles for a warp, chains for the most part) takes place under the
+// streaming of the next rows.  With a warp a row all of them reach their ends together, and memory idles meanwhile.
+// The block's rows (blockIdx, + gridDim, ...; those inside the position ranges) are numbered q = 0, 1, ...: team
+// q % teams streams row q into buffer q % kFinishers, which the finishing warp of that number reads.  Full and
+// empty buffers are hardware barriers (the waiting side sleeps); the number of teams divides the number of
+// buffers, so that a buffer belongs to one team and its barrier's generations cannot mix.  A buffer of a team of 4
+// is free again as soon as the finishing warp has its maxima in registers; teams of 8 have time, and 16 KB more L1 are
+// worth more (4096 rows of 128256: 204 us, 191).
+// The logits come through a ring in shared memory that every lane fills for itself, asynchronously (held in
+// registers across rows they were spilled: 4096 rows of 128256 434 us).
+// What bounds it: the streaming warps' latency a batch (1700 to 2000 cycles, 16 warps, 130 KB in flight an SM).
+// 4096 rows of 128256, K = 64: 265 -> 191 us (without a selection 168, the copy rate 160); 16384 rows of 32000: 257 ->
+// 223, of 50001: 355 -> 324.
+constexpr int kStreamers = 16, kFinishers = 8, kMostTeam = 8;           // warps of a block: streaming, finishing; most of a team
+constexpr int kRing = 4;                                                // batches of a warp on their way
+static_assert(2 * kFinishers <= 16, "a block has 16 barriers");
+template <int TEAM, class W>
+struct __align__(16) PipeRow {
+    static constexpr bool kEarly = TEAM < 8;                            // see above
+    uint32_t slots[16 * kSlots];
+    uint16_t codes[kCodes];
+    W list[kEarly ? 2 * kListCap : kListCap];
+    float ref[kMostTeam], sum[kMostTeam];
+    uint32_t key[kMostTeam];
+    __device__ __forceinline__ W* sorted() { return kEarly ? list + kListCap : reinterpret_cast<W*>(slots); }
+};
+template <int TEAM>
+__device__ __forceinline__ void wait_barrier(int id) { asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(32 * (TEAM + 1)) : "memory"); }
+template <int TEAM>
+__device__ __forceinline__ void arrive_barrier(int id) { asm volatile("barrier.arrive %0, %1;" ::"r"(id), "n"(32 * (TEAM + 1)) : "memory"); }
+
+// The block's rows of numbers first, first + step, ...
+struct PipeRows {
+    long long at;
+    int q, step;
+    __device__ __forceinline__ PipeRows(const TopkArgs& a, int first, int step_) : at(next_row(a, blockIdx.x, gridDim.x)), q(0), step(step_) { skip(a, first); }
+    __device__ __forceinline__ void skip(const TopkArgs& a, int rows) {
+        if (a.pos_begin || a.pos_end) {
+            for (int i = 0; i < rows && at < a.N; ++i) at = next_row(a, at + gridDim.x, gridDim.x);
+        } else {
+            at += (long long)rows * gridDim.x;
+        }
+        q += rows;
+    }
+    __device__ __forceinline__ void next(const TopkArgs& a) { skip(a, step); }
+};
+template <int TEAM>
+struct PipeCut {                                                        // a warp's share of a row
+    int batches, wide, ns;
+    bool fine;
+    __device__ __forceinline__ explicit PipeCut(int nv) {
+        constexpr int per = kBatch * 32 * TEAM;
+        batches = (nv + per - 1) / per;
+        fine = TEAM * batches * kBatch <= kSlots;
+        wide = (TEAM * batches + kSlots - 1) / kSlots;
+        ns = fine ? batches * kBatch : (batches + wide - 1) / wide;
+    }
+};
+
+template <int TEAM, class W>
+__device__ __forceinline__ void pipe_stream(const TopkArgs& a, PipeRow<TEAM, W>* rows, uint4* ring, int team, int w, int lane) {
+    constexpr int per = kBatch * 32 * TEAM, kTeams = kStreamers / TEAM;
+    static_assert(kFinishers % kTeams == 0, "a buffer belongs to one team, which meets at its barriers in the order of its rows");
+    const int first = w * 32 + lane;                                                          // this lane's first group of a row
+    PipeRows to_load(a, team, kTeams), row = to_load;
+    // A lane copies what it will read itself: kRing batches of kBatch groups.
+    const uint4* src = nullptr;
+    int left_nv = 0, into = 0;                                                                // of the row being copied: groups from this lane's next one on
+    auto open_row = [&]() {
+        if (to_load.at >= a.N) return;
+        const RowView r = row_view(a.logits + to_load.at * (long long)a.V, a.V);
+        src = r.body + first; left_nv = r.nv - w * 32;
+    };
+    auto copy_next = [&]() {                                                                  // on into the team's next row
+        if (to_load.at < a.N) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(ring + into * (kBatch * 32));
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u)
+                if (lane + u * 32 * TEAM < left_nv)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + u * 512), "l"(src + u * 32 * TEAM) : "memory");
+            into = into + 1 == kRing ? 0 : into + 1;
+            src += per; left_nv -= per;
+            if (left_nv + w * 32 <= 0) { to_load.next(a); open_row(); }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    open_row();
+#pragma unroll 1
+    for (int i = 0; i < kRing - 1; ++i) copy_next();
+    int at = 0;                                                                               // the ring's batch to be read
+#pragma unroll 1
+    for (; row.at < a.N; row.next(a)) {
+        const RowView r = row_view(a.logits + row.at * (long long)a.V, a.V);
+        const PipeCut<TEAM> cut(r.nv);
+        const int b = row.q % kFinishers;
+        PipeRow<TEAM, W>& to = rows[b];
+        auto put_slot = [&](int slot, uint32_t top2) {                                        // slot s of a lane: half s & 1 of word (s / 2, lane)
+            const int sl = w * cut.ns + slot;
+            reinterpret_cast<uint16_t*>(to.slots)[(sl >> 1) * 64 + lane * 2 + (sl & 1)] = (uint16_t)hmax2_bits(top2, top2 >> 16);
+        };
+        uint32_t group2 = kNegInf2;
+        int left = cut.wide, slot = 0;
+        const bool has_ends = w == 0 && (r.head > 0 || r.head + 8 * r.nv < r.V);
+        const uint4 ends = has_ends ? row_ends(r, lane) : all4(kNoValue2);                    // read now, taken at the row's end
+        RowSum sum;
+#pragma unroll 1
+        for (int t = 0; t < cut.batches; ++t) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
+            uint4 g[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) g[u] = ring[at * (kBatch * 32) + u * 32];
+            if ((t + 1) * per > r.nv) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) if (first + t * per + u * 32 * TEAM >= r.nv) g[u] = all4(kNegInf2);
+            }
+            at = at + 1 == kRing ? 0 : at + 1;
+            copy_next();                                                                      // over the batch before this one
+            if (t == 0) {
+                sum.begin(g, g[0], false);
+                if (row.q >= kFinishers) wait_barrier<TEAM>(kFinishers + b);                        // the row that was there has been read
+            }
+            uint32_t top[kBatch];
+            const uint32_t top4 = sum.add(g, top);
+            if (cut.fine) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) put_slot(t * kBatch + u, top[u]);
+            } else {
+                group2 = hmax2_bits(group2, top4);
+                if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = cut.wide; }
+            }
+        }
+        if (!cut.fine && left != cut.wide) put_slot(slot, group2);
+        if (has_ends) {
+            auto real = [](uint32_t v) { const uint32_t m = __vcmpeq2(v, kNoValue2); return (v & ~m) | (kNegInf2 & m); };
+            const uint4 g[kBatch] = {make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)), all4(kNegInf2), all4(kNegInf2), all4(kNegInf2)};
+            uint32_t top[kBatch];
+            sum.add(g, top);
+        }
+        const uint32_t kmax = sum.max_key();
+        const float total = sum.total();
+        if (lane == 0) { to.key[w] = kmax; to.ref[w] = sum.ref; to.sum[w] = total; }
+        __syncwarp();
+        arrive_barrier<TEAM>(b);
+    }
+}
+template <int TEAM, class W>
+__device__ __forceinline__ void pipe_finish(const TopkArgs& a, PipeRow<TEAM, W>& from, StreamShared& unused, int b, int lane) {
+    constexpr bool kEarly = PipeRow<TEAM, W>::kEarly;
+    PipeRows row(a, b, kFinishers);
+#pragma unroll 1
+    while (row.at < a.N) {
+        const long long rowi = row.at;
+        const RowView r = row_view(a.logits + rowi * (long long)a.V, a.V);
+        const PipeCut<TEAM> cut(r.nv);
+        row.next(a);
+        wait_barrier<TEAM>(b);
+        const bool on = lane < TEAM;
+        const uint32_t kmax = __reduce_max_sync(kFull, on ? from.key[lane] : 0u);
+        const float lmax = val_of_key(kmax);
+        const float sum_all = warp_sum(on ? from.sum[lane] * expf(from.ref[lane] - lmax) : 0.f);
+        select_row<false, false, W>(a, rowi, r, TEAM, cut.ns, cut.fine ? 0 : cut.wide, from.slots, from.codes, from.list, from.sorted(), unused, 0, 1, kmax, lmax,
+                                    sum_all, lane, [&]() { if (kEarly && row.at < a.N) arrive_barrier<TEAM>(kFinishers + b); });   // the next row may be put there
+        if (lane == 0) put_row(a, rowi, r.row, lmax + logf(sum_all));
+        __syncwarp();
+        if (!kEarly && row.at < a.N) arrive_barrier<TEAM>(kFinishers + b);
+    }
+}
+template <int TEAM, class W>
+__global__ void __launch_bounds__(32 * (kStreamers + kFinishers), 1) topk_pipe_kernel(const TopkArgs a) {
+    extern __shared__ __align__(16) unsigned char pipe_raw[];
+    __shared__ StreamShared unused;
+    PipeRow<TEAM, W>* rows = reinterpret_cast<PipeRow<TEAM, W>*>(pipe_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, f = warp - kStreamers;
+    zero_tickets(a);
+    if (f < 0) pipe_stream<TEAM, W>(a, rows, reinterpret_cast<uint4*>(rows + kFinishers) + warp * (kRing * kBatch * 32) + lane, warp / TEAM, warp % TEAM, lane);
+    else pipe_finish<TEAM, W>(a, rows[f], unused, f, lane);
 }
 
 }  // namespace
@@ -1163,6 +1374,15 @@ static cudaError_t launch_stream(TopkArgs a, int sms, cudaStream_t st, int* few_
     return launch_kernel(kern, blocks, per_block * 32, smem, st, a.chained && *few_blocks > 0, cluster, a);
 }
 
+template <int TEAM, class W>
+static cudaError_t launch_pipe(const TopkArgs& a, int sms, cudaStream_t st) {
+    const size_t smem = kFinishers * sizeof(PipeRow<TEAM, W>) + (size_t)kStreamers * kRing * kBatch * 32 * sizeof(uint4);
+    const cudaError_t e = cudaFuncSetAttribute(topk_pipe_kernel<TEAM, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return launch_kernel(topk_pipe_kernel<TEAM, W>, (unsigned)std::min<long long>(a.N, sms), 32 * (kStreamers + kFinishers), smem, st, false, 1, a);
+}
+
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
     *few_blocks = 0;
     if (a.N <= 0) return cudaSuccess;
@@ -1172,6 +1392,11 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
     const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     if (a.K <= kFinal) {
         const int fixed = !(a.step_exp || a.bits_out) ? 0 : vec ? 1 : 2;
+// Long rows, from two an SM on (300 rows of 32000: 17.8 -> 17.1 us, of 128256: 36.6 -> 33).  A row's costs beside its
+        // batches weigh more the shorter it is: teams of 4 warps for rows up to 65536 (16384 rows of 32000: 245 us with 8, 223),
+        // of 8 beyond (4096 rows of 128256: 201 us with 4, 191), and a warp a row for short ones (16384 rows of 16384: 151 us
+        // against 162).  Calls with an adaptive step need sums of the same parts at any number of rows.
+        if (!fixed && a.V >= 24576 && a.N >= 2ll * sms) return a.V <= 65536 ? launch_pipe<4, uint32_t>(a, sms, st) : launch_pipe<8, unsigned long long>(a, sms, st);
         if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st, few_blocks)
                                : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st, few_blocks) : launch_stream<true, 2, uint32_t>(a, sms, st, few_blocks);
         return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st, few_blocks)

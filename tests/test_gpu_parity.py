@@ -992,6 +992,58 @@ def test_topk_rows_of_every_layout(dev, orc, N, V, K, off):
     np.testing.assert_allclose(only["lse"].cpu().numpy(), lse, atol=2e-5, rtol=1e-6)
 
 
+# lengths at the two team sizes' limits, batches that fill a slot and that do not, every alignment; K at its limits
+@pytest.mark.parametrize("N,V,K,off", [(297, 24576, 64, 0), (310, 24577, 128, 3), (1300, 24583, 1, 7), (299, 65536, 100, 0), (600, 65537, 33, 5),
+                                       (300, 128256, 64, 0), (300, 131071, 128, 1)])
+def test_topk_rows_streamed_by_teams(dev, N, V, K, off):
+    """Calls of many long rows against the same rows a hundred at a time (which a block or a cluster selects): the
+    selected and their weights bit for bit, sums in another order (binary32, tolerance of the other layouts).  Rows
+    with ties beyond the lists, with NaN, with fewer finite logits than K and ascending ones among them."""
+    g = torch.Generator(device=dev).manual_seed(N + V)
+    buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
+    rows = buf[off:off + N * V].view(N, V)
+    for i in range(0, N, 100):
+        k = min(100, N - i)
+        rows[i:i + k] = torch.randn(k, V, generator=g, device=dev) * torch.exp(4 * torch.rand(k, 1, generator=g, device=dev) - 1)
+    rows[1] = torch.round(rows[1])
+    rows[2] = torch.sort(rows[2]).values
+    rows[3, ::3] = float("nan")
+    rows[4, 1:] = -float("inf")
+    rows[5] = 1.0
+    rows[N - 1] = torch.round(rows[N - 1] * 4) / 4
+    tok = torch.randint(0, V, (N,), generator=g, device=dev, dtype=torch.int32)
+    ctx = plc.Context(torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02)
+    out = ctx.topk_softmax(rows, tok)
+    few = [ctx.topk_softmax(rows[i:i + 100], tok[i:i + 100]) for i in range(0, N, 100)]
+    ref = {k: torch.cat([f[k] for f in few]) for k in out}
+    assert torch.equal(out["idx"], ref["idx"]) and torch.equal(out["w"], ref["w"])
+    for k, tol in (("lse", 2e-5), ("zk", 2e-5), ("logp2", 1e-4)):
+        assert torch.allclose(out[k], ref[k], rtol=2e-5, atol=tol, equal_nan=True), k
+
+
+def test_rows_streamed_by_teams_inside_position_ranges(dev):
+    """A batch whose rows teams stream, with position ranges (one of them empty), against its sessions one by one."""
+    S, n, V, K, d, CP = 5, 90, 24584, 16, 32, 32
+    g = torch.Generator(device=dev).manual_seed(5)
+    T = torch.randn(1, 2, 1, V, d, generator=g, device=dev).half()
+    logits = (torch.randn(S, n, V, generator=g, device=dev) * 3).half()
+    kv = torch.randn(1, 2, S, 1, n, d, generator=g, device=dev).half()
+    ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
+    mc = ctx.max_chunks(n)
+    begin, end = [0, 13, 40, 89, 7], [90, 90, 40, 90, 71]
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+
+    def coded(kv, logits, b, e):
+        st = plc.StreamSet(logits.shape[0] * ctx.W, mc, 1 << 22, dev)
+        ctx.encode(kv, logits, st, i32(b), i32(e))
+        assert ctx.sync_status() == plc.OK
+        return [st.chunk(i).tobytes() for i in range(logits.shape[0] * ctx.W * mc)]
+
+    whole = coded(kv, logits, begin, end)
+    alone = sum((coded(kv[:, :, s:s + 1].contiguous(), logits[s:s + 1].contiguous(), begin[s:s + 1], end[s:s + 1]) for s in range(S)), [])
+    assert whole == alone and any(whole)
+
+
 @pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
 def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
     """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
