@@ -65,6 +65,8 @@ struct plc_ctx {
     bool finite;                    // T holds neither infinities nor NaN
     int2* pairs;
     int* step_exp;                  // [positions] adaptive step exponents
+    float* s1;                      // [s1_cap][tables] variance terms of large calls, or null
+    long long s1_cap;               // positions
     long long pairs_cap;            // positions
     uint16_t* staging;
     unsigned long long staging_words_per_warp;
@@ -159,17 +161,37 @@ int padded_k(const plc_config& cfg) {
 }
 bool pair_index(const plc_config& cfg) { return (long long)cfg.vocab * cfg.head_dim * 2 >= (1ll << 32); }
 
+// Whether a context keeps what it can do without (a second, bf16 copy of its model's weights; variance terms): only
+// while that leaves the caller three quarters of the memory that is free.
+bool keep_extra(size_t bytes) {
+    size_t free_b = 0, total_b = 0;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4;
+}
+
+// Variance terms formed ahead of the gather (launch_variance): what a call's may take, and from where on the extra
+// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms; 64 streams x 999 positions, 256 KB: 282 -> 277
+// us; 2 x 512: 144 -> 153).
+constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 128 * 1024;
+
 plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (positions <= c->pairs_cap) return PLC_OK;
     if (c->pairs) cudaFree(c->pairs);
     if (c->step_exp) cudaFree(c->step_exp);
-    c->pairs = nullptr; c->step_exp = nullptr; c->pairs_cap = 0;
+    if (c->s1) cudaFree(c->s1);
+    c->pairs = nullptr; c->step_exp = nullptr; c->s1 = nullptr; c->pairs_cap = c->s1_cap = 0;
     if (cudaMalloc(&c->pairs, sizeof(int2) * (size_t)positions * padded_k(c->cfg)) != cudaSuccess ||
         cudaMalloc(&c->step_exp, sizeof(int) * (size_t)positions) != cudaSuccess) {
         cudaGetLastError();                     // the launches that follow ask for the last error
         return PLC_E_CUDA;
     }
     c->pairs_cap = positions;
+    // Where they would take more than a quarter of the free memory, and for calls beyond, the gather forms them itself.
+    const size_t a_position = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads;
+    const long long most = std::min<long long>(positions, (long long)(kMostVariance / a_position));
+    if (c->cfg.variant == PLC_PRED_TOPK && (size_t)most * a_position >= kLeastVariance && keep_extra((size_t)most * a_position)) {
+        if (cudaMalloc(&c->s1, (size_t)most * a_position) == cudaSuccess) c->s1_cap = most;
+        else { cudaGetLastError(); c->s1 = nullptr; }
+    }
     return PLC_OK;
 }
 
@@ -216,13 +238,6 @@ LinearShape linear_shape(const plc_ctx* c, long long rows) {
     sh.resident = c->resident;
     sh.group = layer_group(c, rows, sh.ncols);
     return sh;
-}
-
-// Whether a context keeps a second, bf16 copy of its model's weights: only while that leaves the caller
-// three quarters of the memory that is free when it is created.
-bool keep_weights(size_t bytes) {
-    size_t free_b = 0, total_b = 0;
-    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4;
 }
 
 // Builds a context's model with the kept weights where there is memory for them and for what building them
@@ -334,12 +349,12 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
     if (ok && T_dev) {
         unsigned int not_finite = 0;
         ok = cudaMemset(c->ticket, 0, sizeof(unsigned int)) == cudaSuccess &&
-             launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
+             launch_rownorm(c->T, c->rownorm2, cfg->vocab, 2 * cfg->n_layers * cfg->n_kv_heads, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
              cudaMemcpy(&not_finite, c->ticket, sizeof(unsigned int), cudaMemcpyDeviceToHost) == cudaSuccess;
         c->finite = not_finite == 0;
     }
     if (ok && T_dev && cfg->variant == PLC_PRED_DENSE) {     // operands of every layer, once
-        c->resident = keep_weights((size_t)rows * cfg->head_dim * 2);
+        c->resident = keep_extra((size_t)rows * cfg->head_dim * 2);
         ok = with_or_without_weights(c, [&]() {
             const DenseShape sh = dense_shape(c, 0);
             return sh.nt_all <= 65536 && cudaMalloc(&c->model, dense_model_bytes(sh, c->model_off)) == cudaSuccess &&
@@ -349,7 +364,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
     if (ok && lin) {
         c->lin_E = static_cast<const __half*>(lin->E_dev); c->lin_A = static_cast<const __half*>(lin->A_dev);
         c->lin_c = static_cast<const __half*>(lin->c_dev); c->lin_dm = lin->d_model;
-        c->resident = keep_weights((size_t)cfg->n_layers * 2 * cfg->n_kv_heads * cfg->head_dim * lin->d_model * 2);
+        c->resident = keep_extra((size_t)cfg->n_layers * 2 * cfg->n_kv_heads * cfg->head_dim * lin->d_model * 2);
         ok = with_or_without_weights(c, [&]() {
             const LinearShape sh = linear_shape(c, 0);
             return cudaMalloc(&c->model, linear_model_bytes(sh, c->model_off)) == cudaSuccess &&
@@ -363,7 +378,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
 
 plc_status plc_destroy(plc_ctx* c) {
     if (!c) return PLC_E_INVALID;
-    cudaFree(c->rownorm2); cudaFree(c->pairs); cudaFree(c->step_exp); cudaFree(c->staging);
+    cudaFree(c->rownorm2); cudaFree(c->pairs); cudaFree(c->step_exp); cudaFree(c->s1); cudaFree(c->staging);
     cudaFree(c->ticket); cudaFree(c->status); cudaFree(c->counters); cudaFree(c->dense_scratch); cudaFree(c->model);
     for (int k = 0; k < 3; ++k)
         for (cudaEvent_t e : c->prof_ev[k]) cudaEventDestroy(e);
@@ -481,6 +496,15 @@ static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bo
     return PLC_OK;
 }
 
+// Variance terms of a call that has room for them.
+static cudaError_t form_variance(const plc_ctx* c, CodecArgs& a, cudaStream_t st) {
+    const long long rows = (long long)a.S * a.n;
+    const size_t bytes = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads * rows;
+    if (rows > c->s1_cap || bytes < kLeastVariance) return cudaSuccess;
+    a.s1 = c->s1; a.behind = 0;
+    return launch_variance(a, st);
+}
+
 // tokens_dev non-null <=> adaptive call
 static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* logits_dev, const int32_t* tokens_dev,
                               int32_t S, int32_t n, const int32_t* pos_begin_dev, const int32_t* pos_end_dev,
@@ -506,6 +530,7 @@ static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* log
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
+    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     codec_schedule(a, 2 * a.sh.L * a.sh.H, &c->last_nq, &c->last_g);
     cudaEvent_t* pk = prof_pair(c, 0);
     if (pk) cudaEventRecord(pk[0], st);
@@ -551,6 +576,7 @@ static plc_status decode_impl(plc_ctx* c, const plc_streams* in, const void* log
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
+    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     codec_schedule(a, 2 * a.sh.L * a.sh.H, &c->last_nq, &c->last_g);
     cudaEvent_t* pk = prof_pair(c, 1);
     if (pk) cudaEventRecord(pk[0], st);

@@ -33,24 +33,81 @@ constexpr int kThreads = kWarpsPerBlock * 32;
 constexpr int kBlocksPerSM = 5, kGatherBlocks = 4;
 constexpr int kGatherWarps = kGatherBlocks * kWarpsPerBlock, kFarWarps = 24;
 
+// Squared row norms out[v][t] of tables T[t][v][D]: a warp takes a candidate's rows in kNormTables tables,
+// whose norms are one sector of the output.
+constexpr int kNormTables = 8;
 template <int D>
-__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows,
+__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, int V, int tables,
                                                       unsigned int* not_finite) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
     const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    const int c0 = first_comp<D>(lane);
-    for (long long r = warp; r < rows; r += nw) {
-        float v[G];
+    const int c0 = first_comp<D>(lane), groups = (tables + kNormTables - 1) / kNormTables;
+    for (long long item = warp; item < (long long)groups * V; item += nw) {
+        const int t0 = (int)(item / V) * kNormTables, v = (int)(item % V);
+        float mine = 0.f;
+#pragma unroll 4
+        for (int j = 0; j < kNormTables; ++j) {
+            if (t0 + j >= tables) break;
+            const __half* row = T + ((long long)(t0 + j) * V + v) * D + c0;
+            float x[G];
 #pragma unroll
-        for (int g = 0; g < G; ++g) v[g] = __half2float(T[r * D + c0 + g]);
-        float s = warp_norm2<G>(v);
-        if (lane == 0) {
-            out[r] = s;
-            if (!(s < __int_as_float(0x7f800000))) *not_finite = 1u;          // squares of finite binary16 values sum to less
+            for (int g = 0; g < G; ++g) x[g] = __half2float(row[g]);
+            const float s = warp_norm2<G>(x);
+            if (lane == j) mine = s;
         }
+        if (!(mine < __int_as_float(0x7f800000))) *not_finite = 1u;           // squares of finite binary16 values sum to less
+        if (lane < kNormTables && t0 + lane < tables) out[(long long)v * tables + t0 + lane] = mine;
     }
+}
+
+// Variance terms s1[row][t] = sum_k w_k ||T[t][idx_k]||^2 of every (position, table), ahead of the gather kernels: the
+// norms of a candidate lie beside each other for all tables, so a warp reads them for 32 * VEC tables at
+// once, where the gather, one table a warp, takes a sector a candidate (64 of its 242 L1 wavefronts a vector).  0.36 ms
+// for 1024 tables x 16384 positions, where the gather becomes 1.0 ms shorter.
+// The additions are those of predict's own sum and warp_sum (lane l: candidates l, l + 32, ...; then lanes
+// l and l ^ 16, l ^ 8, ...), so both give the same bits.  Lanes: `width` of them (a power of two) side by side in
+// the tables, 32 / width positions a warp.
+template <int VEC>
+__global__ void __launch_bounds__(256) variance_kernel(const CodecArgs a, int width, int row_shift, int load_shift) {
+    using Vec = std::conditional_t<VEC == 4, float4, float2>;
+    const int lane = threadIdx.x & 31, W = 2 * a.sh.L * a.sh.H, Kp = a.sh.Kp, iters = Kp >> load_shift, per_warp = 32 / width;
+    const int t0 = ((int)blockIdx.y * width + (lane & (width - 1))) * VEC;
+    const long long N = (long long)a.S * a.n, row = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per_warp + lane / width;
+    if (row >= N || t0 >= W) return;
+    if (a.pos_begin || a.pos_end) {
+        const int s = (int)(row / a.n), i = (int)(row % a.n);
+        if (i < (a.pos_begin ? a.pos_begin[s] : 0) || i >= (a.pos_end ? a.pos_end[s] : a.n)) return;   // no pairs there
+    }
+    const int2* pairs = a.pairs + row * Kp;
+    float stack[5][VEC], sum[VEC];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        const int l = (i & 1) * 16 + (i >> 1 & 1) * 8 + (i >> 2 & 1) * 4 + (i >> 3 & 1) * 2 + (i >> 4);
+#pragma unroll
+        for (int j = 0; j < VEC; ++j) sum[j] = 0.f;
+#pragma unroll 2
+        for (int k = l; k < Kp; k += 32) {
+            const int2 pr = __ldg(pairs + (k & ((1 << load_shift) - 1)) * iters + (k >> load_shift));
+            const uint32_t at = (uint32_t)pr.x >> row_shift;
+            const Vec n = __ldg(reinterpret_cast<const Vec*>(a.rownorm2 + (size_t)at * W + t0));
+            const float w = __int_as_float(pr.y);
+            sum[0] = __fmaf_rn(w, n.x, sum[0]); sum[1] = __fmaf_rn(w, n.y, sum[1]);
+            if constexpr (VEC == 4) { sum[2] = __fmaf_rn(w, n.z, sum[2]); sum[3] = __fmaf_rn(w, n.w, sum[3]); }
+        }
+        int level = 0;
+#pragma unroll
+        for (; level < 5 && (i >> level & 1); ++level)
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) sum[j] = stack[level][j] + sum[j];
+        if (level < 5)
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) stack[level][j] = sum[j];
+    }
+    float* out = a.s1 + row * W + t0;
+    if constexpr (VEC == 4) *reinterpret_cast<float4*>(out) = make_float4(sum[0], sum[1], sum[2], sum[3]);
+    else *reinterpret_cast<float2*>(out) = make_float2(sum[0], sum[1]);
 }
 
 // ZR: the zero-rate rule (Thm. 3) is on; a separate instantiation keeps the plain coder's loop free of it.
@@ -98,7 +155,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
             continue;
         }
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
+        const float* n2 = a.rownorm2 + it.t;
         uint32_t x = kRansL;
         int wp = cap_words;
         unsigned n_escapes = 0;
@@ -106,10 +163,13 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
         float ideal = 0.f;                                                         // this lane's share, if asked for
         const int2* gp = nullptr;
         const __half* kvp = nullptr;
+        const float* s1_at = nullptr;
         int buf = 0;
         if (!FROM_OPEN) {
             if (!DENSE) {
-                gp = a.pairs + ((long long)it.s * a.n + it.p0 + it.P - 1) * Kp;  // last position first
+                const long long row = (long long)it.s * a.n + it.p0 + it.P - 1;  // last position first
+                gp = a.pairs + row * Kp;
+                if (a.s1) s1_at = a.s1 + row * Wt + it.t;
                 __syncwarp();                                                    // slot 0 is free again
                 prefetch_pairs(sp0, gp, Kp, lane);
             }
@@ -151,7 +211,8 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, Wt, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                    if (s1_at) s1_at -= Wt;
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
                 int zero_q = ZR ? a.sh.zero_q : 0;
@@ -237,8 +298,9 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
         auto read_word = [&](int i) { return (uint32_t)__ldg(words + min(i, last)); };   // past the end: the last word
         int rp = 0;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
+        const float* n2 = a.rownorm2 + it.t;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
+        const float* s1_at = !DENSE && a.s1 ? a.s1 + ((long long)it.s * a.n + it.p0) * Wt + it.t : nullptr;
         __syncwarp();
         if (!DENSE) prefetch_pairs(sp0, gp, Kp, lane);
         int buf = 0;
@@ -265,7 +327,8 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, Wt, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                if (s1_at) s1_at += Wt;
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
             int zero_q = ZR ? a.sh.zero_q : 0;
@@ -356,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
         const Item it = bulk_item(a, item);
         if (it.P <= 0) continue;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
+        const float* n2 = a.rownorm2 + it.t;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
         __syncwarp();
         prefetch_pairs(sp0, gp, Kp, lane);
@@ -374,7 +437,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D, true>(col, n2, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D, true>(col, n2, Wt, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -451,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) append_quantise_kerne
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + t, Wt, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;
@@ -529,14 +592,26 @@ static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
     a.sched_g = (int)g; a.sched_nq = nq;
 }
 
-cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, unsigned int* not_finite, cudaStream_t st) {
+cudaError_t launch_rownorm(const __half* T, float* out, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st) {
     return dispatch_d(d, [&](auto D) {
-        long long blocks = (rows + 7) / 8;
-        if (blocks > (long long)sm_count() * 16) blocks = (long long)sm_count() * 16;
-        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, rows, not_finite);
+        const long long blocks = std::min(((long long)(tables + kNormTables - 1) / kNormTables * V + 7) / 8, (long long)sm_count() * 16);
+        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, V, tables, not_finite);
         count_launch();
         return cudaGetLastError();
     });
+}
+
+static int log2_of(int v) { return v > 1 ? 1 + log2_of(v >> 1) : 0; }
+
+cudaError_t launch_variance(const CodecArgs& a, cudaStream_t st) {
+    const int W = 2 * a.sh.L * a.sh.H, vec = W % 4 == 0 ? 4 : 2;
+    int width = 1;
+    while (width < 32 && width * vec < W) width *= 2;
+    const long long rows = (long long)a.S * a.n, a_block = 8 * (32 / width);
+    auto kern = vec == 4 ? variance_kernel<4> : variance_kernel<2>;
+    kern<<<dim3((unsigned)((rows + a_block - 1) / a_block), (unsigned)((W + width * vec - 1) / (width * vec))), 256, 0, st>>>(a, width, a.row_form == kRowIndices ? 0 : log2_of(2 * a.sh.d), log2_of(256 / a.sh.d));
+    count_launch();
+    return cudaGetLastError();
 }
 
 cudaError_t launch_encode(const CodecArgs& a0, cudaStream_t st) {

@@ -65,7 +65,8 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
 // offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
 // multiple of 2 ROWS (the padding has weight 0 and a valid offset).  table, n2: the table's rows and
-// their squared norms, the same pointers in every lane.
+// their squared norms (`tables` apart), s1_at: the position's variance term where it was formed ahead
+// (launch_variance), or null; the same pointers in every lane.
 // What bounds it: issue slots (per row and lane 8 conversions, 4 packed FMAs, a load), with the rows'
 // latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
 // beside its load.
@@ -79,7 +80,7 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // block-per-chunk kernel, 128 streams x 4096 positions, both calls 2075 -> 2002); the others lose loads in flight
 // (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
 template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN>
-__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, int row_form,
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, size_t tables, const float* s1_at, int row_form,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
@@ -89,10 +90,14 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
     auto row_at = [&](int off) { return LANE_BASE ? lane_table + (uint32_t)off : table + ((uint32_t)off + lane_off); };
     // variance term first: its row-norm loads are in flight while the rows are gathered
     float s1 = 0.f;
-    for (int k = lane; k < Kp; k += 32) {
-        const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
-        const uint32_t at = row_form == kRowIndices ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
-        s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
+    if (s1_at) {                                  // formed ahead: lane 0 brings the sum into the butterfly below
+        if (lane == 0) s1 = __ldg(s1_at);
+    } else {
+        for (int k = lane; k < Kp; k += 32) {
+            const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
+            const uint32_t at = row_form == kRowIndices ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
+            s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at * tables), s1);
+        }
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
     if (WIDEN ? row_form == kRowOffsets : row_form != kRowIndices) {

@@ -1044,6 +1044,39 @@ def test_rows_streamed_by_teams_inside_position_ranges(dev):
     assert whole == alone and any(whole)
 
 
+# two and four tables a lane, tables beyond one warp's, several positions a warp; K below, at and off the lanes of a warp
+@pytest.mark.parametrize("L,H,d,K,n,ranges", [(1, 1, 32, 17, 5000, False), (3, 1, 64, 64, 1500, True), (4, 4, 32, 100, 300, False), (2, 33, 32, 5, 80, True),
+                                              (1, 8, 128, 64, 600, False), (1, 4, 256, 33, 1100, True)])
+def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
+    """A batch large enough for its variance terms to be formed ahead gives the same bytes as its sessions one by
+    one, in pieces too small for it."""
+    S, V, CP = 4, 500, 50
+    _, logits, T, kv = make_workload(31 + d + K, S, n, L, H, d, V, K, pp=20.0)
+    T, logits, kv = T.to(dev), logits.to(dev), kv.to(dev)
+    ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
+    assert 4 * S * n * ctx.W >= 128 * 1024
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+    begin, end = ([0, n // 3, 7, n // 2], [n, n, n // 2, n // 2]) if ranges else ([0] * S, [n] * S)
+
+    def coded(kv, logits, b, e):
+        mc = ctx.max_chunks(logits.shape[1])
+        st = plc.StreamSet(logits.shape[0] * ctx.W, mc, 4 * logits.shape[0] * logits.shape[1] * ctx.W * d + (1 << 20), dev)
+        ctx.encode(kv, logits, st, i32(b), i32(e))
+        assert ctx.sync_status() == plc.OK
+        return [[st.chunk(i * mc + c).tobytes() for c in range(mc)] for i in range(logits.shape[0] * ctx.W)]
+
+    whole = coded(kv, logits, begin, end)
+    step = max(CP, 28000 // ctx.W // CP * CP)                        # positions of a piece: whole chunks, fewer than 32768 vectors
+    for s in range(S):
+        alone = [[] for _ in range(ctx.W)]
+        for p in range(begin[s], end[s], step):
+            q = min(p + step, end[s])
+            for t, chunks in enumerate(coded(kv[:, :, s:s + 1, :, p:q].contiguous(), logits[s:s + 1, p:q].contiguous(), [0], [q - p])):
+                alone[t] += chunks
+        for t in range(ctx.W):
+            assert [c for c in whole[s * ctx.W + t] if c] == alone[t]
+
+
 @pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
 def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
     """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
