@@ -124,13 +124,20 @@ __device__ __forceinline__ void slot_get_entries(const int* slot, int lane, EncE
     }
 }
 
-size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc, bool roomy) {
+__host__ __device__ constexpr size_t coop_smem(int warps, int Kp, int d, bool dense, bool enc, bool roomy) {
     const int NP = coop_predictors(warps), G = d / 32, slot = (enc ? 64 : 32) * G + kTailWords;
     return (size_t)(dense ? 0 : NP * 2 * Kp * (int)sizeof(int2)) + (size_t)2 * NP * slot * 4 + (enc ? 0 : ring_bytes(G, roomy));
 }
 
-// All warps of the block meet here; the two roles reach it from different places in the code.
-__device__ __forceinline__ void block_barrier() { asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)(32 + 32 * coop_predictors(blockDim.x >> 5))) : "memory"); }
+// All warps of a chunk meet here, from different places in the code: those of the block, or of a group of GW.
+template <int GW>
+struct Meet {
+    int group;
+    __device__ __forceinline__ void operator()() const {
+        if constexpr (GW == 0) asm volatile("barrier.sync 1, %0;" ::"r"((unsigned)(32 + 32 * coop_predictors(blockDim.x >> 5))) : "memory");
+        else asm volatile("barrier.sync %0, %1;" ::"r"(1 + group), "n"(32 * GW) : "memory");
+    }
+};
 
 // The block's current chunk.
 struct CoopItem {
@@ -149,9 +156,9 @@ struct CoopShared {
 
 // Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a batch; the inputs
 // of the next are fetched while it works on one.
-template <int D, bool DENSE, bool ENC, class Tab>
+template <int D, bool DENSE, bool ENC, int GW, class Tab>
 __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
-                                             const LaneCode& lc) {
+                                             const Meet<GW>& meet, const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
     const int P = sh.item.it.P, Kp = DENSE ? 0 : a.sh.Kp, n_batches = (P + NP - 1) / NP, c0 = first_comp<D>(lane);
@@ -302,7 +309,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
             if (lane == 0) sh.meta[b & 1][w] = SlotMeta{s, qp - kQMin, esc, 0};
             __syncwarp();                                                      // readers of the pair slot are done
         }
-        block_barrier();
+        meet();
         finish(b - 1);
 #pragma unroll
         for (int g = 0; g < G; ++g) mu_old[g] = mu[g];
@@ -311,7 +318,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
         s_old = s; e_old = e; esc_old = esc;
         __syncwarp();                                                          // the slot's readers are done before it is filled again
     }
-    block_barrier();
+    meet();
     finish(n_batches - 1);
     if (ENC && a.dbg.ideal) {
         ideal = warp_sum(ideal);
@@ -320,8 +327,9 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
 }
 
 // Coder of the block's chunk, one batch behind the predictions.
-template <int D, bool ENC, bool ROOMY, class Tab>
-__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const LaneCode& lc) {
+template <int D, bool ENC, bool ROOMY, int GW, class Tab>
+__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const Meet<GW>& meet,
+                                          const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
     const int P = sh.item.it.P, n_batches = (P + NP - 1) / NP;
@@ -333,7 +341,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
         int wp = cap_words, n_skipped = 0;
         unsigned n_escapes = 0;
         for (int b = 0; b < n_batches; ++b) {
-            block_barrier();                                                   // batch b is there
+            meet();                                                   // batch b is there
             const int cnt = min(NP, P - b * NP);
             int* slot = slots + (b & 1) * NP * SW;
             const SlotMeta* meta = sh.meta[b & 1];
@@ -383,7 +391,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                 }
             }
         }
-        block_barrier();
+        meet();
         uint8_t* dst = reserve_chunk(a, sh.item.it.slot, x, cap_words - wp, lane, P, n_escapes, n_skipped);
         if (lane == 0) { sh.dst = dst; sh.wp = wp; }
     } else {
@@ -415,7 +423,7 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
             }
         };
         for (int b = 0; b < n_batches; ++b) {
-            block_barrier();                                                   // the classes of batch b are there
+            meet();                                                   // the classes of batch b are there
             const int cnt = min(NP, P - b * NP);
             int* slot = slots + (b & 1) * NP * SW;
             SlotMeta* meta = sh.meta[b & 1];
@@ -455,26 +463,38 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
                 }
             }
         }
-        block_barrier();
+        meet();
         bad = bad || x != kRansL || rp != nwords;
         if (__any_sync(kFull, bad) && lane == 0) atomicOr(a.status, kStCorrupt);
         asm volatile("cp.async.wait_all;" ::: "memory");                       // of a damaged chunk: nothing may land later
     }
 }
 
+// GW: warps of a chunk's group, several groups a block (decoding where predictions come from memory: the coder's
+// chain is all that takes time then, and one block of eight coders an SM shares the 33 KB of tables that keep blocks
+// of one coder to four an SM), or 0: the block has one chunk.
+constexpr int kGroupWarps = 4;
+template <int D>
+constexpr int kGroups = D == 256 ? 4 : 8;                // by the registers
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
-template <int D, bool DENSE, bool ENC, bool ROOMY>
-__global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
+template <int D, bool DENSE, bool ENC, bool ROOMY, int GW = 0>
+__global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : kCoopMaxWarps * 32, GW || D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
+    static_assert(GW == 0 || (DENSE && !ENC), "staging is addressed by block");
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
-    __shared__ CoopShared sh;
+    __shared__ CoopShared shared[GW ? kGroups<D> : 1];
     // Warps go to an SM's four schedulers in turn.  A block that has its SM to itself (16 warps) leaves the
-    // coder's scheduler to the coder: the warps that would share it stay idle.
-    const int lane = threadIdx.x & 31, hw = threadIdx.x >> 5, NP = coop_predictors(blockDim.x >> 5);   // NP predicting warps
-    const int warp = NP < (int)(blockDim.x >> 5) - 1 ? ((hw & 3) == 0 ? (hw == 0 ? 0 : -1) : hw - (hw >> 2)) : hw;
+    // coder's scheduler to the coder: the warps that would share it stay idle.  The coders of groups lie on
+    // different schedulers.
+    const int lane = threadIdx.x & 31, hw = threadIdx.x >> 5, warps = GW ? GW : (int)(blockDim.x >> 5), NP = coop_predictors(warps);   // NP predicting warps
+    const int group = GW ? hw / GW : 0;
+    const int warp = GW ? (hw - group) & (GW - 1) : NP < warps - 1 ? ((hw & 3) == 0 ? (hw == 0 ? 0 : -1) : hw - (hw >> 2)) : hw;
     const int Kp = DENSE ? 0 : a.sh.Kp;
-    int* slots = reinterpret_cast<int*>(g_pair_smem + NP * 2 * Kp);                          // [2][NP] slots
+    CoopShared& sh = shared[group];
+    int2* pairs = GW ? reinterpret_cast<int2*>(reinterpret_cast<unsigned char*>(g_pair_smem) + group * coop_smem(GW, 0, D, DENSE, ENC, ROOMY)) : g_pair_smem;
+    int* slots = reinterpret_cast<int*>(pairs + NP * 2 * Kp);                                // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
+    const Meet<GW> meet{group};
     const LaneCode lc = lane_code(lane);
     load_tables(&tb, ENC ? reinterpret_cast<const Tab*>(&a.tables->enc) : reinterpret_cast<const Tab*>(&a.tables->wide));
     chain_wait();
@@ -482,6 +502,8 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
     const unsigned per_table = (unsigned)a.S * (unsigned)a.chunks, total = (unsigned)Wl * per_table;
     if (ENC) clear_unused_slots(a, DENSE ? a.dense_t0 : 0, Wl);
     QueueCursor qc = DENSE ? QueueCursor{0, 0} : queue_of_this_sm(a);
+    auto all_meet = [&]() { if (GW) meet(); else __syncthreads(); };
+    if (GW) __syncthreads();                                                   // the tables are there
 
     for (;;) {
         if (warp == 0) {
@@ -507,14 +529,14 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, D == 256 ? 1 : 2) coop_ker
                 sh.item = ci;
             }
         }
-        __syncthreads();
+        all_meet();
         const int go = sh.item.go;
         if (go < 0) break;
         if (go > 0) {
-            if (warp == 0) coop_code<D, ENC, ROOMY>(a, sh, tb, slots, ring, NP, lc);
-            else if (warp > 0) coop_predict<D, DENSE, ENC>(a, sh, tb, g_pair_smem + (warp - 1) * 2 * Kp, slots, warp - 1, NP, lc);
+            if (warp == 0) coop_code<D, ENC, ROOMY, GW>(a, sh, tb, slots, ring, NP, meet, lc);
+            else if (warp > 0) coop_predict<D, DENSE, ENC, GW>(a, sh, tb, pairs + (warp - 1) * 2 * Kp, slots, warp - 1, NP, meet, lc);
         }
-        __syncthreads();                                                       // the chunk is coded; its item has been read
+        all_meet();                                                            // the chunk is coded; its item has been read
         if (ENC && go > 0 && sh.dst)
             copy_words(sh.dst, a.staging + (long long)blockIdx.x * a.staging_words_per_warp + sh.wp,
                        (int)a.staging_words_per_warp - sh.wp, threadIdx.x, blockDim.x);
@@ -533,6 +555,16 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         // there is a chunk an SM at most.
         const bool alone = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode, true) <= kMostSmem;
         const bool roomy = dense || alone;
+        // Coders alone with their chains: eight an SM, in groups of one block, once there are more chunks than the four
+        // that blocks of eight warps hold (2048 chunks of 256 positions: 745 -> 548 us with 128 components, 1180 -> 703 with 256; 1024 of 128: 337 -> 252).
+        if (dense && !encode && items > 4ll * sm_count()) {
+            auto kern = coop_kernel<d, true, false, true, kGroupWarps>;
+            const size_t smem = kGroups<d> * coop_smem(kGroupWarps, 0, d, true, false, true);
+            const cudaError_t e = allow_smem(kern, smem);
+            if (e != cudaSuccess) return e;
+            count_launch();
+            return launch_kernel(kern, (unsigned)sm_count(), 32 * kGroupWarps * kGroups<d>, smem, st, false, 1, a);
+        }
         auto kern = dense ? (encode ? coop_kernel<d, true, true, true> : coop_kernel<d, true, false, true>)
                   : roomy ? (encode ? coop_kernel<d, false, true, true> : coop_kernel<d, false, false, true>)
                           : (encode ? coop_kernel<d, false, true, false> : coop_kernel<d, false, false, false>);

@@ -1044,6 +1044,41 @@ def test_rows_streamed_by_teams_inside_position_ranges(dev):
     assert whole == alone and any(whole)
 
 
+@pytest.mark.parametrize("d,CP,n,kind", [(128, 17, 133, "plain"), (64, 64, 520, "escapes"), (32, 3, 30, "ranges"), (256, 20, 155, "escapes"), (128, 90, 700, "zero")])
+def test_coders_in_groups(dev, d, CP, n, kind):
+    """Decoding with the full-vocabulary predictor and more than four chunks an SM: eight coders a block (four of 256
+    components).  The symbols that were coded come back; sessions decoded one by one, a block per chunk, give the same
+    bits.  Chunks shorter and longer than the word ring, empty ones, escapes, skipped positions."""
+    S, L, H, V = 6, 2, 4, 300
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    delta = 1.0 / 256 if kind == "escapes" else 0.02
+    _, logits, T, kv = make_workload(40 + d + CP, S, n, L, H, d, V, 16, pp=6.0, sigma=0.1)
+    if kind == "escapes":
+        kv.view(-1)[::701] += 60.0
+    T, logits, kv = T.to(dev), logits.to(dev), kv.to(dev)
+    ctx = plc.Context(T, 16, delta, chunk_pos=CP, variant=plc.PRED_DENSE, zero_rate_D=0.5 if kind == "zero" else 0.0)
+    W, mc = ctx.W, ctx.max_chunks(n)
+    assert 4 * sms < S * W * mc <= 40 * sms and W * mc <= 4 * sms
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+    begin, end = ([0, 1, n, n // 2, 5, 0], [n, n - 1, n, n, 5, 1]) if kind == "ranges" else ([0] * S, [n] * S)
+    st = plc.StreamSet(S * W, mc, 6 * S * n * W * d + (1 << 20), dev)
+    sym = torch.zeros(S, n, W, d, dtype=torch.int32, device=dev)
+    ctx.encode(kv, logits, st, i32(begin), i32(end), debug=plc.DebugBuffers(sym.data_ptr(), None, None))
+    out, back = torch.zeros(kv.shape, dtype=torch.float32, device=dev), torch.zeros_like(sym)
+    ctx.decode(st, logits, out, i32(begin), i32(end), debug=plc.DebugBuffers(back.data_ptr(), None, None))
+    assert ctx.sync_status() == plc.OK and torch.equal(back, sym)
+    stats = ctx.stats()
+    assert stats.n_escapes > 0 or kind != "escapes"
+    assert (stats.skipped_vectors > 0) == (kind == "zero")
+    alone = torch.zeros_like(out)
+    for s in range(S):
+        one = plc.StreamSet(W, mc, 16, dev)
+        one.payload, one.capacity, one.total_bytes = st.payload, st.capacity, st.total_bytes
+        one.chunk_offset, one.chunk_bytes = st.chunk_offset[s * W * mc:(s + 1) * W * mc], st.chunk_bytes[s * W * mc:(s + 1) * W * mc]
+        ctx.decode(one, logits[s:s + 1].contiguous(), alone[:, :, s:s + 1], i32(begin[s:s + 1]), i32(end[s:s + 1]))
+    assert ctx.sync_status() == plc.OK and torch.equal(alone, out)
+
+
 # two and four tables a lane, tables beyond one warp's, several positions a warp; K below, at and off the lanes of a warp
 @pytest.mark.parametrize("L,H,d,K,n,ranges", [(1, 1, 32, 17, 5000, False), (3, 1, 64, 64, 1500, True), (4, 4, 32, 100, 300, False), (2, 33, 32, 5, 80, True),
                                               (1, 8, 128, 64, 600, False), (1, 4, 256, 33, 1100, True)])
