@@ -21,9 +21,9 @@
 namespace plc {
 namespace {
 
-constexpr int kCoopMaxWarps = 16;
+constexpr int kCoopMaxWarps = 32;
 // Predicting warps of a block.
-__host__ __device__ constexpr int coop_predictors(int warps) { return warps == kCoopMaxWarps ? 3 * warps / 4 : warps - 1; }
+__host__ __device__ constexpr int coop_predictors(int warps) { return warps >= 16 ? 3 * warps / 4 : warps - 1; }
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
 // Ring size: a position takes at most G * (2 * 15 + 32 + 64) words.  The roomy ring holds two positions at a
 // time for the coder (of blocks whose predictions come from memory, or that have an SM to themselves);
@@ -476,14 +476,18 @@ __device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, co
 constexpr int kGroupWarps = 4;
 template <int D>
 constexpr int kGroups = D == 256 ? 4 : 8;                // by the registers
+// Warps of a block that has its SM to itself: 24 beside the coder (7 idle), since a prediction's latency (4000 cycles)
+// is what an encoder waits for (2 x 512 positions of 64: 55 -> 43 us, 64 chunks of 256 x 128: 121 -> 92; with 12).
+template <int D>
+constexpr int kAloneWarps = D == 256 ? 16 : 32;
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
 template <int D, bool DENSE, bool ENC, bool ROOMY, int GW = 0>
-__global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : kCoopMaxWarps * 32, GW || D == 256 ? 1 : 2) coop_kernel(const CodecArgs a) {
+__global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 32 * kAloneWarps<D> : 512, GW || D == 256 || (ROOMY && !DENSE) ? 1 : 2) coop_kernel(const CodecArgs a) {
     static_assert(GW == 0 || (DENSE && !ENC), "staging is addressed by block");
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
     __shared__ CoopShared shared[GW ? kGroups<D> : 1];
-    // Warps go to an SM's four schedulers in turn.  A block that has its SM to itself (16 warps) leaves the
+    // Warps go to an SM's four schedulers in turn.  A block that has its SM to itself (16 warps or more) leaves the
     // coder's scheduler to the coder: the warps that would share it stay idle.  The coders of groups lie on
     // different schedulers.
     const int lane = threadIdx.x & 31, hw = threadIdx.x >> 5, warps = GW ? GW : (int)(blockDim.x >> 5), NP = coop_predictors(warps);   // NP predicting warps
@@ -551,9 +555,11 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         const bool dense = a.mu_dense != nullptr;
         const long long items = (long long)(dense ? a.dense_nt : 2 * a.sh.L * a.sh.H) * a.S * a.chunks;
         // Seven warps beside the coder: with three the coder waits, with fifteen two coders an SM are too few
-        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  A block of sixteen where
-        // there is a chunk an SM at most.
-        const bool alone = items <= sm_count() && coop_smem(kCoopMaxWarps, a.sh.Kp, d, dense, encode, true) <= kMostSmem;
+        // (encode + decode of 4096 positions x 128 streams: 2.9, 2.3 and 3.2 ms).  Where there is a chunk an SM at
+        // most, a block of kAloneWarps, or of 16 (streamed predictions, and where the pairs of more do not fit).
+        const int most = dense ? 16 : kAloneWarps<d>;
+        const int fit = coop_smem(most, a.sh.Kp, d, dense, encode, true) <= kMostSmem ? most : 16;
+        const bool alone = items <= sm_count() && coop_smem(fit, a.sh.Kp, d, dense, encode, true) <= kMostSmem;
         const bool roomy = dense || alone;
         // Coders alone with their chains: eight an SM, in groups of one block, once there are more chunks than the four
         // that blocks of eight warps hold (2048 chunks of 256 positions: 745 -> 548 us with 128 components, 1180 -> 703 with 256; 1024 of 128: 337 -> 252).
@@ -568,7 +574,7 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         auto kern = dense ? (encode ? coop_kernel<d, true, true, true> : coop_kernel<d, true, false, true>)
                   : roomy ? (encode ? coop_kernel<d, false, true, true> : coop_kernel<d, false, false, true>)
                           : (encode ? coop_kernel<d, false, true, false> : coop_kernel<d, false, false, false>);
-        const int warps = alone ? kCoopMaxWarps : kCoopMaxWarps / 2;
+        const int warps = alone ? fit : 8;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode, roomy);
         const cudaError_t e = allow_smem(kern, smem);
         if (e != cudaSuccess) return e;
