@@ -61,7 +61,8 @@ using namespace plc;
 struct plc_ctx {
     plc_config cfg;
     const __half* T;
-    float* rownorm2;
+    float* rownorm2;                // squared row norms [tables][V]
+    float* norms_by_row;            // the same [V][tables], for variance terms formed ahead (where the memory is to be had)
     bool finite;                    // T holds neither infinities nor NaN
     int2* pairs;
     int* step_exp;                  // [positions] adaptive step exponents
@@ -169,9 +170,9 @@ bool keep_extra(size_t bytes) {
 }
 
 // Variance terms formed ahead of the gather (launch_variance): what a call's may take, and from where on the extra
-// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms; 64 streams x 999 positions, 256 KB: 282 -> 277
-// us; 2 x 512: 144 -> 153).
-constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 128 * 1024;
+// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms; 128 x 1024 with the adaptive step 736 -> 729 us; 64 x
+// 999, half of them in range: 3 % slower; 2 x 512: 144 -> 153).
+constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 256 * 1024;
 
 plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (positions <= c->pairs_cap) return PLC_OK;
@@ -188,7 +189,7 @@ plc_status ensure_pairs(plc_ctx* c, long long positions) {
     // Where they would take more than a quarter of the free memory, and for calls beyond, the gather forms them itself.
     const size_t a_position = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads;
     const long long most = std::min<long long>(positions, (long long)(kMostVariance / a_position));
-    if (c->cfg.variant == PLC_PRED_TOPK && (size_t)most * a_position >= kLeastVariance && keep_extra((size_t)most * a_position)) {
+    if (c->norms_by_row && (size_t)most * a_position >= kLeastVariance && keep_extra((size_t)most * a_position)) {
         if (cudaMalloc(&c->s1, (size_t)most * a_position) == cudaSuccess) c->s1_cap = most;
         else { cudaGetLastError(); c->s1 = nullptr; }
     }
@@ -207,7 +208,7 @@ CodecArgs base_args(const plc_ctx* c) {
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
     a.tables = c->tables;
-    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs; 
+    a.T = c->T; a.rownorm2 = c->rownorm2; a.norms_by_row = c->norms_by_row; a.pairs = c->pairs; 
     a.row_form = pair_index(c->cfg) ? kRowIndices : c->finite ? kRowOffsets : kRowOffsetsPlain;
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
@@ -348,8 +349,13 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
     if (ok && T_dev) {
         unsigned int not_finite = 0;
+        if (cfg->variant == PLC_PRED_TOPK && keep_extra(sizeof(float) * (size_t)rows) &&
+            cudaMalloc(&c->norms_by_row, sizeof(float) * (size_t)rows) != cudaSuccess) {
+            cudaGetLastError();
+            c->norms_by_row = nullptr;
+        }
         ok = cudaMemset(c->ticket, 0, sizeof(unsigned int)) == cudaSuccess &&
-             launch_rownorm(c->T, c->rownorm2, cfg->vocab, 2 * cfg->n_layers * cfg->n_kv_heads, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
+             launch_rownorm(c->T, c->rownorm2, c->norms_by_row, cfg->vocab, 2 * cfg->n_layers * cfg->n_kv_heads, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
              cudaMemcpy(&not_finite, c->ticket, sizeof(unsigned int), cudaMemcpyDeviceToHost) == cudaSuccess;
         c->finite = not_finite == 0;
     }
@@ -378,7 +384,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
 
 plc_status plc_destroy(plc_ctx* c) {
     if (!c) return PLC_E_INVALID;
-    cudaFree(c->rownorm2); cudaFree(c->pairs); cudaFree(c->step_exp); cudaFree(c->s1); cudaFree(c->staging);
+    cudaFree(c->rownorm2); cudaFree(c->norms_by_row); cudaFree(c->pairs); cudaFree(c->step_exp); cudaFree(c->s1); cudaFree(c->staging);
     cudaFree(c->ticket); cudaFree(c->status); cudaFree(c->counters); cudaFree(c->dense_scratch); cudaFree(c->model);
     for (int k = 0; k < 3; ++k)
         for (cudaEvent_t e : c->prof_ev[k]) cudaEventDestroy(e);

@@ -33,11 +33,11 @@ constexpr int kThreads = kWarpsPerBlock * 32;
 constexpr int kBlocksPerSM = 5, kGatherBlocks = 4;
 constexpr int kGatherWarps = kGatherBlocks * kWarpsPerBlock, kFarWarps = 24;
 
-// Squared row norms out[v][t] of tables T[t][v][D]: a warp takes a candidate's rows in kNormTables tables,
-// whose norms are one sector of the output.
+// Squared row norms of tables T[t][v][D], out[t][v] and (unless it is null) by_row[v][t]: a warp takes a candidate's rows in
+// kNormTables tables, whose norms are one sector of the latter.
 constexpr int kNormTables = 8;
 template <int D>
-__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, int V, int tables,
+__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, float* __restrict__ by_row, int V, int tables,
                                                       unsigned int* not_finite) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
@@ -58,7 +58,10 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__
             if (lane == j) mine = s;
         }
         if (!(mine < __int_as_float(0x7f800000))) *not_finite = 1u;           // squares of finite binary16 values sum to less
-        if (lane < kNormTables && t0 + lane < tables) out[(long long)v * tables + t0 + lane] = mine;
+        if (lane < kNormTables && t0 + lane < tables) {
+            out[(long long)(t0 + lane) * V + v] = mine;
+            if (by_row) by_row[(long long)v * tables + t0 + lane] = mine;
+        }
     }
 }
 
@@ -91,7 +94,7 @@ __global__ void __launch_bounds__(256) variance_kernel(const CodecArgs a, int wi
         for (int k = l; k < Kp; k += 32) {
             const int2 pr = __ldg(pairs + (k & ((1 << load_shift) - 1)) * iters + (k >> load_shift));
             const uint32_t at = (uint32_t)pr.x >> row_shift;
-            const Vec n = __ldg(reinterpret_cast<const Vec*>(a.rownorm2 + (size_t)at * W + t0));
+            const Vec n = __ldg(reinterpret_cast<const Vec*>(a.norms_by_row + (size_t)at * W + t0));
             const float w = __int_as_float(pr.y);
             sum[0] = __fmaf_rn(w, n.x, sum[0]); sum[1] = __fmaf_rn(w, n.y, sum[1]);
             if constexpr (VEC == 4) { sum[2] = __fmaf_rn(w, n.z, sum[2]); sum[3] = __fmaf_rn(w, n.w, sum[3]); }
@@ -155,7 +158,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
             continue;
         }
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + it.t;
+        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         uint32_t x = kRansL;
         int wp = cap_words;
         unsigned n_escapes = 0;
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, Wt, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
                     if (s1_at) s1_at -= Wt;
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
         auto read_word = [&](int i) { return (uint32_t)__ldg(words + min(i, last)); };   // past the end: the last word
         int rp = 0;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + it.t;
+        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
         const float* s1_at = !DENSE && a.s1 ? a.s1 + ((long long)it.s * a.n + it.p0) * Wt + it.t : nullptr;
         __syncwarp();
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, Wt, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
                 if (s1_at) s1_at += Wt;
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
         const Item it = bulk_item(a, item);
         if (it.P <= 0) continue;
         const char* col = reinterpret_cast<const char*>(a.T + (size_t)it.t * a.sh.V * D);
-        const float* n2 = a.rownorm2 + it.t;
+        const float* n2 = a.rownorm2 + (size_t)it.t * a.sh.V;
         const int2* gp = a.pairs + ((long long)it.s * a.n + it.p0) * Kp;
         __syncwarp();
         prefetch_pairs(sp0, gp, Kp, lane);
@@ -437,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D, true>(col, n2, Wt, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D, true>(col, n2, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -514,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) append_quantise_kerne
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + t, Wt, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;
@@ -592,10 +595,10 @@ static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
     a.sched_g = (int)g; a.sched_nq = nq;
 }
 
-cudaError_t launch_rownorm(const __half* T, float* out, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st) {
+cudaError_t launch_rownorm(const __half* T, float* out, float* by_row, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st) {
     return dispatch_d(d, [&](auto D) {
         const long long blocks = std::min(((long long)(tables + kNormTables - 1) / kNormTables * V + 7) / 8, (long long)sm_count() * 16);
-        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, V, tables, not_finite);
+        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, by_row, V, tables, not_finite);
         count_launch();
         return cudaGetLastError();
     });

@@ -65,7 +65,7 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
 // offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
 // multiple of 2 ROWS (the padding has weight 0 and a valid offset).  table, n2: the table's rows and
-// their squared norms (`tables` apart), s1_at: the position's variance term where it was formed ahead
+// their squared norms, s1_at: the position's variance term where it was formed ahead
 // (launch_variance), or null; the same pointers in every lane.
 // What bounds it: issue slots (per row and lane 8 conversions, 4 packed FMAs, a load), with the rows'
 // latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
@@ -80,13 +80,13 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // block-per-chunk kernel, 128 streams x 4096 positions, both calls 2075 -> 2002); the others lose loads in flight
 // (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
 template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN>
-__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, size_t tables, const float* s1_at, int row_form,
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, const float* s1_at, int row_form,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
     const int h = lane / R, iters = Kp / ROWS;
     const uint32_t lane_off = 16u * (lane % R);
-    const char* lane_table = table + lane_off;
+    const char* lane_table = LANE_BASE ? table + lane_off : table;
     auto row_at = [&](int off) { return LANE_BASE ? lane_table + (uint32_t)off : table + ((uint32_t)off + lane_off); };
     // variance term first: its row-norm loads are in flight while the rows are gathered
     float s1 = 0.f;
@@ -96,7 +96,7 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
         for (int k = lane; k < Kp; k += 32) {
             const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
             const uint32_t at = row_form == kRowIndices ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
-            s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at * tables), s1);
+            s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
         }
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
@@ -134,7 +134,7 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
 #pragma unroll 1
         for (int it = 0; it < iters; ++it) {
             const int2 pr = sp[h * iters + it];
-            add_row<false>(lane_table + (size_t)(uint32_t)pr.x * unit, __int_as_float(pr.y), 0u, acc2);
+            add_row<false>(table + ((size_t)(uint32_t)pr.x * unit + lane_off), __int_as_float(pr.y), 0u, acc2);
         }
     }
     float acc[8];

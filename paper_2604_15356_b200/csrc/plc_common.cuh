@@ -247,7 +247,8 @@ enum { kRowOffsets = 0, kRowOffsetsPlain = 1, kRowIndices = 2 };
 struct CodecArgs {
     CodecShape sh;
     const CoderTables* tables;                     // frequency tables of the coder
-    const __half* T; const float* rownorm2;        // [tables][V][d], [V][tables]
+    const __half* T; const float* rownorm2;        // [tables][V][d], [tables][V]
+    const float* norms_by_row;                     // [V][tables], for launch_variance
     float* s1;                                     // [S*n][tables] variance terms where they were formed ahead (launch_variance), or null
     const int2* pairs;                             // [S*n][Kp] (written by the top-K kernels, put_pair)
     int row_form;                                  // kRow...: what the pairs hold, and whether T may go through the tensor cores
@@ -318,7 +319,7 @@ cudaError_t linear_begin(const __half* logits, const LinearShape& sh, const uint
 cudaError_t linear_layers(const __half* A, int l0, int nl, const LinearShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
                           const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
 // Sets *not_finite where a row holds an infinity or NaN.
-cudaError_t launch_rownorm(const __half* T, float* out, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st);
+cudaError_t launch_rownorm(const __half* T, float* out, float* by_row, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st);
 cudaError_t launch_variance(const CodecArgs& a, cudaStream_t st);            // fills a.s1 for the pairs
 cudaError_t launch_encode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_decode(const CodecArgs& a, cudaStream_t st);

@@ -167,7 +167,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
     const long long row0 = sh.item.row0;
     const char* col = reinterpret_cast<const char*>(a.T + (size_t)t * a.sh.V * D);
     const int Wt = 2 * a.sh.L * a.sh.H;
-    const float* n2 = a.rownorm2 + t;
+    const float* n2 = a.rownorm2 + (size_t)t * a.sh.V;
     const bool zr = a.sh.zero_q != kZeroOff;
     int buf = 0;
     float m_next[G] = {}, s1_next = 0.f, ideal = 0.f;
@@ -254,7 +254,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                 if (k + NP < P) { fetch(k + NP, buf ^ 1); pairs_ready<1>(); }
                 else pairs_ready<0>();
                 buf ^= 1;
-                predict<D, false, true>(col, n2, Wt, a.s1 ? a.s1 + (row0 + p) * Wt + t : nullptr, a.row_form, sp, Kp, lane, 1.0f / D, mu, sigma2);
+                predict<D, false, true>(col, n2, a.s1 ? a.s1 + (row0 + p) * Wt + t : nullptr, a.row_form, sp, Kp, lane, 1.0f / D, mu, sigma2);
             }
             float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
             int zero_q = a.sh.zero_q;

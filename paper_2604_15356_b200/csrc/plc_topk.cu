@@ -1396,7 +1396,8 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
         // batches weigh more the shorter it is: teams of 4 warps for rows up to 65536 (16384 rows of 32000: 245 us with 8, 223),
         // of 8 beyond (4096 rows of 128256: 201 us with 4, 191), and a warp a row for short ones (16384 rows of 16384: 151 us
         // against 162).  Calls with an adaptive step need sums of the same parts at any number of rows.
-        if (!fixed && a.V >= 24576 && a.N >= 2ll * sms) return a.V <= 65536 ? launch_pipe<4, uint32_t>(a, sms, st) : launch_pipe<8, unsigned long long>(a, sms, st);
+        const bool ranges = a.pos_begin || a.pos_end;
+        if (!fixed && !ranges && a.V >= 24576 && a.N >= 2ll * sms) return a.V <= 65536 ? launch_pipe<4, uint32_t>(a, sms, st) : launch_pipe<8, unsigned long long>(a, sms, st);
         if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st, few_blocks)
                                : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st, few_blocks) : launch_stream<true, 2, uint32_t>(a, sms, st, few_blocks);
         return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st, few_blocks)

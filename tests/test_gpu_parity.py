@@ -1080,8 +1080,8 @@ def test_coders_in_groups(dev, d, CP, n, kind):
 
 
 # two and four tables a lane, tables beyond one warp's, several positions a warp; K below, at and off the lanes of a warp
-@pytest.mark.parametrize("L,H,d,K,n,ranges", [(1, 1, 32, 17, 5000, False), (3, 1, 64, 64, 1500, True), (4, 4, 32, 100, 300, False), (2, 33, 32, 5, 80, True),
-                                              (1, 8, 128, 64, 600, False), (1, 4, 256, 33, 1100, True)])
+@pytest.mark.parametrize("L,H,d,K,n,ranges", [(1, 1, 32, 17, 9000, False), (3, 1, 64, 64, 2800, True), (4, 4, 32, 100, 520, False), (2, 33, 32, 5, 130, True),
+                                              (1, 8, 128, 64, 1100, False), (1, 4, 256, 33, 2100, True)])
 def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
     """A batch large enough for its variance terms to be formed ahead gives the same bytes as its sessions one by
     one, in pieces too small for it."""
@@ -1089,7 +1089,7 @@ def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
     _, logits, T, kv = make_workload(31 + d + K, S, n, L, H, d, V, K, pp=20.0)
     T, logits, kv = T.to(dev), logits.to(dev), kv.to(dev)
     ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
-    assert 4 * S * n * ctx.W >= 128 * 1024
+    assert 4 * S * n * ctx.W >= 256 * 1024
     i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
     begin, end = ([0, n // 3, 7, n // 2], [n, n, n // 2, n // 2]) if ranges else ([0] * S, [n] * S)
 
@@ -1101,7 +1101,7 @@ def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
         return [[st.chunk(i * mc + c).tobytes() for c in range(mc)] for i in range(logits.shape[0] * ctx.W)]
 
     whole = coded(kv, logits, begin, end)
-    step = max(CP, 28000 // ctx.W // CP * CP)                        # positions of a piece: whole chunks, fewer than 32768 vectors
+    step = max(CP, 28000 // ctx.W // CP * CP)                        # positions of a piece: whole chunks, fewer than 65536 vectors
     for s in range(S):
         alone = [[] for _ in range(ctx.W)]
         for p in range(begin[s], end[s], step):
