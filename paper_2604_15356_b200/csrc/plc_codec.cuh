@@ -50,17 +50,20 @@ template <bool WIDEN>
 __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand, unsigned long long (&acc2)[4]) {
     const uint4 r = __ldg(reinterpret_cast<const uint4*>(p));
     const unsigned long long ww = pack2(w, w);
-    unsigned long long v[4];
     if constexpr (WIDEN) {
+        unsigned long long v[4];
         widen(r.x, r.y, operand, v[0], v[1]);
         widen(r.z, r.w, operand, v[2], v[3]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc2[j] = fma2(ww, v[j], acc2[j]);
     } else {
         const __half2* hp = reinterpret_cast<const __half2*>(&r);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(hp[j]); v[j] = pack2(f.x, f.y); }
+        for (int j = 0; j < 4; ++j) {
+            const float2 f = __half22float2(hp[j]);
+            acc2[j] = fma2(ww, pack2(f.x, f.y), acc2[j]);
+        }
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc2[j] = fma2(ww, v[j], acc2[j]);
 }
 // Mixture of one position for one table.  sp: the position's Kp pairs in shared memory (put_pair: byte
 // offset of the candidate's row and weight, the Kp / ROWS entries of each row group together), Kp a
