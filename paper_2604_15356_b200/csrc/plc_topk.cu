@@ -865,10 +865,9 @@ struct RowSum {
 // of a block (SHARE) or by one.  ACROSS: rows may lie off 16-byte boundaries with their groups counted from the
 // first logit.
 template <bool SHARE, bool ACROSS, class W, class Read>
-__device__ __forceinline__ void select_row(const TopkArgs& a, long long rowi, const RowView& r, int NW, int ns, int wide, uint32_t* slots, uint16_t* codes, W* list,
+__device__ __forceinline__ void select_row(const TopkArgs& a, long long rowi, const RowView& r, int NW, int ns, int wide, bool fine, uint32_t* slots, uint16_t* codes, W* list,
                                            W* sorted, StreamShared& local_sh, int tw, int tws, uint32_t kmax, float lmax, float sum_all, int lane, Read&& read) {
     const int K = a.K;
-    const bool fine = wide == 0;
     auto sync = [&]() { if (SHARE) __syncthreads(); else __syncwarp(); };
     // With three quarters as many selected as there are groups the bound holds back little: the logits are
     // counted instead (V = 256, K = 64, 32768 rows: 438 -> 120 us).
@@ -1150,7 +1149,7 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
         }
 
         if (SELECT && (!SHARE || wfirst < nwarps))                                        // the row's own warp, or all warps of the first block
-            select_row<SHARE, FIXED == 2, W>(a, rowi, r, NW, ns, fine ? 0 : wide, slots, codes, list,
+            select_row<SHARE, FIXED == 2, W>(a, rowi, r, NW, ns, wide, fine, slots, codes, list,
                                              reinterpret_cast<W*>(slots), local_sh, SHARE ? warp : 0, SHARE ? nwarps : 1, kmax, lmax, sum_all, lane, []() {});
         if (lane == 0 && wfirst == 0) put_row(a, rowi, r.row, lmax + logf(sum_all));
         __syncwarp();
@@ -1320,7 +1319,7 @@ __device__ __forceinline__ void pipe_finish(const TopkArgs& a, PipeRow<TEAM, W>&
         const uint32_t kmax = __reduce_max_sync(kFull, on ? from.key[lane] : 0u);
         const float lmax = val_of_key(kmax);
         const float sum_all = warp_sum(on ? from.sum[lane] * expf(from.ref[lane] - lmax) : 0.f);
-        select_row<false, false, W>(a, rowi, r, TEAM, cut.ns, cut.fine ? 0 : cut.wide, from.slots, from.codes, from.list, from.sorted(), unused, 0, 1, kmax, lmax,
+        select_row<false, false, W>(a, rowi, r, TEAM, cut.ns, cut.wide, cut.fine, from.slots, from.codes, from.list, from.sorted(), unused, 0, 1, kmax, lmax,
                                     sum_all, lane, [&]() { if (kEarly && row.at < a.N) arrive_barrier<TEAM>(kFinishers + b); });   // the next row may be put there
         if (lane == 0) put_row(a, rowi, r.row, lmax + logf(sum_all));
         __syncwarp();
