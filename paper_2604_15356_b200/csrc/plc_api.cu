@@ -208,8 +208,8 @@ CodecArgs base_args(const plc_ctx* c) {
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
     a.tables = c->tables;
-    a.T = c->T; a.rownorm2 = c->rownorm2; a.norms_by_row = c->norms_by_row; a.pairs = c->pairs; 
-    a.row_form = pair_index(c->cfg) ? kRowIndices : c->finite ? kRowOffsets : kRowOffsetsPlain;
+    a.T = c->T; a.rownorm2 = c->rownorm2; a.norms_by_row = c->norms_by_row; a.pairs = c->pairs;
+    a.pair_index = pair_index(c->cfg); a.finite = c->finite;
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
     return a;

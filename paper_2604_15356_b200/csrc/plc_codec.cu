@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) encode_kernel(const CodecA
                         pairs_ready<0>();
                     }
                     buf ^= 1;
-                    predict<D>(col, n2, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                    predict<D>(col, n2, s1_at, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
                     if (s1_at) s1_at -= Wt;
                 }
                 float inv_delta_p = inv_delta, inv_delta2_p = inv_delta2;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(32 * WARPS, BLOCKS) decode_kernel(const CodecA
                     pairs_ready<0>();
                 }
                 buf ^= 1;
-                predict<D>(col, n2, s1_at, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+                predict<D>(col, n2, s1_at, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
                 if (s1_at) s1_at += Wt;
             }
             float delta_p = delta, inv_delta2_p = inv_delta2;
@@ -404,8 +404,10 @@ __device__ __forceinline__ void hadamard(float (&v)[Geo<D>::G], int lane) {
 // x = eps * R, y = H x (orthonormal Hadamard), s = max |y|, b-bit mid-rise codes on [-s, s]; the
 // record is s followed by one ballot word per (register, code bit).  ENC: KV -> records;
 // otherwise records -> KV' = KV^ + eps * H y^.  One warp per (stream, chunk of positions).
-template <int D, bool ENC>
-__global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
+template <int D, bool WIDEN>
+constexpr int kRotqBlocks = WIDEN && D != 256 ? 3 : kGatherBlocks;       // an SM; see launch_rotq
+template <int D, bool ENC, bool WIDEN>
+__global__ void __launch_bounds__(kThreads, (kRotqBlocks<D, WIDEN>)) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
     const int Wt = 2 * a.sh.L * a.sh.H, H = a.sh.H, Kp = a.sh.Kp, B = rq.bits;
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) rotq_kernel(const Cod
             }
             buf ^= 1;
             float mu[G], sigma2;
-            predict<D, true>(col, n2, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+            predict<D, WIDEN, WIDEN, true>(col, n2, nullptr, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
             __syncwarp();                                                         // readers of this slot are done
             float y[G];
             if (ENC) {
@@ -517,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, kGatherBlocks) append_quantise_kerne
         float kvv[G];
         load_half_vec<G>(reinterpret_cast<const __half*>(a.kv.base) + kv_elem(a.kv, t, H, b, 0) + c0, kvv);
         float mu[G], sigma2;
-        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, nullptr, a.row_form, sp, Kp, lane, inv_d, mu, sigma2);
+        predict<D>(col, a.rownorm2 + (size_t)t * a.sh.V, nullptr, a.pair_index, sp, Kp, lane, inv_d, mu, sigma2);
         const int q = scale_class(sigma2, floor2, inv_delta2);
         const long long o = ((long long)b * Wt + t) * a.sh.chunk_pos + a.open_slot;
         if (lane == 0) a.open_q[o] = q;
@@ -612,7 +614,7 @@ cudaError_t launch_variance(const CodecArgs& a, cudaStream_t st) {
     while (width < 32 && width * vec < W) width *= 2;
     const long long rows = (long long)a.S * a.n, a_block = 8 * (32 / width);
     auto kern = vec == 4 ? variance_kernel<4> : variance_kernel<2>;
-    kern<<<dim3((unsigned)((rows + a_block - 1) / a_block), (unsigned)((W + width * vec - 1) / (width * vec))), 256, 0, st>>>(a, width, a.row_form == kRowIndices ? 0 : log2_of(2 * a.sh.d), log2_of(256 / a.sh.d));
+    kern<<<dim3((unsigned)((rows + a_block - 1) / a_block), (unsigned)((W + width * vec - 1) / (width * vec))), 256, 0, st>>>(a, width, a.pair_index ? 0 : log2_of(2 * a.sh.d), log2_of(256 / a.sh.d));
     count_launch();
     return cudaGetLastError();
 }
@@ -691,16 +693,28 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
     });
 }
 
+// Rows are widened on the tensor cores where a queue is served by a few SMs (set_queues: the tables in flight are more
+// than L2 holds), with 24 warps an SM at 80 registers (32 at 64 for 256 components); where all SMs share a queue, and for
+// T that the tensor cores cannot take, value by value with 32 warps.  Widening lets the few rows in flight that L1
+// has room for beside the shared ones do more work; where L2 holds the tables the packed conversions are the quicker
+// chain.  4000 positions, 8 x 8 heads of 128, K = 64, both calls, value by value with stretches of 32 rows / widened
+// with 32 warps / as now, us: V = 32000, skewed candidates (many queues) 1693 / 1457 / 1433, uniform 2742 / 3103 / 2616,
+// uniform K = 128 4925 / 5802 / 4720; V = 5000 (one queue) 1360 / 1480 / 1319; 4 layers (one queue) skewed 834 / 854 /
+// 814, uniform 1055 / 1290 / 996; 256 components, 4 layers, skewed 1648 / 1398 / 1355 (24 warps 1387), uniform 2725 /
+// 2744 / 2740 (3000).
 cudaError_t launch_rotq(const CodecArgs& a0, const RotqArgs& r, bool encode, cudaStream_t st) {
     CodecArgs a = a0;
     set_queues(a, 2 * a.sh.L * a.sh.H);
+    const bool widen = a.sched_nq > 1 && a.finite && !a.pair_index;
     return dispatch_d(a.sh.d, [&](auto D) {
-        auto kern = encode ? rotq_kernel<decltype(D)::value, true> : rotq_kernel<decltype(D)::value, false>;
+        constexpr int d = decltype(D)::value;
+        auto kern = widen ? (encode ? rotq_kernel<d, true, true> : rotq_kernel<d, false, true>)
+                          : (encode ? rotq_kernel<d, true, false> : rotq_kernel<d, false, false>);
         size_t sm = 0;
         cudaError_t e2 = pair_smem_bytes(kern, a.sh.Kp, sm);
         if (e2 != cudaSuccess) return e2;
         count_launch();
-        return launch_kernel(kern, sm_count() * kGatherBlocks, kThreads, sm, st, false, 1, a, r);
+        return launch_kernel(kern, sm_count() * (widen ? kRotqBlocks<d, true> : kRotqBlocks<d, false>), kThreads, sm, st, false, 1, a, r);
     });
 }
 

@@ -74,16 +74,15 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // latency on top; pairs are read two at a time and hold byte offsets, so that a row costs one addition
 // beside its load.
 // WIDEN: the conversions on the tensor cores, 2 instructions for 8 on the pipe that the packed FMAs need too (392
-// of the 570 instructions that 64 rows of 128 take), in stretches of 16 rows at most.  Right where a warp has
-// little else to do (rotated quantiser, 8 x 8 heads, 4000 positions: both calls 1700 -> 1500 us; stretches of 32 rows
-// 1530).  The coder's kernels lose more to the tensor instructions' latency than they gain (32 heads of 128, 8 layers,
-// 16384 positions: 20.6 -> 21.8 ms at 64 registers, 25.2 at 48 with more warps).
+// of the 570 instructions that 64 rows of 128 take); for finite T and pairs that hold byte offsets.  Where it pays:
+// see launch_rotq.  The coder's kernels lose more to the tensor instructions' latency than they gain (32 heads of
+// 128, 8 layers, 16384 positions: 20.6 -> 21.8 ms at 64 registers, 25.2 at 48 with more warps).
 // LANE_BASE: a row's address as the lane's own 64-bit base and the offset, one addition of three fewer, but two
-// registers more.  It pays in kernels with little state beside the gather (rotated quantiser 1500 -> 1475 us,
-// block-per-chunk kernel, 128 streams x 4096 positions, both calls 2075 -> 2002); the others lose loads in flight
-// (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
-template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN>
-__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, const float* s1_at, int row_form,
+// registers more.  It pays in the block-per-chunk kernel (128 streams x 4096 positions, both calls 2075 -> 2002 us)
+// and beside WIDEN; the others lose loads in flight (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
+// SHORT: straight-line stretches of 16 rows at most.
+template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN, bool SHORT = WIDEN>
+__device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, const float* s1_at, bool pair_index,
                                         const int2* sp, int Kp, int lane, float inv_d,
                                         float (&mu)[Geo<D>::G], float& sigma2) {
     constexpr int R = Geo<D>::R, G = Geo<D>::G, ROWS = Geo<D>::ROWS;
@@ -98,12 +97,12 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
     } else {
         for (int k = lane; k < Kp; k += 32) {
             const int2 pr = sp[(k % ROWS) * iters + k / ROWS];
-            const uint32_t at = row_form == kRowIndices ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
+            const uint32_t at = pair_index ? (uint32_t)pr.x : (uint32_t)pr.x / (2u * D);
             s1 = __fmaf_rn(__int_as_float(pr.y), __ldg(n2 + at), s1);
         }
     }
     unsigned long long acc2[4] = {0ull, 0ull, 0ull, 0ull};   // four pairs of +0.f
-    if (WIDEN ? row_form == kRowOffsets : row_form != kRowIndices) {
+    if (WIDEN || !pair_index) {
         const uint32_t operand = WIDEN ? widen_operand(lane) : 0u;
         // Straight-line stretches of 32, 16 and 8 rows: the loads of a stretch are issued as far ahead as the
         // kernel's registers allow (64 rows of 128 components, uniform candidates, 24 warps an SM: 8.0 ms
@@ -121,7 +120,7 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
             pl += N;
             left -= N;
         };
-        if constexpr (WIDEN) {
+        if constexpr (SHORT) {
 #pragma unroll 1
             while (left >= 8) rows(std::integral_constant<int, 8>{});
         } else {
@@ -132,12 +131,11 @@ __device__ __forceinline__ void predict(const char* __restrict__ table, const fl
         if (left >= 4) rows(std::integral_constant<int, 4>{});
 #pragma unroll 1
         while (left > 0) rows(std::integral_constant<int, 1>{});
-    } else {                                                 // tables of 4 GB or more (64-bit offsets), values that are not finite
-        const uint32_t unit = row_form == kRowIndices ? 2 * D : 1;
+    } else {                                                 // tables of 4 GB or more: 64-bit offsets
 #pragma unroll 1
         for (int it = 0; it < iters; ++it) {
             const int2 pr = sp[h * iters + it];
-            add_row<false>(table + ((size_t)(uint32_t)pr.x * unit + lane_off), __int_as_float(pr.y), 0u, acc2);
+            add_row<false>(table + ((size_t)(uint32_t)pr.x * (2 * D) + lane_off), __int_as_float(pr.y), 0u, acc2);
         }
     }
     float acc[8];

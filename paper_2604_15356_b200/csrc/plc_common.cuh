@@ -240,10 +240,6 @@ struct DebugDev {
 
 struct CoderTables;                                // plc_coder.cuh
 
-// The pairs' candidates: byte offsets of rows; byte offsets where T holds infinities or NaN; row indices (tables of
-// 4 GB or more).
-enum { kRowOffsets = 0, kRowOffsetsPlain = 1, kRowIndices = 2 };
-
 struct CodecArgs {
     CodecShape sh;
     const CoderTables* tables;                     // frequency tables of the coder
@@ -251,7 +247,8 @@ struct CodecArgs {
     const float* norms_by_row;                     // [V][tables], for launch_variance
     float* s1;                                     // [S*n][tables] variance terms where they were formed ahead (launch_variance), or null
     const int2* pairs;                             // [S*n][Kp] (written by the top-K kernels, put_pair)
-    int row_form;                                  // kRow...: what the pairs hold, and whether T may go through the tensor cores
+    bool pair_index;                               // pairs hold row indices instead of byte offsets (tables of 4 GB or more)
+    bool finite;                                   // T holds neither infinities nor NaN
     const int* step_exp;                           // [S*n] adaptive step exponent, or null
     KvView kv;                                     // encode: input f16; decode: output
     int S, n; const int32_t* pos_begin; const int32_t* pos_end;

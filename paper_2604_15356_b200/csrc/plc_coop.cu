@@ -254,7 +254,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
                 if (k + NP < P) { fetch(k + NP, buf ^ 1); pairs_ready<1>(); }
                 else pairs_ready<0>();
                 buf ^= 1;
-                predict<D, false, true>(col, n2, a.s1 ? a.s1 + (row0 + p) * Wt + t : nullptr, a.row_form, sp, Kp, lane, 1.0f / D, mu, sigma2);
+                predict<D, false, true>(col, n2, a.s1 ? a.s1 + (row0 + p) * Wt + t : nullptr, a.pair_index, sp, Kp, lane, 1.0f / D, mu, sigma2);
             }
             float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
             int zero_q = a.sh.zero_q;

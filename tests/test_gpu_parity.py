@@ -397,17 +397,21 @@ def test_rotated_quantiser_parity(dev, orc, d, bits, ranges):
 
 @pytest.mark.parametrize("d,K", [(128, 64), (128, 1), (128, 37), (64, 50), (64, 64), (32, 100), (256, 16), (256, 70)])
 def test_rows_widened_by_the_tensor_cores(dev, d, K):
-    """The rotated quantiser's rows go through the tensor cores while T is finite, value by value where it is not:
-    an infinity and a NaN in a row that is never a candidate must not change a bit.  T holds every kind of finite
-    value (both zeros, subnormal, largest); K covers stretches of 16, 8 and 2 rows and what remains."""
-    S, n, L, H, V, bits = 2, 40, 1, 2, 600, 6
-    _, logits, T, kv = make_workload(77 + d + K, S, n, L, H, d, V, K, pp=30.0)
+    """The rotated quantiser's rows go through the tensor cores where the tables are more than L2 holds and T is finite,
+    value by value where it is not: an infinity and a NaN in a row that is never a candidate must not change a bit.
+    T holds every kind of finite value (both zeros, subnormal, largest); K covers stretches of 16, 8 and 2 rows and
+    what remains."""
+    S, n, L, H, bits = 2, 40, 8, 2, 6
+    V = torch.cuda.get_device_properties(dev).L2_cache_size // (2 * L * H * d * 2) * 9 // 8 | 1
+    g = torch.Generator(device=dev).manual_seed(77 + d + K)
     rng = np.random.default_rng(d + K)
-    raw = rng.integers(0, 1 << 16, T.numel()).astype(np.uint16)
-    raw[(raw & 0x7c00) == 0x7c00] &= 0x83ff
-    T = torch.from_numpy(raw.view(np.float16)).reshape(T.shape).to(dev)
-    logits[..., V - 1] = -float("inf")
-    kvd, lgd = kv.to(dev), logits.to(dev)
+    raw = torch.randint(0, 1 << 16, (L, 2, H, V, d), generator=g, device=dev, dtype=torch.int32)
+    raw = torch.where((raw & 0x7c00) == 0x7c00, raw & 0x83ff, raw)
+    T = torch.where(raw >= 1 << 15, raw - (1 << 16), raw).to(torch.int16).view(torch.float16)
+    assert torch.isfinite(T).all()
+    lgd = (torch.randn(S, n, V, generator=g, device=dev) * 3).half()
+    lgd[..., V - 1] = -float("inf")
+    kvd = kv = torch.randn(L, 2, S, H, n, d, generator=g, device=dev).half()
     got = []
     for special in (False, True):
         if special:
