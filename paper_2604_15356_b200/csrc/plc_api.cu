@@ -170,9 +170,20 @@ bool keep_extra(size_t bytes) {
 }
 
 // Variance terms formed ahead of the gather (launch_variance): what a call's may take, and from where on the extra
-// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms; 128 x 1024 with the adaptive step 736 -> 729 us; 64 x
-// 999, half of them in range: 3 % slower; 2 x 512: 144 -> 153).
-constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 256 * 1024;
+// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms).  Both calls' time with the terms formed in
+// the gather over that with the terms formed ahead, K = 64, by the terms' bytes (streams: components, vocabulary):
+//                            128 KB  256 KB  384 KB  512 KB  768 KB    1 MB
+//     2: 64, 4000             0.94    0.96    0.98    0.97    0.98    0.98
+//    32: 128, 4000            0.94    0.96    0.99    0.99    1.01    1.01    (K = 16 and 128 at 512 KB: 0.99, 1.02)
+//    32: 128, 32000           0.97    0.97    1.01    1.00    1.03    1.03    (uniform candidates at 512 KB: 1.06)
+//   128: 128, 32000           0.96    0.99    1.03    1.03    1.04    1.06    (1.10; K = 16 1.00)
+//   512: 128, 4000            0.98    0.99    0.98    1.00    1.01    1.02
+//   512: 64, 32000            0.95    1.02    1.03    1.07    1.08    1.12    (1.19; K = 16 0.98)
+//  2048: 64, 16000            1.07    1.07    1.06    1.08    1.09    1.11    (1.13; K = 16 1.02)
+// and with a quarter to a half of the positions out of range, at 512 KB, in this order: 0.98, 0.98, 1.01, 1.03, 1.00, 1.04,
+// 1.06.  A few streams use little of the sector that a candidate's norms lie in.
+constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 512 * 1024;
+constexpr int kLeastVarianceTables = 16;
 
 plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (positions <= c->pairs_cap) return PLC_OK;
@@ -349,7 +360,7 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
     if (ok && T_dev) {
         unsigned int not_finite = 0;
-        if (cfg->variant == PLC_PRED_TOPK && keep_extra(sizeof(float) * (size_t)rows) &&
+        if (cfg->variant == PLC_PRED_TOPK && 2 * cfg->n_layers * cfg->n_kv_heads >= kLeastVarianceTables && keep_extra(sizeof(float) * (size_t)rows) &&
             cudaMalloc(&c->norms_by_row, sizeof(float) * (size_t)rows) != cudaSuccess) {
             cudaGetLastError();
             c->norms_by_row = nullptr;
