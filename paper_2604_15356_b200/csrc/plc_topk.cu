@@ -1170,8 +1170,8 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 4) topk_stream_kernel(const
 // The logits come through a ring in shared memory that every lane fills for itself, asynchronously (held in
 // registers across rows they were spilled: 4096 rows of 128256 434 us).
 // What bounds it: the streaming warps' latency a batch (1700 to 2000 cycles, 16 warps, 130 KB in flight an SM).
-// 4096 rows of 128256, K = 64: 265 -> 191 us (without a selection 168, the copy rate 160); 16384 rows of 32000: 257 ->
-// 223, of 50001: 355 -> 324.
+// 4000 rows of 128256, K = 64, every output: 270 -> 191 us (idx and w only 263, 186; without a selection 168, the copy
+// rate 156); 16384 rows of 32000: 268 -> 242.
 constexpr int kStreamers = 16, kFinishers = 8, kMostTeam = 8;           // warps of a block: streaming, finishing; most of a team
 constexpr int kRing = 4;                                                // batches of a warp on their way
 static_assert(2 * kFinishers <= 16, "a block has 16 barriers");
@@ -1205,16 +1205,16 @@ struct PipeRows {
     }
     __device__ __forceinline__ void next(const TopkArgs& a) { skip(a, step); }
 };
+constexpr int kPipeLeast = 24576;                                       // shortest row
 template <int TEAM>
-struct PipeCut {                                                        // a warp's share of a row
+struct PipeCut {                                                        // a warp's share of a row: a slot every `wide` batches
     int batches, wide, ns;
-    bool fine;
     __device__ __forceinline__ explicit PipeCut(int nv) {
         constexpr int per = kBatch * 32 * TEAM;
+        static_assert((kPipeLeast - 7) / 8 * kBatch * TEAM > kSlots * per, "more groups than slots");
         batches = (nv + per - 1) / per;
-        fine = TEAM * batches * kBatch <= kSlots;
         wide = (TEAM * batches + kSlots - 1) / kSlots;
-        ns = fine ? batches * kBatch : (batches + wide - 1) / wide;
+        ns = (batches + wide - 1) / wide;
     }
 };
 
@@ -1281,16 +1281,10 @@ __device__ __forceinline__ void pipe_stream(const TopkArgs& a, PipeRow<TEAM, W>*
                 if (row.q >= kFinishers) wait_barrier<TEAM>(kFinishers + b);                        // the row that was there has been read
             }
             uint32_t top[kBatch];
-            const uint32_t top4 = sum.add(g, top);
-            if (cut.fine) {
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) put_slot(t * kBatch + u, top[u]);
-            } else {
-                group2 = hmax2_bits(group2, top4);
-                if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = cut.wide; }
-            }
+            group2 = hmax2_bits(group2, sum.add(g, top));
+            if (--left == 0) { put_slot(slot++, group2); group2 = kNegInf2; left = cut.wide; }
         }
-        if (!cut.fine && left != cut.wide) put_slot(slot, group2);
+        if (left != cut.wide) put_slot(slot, group2);
         if (has_ends) {
             auto real = [](uint32_t v) { const uint32_t m = __vcmpeq2(v, kNoValue2); return (v & ~m) | (kNegInf2 & m); };
             const uint4 g[kBatch] = {make_uint4(real(ends.x), real(ends.y), real(ends.z), real(ends.w)), all4(kNegInf2), all4(kNegInf2), all4(kNegInf2)};
@@ -1319,7 +1313,7 @@ __device__ __forceinline__ void pipe_finish(const TopkArgs& a, PipeRow<TEAM, W>&
         const uint32_t kmax = __reduce_max_sync(kFull, on ? from.key[lane] : 0u);
         const float lmax = val_of_key(kmax);
         const float sum_all = warp_sum(on ? from.sum[lane] * expf(from.ref[lane] - lmax) : 0.f);
-        select_row<false, false, W>(a, rowi, r, TEAM, cut.ns, cut.wide, cut.fine, from.slots, from.codes, from.list, from.sorted(), unused, 0, 1, kmax, lmax,
+        select_row<false, false, W>(a, rowi, r, TEAM, cut.ns, cut.wide, false, from.slots, from.codes, from.list, from.sorted(), unused, 0, 1, kmax, lmax,
                                     sum_all, lane, [&]() { if (kEarly && row.at < a.N) arrive_barrier<TEAM>(kFinishers + b); });   // the next row may be put there
         if (lane == 0) put_row(a, rowi, r.row, lmax + logf(sum_all));
         __syncwarp();
@@ -1382,6 +1376,26 @@ static cudaError_t launch_pipe(const TopkArgs& a, int sms, cudaStream_t st) {
     return launch_kernel(topk_pipe_kernel<TEAM, W>, (unsigned)std::min<long long>(a.N, sms), 32 * (kStreamers + kFinishers), smem, st, false, 1, a);
 }
 
+// Where topk_pipe_kernel is the quicker one (times of topk_stream_kernel / of teams, idx and w only unless said).
+// Long rows, from two an SM on: 300 rows of 32000: 17.6 / 14.6 us, of 128256: 37.7 / 33.0.  A row's costs beside its
+// batches weigh more the shorter it is: teams of 4 warps for rows up to 65536 (16384 rows of 32000: 245 us with 8, 223),
+// of 8 beyond (4096 rows of 128256: 201 us with 4, 191), and a warp a row for short ones (16384 rows of 16384: 151 us
+// against 162).
+// More than 64 rows an SM of up to 65536: a warp a row has no last wave to speak of, and teams pay only where the
+// ends of rows are long (large K) but not so long against a row that they keep the finishing warps busier than the
+// streaming ones.  10000 rows: of 24576 K = 16 102 / 107, 64 135 / 130, 80 140 / 144, 128 167 / 183; of 32000 16 136 / 134, 40 156 /
+// 148, 64 168 / 152, 128 206 / 212; of 50001 16 207 / 224, 40 222 / 234, 64 239 / 240, 100 280 / 256; 32768 rows of 32000: 16
+// 424 / 457, 64 523 / 505; 8000 rows: of 24576 16 91 / 87, 128 153 / 148.
+// With position ranges the rows are counted off one by one, and half of them may be missing: rows beyond 65536 only,
+// and from where the other kernel gives a warp a row (both calls with 2 streams of 32, half in range: 4000 rows of
+// 32000 152 / 164 us; 3000 rows of 65544 289 / 187, of 128256 406 / 240; 2100 rows of 65544 184 / 180, of 100001 250 /
+// 258; 1000 rows of 100001 137 / 144).
+static bool teams_pay(const TopkArgs& a, int sms) {
+    if (a.V < kPipeLeast || a.N < 2ll * sms) return false;
+    if (a.pos_begin || a.pos_end) return a.V > 65536 && a.N > 16ll * sms;
+    return a.V > 65536 || a.N <= 64ll * sms || (a.K >= 48 && (a.K < 80 || a.V >= 32000));
+}
+
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
     *few_blocks = 0;
     if (a.N <= 0) return cudaSuccess;
@@ -1391,12 +1405,8 @@ cudaError_t launch_topk(const TopkArgs& a, cudaStream_t st, int* few_blocks) {
     const bool vec = (a.V % 8 == 0) && ((reinterpret_cast<uintptr_t>(a.logits) & 15) == 0);
     if (a.K <= kFinal) {
         const int fixed = !(a.step_exp || a.bits_out) ? 0 : vec ? 1 : 2;
-// Long rows, from two an SM on (300 rows of 32000: 17.8 -> 17.1 us, of 128256: 36.6 -> 33).  A row's costs beside its
-        // batches weigh more the shorter it is: teams of 4 warps for rows up to 65536 (16384 rows of 32000: 245 us with 8, 223),
-        // of 8 beyond (4096 rows of 128256: 201 us with 4, 191), and a warp a row for short ones (16384 rows of 16384: 151 us
-        // against 162).  Calls with an adaptive step need sums of the same parts at any number of rows.
-        const bool ranges = a.pos_begin || a.pos_end;
-        if (!fixed && !ranges && a.V >= 24576 && a.N >= 2ll * sms) return a.V <= 65536 ? launch_pipe<4, uint32_t>(a, sms, st) : launch_pipe<8, unsigned long long>(a, sms, st);
+        // Calls with an adaptive step need sums of the same parts at any number of rows.
+        if (!fixed && teams_pay(a, sms)) return a.V <= 65536 ? launch_pipe<4, uint32_t>(a, sms, st) : launch_pipe<8, unsigned long long>(a, sms, st);
         if (a.V <= 65536) return fixed == 0 ? launch_stream<true, 0, uint32_t>(a, sms, st, few_blocks)
                                : fixed == 1 ? launch_stream<true, 1, uint32_t>(a, sms, st, few_blocks) : launch_stream<true, 2, uint32_t>(a, sms, st, few_blocks);
         return fixed == 0 ? launch_stream<true, 0, unsigned long long>(a, sms, st, few_blocks)

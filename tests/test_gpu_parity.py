@@ -997,12 +997,13 @@ def test_topk_rows_of_every_layout(dev, orc, N, V, K, off):
 
 
 # lengths at the two team sizes' limits, batches that fill a slot and that do not, every alignment; K at its limits
-@pytest.mark.parametrize("N,V,K,off", [(297, 24576, 64, 0), (310, 24577, 128, 3), (1300, 24583, 1, 7), (299, 65536, 100, 0), (600, 65537, 33, 5),
-                                       (300, 128256, 64, 0), (300, 131071, 128, 1)])
-def test_topk_rows_streamed_by_teams(dev, N, V, K, off):
-    """Calls of many long rows against the same rows a hundred at a time (which a block or a cluster selects): the
+@pytest.mark.parametrize("extra,V,K,off", [(1, 24576, 64, 0), (14, 24577, 128, 3), (1004, 24583, 1, 7), (3, 65536, 100, 0), (304, 65537, 33, 5),
+                                           (0, 128256, 64, 0), (4, 131071, 128, 1)])
+def test_topk_rows_streamed_by_teams(dev, extra, V, K, off):
+    """Calls of at least two long rows an SM against the same rows a hundred at a time (which a block or a cluster selects): the
     selected and their weights bit for bit, sums in another order (binary32, tolerance of the other layouts).  Rows
     with ties beyond the lists, with NaN, with fewer finite logits than K and ascending ones among them."""
+    N = 2 * torch.cuda.get_device_properties(dev).multi_processor_count + extra
     g = torch.Generator(device=dev).manual_seed(N + V)
     buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
     rows = buf[off:off + N * V].view(N, V)
@@ -1026,15 +1027,19 @@ def test_topk_rows_streamed_by_teams(dev, N, V, K, off):
 
 
 def test_rows_streamed_by_teams_inside_position_ranges(dev):
-    """A batch whose rows teams stream, with position ranges (one of them empty), against its sessions one by one."""
-    S, n, V, K, d, CP = 5, 90, 24584, 16, 32, 32
+    """A batch whose rows teams stream (more than 16 an SM, of more than 65536 logits), with position ranges (empty ones
+    among them), against its sessions one by one, whose rows blocks or clusters select."""
+    S, V, K, d, CP = 9, 65544, 16, 32, 32
+    n = 16 * torch.cuda.get_device_properties(dev).multi_processor_count // S + 1
     g = torch.Generator(device=dev).manual_seed(5)
     T = torch.randn(1, 2, 1, V, d, generator=g, device=dev).half()
-    logits = (torch.randn(S, n, V, generator=g, device=dev) * 3).half()
+    logits = torch.empty(S, n, V, dtype=torch.float16, device=dev)
+    for s in range(S):
+        logits[s] = torch.randn(n, V, generator=g, device=dev) * 3
     kv = torch.randn(1, 2, S, 1, n, d, generator=g, device=dev).half()
     ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
     mc = ctx.max_chunks(n)
-    begin, end = [0, 13, 40, 89, 7], [90, 90, 40, 90, 71]
+    begin, end = [0, 13, 40, n - 1, 7, 0, 0, n, 0], [n, n, 40, n, 71, n // 2, 0, n, n]
     i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
 
     def coded(kv, logits, b, e):
