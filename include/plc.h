@@ -359,7 +359,8 @@ plc_status plc_get_stats(plc_ctx* ctx, plc_stats* out, int32_t reset, void* stre
 plc_status plc_table_constants(int32_t qp, uint32_t* theta, uint32_t* rho);
 plc_status plc_build_table(int32_t qp, uint32_t* f, uint32_t* c);
 /* With profiling on, plc_encode / plc_decode record CUDA events on the caller's stream directly
- * around their fused predict+code kernel (the top-K kernel that precedes it is outside);
+ * around their fused predict+code kernel and the launch that forms its variance terms ahead in large
+ * calls (the top-K kernel that precedes them is outside);
  * plc_last_kernel_ms waits for the most recent such launch (which = 0 encode, 1 decode, 2 the dense and
  * linear variants' tensor-core contraction of the last group of layers; small calls form all layers
  * in one) and returns its duration.  PLC_E_STATE if

@@ -547,10 +547,10 @@ static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* log
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
-    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     codec_schedule(a, 2 * a.sh.L * a.sh.H, &c->last_nq, &c->last_g);
     cudaEvent_t* pk = prof_pair(c, 0);
     if (pk) cudaEventRecord(pk[0], st);
+    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     cudaError_t e = launch_encode(a, st);
     if (pk) cudaEventRecord(pk[1], st);
     return e == cudaSuccess ? PLC_OK : PLC_E_CUDA;
@@ -593,10 +593,10 @@ static plc_status decode_impl(plc_ctx* c, const plc_streams* in, const void* log
     if (rc) return rc;
     a.pairs = c->pairs;
     a.step_exp = tokens_dev ? c->step_exp : nullptr;
-    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     codec_schedule(a, 2 * a.sh.L * a.sh.H, &c->last_nq, &c->last_g);
     cudaEvent_t* pk = prof_pair(c, 1);
     if (pk) cudaEventRecord(pk[0], st);
+    if (form_variance(c, a, st) != cudaSuccess) return PLC_E_CUDA;
     cudaError_t e = launch_decode(a, st);
     if (pk) cudaEventRecord(pk[1], st);
     return e == cudaSuccess ? PLC_OK : PLC_E_CUDA;

@@ -232,6 +232,37 @@ def test_status_and_profiling_read_outs(dev):
     assert ctx.sync_status() == plc.E_CORRUPT and ctx.poll_status() == (plc.OK, 0)
 
 
+def test_profiled_time_holds_the_terms_formed_ahead(dev):
+    """An encode's or decode's profiled time, the top-K's and what the launches cost are all of the call's time: the
+    variance terms that a large call forms ahead of the gather are part of the first."""
+    L, H, V, d, K, n = 16, 32, 256, 32, 16, 12288
+    g = torch.Generator(device=dev).manual_seed(3)
+    T = torch.randn(L, 2, H, V, d, generator=g, device=dev).half()
+    logits = (torch.randn(1, n, V, generator=g, device=dev) * 3).half()
+    kv = torch.randn(L, 2, 1, H, n, d, generator=g, device=dev).half()
+    ctx = plc.Context(T, K, 0.02)
+    mc = ctx.max_chunks(n)
+    st = plc.StreamSet(ctx.W, mc, 2 * n * ctx.W * d + ctx.W * mc * 160, dev)
+    out = torch.empty(kv.shape, dtype=torch.float32, device=dev)
+    ctx.set_profiling(True)
+
+    def ms(f):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record(); f(); b.record(); b.synchronize()
+        return a.elapsed_time(b)
+
+    def encode():
+        st.total_bytes.zero_()
+        ctx.encode(kv, logits, st)
+
+    topk = min(ms(lambda: ctx.topk_softmax(logits, want=("idx", "w"))) for _ in range(8))
+    for which, f in ((0, encode), (1, lambda: ctx.decode(st, logits, out))):
+        f()
+        rest = min(ms(f) - ctx.last_kernel_ms(which) for _ in range(8))
+        assert rest < topk + 0.05
+    assert ctx.sync_status() == plc.OK
+
+
 def test_tiny_config_full_parity(dev, orc):
     """Tiny: 1 session x 512 tokens, 1 layer, 1 head, d=64, V=256, K=16, delta=0.02, perplexity 12."""
     tokens, logits, T, kv = make_workload(20260416, 1, 512, 1, 1, 64, 256, 16)
