@@ -179,8 +179,9 @@ plc_status plc_create_linear(plc_ctx** out, const plc_config* cfg, const plc_lin
 plc_status plc_destroy(plc_ctx* ctx);
 
 /* Grows the context's scratch so that calls over up to max_positions = S*n positions allocate
- * nothing (top-K results: 8*K bytes per position; the prediction's variance terms: 4 bytes per position and
- * stream, up to 1 GB and while that much can be had; encoder staging: fixed per device). */
+ * nothing (top-K results: 8*K bytes per position; from 512 KB and 16 tables on the prediction's variance terms, 4 bytes
+ * per position and table, up to 1 GB, and the row norms once more, while a quarter of the free memory holds them;
+ * encoder staging: fixed per device).  Without it they are allocated by the first call that needs them. */
 plc_status plc_reserve(plc_ctx* ctx, int64_t max_positions);
 
 /* Top-K softmax of N rows of logits (Sec. 5.1: P(t | t_<i) = softmax; Sec. 7.1: renormalised top-k;

@@ -62,12 +62,12 @@ struct plc_ctx {
     plc_config cfg;
     const __half* T;
     float* rownorm2;                // squared row norms [tables][V]
-    float* norms_by_row;            // the same [V][tables], for variance terms formed ahead (where the memory is to be had)
+    float* norms_by_row;            // the same [V][tables], for variance terms formed ahead, or null
     bool finite;                    // T holds neither infinities nor NaN
     int2* pairs;
     int* step_exp;                  // [positions] adaptive step exponents
     float* s1;                      // [s1_cap][tables] variance terms of large calls, or null
-    long long s1_cap;               // positions
+    long long s1_cap, s1_asked;     // positions: that it holds, that it has been asked to hold
     long long pairs_cap;            // positions
     uint16_t* staging;
     unsigned long long staging_words_per_warp;
@@ -189,22 +189,42 @@ plc_status ensure_pairs(plc_ctx* c, long long positions) {
     if (positions <= c->pairs_cap) return PLC_OK;
     if (c->pairs) cudaFree(c->pairs);
     if (c->step_exp) cudaFree(c->step_exp);
-    if (c->s1) cudaFree(c->s1);
-    c->pairs = nullptr; c->step_exp = nullptr; c->s1 = nullptr; c->pairs_cap = c->s1_cap = 0;
+    c->pairs = nullptr; c->step_exp = nullptr; c->pairs_cap = 0;
     if (cudaMalloc(&c->pairs, sizeof(int2) * (size_t)positions * padded_k(c->cfg)) != cudaSuccess ||
         cudaMalloc(&c->step_exp, sizeof(int) * (size_t)positions) != cudaSuccess) {
         cudaGetLastError();                     // the launches that follow ask for the last error
         return PLC_E_CUDA;
     }
     c->pairs_cap = positions;
-    // Where they would take more than a quarter of the free memory, and for calls beyond, the gather forms them itself.
-    const size_t a_position = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads;
-    const long long most = std::min<long long>(positions, (long long)(kMostVariance / a_position));
-    if (c->norms_by_row && (size_t)most * a_position >= kLeastVariance && keep_extra((size_t)most * a_position)) {
-        if (cudaMalloc(&c->s1, (size_t)most * a_position) == cudaSuccess) c->s1_cap = most;
-        else { cudaGetLastError(); c->s1 = nullptr; }
-    }
     return PLC_OK;
+}
+
+// Room for the variance terms of calls over `positions`, and the norms that they are formed from: on reserve, or on the
+// first encode or decode that can use them (no other call does).  Where they would take more than a quarter of the free
+// memory, for calls beyond, and while the stream is being captured, the gather forms the terms itself.
+void ensure_variance(plc_ctx* c, long long positions, cudaStream_t st) {
+    const int tables = 2 * c->cfg.n_layers * c->cfg.n_kv_heads;
+    const size_t a_position = sizeof(float) * tables, norms = a_position * c->cfg.vocab;
+    const long long most = std::min<long long>(positions, (long long)(kMostVariance / a_position));
+    if (c->cfg.variant != PLC_PRED_TOPK || tables < kLeastVarianceTables || positions <= c->s1_asked || (size_t)most * a_position < kLeastVariance) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
+    c->s1_asked = positions;
+    if (most <= c->s1_cap) return;
+    if (c->s1) cudaFree(c->s1);
+    c->s1 = nullptr; c->s1_cap = 0;
+    if (!keep_extra((size_t)most * a_position + (c->norms_by_row ? 0 : norms))) return;
+    if (!c->norms_by_row) {
+        if (cudaMalloc(&c->norms_by_row, norms) != cudaSuccess) { cudaGetLastError(); c->norms_by_row = nullptr; return; }
+        if (launch_norms_by_row(c->rownorm2, c->norms_by_row, c->cfg.vocab, tables, c->side_stream) != cudaSuccess ||
+            cudaStreamSynchronize(c->side_stream) != cudaSuccess) {
+            cudaFree(c->norms_by_row);
+            c->norms_by_row = nullptr;
+            return;
+        }
+    }
+    if (cudaMalloc(&c->s1, (size_t)most * a_position) == cudaSuccess) c->s1_cap = most;
+    else { cudaGetLastError(); c->s1 = nullptr; }
 }
 
 CodecArgs base_args(const plc_ctx* c) {
@@ -219,7 +239,7 @@ CodecArgs base_args(const plc_ctx* c) {
         ? (int)floor(4.0 * log2((double)c->cfg.zero_rate_D / ((double)c->cfg.delta * (double)c->cfg.delta)) - 0.5)
         : kZeroOff;
     a.tables = c->tables;
-    a.T = c->T; a.rownorm2 = c->rownorm2; a.norms_by_row = c->norms_by_row; a.pairs = c->pairs;
+    a.T = c->T; a.rownorm2 = c->rownorm2; a.pairs = c->pairs;
     a.pair_index = pair_index(c->cfg); a.finite = c->finite;
     a.staging = c->staging; a.staging_words_per_warp = c->staging_words_per_warp;
     a.ticket = c->ticket; a.status = c->status; a.counters = c->counters;
@@ -360,13 +380,8 @@ static plc_status create_common(plc_ctx** out, const plc_config* cfg, const void
                  cudaMemset(c->counters, 0, sizeof(Counters)) == cudaSuccess;
     if (ok && T_dev) {
         unsigned int not_finite = 0;
-        if (cfg->variant == PLC_PRED_TOPK && 2 * cfg->n_layers * cfg->n_kv_heads >= kLeastVarianceTables && keep_extra(sizeof(float) * (size_t)rows) &&
-            cudaMalloc(&c->norms_by_row, sizeof(float) * (size_t)rows) != cudaSuccess) {
-            cudaGetLastError();
-            c->norms_by_row = nullptr;
-        }
         ok = cudaMemset(c->ticket, 0, sizeof(unsigned int)) == cudaSuccess &&
-             launch_rownorm(c->T, c->rownorm2, c->norms_by_row, cfg->vocab, 2 * cfg->n_layers * cfg->n_kv_heads, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
+             launch_rownorm(c->T, c->rownorm2, rows, cfg->head_dim, c->ticket, 0) == cudaSuccess &&
              cudaMemcpy(&not_finite, c->ticket, sizeof(unsigned int), cudaMemcpyDeviceToHost) == cudaSuccess;
         c->finite = not_finite == 0;
     }
@@ -410,7 +425,9 @@ plc_status plc_destroy(plc_ctx* c) {
 
 plc_status plc_reserve(plc_ctx* c, int64_t max_positions) {
     if (!c || max_positions < 0) return PLC_E_INVALID;
-    return ensure_pairs(c, max_positions);
+    const plc_status rc = ensure_pairs(c, max_positions);
+    if (rc == PLC_OK) ensure_variance(c, max_positions, c->side_stream);
+    return rc;
 }
 
 plc_status plc_topk_softmax(plc_ctx* c, const void* logits_dev, const int32_t* tokens_dev, int64_t N, int32_t* idx_dev,
@@ -513,12 +530,12 @@ static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bo
     return PLC_OK;
 }
 
-// Variance terms of a call that has room for them.
+// Variance terms of a call that has room for them (ensure_variance).
 static cudaError_t form_variance(const plc_ctx* c, CodecArgs& a, cudaStream_t st) {
     const long long rows = (long long)a.S * a.n;
     const size_t bytes = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads * rows;
     if (rows > c->s1_cap || bytes < kLeastVariance) return cudaSuccess;
-    a.s1 = c->s1; a.behind = 0;
+    a.s1 = c->s1; a.norms_by_row = c->norms_by_row; a.behind = 0;
     return launch_variance(a, st);
 }
 
@@ -543,6 +560,9 @@ static plc_status encode_impl(plc_ctx* c, const plc_kv_view* kv, const void* log
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, true, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, true, st);
+    rc = ensure_pairs(c, (long long)S * n);
+    if (rc) return rc;
+    ensure_variance(c, (long long)S * n, st);
     rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, false, &a.behind, tokens_dev, dbg ? dbg->bits_dev : nullptr);
     if (rc) return rc;
     a.pairs = c->pairs;
@@ -589,6 +609,9 @@ static plc_status decode_impl(plc_ctx* c, const plc_streams* in, const void* log
     if (dbg) a.dbg = DebugDev{dbg->sym_dev, dbg->q_dev, dbg->mu_dev, dbg->count_ideal_bits};
     if (c->cfg.variant == PLC_PRED_DENSE) return run_dense(c, a, logits_dev, false, st);
     if (c->cfg.variant == PLC_PRED_LINEAR) return run_linear(c, a, logits_dev, false, st);
+    rc = ensure_pairs(c, (long long)S * n);
+    if (rc) return rc;
+    ensure_variance(c, (long long)S * n, st);
     rc = run_topk_for(c, logits_dev, S, n, pos_begin_dev, pos_end_dev, st, false, &a.behind, tokens_dev, dbg ? dbg->bits_dev : nullptr);
     if (rc) return rc;
     a.pairs = c->pairs;

@@ -33,24 +33,21 @@ constexpr int kThreads = kWarpsPerBlock * 32;
 constexpr int kBlocksPerSM = 5, kGatherBlocks = 4;
 constexpr int kGatherWarps = kGatherBlocks * kWarpsPerBlock, kFarWarps = 24;
 
-// Squared row norms of tables T[t][v][D], out[t][v] and (unless it is null) by_row[v][t]: a warp takes a candidate's rows in
-// kNormTables tables, whose norms are one sector of the latter.
-constexpr int kNormTables = 8;
+// Squared row norms; a warp takes kNormRows rows, whose norms are one sector.
+constexpr int kNormRows = 8;
 template <int D>
-__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, float* __restrict__ by_row, int V, int tables,
-                                                      unsigned int* not_finite) {
+__global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__ T, float* __restrict__ out, long long rows, unsigned int* not_finite) {
     constexpr int G = Geo<D>::G;
     const int lane = threadIdx.x & 31;
     const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    const int c0 = first_comp<D>(lane), groups = (tables + kNormTables - 1) / kNormTables;
-    for (long long item = warp; item < (long long)groups * V; item += nw) {
-        const int t0 = (int)(item / V) * kNormTables, v = (int)(item % V);
+    const int c0 = first_comp<D>(lane);
+    for (long long r0 = warp * kNormRows; r0 < rows; r0 += nw * kNormRows) {
         float mine = 0.f;
 #pragma unroll 4
-        for (int j = 0; j < kNormTables; ++j) {
-            if (t0 + j >= tables) break;
-            const __half* row = T + ((long long)(t0 + j) * V + v) * D + c0;
+        for (int j = 0; j < kNormRows; ++j) {
+            if (r0 + j >= rows) break;
+            const __half* row = T + (r0 + j) * D + c0;
             float x[G];
 #pragma unroll
             for (int g = 0; g < G; ++g) x[g] = __half2float(row[g]);
@@ -58,11 +55,19 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const __half* __restrict__
             if (lane == j) mine = s;
         }
         if (!(mine < __int_as_float(0x7f800000))) *not_finite = 1u;           // squares of finite binary16 values sum to less
-        if (lane < kNormTables && t0 + lane < tables) {
-            out[(long long)(t0 + lane) * V + v] = mine;
-            if (by_row) by_row[(long long)v * tables + t0 + lane] = mine;
-        }
+        if (lane < kNormRows && r0 + lane < rows) out[r0 + lane] = mine;
     }
+}
+
+// by_row[v][t] = norms[t][v], by tiles of 32 x 32.
+__global__ void __launch_bounds__(256) norms_by_row_kernel(const float* __restrict__ norms, float* __restrict__ by_row, int V, int tables) {
+    __shared__ float tile[32][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5, v0 = blockIdx.x * 32, t0 = blockIdx.y * 32;
+    for (int j = y; j < 32; j += 8)
+        if (t0 + j < tables && v0 + x < V) tile[j][x] = norms[(long long)(t0 + j) * V + v0 + x];
+    __syncthreads();
+    for (int j = y; j < 32; j += 8)
+        if (v0 + j < V && t0 + x < tables) by_row[(long long)(v0 + j) * tables + t0 + x] = tile[x][j];
 }
 
 // Variance terms s1[row][t] = sum_k w_k ||T[t][idx_k]||^2 of every (position, table), ahead of the gather kernels: the
@@ -400,12 +405,12 @@ __device__ __forceinline__ void hadamard(float (&v)[Geo<D>::G], int lane) {
     for (int g = 0; g < G; ++g) v[g] *= norm;
 }
 
+template <int D, bool WIDEN>
+constexpr int kRotqBlocks = WIDEN && D != 256 ? 3 : kGatherBlocks;       // an SM; see launch_rotq
 // Rotated fixed-rate quantiser (Prop. 3 step 3: a per-vector quantiser on the residual R = KV - KV^):
 // x = eps * R, y = H x (orthonormal Hadamard), s = max |y|, b-bit mid-rise codes on [-s, s]; the
 // record is s followed by one ballot word per (register, code bit).  ENC: KV -> records;
 // otherwise records -> KV' = KV^ + eps * H y^.  One warp per (stream, chunk of positions).
-template <int D, bool WIDEN>
-constexpr int kRotqBlocks = WIDEN && D != 256 ? 3 : kGatherBlocks;       // an SM; see launch_rotq
 template <int D, bool ENC, bool WIDEN>
 __global__ void __launch_bounds__(kThreads, (kRotqBlocks<D, WIDEN>)) rotq_kernel(const CodecArgs a, const RotqArgs rq) {
     constexpr int G = Geo<D>::G;
@@ -597,13 +602,20 @@ static void set_queues(CodecArgs& a, int n_tables, int items_per_sm) {
     a.sched_g = (int)g; a.sched_nq = nq;
 }
 
-cudaError_t launch_rownorm(const __half* T, float* out, float* by_row, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st) {
+cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, unsigned int* not_finite, cudaStream_t st) {
     return dispatch_d(d, [&](auto D) {
-        const long long blocks = std::min(((long long)(tables + kNormTables - 1) / kNormTables * V + 7) / 8, (long long)sm_count() * 16);
-        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, by_row, V, tables, not_finite);
+        constexpr int a_block = 8 * kNormRows;
+        const long long blocks = std::min((rows + a_block - 1) / a_block, (long long)sm_count() * 16);
+        rownorm_kernel<decltype(D)::value><<<(unsigned)blocks, 256, 0, st>>>(T, out, rows, not_finite);
         count_launch();
         return cudaGetLastError();
     });
+}
+
+cudaError_t launch_norms_by_row(const float* norms, float* by_row, int V, int tables, cudaStream_t st) {
+    norms_by_row_kernel<<<dim3((unsigned)((V + 31) / 32), (unsigned)((tables + 31) / 32)), 256, 0, st>>>(norms, by_row, V, tables);
+    count_launch();
+    return cudaGetLastError();
 }
 
 static int log2_of(int v) { return v > 1 ? 1 + log2_of(v >> 1) : 0; }

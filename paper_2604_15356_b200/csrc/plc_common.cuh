@@ -316,7 +316,8 @@ cudaError_t linear_begin(const __half* logits, const LinearShape& sh, const uint
 cudaError_t linear_layers(const __half* A, int l0, int nl, const LinearShape& sh, const uint8_t* model, const size_t* moff, uint8_t* scratch,
                           const size_t* off, unsigned int* status, cudaStream_t st, cudaEvent_t ev0, cudaEvent_t ev1);
 // Sets *not_finite where a row holds an infinity or NaN.
-cudaError_t launch_rownorm(const __half* T, float* out, float* by_row, int V, int tables, int d, unsigned int* not_finite, cudaStream_t st);
+cudaError_t launch_rownorm(const __half* T, float* out, long long rows, int d, unsigned int* not_finite, cudaStream_t st);
+cudaError_t launch_norms_by_row(const float* norms, float* by_row, int V, int tables, cudaStream_t st);
 cudaError_t launch_variance(const CodecArgs& a, cudaStream_t st);            // fills a.s1 for the pairs
 cudaError_t launch_encode(const CodecArgs& a, cudaStream_t st);
 cudaError_t launch_decode(const CodecArgs& a, cudaStream_t st);

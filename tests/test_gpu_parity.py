@@ -1152,6 +1152,46 @@ def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
             assert [c for c in whole[s * ctx.W + t] if c] == alone[t]
 
 
+def test_scratch_of_the_terms_formed_ahead(dev):
+    """The terms' scratch (16 MB here) and the second copy of the norms (20 MB) are taken by the first call that reads
+    them, or on reserve, not by one that predicts without them; a call that is being captured does without."""
+    L, H, V, d, K, n, bits = 4, 32, 20000, 32, 16, 16384, 4
+    g = torch.Generator(device=dev).manual_seed(9)
+    T = torch.randn(L, 2, H, V, d, generator=g, device=dev).half()
+    logits = torch.randn(1, n, V, generator=g, device=dev).half()
+    kv = torch.randn(L, 2, 1, H, n, d, generator=g, device=dev).half()
+
+    def used(f):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info(dev)[0]
+        f()
+        torch.cuda.synchronize()
+        return (before - torch.cuda.mem_get_info(dev)[0]) / 2**20
+
+    ctx, reserved = plc.Context(T, K, 0.02), plc.Context(T, K, 0.02)
+    W, mc = ctx.W, ctx.max_chunks(n)
+    records = torch.zeros(W * n * ctx.rotq_record_bytes(bits), dtype=torch.uint8, device=dev)
+    streams = [plc.StreamSet(W, mc, 2 * n * W * d + W * mc * 160, dev) for _ in range(3)]
+    params = ctx.rotq_params(bits, [0] * d)
+    assert used(lambda: ctx.encode_rotq(kv, logits, params, records)) < 8          # 2 MB of candidates
+    graph = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+
+    def capture():
+        with torch.cuda.graph(graph, stream=side):
+            ctx.encode(kv, logits, streams[0])
+
+    capture()
+    graph.replay()
+    assert used(lambda: ctx.encode(kv, logits, streams[1])) >= 32
+    assert used(lambda: reserved.reserve(n)) >= 32
+    assert used(lambda: reserved.encode(kv, logits, streams[2])) < 8
+    assert ctx.sync_status() == plc.OK and reserved.sync_status() == plc.OK
+    for s in range(0, W * mc, 97):
+        assert streams[0].chunk(s).tobytes() == streams[1].chunk(s).tobytes() == streams[2].chunk(s).tobytes()
+
+
 @pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
 def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
     """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
