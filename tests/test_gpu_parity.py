@@ -1192,7 +1192,8 @@ def test_scratch_of_the_terms_formed_ahead(dev):
         assert streams[0].chunk(s).tobytes() == streams[1].chunk(s).tobytes() == streams[2].chunk(s).tobytes()
 
 
-@pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
+@pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False),
+                                             (64, 200, 500, 1, True), (32, 426, 600, 1, False), (32, 429, 600, 1, False), (64, 1000, 1100, 1, False)])
 def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
     """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
     (fewer chunks get a block each); candidate counts that leave remainders of the gather's stretches."""
@@ -1203,6 +1204,40 @@ def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, rang
     assert g["rc"] == plc.OK and g["W"] * S * g["mc"] > 32 * torch.cuda.get_device_properties(dev).multi_processor_count
     check_against_oracle(orc, g, T, kv, logits, K, 0.02, CP, pb, pe)
     gpu_decode_check(g, kv, 0.02, n, pb, pe)
+
+
+@pytest.mark.parametrize("K,ranges", [(200, False), (320, True), (321, False), (1000, True)])
+def test_pairs_beside_each_other_or_in_blocks_of_eight(dev, K, ranges):
+    """More than a chunk a warp and tables beyond L2 (many queues): the pairs of an SM's 32 warps lie beside each other in
+    one block up to K = 320, in blocks of eight beyond.  The sessions one by one (a block per chunk) give the same
+    bytes and vectors."""
+    S, n, L, H, d, CP = 5, 8, 8, 8, 32, 1
+    V = torch.cuda.get_device_properties(dev).L2_cache_size // (2 * L * H * d * 2) * 9 // 8 | 1
+    g = torch.Generator(device=dev).manual_seed(K)
+    T = torch.randn(L, 2, H, V, d, generator=g, device=dev).half()
+    logits = (torch.randn(S, n, V, generator=g, device=dev) * 2).half()
+    kv = torch.randn(L, 2, S, H, n, d, generator=g, device=dev).half()
+    ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
+    W, mc = ctx.W, ctx.max_chunks(n)
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+    begin, end = ([0, 1, 3, n, 0], [n, n, n - 1, n, 1]) if ranges else ([0] * S, [n] * S)
+
+    def both(kv, logits, b, e):
+        st = plc.StreamSet(logits.shape[0] * W, mc, 4 * kv.numel() + logits.shape[0] * W * mc * 160, dev)
+        ctx.encode(kv, logits, st, i32(b), i32(e))
+        out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+        ctx.decode(st, logits, out, i32(b), i32(e))
+        assert ctx.sync_status() == plc.OK
+        return [st.chunk(i).tobytes() for i in range(logits.shape[0] * W * mc)], out
+
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    assert W * S * mc > 32 * sms >= W * mc
+    whole, out = both(kv, logits, begin, end)
+    assert ctx.last_schedule()[0] > 1
+    for s in range(S):
+        alone, out_s = both(kv[:, :, s:s + 1].contiguous(), logits[s:s + 1].contiguous(), begin[s:s + 1], end[s:s + 1])
+        assert whole[s * W * mc:(s + 1) * W * mc] == alone and torch.equal(out[:, :, s:s + 1], out_s)
+    assert any(whole)
 
 
 def test_long_chunks_with_escapes_and_wide_planes(dev, orc):
