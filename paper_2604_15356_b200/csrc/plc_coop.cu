@@ -21,7 +21,6 @@
 namespace plc {
 namespace {
 
-constexpr int kCoopMaxWarps = 32;
 // Predicting warps of a block.
 __host__ __device__ constexpr int coop_predictors(int warps) { return warps >= 16 ? 3 * warps / 4 : warps - 1; }
 constexpr int kRingBlock = 512;                          // bytes one warp-wide copy brings to the word ring of a decoding coder
@@ -147,17 +146,18 @@ struct CoopItem {
     unsigned nbytes;
     int go;                              // 0: nothing to do for this chunk, -1: no chunks left
 };
+template <int NP>                        // predicting warps at most
 struct CoopShared {
     CoopItem item;
-    SlotMeta meta[2][kCoopMaxWarps];
+    SlotMeta meta[2][NP];
     uint8_t* dst;                        // encoding: where the finished chunk's words go (null: nowhere)
     int wp;
 };
 
 // Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a batch; the inputs
 // of the next are fetched while it works on one.
-template <int D, bool DENSE, bool ENC, int GW, class Tab>
-__device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
+template <int D, bool DENSE, bool ENC, int GW, class Tab, class Shared>
+__device__ __forceinline__ void coop_predict(const CodecArgs& a, Shared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
                                              const Meet<GW>& meet, const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
@@ -327,8 +327,8 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, CoopShared& sh,
 }
 
 // Coder of the block's chunk, one batch behind the predictions.
-template <int D, bool ENC, bool ROOMY, int GW, class Tab>
-__device__ __forceinline__ void coop_code(const CodecArgs& a, CoopShared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const Meet<GW>& meet,
+template <int D, bool ENC, bool ROOMY, int GW, class Tab, class Shared>
+__device__ __forceinline__ void coop_code(const CodecArgs& a, Shared& sh, const Tab& tb, int* slots, uint16_t* ring, int NP, const Meet<GW>& meet,
                                           const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
     const int lane = lc.lane;
@@ -486,7 +486,8 @@ __global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 
     static_assert(GW == 0 || (DENSE && !ENC), "staging is addressed by block");
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
     __shared__ Tab tb;
-    __shared__ CoopShared shared[GW ? kGroups<D> : 1];
+    using Shared = CoopShared<GW ? GW - 1 : ROOMY ? coop_predictors(DENSE ? 16 : kAloneWarps<D>) : 7>;
+    __shared__ Shared shared[GW ? kGroups<D> : 1];
     // Warps go to an SM's four schedulers in turn.  A block that has its SM to itself (16 warps or more) leaves the
     // coder's scheduler to the coder: the warps that would share it stay idle.  The coders of groups lie on
     // different schedulers.
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 
     const int group = GW ? hw / GW : 0;
     const int warp = GW ? (hw - group) & (GW - 1) : NP < warps - 1 ? ((hw & 3) == 0 ? (hw == 0 ? 0 : -1) : hw - (hw >> 2)) : hw;
     const int Kp = DENSE ? 0 : a.sh.Kp;
-    CoopShared& sh = shared[group];
+    Shared& sh = shared[group];
     int2* pairs = GW ? reinterpret_cast<int2*>(reinterpret_cast<unsigned char*>(g_pair_smem) + group * coop_smem(GW, 0, D, DENSE, ENC, ROOMY)) : g_pair_smem;
     int* slots = reinterpret_cast<int*>(pairs + NP * 2 * Kp);                                // [2][NP] slots
     uint16_t* ring = reinterpret_cast<uint16_t*>(slots + 2 * NP * kDecSlotWords<Geo<D>::G>);  // decoding
@@ -548,6 +549,10 @@ __global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 
 }
 
 }  // namespace
+
+// Four decoding blocks of eight warps fit an SM (228 KB, 1 KB of them each block's own) up to K = 100: with 512 bytes more a
+// block three did, and 168 streams x 768 positions, K = 100, decoded in 652 us instead of 484.
+static_assert(sizeof(WideDecTables) + sizeof(CoopShared<7>) + coop_smem(8, 100, 128, false, false, false) + 1024 <= 228 * 1024 / 4, "shared memory of a block");
 
 cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
     return dispatch_d(a.sh.d, [&](auto D) {
