@@ -179,7 +179,7 @@ plc_status plc_create_linear(plc_ctx** out, const plc_config* cfg, const plc_lin
 plc_status plc_destroy(plc_ctx* ctx);
 
 /* Grows the context's scratch so that calls over up to max_positions = S*n positions allocate
- * nothing (top-K results: 8*K bytes per position; from 512 KB and 16 tables on the prediction's variance terms, 4 bytes
+ * nothing (top-K results: 8*K bytes per position; from 288 KB and 16 tables on the prediction's variance terms, 4 bytes
  * per position and table, up to 1 GB, and the row norms once more, while a quarter of the free memory holds them;
  * encoder staging: fixed per device).  Without it they are allocated by the first call that needs them. */
 plc_status plc_reserve(plc_ctx* ctx, int64_t max_positions);

@@ -170,19 +170,20 @@ bool keep_extra(size_t bytes) {
 }
 
 // Variance terms formed ahead of the gather (launch_variance): what a call's may take, and from where on the extra
-// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms).  Both calls' time with the terms formed in
-// the gather over that with the terms formed ahead, K = 64, by the terms' bytes (streams: components, vocabulary):
+// launch pays (1024 streams x 16384 positions, both calls 41.12 -> 39.70 ms): earlier where many queues serve the tables
+// (more than L2 holds: the norms come from afar too).  Both calls' time with the terms formed in the gather over that with
+// the terms formed ahead, K = 64, by the terms' bytes (streams: components, vocabulary; the first and the fourth row are
+// tables that one queue serves):
 //                            128 KB  256 KB  384 KB  512 KB  768 KB    1 MB
-//     2: 64, 4000             0.94    0.96    0.98    0.97    0.98    0.98
 //    32: 128, 4000            0.94    0.96    0.99    0.99    1.01    1.01    (K = 16 and 128 at 512 KB: 0.99, 1.02)
-//    32: 128, 32000           0.97    0.97    1.01    1.00    1.03    1.03    (uniform candidates at 512 KB: 1.06)
-//   128: 128, 32000           0.96    0.99    1.03    1.03    1.04    1.06    (1.10; K = 16 1.00)
+//    64: 128, 32000           0.96    0.98    1.06    1.02    1.03    1.04    (uniform candidates 0.98 1.06 1.08 1.07 1.09 1.10)
+//   128: 128, 32000           0.96    0.99    1.03    1.03    1.04    1.06    (uniform 1.01 1.10 1.14 1.10 1.10 1.11; K = 16 at 512 KB 1.00)
 //   512: 128, 4000            0.98    0.99    0.98    1.00    1.01    1.02
-//   512: 64, 32000            0.95    1.02    1.03    1.07    1.08    1.12    (1.19; K = 16 0.98)
-//  2048: 64, 16000            1.07    1.07    1.06    1.08    1.09    1.11    (1.13; K = 16 1.02)
-// and with a quarter to a half of the positions out of range, at 512 KB, in this order: 0.98, 0.98, 1.01, 1.03, 1.00, 1.04,
-// 1.06.  A few streams use little of the sector that a candidate's norms lie in.
-constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVariance = 512 * 1024;
+//   512: 64, 32000            0.95    1.02    1.03    1.07    1.08    1.12    (uniform 1.03 1.12 1.16 1.19 1.19 1.16; K = 16 0.98)
+//  2048: 64, 16000            1.07    1.07    1.06    1.08    1.09    1.11    (uniform 1.01 1.08 1.10 1.13 1.16 1.17; K = 16 1.02)
+// and with a quarter to a half of the positions out of range, at 512 KB, in this order: 0.98, 1.02, 1.03, 1.00, 1.04, 1.06.
+// Two streams use little of the sector that a candidate's norms lie in: 0.94 to 0.98 at any size.
+constexpr size_t kMostVariance = (size_t)1 << 30, kLeastVarianceFar = 288 * 1024, kLeastVariance = 512 * 1024;
 constexpr int kLeastVarianceTables = 16;
 
 plc_status ensure_pairs(plc_ctx* c, long long positions) {
@@ -206,7 +207,7 @@ void ensure_variance(plc_ctx* c, long long positions, cudaStream_t st) {
     const int tables = 2 * c->cfg.n_layers * c->cfg.n_kv_heads;
     const size_t a_position = sizeof(float) * tables, norms = a_position * c->cfg.vocab;
     const long long most = std::min<long long>(positions, (long long)(kMostVariance / a_position));
-    if (c->cfg.variant != PLC_PRED_TOPK || tables < kLeastVarianceTables || positions <= c->s1_asked || (size_t)most * a_position < kLeastVariance) return;
+    if (c->cfg.variant != PLC_PRED_TOPK || tables < kLeastVarianceTables || positions <= c->s1_asked || (size_t)most * a_position < kLeastVarianceFar) return;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) { cudaGetLastError(); return; }
     c->s1_asked = positions;
@@ -530,11 +531,11 @@ static plc_status run_linear(plc_ctx* c, CodecArgs a, const void* logits_dev, bo
     return PLC_OK;
 }
 
-// Variance terms of a call that has room for them (ensure_variance).
+// Variance terms of a call that has room for them (ensure_variance) and is large enough, its queues set.
 static cudaError_t form_variance(const plc_ctx* c, CodecArgs& a, cudaStream_t st) {
     const long long rows = (long long)a.S * a.n;
     const size_t bytes = sizeof(float) * 2 * c->cfg.n_layers * c->cfg.n_kv_heads * rows;
-    if (rows > c->s1_cap || bytes < kLeastVariance) return cudaSuccess;
+    if (rows > c->s1_cap || bytes < (c->last_nq > 1 ? kLeastVarianceFar : kLeastVariance)) return cudaSuccess;
     a.s1 = c->s1; a.norms_by_row = c->norms_by_row; a.behind = 0;
     return launch_variance(a, st);
 }
