@@ -707,9 +707,7 @@ cudaError_t launch_decode(const CodecArgs& a0, cudaStream_t st) {
 
 // Rows are widened on the tensor cores where a queue is served by a few SMs (set_queues: the tables in flight are more
 // than L2 holds), with 24 warps an SM at 80 registers (32 at 64 for 256 components); where all SMs share a queue, and for
-// T that the tensor cores cannot take, value by value with 32 warps.  Widening lets the few rows in flight that L1
-// has room for beside the shared ones do more work; where L2 holds the tables the packed conversions are the quicker
-// chain.  4000 positions, 8 x 8 heads of 128, K = 64, both calls, value by value with stretches of 32 rows / widened
+// T that the tensor cores cannot take, value by value with 32 warps.  4000 positions, 8 x 8 heads of 128, K = 64, both calls, value by value with stretches of 32 rows / widened
 // with 32 warps / as now, us: V = 32000, skewed candidates (many queues) 1693 / 1457 / 1433, uniform 2742 / 3103 / 2616,
 // uniform K = 128 4925 / 5802 / 4720; V = 5000 (one queue) 1360 / 1480 / 1319; 4 layers (one queue) skewed 834 / 854 /
 // 814, uniform 1055 / 1290 / 996; 256 components, 4 layers, skewed 1648 / 1398 / 1355 (24 warps 1387), uniform 2725 /

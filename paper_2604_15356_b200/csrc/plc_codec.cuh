@@ -78,8 +78,9 @@ __device__ __forceinline__ void add_row(const char* p, float w, uint32_t operand
 // see launch_rotq.  The coder's kernels lose more to the tensor instructions' latency than they gain (32 heads of
 // 128, 8 layers, 16384 positions: 20.6 -> 21.8 ms at 64 registers, 25.2 at 48 with more warps).
 // LANE_BASE: a row's address as the lane's own 64-bit base and the offset, one addition of three fewer, but two
-// registers more.  It pays in the block-per-chunk kernel (128 streams x 4096 positions, both calls 2075 -> 2002 us)
-// and beside WIDEN; the others lose loads in flight (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
+// registers more.  It pays beside WIDEN and in the block-per-chunk kernel (128 streams x 4096 positions, both calls 1977 ->
+// 1933 us, 3 x 333 x 64 streams 282 -> 275, although encoding then spills 46 bytes for 26), with 256 components only where the
+// variance terms were formed ahead; the others lose loads in flight (131072 positions x 64 streams: decode 13.5 -> 15.5 ms).
 // SHORT: straight-line stretches of 16 rows at most.
 template <int D, bool WIDEN = false, bool LANE_BASE = WIDEN, bool SHORT = WIDEN>
 __device__ __forceinline__ void predict(const char* __restrict__ table, const float* __restrict__ n2, const float* s1_at, bool pair_index,

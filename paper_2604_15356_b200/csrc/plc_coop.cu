@@ -156,7 +156,7 @@ struct CoopShared {
 
 // Warp w (of NP) beside the coder: positions w, w + NP, ... in the coder's order, one a batch; the inputs
 // of the next are fetched while it works on one.
-template <int D, bool DENSE, bool ENC, int GW, class Tab, class Shared>
+template <int D, bool DENSE, bool ENC, bool AHEAD, int GW, class Tab, class Shared>
 __device__ __forceinline__ void coop_predict(const CodecArgs& a, Shared& sh, const Tab& tb, int2* sp0, int* slots, int w, int NP,
                                              const Meet<GW>& meet, const LaneCode& lc) {
     constexpr int G = Geo<D>::G, SW = ENC ? kEncSlotWords<G> : kDecSlotWords<G>;
@@ -254,7 +254,7 @@ __device__ __forceinline__ void coop_predict(const CodecArgs& a, Shared& sh, con
                 if (k + NP < P) { fetch(k + NP, buf ^ 1); pairs_ready<1>(); }
                 else pairs_ready<0>();
                 buf ^= 1;
-                predict<D, false, true>(col, n2, a.s1 ? a.s1 + (row0 + p) * Wt + t : nullptr, a.pair_index, sp, Kp, lane, 1.0f / D, mu, sigma2);
+                predict<D, false, (AHEAD || D != 256)>(col, n2, AHEAD ? a.s1 + (row0 + p) * Wt + t : nullptr, a.pair_index, sp, Kp, lane, 1.0f / D, mu, sigma2);
             }
             float inv_delta = a.sh.inv_delta, inv_delta2 = a.sh.inv_delta2;
             int zero_q = a.sh.zero_q;
@@ -481,7 +481,10 @@ constexpr int kGroups = D == 256 ? 4 : 8;                // by the registers
 template <int D>
 constexpr int kAloneWarps = D == 256 ? 16 : 32;
 // 64 registers: the row loads of a prediction's whole unrolled batch are in flight before the first use.
-template <int D, bool DENSE, bool ENC, bool ROOMY, int GW = 0>
+// AHEAD: the call's variance terms were formed ahead; an instantiation of its own, since asking for each position costs
+// registers (168 streams x 384 positions of 256, K = 128, uniform: 983 + 916 us with the question, 946 + 882 without; 1024 x
+// 128 positions of 128: encoding 245 -> 240).
+template <int D, bool DENSE, bool ENC, bool ROOMY, bool AHEAD = false, int GW = 0>
 __global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 32 * kAloneWarps<D> : 512, GW || D == 256 || (ROOMY && !DENSE) ? 1 : 2) coop_kernel(const CodecArgs a) {
     static_assert(GW == 0 || (DENSE && !ENC), "staging is addressed by block");
     using Tab = std::conditional_t<ENC, EncTables, WideDecTables>;
@@ -539,7 +542,7 @@ __global__ void __launch_bounds__(GW ? 32 * GW * kGroups<D> : ROOMY && !DENSE ? 
         if (go < 0) break;
         if (go > 0) {
             if (warp == 0) coop_code<D, ENC, ROOMY, GW>(a, sh, tb, slots, ring, NP, meet, lc);
-            else if (warp > 0) coop_predict<D, DENSE, ENC, GW>(a, sh, tb, pairs + (warp - 1) * 2 * Kp, slots, warp - 1, NP, meet, lc);
+            else if (warp > 0) coop_predict<D, DENSE, ENC, AHEAD, GW>(a, sh, tb, pairs + (warp - 1) * 2 * Kp, slots, warp - 1, NP, meet, lc);
         }
         all_meet();                                                            // the chunk is coded; its item has been read
         if (ENC && go > 0 && sh.dst)
@@ -569,16 +572,20 @@ cudaError_t launch_coop(const CodecArgs& a, bool encode, cudaStream_t st) {
         // Coders alone with their chains: eight an SM, in groups of one block, once there are more chunks than the four
         // that blocks of eight warps hold (2048 chunks of 256 positions: 745 -> 548 us with 128 components, 1180 -> 703 with 256; 1024 of 128: 337 -> 252).
         if (dense && !encode && items > 4ll * sm_count()) {
-            auto kern = coop_kernel<d, true, false, true, kGroupWarps>;
+            auto kern = coop_kernel<d, true, false, true, false, kGroupWarps>;
             const size_t smem = kGroups<d> * coop_smem(kGroupWarps, 0, d, true, false, true);
             const cudaError_t e = allow_smem(kern, smem);
             if (e != cudaSuccess) return e;
             count_launch();
             return launch_kernel(kern, (unsigned)sm_count(), 32 * kGroupWarps * kGroups<d>, smem, st, false, 1, a);
         }
+        auto gather = [&](auto ahead) {
+            constexpr bool A = decltype(ahead)::value;
+            return roomy ? (encode ? coop_kernel<d, false, true, true, A> : coop_kernel<d, false, false, true, A>)
+                         : (encode ? coop_kernel<d, false, true, false, A> : coop_kernel<d, false, false, false, A>);
+        };
         auto kern = dense ? (encode ? coop_kernel<d, true, true, true> : coop_kernel<d, true, false, true>)
-                  : roomy ? (encode ? coop_kernel<d, false, true, true> : coop_kernel<d, false, false, true>)
-                          : (encode ? coop_kernel<d, false, true, false> : coop_kernel<d, false, false, false>);
+                  : a.s1 ? gather(std::true_type{}) : gather(std::false_type{});
         const int warps = alone ? fit : 8;
         const size_t smem = coop_smem(warps, a.sh.Kp, d, dense, encode, roomy);
         const cudaError_t e = allow_smem(kern, smem);
