@@ -146,10 +146,11 @@ typedef struct plc_ctx plc_ctx;
 
 /* Creates a context for one parameter set and one candidate table.
  * T_dev: [L][2][H][V][d] f16, the stand-in for F_M(t_<i, t) of Def. 5 (one d-vector per layer, K/V,
- * head and candidate token); 16-byte aligned; must outlive the context (it is not copied;
+ * head and candidate token); 16-byte aligned; must outlive the context and stay as it is for as long (it is not
+ * copied, but what is read off it at creation is kept: the squared norm of every row, and whether T
+ * holds infinities or NaN, by which plc_encode_rotq / plc_decode_rotq choose their kernel;
  * PLC_PRED_DENSE contexts keep its bf16 transpose while that takes at most a quarter of the memory
- * free at creation, and form a layer's at a time per call otherwise).
- * Synchronises the device once (it pre-computes the squared norm of every row of T).
+ * free at creation, and form a layer's at a time per call otherwise).  Synchronises the device once.
  * Errors: PLC_E_INVALID / PLC_E_SHAPE / PLC_E_ALIGN on bad arguments, PLC_E_CUDA. */
 plc_status plc_create(plc_ctx** out, const plc_config* cfg, const void* T_dev);
 
@@ -158,8 +159,9 @@ plc_status plc_create(plc_ctx** out, const plc_config* cfg, const void* T_dev);
  *     KV^ = c + A * Ebar,   Ebar = sum_v P(v) E(v)   over the whole vocabulary,
  *     sigma_mix^2 = sum_v P(v) ||c + A E(v)||^2 / d - ||KV^||^2 / d          (Thm. 2 with F := c + A E).
  * E_dev [V][d_model], A_dev [L][2][H][d][d_model], c_dev [L][2][H][d], all f16, 16-byte aligned; they
- * must outlive the context (which keeps a bf16 copy of A while that takes at most a quarter of the
- * memory free at creation, and converts a layer at a time per call otherwise).  d_model: a multiple of 64, at most 16384.
+ * must outlive the context and stay as they are for as long (it keeps what it has formed from them, and a bf16 copy of A
+ * while that takes at most a quarter of the memory free at creation; it converts a layer at a time per call otherwise).
+ * d_model: a multiple of 64, at most 16384.
  * Arithmetic: P, E, A and Ebar are rounded to bfloat16 and contracted on the tensor cores with
  * binary32 accumulation; c is added in binary32. */
 typedef struct {
