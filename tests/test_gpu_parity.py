@@ -428,6 +428,37 @@ def test_rotated_quantiser_parity(dev, orc, d, bits, ranges):
 
 @pytest.mark.parametrize("d,K", [(128, 64), (128, 1), (128, 37), (64, 50), (64, 64), (32, 100), (256, 16), (256, 70)])
 def test_rows_widened_by_the_tensor_cores(dev, d, K):
+    """The rotated quantiser's rows go through the tensor cores while T is finite, value by value where it is not:
+    an infinity and a NaN in a row that is never a candidate must not change a bit.  T holds every kind of finite
+    value (both zeros, subnormal, largest); K covers stretches of 16, 8 and 2 rows and what remains."""
+    S, n, L, H, V, bits = 2, 40, 1, 2, 600, 6
+    _, logits, T, kv = make_workload(77 + d + K, S, n, L, H, d, V, K, pp=30.0)
+    rng = np.random.default_rng(d + K)
+    raw = rng.integers(0, 1 << 16, T.numel()).astype(np.uint16)
+    raw[(raw & 0x7c00) == 0x7c00] &= 0x83ff
+    T = torch.from_numpy(raw.view(np.float16)).reshape(T.shape).to(dev)
+    logits[..., V - 1] = -float("inf")
+    kvd, lgd = kv.to(dev), logits.to(dev)
+    got = []
+    for special in (False, True):
+        if special:
+            T = T.clone()
+            T[..., V - 1, 0], T[..., V - 1, 5] = float("inf"), float("nan")
+        ctx = plc.Context(T, K, 0.02)
+        params = ctx.rotq_params(bits, rng.integers(0, 2, d) if not special else neg)
+        neg = [(params.sign_bits[j >> 5] >> (j & 31)) & 1 for j in range(d)]
+        records = torch.zeros(S * ctx.W * n * ctx.rotq_record_bytes(bits), dtype=torch.uint8, device=dev)
+        out = torch.zeros(kv.shape, dtype=torch.float32, device=dev)
+        ctx.encode_rotq(kvd, lgd, params, records)
+        ctx.decode_rotq(records, lgd, params, out)
+        assert ctx.sync_status() == plc.OK
+        got.append((records, out))
+    assert torch.isfinite(got[0][1]).all() and got[0][0].any()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("d,K", [(128, 64), (128, 1), (128, 37), (64, 50), (64, 64), (32, 100), (256, 16), (256, 70)])
+def test_rows_widened_where_tables_are_beyond_l2(dev, d, K):
     """The rotated quantiser's rows go through the tensor cores where the tables are more than L2 holds and T is finite,
     value by value where it is not: an infinity and a NaN in a row that is never a candidate must not change a bit.
     T holds every kind of finite value (both zeros, subnormal, largest); K covers stretches of 16, 8 and 2 rows and
@@ -1028,9 +1059,38 @@ def test_topk_rows_of_every_layout(dev, orc, N, V, K, off):
 
 
 # lengths at the two team sizes' limits, batches that fill a slot and that do not, every alignment; K at its limits
+@pytest.mark.parametrize("N,V,K,off", [(297, 24576, 64, 0), (310, 24577, 128, 3), (1300, 24583, 1, 7), (299, 65536, 100, 0), (600, 65537, 33, 5),
+                                       (300, 128256, 64, 0), (300, 131071, 128, 1)])
+def test_topk_rows_streamed_by_teams(dev, N, V, K, off):
+    """Calls of many long rows against the same rows a hundred at a time (which a block or a cluster selects): the
+    selected and their weights bit for bit, sums in another order (binary32, tolerance of the other layouts).  Rows
+    with ties beyond the lists, with NaN, with fewer finite logits than K and ascending ones among them."""
+    g = torch.Generator(device=dev).manual_seed(N + V)
+    buf = torch.zeros(N * V + 16, dtype=torch.float16, device=dev)
+    rows = buf[off:off + N * V].view(N, V)
+    for i in range(0, N, 100):
+        k = min(100, N - i)
+        rows[i:i + k] = torch.randn(k, V, generator=g, device=dev) * torch.exp(4 * torch.rand(k, 1, generator=g, device=dev) - 1)
+    rows[1] = torch.round(rows[1])
+    rows[2] = torch.sort(rows[2]).values
+    rows[3, ::3] = float("nan")
+    rows[4, 1:] = -float("inf")
+    rows[5] = 1.0
+    rows[N - 1] = torch.round(rows[N - 1] * 4) / 4
+    tok = torch.randint(0, V, (N,), generator=g, device=dev, dtype=torch.int32)
+    ctx = plc.Context(torch.zeros(1, 2, 1, V, 32, dtype=torch.float16, device=dev), K, 0.02)
+    out = ctx.topk_softmax(rows, tok)
+    few = [ctx.topk_softmax(rows[i:i + 100], tok[i:i + 100]) for i in range(0, N, 100)]
+    ref = {k: torch.cat([f[k] for f in few]) for k in out}
+    assert torch.equal(out["idx"], ref["idx"]) and torch.equal(out["w"], ref["w"])
+    for k, tol in (("lse", 2e-5), ("zk", 2e-5), ("logp2", 1e-4)):
+        assert torch.allclose(out[k], ref[k], rtol=2e-5, atol=tol, equal_nan=True), k
+
+
+# lengths at the two team sizes' limits, batches that fill a slot and that do not, every alignment; K at its limits
 @pytest.mark.parametrize("extra,V,K,off", [(1, 24576, 64, 0), (14, 24577, 128, 3), (1004, 24583, 1, 7), (3, 65536, 100, 0), (304, 65537, 33, 5),
                                            (0, 128256, 64, 0), (4, 131071, 128, 1)])
-def test_topk_rows_streamed_by_teams(dev, extra, V, K, off):
+def test_topk_rows_streamed_by_teams_from_two_an_sm(dev, extra, V, K, off):
     """Calls of at least two long rows an SM against the same rows a hundred at a time (which a block or a cluster selects): the
     selected and their weights bit for bit, sums in another order (binary32, tolerance of the other layouts).  Rows
     with ties beyond the lists, with NaN, with fewer finite logits than K and ascending ones among them."""
@@ -1058,6 +1118,29 @@ def test_topk_rows_streamed_by_teams(dev, extra, V, K, off):
 
 
 def test_rows_streamed_by_teams_inside_position_ranges(dev):
+    """A batch whose rows teams stream, with position ranges (one of them empty), against its sessions one by one."""
+    S, n, V, K, d, CP = 5, 90, 24584, 16, 32, 32
+    g = torch.Generator(device=dev).manual_seed(5)
+    T = torch.randn(1, 2, 1, V, d, generator=g, device=dev).half()
+    logits = (torch.randn(S, n, V, generator=g, device=dev) * 3).half()
+    kv = torch.randn(1, 2, S, 1, n, d, generator=g, device=dev).half()
+    ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
+    mc = ctx.max_chunks(n)
+    begin, end = [0, 13, 40, 89, 7], [90, 90, 40, 90, 71]
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+
+    def coded(kv, logits, b, e):
+        st = plc.StreamSet(logits.shape[0] * ctx.W, mc, 1 << 22, dev)
+        ctx.encode(kv, logits, st, i32(b), i32(e))
+        assert ctx.sync_status() == plc.OK
+        return [st.chunk(i).tobytes() for i in range(logits.shape[0] * ctx.W * mc)]
+
+    whole = coded(kv, logits, begin, end)
+    alone = sum((coded(kv[:, :, s:s + 1].contiguous(), logits[s:s + 1].contiguous(), begin[s:s + 1], end[s:s + 1]) for s in range(S)), [])
+    assert whole == alone and any(whole)
+
+
+def test_long_rows_streamed_by_teams_inside_position_ranges(dev):
     """A batch whose rows teams stream (more than 16 an SM, of more than 65536 logits), with position ranges (empty ones
     among them), against its sessions one by one, whose rows blocks or clusters select."""
     S, V, K, d, CP = 9, 65544, 16, 32, 32
@@ -1120,9 +1203,42 @@ def test_coders_in_groups(dev, d, CP, n, kind):
 
 
 # two and four tables a lane, tables beyond one warp's, several positions a warp; K below, at and off the lanes of a warp
+@pytest.mark.parametrize("L,H,d,K,n,ranges", [(1, 1, 32, 17, 9000, False), (3, 1, 64, 64, 2800, True), (4, 4, 32, 100, 520, False), (2, 33, 32, 5, 130, True),
+                                              (1, 8, 128, 64, 1100, False), (1, 4, 256, 33, 2100, True)])
+def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
+    """A batch large enough for its variance terms to be formed ahead gives the same bytes as its sessions one by
+    one, in pieces too small for it."""
+    S, V, CP = 4, 500, 50
+    _, logits, T, kv = make_workload(31 + d + K, S, n, L, H, d, V, K, pp=20.0)
+    T, logits, kv = T.to(dev), logits.to(dev), kv.to(dev)
+    ctx = plc.Context(T, K, 0.02, chunk_pos=CP)
+    assert 4 * S * n * ctx.W >= 256 * 1024
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=dev)
+    begin, end = ([0, n // 3, 7, n // 2], [n, n, n // 2, n // 2]) if ranges else ([0] * S, [n] * S)
+
+    def coded(kv, logits, b, e):
+        mc = ctx.max_chunks(logits.shape[1])
+        st = plc.StreamSet(logits.shape[0] * ctx.W, mc, 4 * logits.shape[0] * logits.shape[1] * ctx.W * d + (1 << 20), dev)
+        ctx.encode(kv, logits, st, i32(b), i32(e))
+        assert ctx.sync_status() == plc.OK
+        return [[st.chunk(i * mc + c).tobytes() for c in range(mc)] for i in range(logits.shape[0] * ctx.W)]
+
+    whole = coded(kv, logits, begin, end)
+    step = max(CP, 28000 // ctx.W // CP * CP)                        # positions of a piece: whole chunks, fewer than 65536 vectors
+    for s in range(S):
+        alone = [[] for _ in range(ctx.W)]
+        for p in range(begin[s], end[s], step):
+            q = min(p + step, end[s])
+            for t, chunks in enumerate(coded(kv[:, :, s:s + 1, :, p:q].contiguous(), logits[s:s + 1, p:q].contiguous(), [0], [q - p])):
+                alone[t] += chunks
+        for t in range(ctx.W):
+            assert [c for c in whole[s * ctx.W + t] if c] == alone[t]
+
+
+# two and four tables a lane, tables beyond one warp's, several positions a warp; K below, at and off the lanes of a warp
 @pytest.mark.parametrize("L,H,d,K,n,ranges", [(3, 3, 32, 17, 1900, False), (5, 3, 64, 64, 1150, True), (4, 4, 32, 100, 1050, False), (2, 33, 32, 5, 260, True),
                                               (1, 8, 128, 64, 2100, False), (2, 4, 256, 33, 2100, True)])
-def test_variance_terms_formed_ahead(dev, L, H, d, K, n, ranges):
+def test_variance_terms_formed_ahead_from_their_limits(dev, L, H, d, K, n, ranges):
     """A batch large enough for its variance terms to be formed ahead gives the same bytes as its sessions one by
     one, in pieces too small for it."""
     S, V, CP = 4, 500, 50
@@ -1192,8 +1308,7 @@ def test_scratch_of_the_terms_formed_ahead(dev):
         assert streams[0].chunk(s).tobytes() == streams[1].chunk(s).tobytes() == streams[2].chunk(s).tobytes()
 
 
-@pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False),
-                                             (64, 200, 500, 1, True), (32, 426, 600, 1, False), (32, 429, 600, 1, False), (64, 1000, 1100, 1, False)])
+@pytest.mark.parametrize("d,K,V,CP,ranges", [(128, 64, 2000, 1, False), (64, 50, 777, 2, True), (32, 128, 300, 1, False), (256, 21, 500, 2, False)])
 def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges):
     """4800 short chunks: more than a warp each on the whole GPU, so the kernels that give a chunk to a warp run
     (fewer chunks get a block each); candidate counts that leave remainders of the gather's stretches."""
@@ -1204,6 +1319,12 @@ def test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, rang
     assert g["rc"] == plc.OK and g["W"] * S * g["mc"] > 32 * torch.cuda.get_device_properties(dev).multi_processor_count
     check_against_oracle(orc, g, T, kv, logits, K, 0.02, CP, pb, pe)
     gpu_decode_check(g, kv, 0.02, n, pb, pe)
+
+
+@pytest.mark.parametrize("d,K,V,CP,ranges", [(64, 200, 500, 1, True), (32, 426, 600, 1, False), (32, 429, 600, 1, False), (64, 1000, 1100, 1, False)])
+def test_many_chunks_with_many_candidates(dev, orc, d, K, V, CP, ranges):
+    """The same with candidate counts up to and beyond what the pairs of 24 warps beside each other take (K = 426)."""
+    test_many_chunks_take_the_warp_per_chunk_kernels(dev, orc, d, K, V, CP, ranges)
 
 
 @pytest.mark.parametrize("K,ranges", [(200, False), (320, True), (321, False), (1000, True)])
