@@ -56,7 +56,7 @@ def parse_over(pairs):
 
 
 # Issue-slot use of the fused kernels (smsp__issue_active) from an ncu capture; quoted beside the roofline fraction, not part of it.
-NCU_ISSUE_SLOT_USE = {"encode_kernel": 0.684, "decode_kernel": 0.654}
+NCU_ISSUE_SLOT_USE = {"encode_kernel": 0.727, "decode_kernel": 0.722}
 
 
 def fused_roofline(vecs, K, d, t_bytes, kv_bytes, payload, ek, dk, sm_mhz, sms, peak, peak_kind, traffic_per_vector=None):
@@ -83,8 +83,8 @@ def fused_roofline(vecs, K, d, t_bytes, kv_bytes, payload, ek, dk, sm_mhz, sms, 
          "fp32_fma": {"achieved": flop_ach, "peak": flop_peak, "unit": "TFLOP/s", "frac": alu_frac,
                       "peak_kind": "SMs x 128 lanes x 2 flop x sampled SM clock (%d x %.0f MHz)" % (sms, sm_mhz)},
          "issue_slot_use_ncu": NCU_ISSUE_SLOT_USE.get(name),
-         "busiest_units_ncu": "issue slots 65-68 % (ncu capture); heavy half of the FMA pipe and L1 data pipe level behind "
-                              "them (capture of an earlier form): no single unit saturated",
+         "busiest_units_ncu": "issue slots 72-73 %, heavy half of the FMA pipe 67 / 65 %, L1 data pipe 60 / 62 % (ncu capture, "
+                              "encode / decode): no single unit saturated",
          "gathered_row_bytes_frac": bytes_ns / sec / 1e9 / peak,
          "gathered_row_note": "KV + K*d*2 B of gathered rows per vector + bitstream over the HBM copy peak; the rows are "
                            "L1 / L2 hits, so this is an on-chip gather rate, not an HBM utilisation",
@@ -136,10 +136,10 @@ class ClockSampler:
                 "power_w_max": max(power) if power else None, "samples": len(sm), "reasons": sorted(reasons)}
 
 
-# DRAM bytes per vector of the fused kernels, from the ncu capture summarised in
-# profiles/gather_and_topk_after_rework.md (dram__bytes_read.sum + dram__bytes_write.sum over 4.19 M vectors;
-# traffic grows in proportion to the vectors).  Valid for the default workload and chunk size only.
-NCU_DRAM_BYTES_PER_VECTOR = {"encode_kernel": 664.9, "decode_kernel": 423.5}
+# DRAM bytes per vector of the fused kernels and the launch that forms their variance terms (2.2 of them), from the ncu
+# capture summarised in profiles/gather_one_block_and_variance.md (dram__bytes_read.sum + dram__bytes_write.sum over 4.19 M
+# vectors; traffic grows in proportion to the vectors).  Valid for the default workload and chunk size only.
+NCU_DRAM_BYTES_PER_VECTOR = {"encode_kernel": 655.7, "decode_kernel": 418.4}
 NCU_TRAFFIC_NOTE = ("dram__bytes_read + dram__bytes_write of a 4-layer ncu capture "
                     "scaled by the vectors of a launch")
 
